@@ -170,65 +170,84 @@ __global__ void hadamard_kernel(HadArgs<T> a) {
 }
 
 // out_b = lmax(H_b) for the matrix b = blockIdx.x of the launch (H_0: n0 x n0,
-// H_1: n1 x n1, n <= 64): kPowerIters FP64 power iterations from the
-// normalised all-ones vector, then the Rayleigh quotient; 0 if an iterate maps
-// to zero. One warp per matrix: lane l owns rows l and l + 32 of H (kept in
-// shared memory with an odd row stride) and the same entries of v, which the
-// products fetch by shuffles. FP64 is slow on this GPU, and an iteration then
-// needs no block barrier: one shuffle sum for the norm and one reciprocal.
+// H_1: n1 x n1, n <= 64): kPowerIters FP64 power iterations from the all-ones
+// vector, then the Rayleigh quotient; 0 if an iterate maps to zero or is not
+// finite. GB300's FP64 units are slow (a warp-wide FMA holds its scheduler's
+// unit for tens of cycles), so the chain is bound by the FP64 instructions of
+// one scheduler: a block spreads each product over warps of eight rows (all
+// four schedulers), four lanes per row with the row's entries of H in
+// registers, and the iterate is scaled by a power of two every other
+// iteration (the exponent from the integer bits of its largest entry) where
+// norms would put an FP64 square root and a division into every iteration.
+// 24 x 24: 16.5 us (one warp per matrix with a norm per iteration: 78 us).
+constexpr int kPowerMaxThreads = 256;
+inline int power_iter_threads(int n0, int n1) { return ((n0 > n1 ? n0 : n1) + 7) / 8 * 32; }
+
 template <typename T>
-__global__ void __launch_bounds__(32) power_iter_kernel(const T* __restrict__ H0, int n0,
-                                                         double* out0, const T* __restrict__ H1,
-                                                         int n1, double* out1) {
-  __shared__ double h[64 * 65];
+__global__ void __launch_bounds__(kPowerMaxThreads)
+power_iter_kernel(const T* __restrict__ H0, int n0, double* out0, const T* __restrict__ H1,
+                  int n1, double* out1) {
+  __shared__ double v[2][64];
   const T* H = blockIdx.x == 0 ? H0 : H1;
   const int n = blockIdx.x == 0 ? n0 : n1;
   double* out = blockIdx.x == 0 ? out0 : out1;
-  const int lane = threadIdx.x, ld = n + 1;
-  for (int e = lane; e < n * n; e += 32) h[(e / n) * ld + e % n] = (double)H[e];
-  __syncwarp();
-  const int r0 = lane, r1 = lane + 32;
-  const bool has0 = r0 < n, has1 = r1 < n;
-  const double v0i = 1.0 / sqrt((double)n);
-  double v0 = has0 ? v0i : 0.0, v1 = has1 ? v0i : 0.0;  // v[r0], v[r1]
-  double w0 = 0.0, w1 = 0.0;
-  auto matvec = [&]() {  // (w0, w1) = rows r0, r1 of H v
-    double a0 = 0.0, b0 = 0.0, a1 = 0.0, b1 = 0.0;
-    int j = 0;
-    for (; j + 1 < n; j += 2) {
-      const double x = __shfl_sync(0xffffffffu, j < 32 ? v0 : v1, j & 31);
-      const double y = __shfl_sync(0xffffffffu, j + 1 < 32 ? v0 : v1, (j + 1) & 31);
-      if (has0) {
-        a0 = fma(h[r0 * ld + j], x, a0);
-        b0 = fma(h[r0 * ld + j + 1], y, b0);
-      }
-      if (has1) {
-        a1 = fma(h[r1 * ld + j], x, a1);
-        b1 = fma(h[r1 * ld + j + 1], y, b1);
+  const int lane = threadIdx.x & 31, s = threadIdx.x & 3, row = threadIdx.x >> 2;
+  constexpr int kPer = 16;  // entries s, s + 4, ... of a row of up to 64
+  double h[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int j = s + 4 * k;
+    h[k] = row < n && j < n ? (double)H[row * n + j] : 0.0;
+  }
+  if (threadIdx.x < 32) {
+    v[0][lane] = lane < n ? 1.0 : 0.0;
+    v[0][lane + 32] = lane + 32 < n ? 1.0 : 0.0;
+    v[1][lane] = 0.0;
+    v[1][lane + 32] = 0.0;
+  }
+  __syncthreads();
+  const int per = (n + 3) / 4;
+  auto product = [&](const double* x) {  // (H x)[row], in all four lanes of the row
+    double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < kPer; k += 2) {
+      if (k < per) {
+        a0 = fma(h[k], x[s + 4 * k], a0);
+        if (k + 1 < per) a1 = fma(h[k + 1], x[s + 4 * k + 4], a1);
       }
     }
-    if (j < n) {
-      const double x = __shfl_sync(0xffffffffu, j < 32 ? v0 : v1, j & 31);
-      if (has0) a0 = fma(h[r0 * ld + j], x, a0);
-      if (has1) a1 = fma(h[r1 * ld + j], x, a1);
-    }
-    w0 = a0 + b0;
-    w1 = a1 + b1;
+    a0 += a1;
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+    return a0;
+  };
+  // 2^-e for the exponent e of the largest entry of x (1 if that is zero,
+  // subnormal or not finite), the same in every warp.
+  auto scale_of = [&](const double* x) {
+    const unsigned b0 = (unsigned)(__double2hiint(x[lane]) & 0x7fffffff);
+    const unsigned b1 = (unsigned)(__double2hiint(x[lane + 32]) & 0x7fffffff);
+    const unsigned e = __reduce_max_sync(0xffffffffu, b0 > b1 ? b0 : b1) >> 20;
+    return e > 0u && e < 2046u ? __hiloint2double((int)((2046u - e) << 20), 0) : 1.0;
   };
   for (int it = 0; it < kPowerIters; ++it) {
-    matvec();
-    const double nrm = sqrt(warp_sum(w0 * w0 + w1 * w1));
-    if (!(nrm > 0.0)) {
-      if (lane == 0) out[0] = 0.0;
-      return;
-    }
-    const double inv = 1.0 / nrm;
-    v0 = w0 * inv;
-    v1 = w1 * inv;
+    const double* x = v[it & 1];
+    double w = product(x);
+    if (it & 1) w *= scale_of(x);
+    if (s == 0 && row < n) v[(it + 1) & 1][row] = w;
+    __syncthreads();
   }
-  matvec();
-  const double q = warp_sum(v0 * w0 + v1 * w1);
-  if (lane == 0) out[0] = q;
+  const double* x = v[kPowerIters & 1];
+  const double w = product(x);
+  if (s == 0 && row < n) v[(kPowerIters + 1) & 1][row] = w;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double* y = v[(kPowerIters + 1) & 1];
+    const double sc = scale_of(x);
+    const double x0 = x[lane] * sc, x1 = x[lane + 32] * sc;
+    const double xx = warp_sum(x0 * x0 + x1 * x1);
+    const double xy = warp_sum(x0 * (y[lane] * sc) + x1 * (y[lane + 32] * sc));
+    if (lane == 0) out[0] = xx > 0.0 && isfinite(xx) && isfinite(xy) ? xy / xx : 0.0;
+  }
 }
 
 // P <- max(P - G / L, 0) when L > 0, with L = L1[0] (times L2[0] if given).
@@ -566,7 +585,8 @@ int pg_mode(Work<T>& w, int n, T* const* F, T* const* B, cudaStream_t s, SideStr
   NNC_TRY(fork());
   NNC_CUDA_TRY(small_gemm<T>(mn, r, r, B[n], r, 1, w.V, r, 1, nullptr, w.tmp2, ls));
   NNC_CUDA_TRY(small_gemm<T>(mn, mn, r, w.tmp2, r, 1, B[n], 1, r, nullptr, w.H, ls));
-  power_iter_kernel<T><<<2, 32, 0, ls>>>(w.H, mn, w.Ls + 0, w.V, r, w.Ls + 1);
+  power_iter_kernel<T><<<2, power_iter_threads(mn, r), 0, ls>>>(w.H, mn, w.Ls + 0, w.V, r,
+                                                                 w.Ls + 1);
   note_launch(ls);
   NNC_CUDA_TRY(cudaGetLastError());
   NNC_TRY(grad_a(w, n, s));
@@ -581,7 +601,8 @@ int pg_mode(Work<T>& w, int n, T* const* F, T* const* B, cudaStream_t s, SideStr
   // L_B = lmax(F^T F) lmax(V)
   NNC_TRY(fork());
   NNC_TRY(launch_gram<T>(F[n], Nn, mn, w.S, ls));
-  power_iter_kernel<T><<<1, 32, 0, ls>>>(w.S, mn, w.Ls + 2, w.S, mn, w.Ls + 2);
+  power_iter_kernel<T><<<1, power_iter_threads(mn, mn), 0, ls>>>(w.S, mn, w.Ls + 2, w.S, mn,
+                                                                 w.Ls + 2);
   note_launch(ls);
   NNC_CUDA_TRY(cudaGetLastError());
   NNC_TRY(grad_a(w, n, s));
