@@ -324,14 +324,15 @@ __device__ void pass_cols(const T* __restrict__ X, int N1, int C, const T* F, in
 }
 
 // sum (X - X_hat)^2 and sum X^2 in FP64 with X_hat[r, k] = sum_c U[r, c] W[k, c]
-// (X viewed R x N3 in global memory, U: R x K and W: N3 x K in shared memory).
+// (X viewed R x N3 in global memory, U: R x K and W: N3 x K, rows wp apart, in
+// shared memory).
 template <typename T>
 __device__ void stream_residual(const T* __restrict__ X, int R, int N3, const T* U, const T* W,
-                                int K, double* red, double* out2) {
+                                int K, int wp, double* red, double* out2) {
   const double2 r2 = fixed_sums2((int64_t)R * N3, [&](int64_t e) {
     const int r = (int)(e / N3), k = (int)(e - (int64_t)r * N3);
     T h = T(0);
-    for (int c = 0; c < K; ++c) h = fma(U[r * K + c], W[k * K + c], h);
+    for (int c = 0; c < K; ++c) h = fma(U[r * K + c], W[k * wp + c], h);
     const double xv = (double)__ldg(X + e), dv = xv - (double)h;
     return make_double2(dv * dv, xv * xv);
   }, red);
@@ -372,6 +373,8 @@ size_t ntd_l2_elems(const ntd_small_job& j) {
   return f + s + (size_t)z.p + z.y + 2 * (size_t)z.nm + z.mm + 4 * (size_t)z.ng;
 }
 
+// (ntd_blk_kernel below takes the jobs it fits; this one those whose T = X x_2
+// F2^T would not fit where P3 does, N2 far below N1 and N3.)
 // nnTD of one job per block with X in global memory: the sweep of ntd_fit,
 // F^(1), F^(2), F^(3) by MU (Num_n from the pass results, H_n from the core
 // and the Grams), then G with M = Y3 x_3 F^(3)T and D = (G x_1 S1 x_2 S2) x_3
@@ -453,10 +456,464 @@ ntd_l2_kernel(const ntd_small_job* __restrict__ jobs, int iters, T eps, double* 
   const int dg[3] = {m[0], m[1], m[2]};
   mp3(G, dg, 0, F[0], m[0], 1, N[0], Y);
   mp3(Y, y1, 1, F[1], m[1], 1, N[1], P);
-  stream_residual(X, N[0] * N[1], N[2], P, F[2], m[2], red, nrm);
+  stream_residual(X, N[0] * N[1], N[2], P, F[2], m[2], m[2], red, nrm);
   if (threadIdx.x == 0 && rel_errs) rel_errs[blockIdx.x] = sqrt(nrm[0] / nrm[1]);
   for (int k = 0; k < 3; ++k) store(static_cast<T*>(jb.F[k]), F[k], N[k] * m[k]);
   store(static_cast<T*>(jb.G), G, z.ng);
+}
+
+// ---- nnTD of one job per block, two column passes over X ---------------------
+//
+// One thread block per problem: X in global memory (with several blocks per SM
+// in flight, their tensors stay in L2, small ones in L1); factors, core, Grams and pass
+// results in shared memory. A sweep reads X twice, each time
+// along an axis whose neighbours are contiguous (16-byte loads, VL entries a
+// thread, when N3 and X allow it):
+//   T  = X x_2 F2^T   (N1, m2, N3)   mode 1: Y1 = T x_3 F3^T
+//   P1 = X x_1 F1^T   (m1, N2, N3)   mode 2: Y2 = P1 x_3 F3^T, mode 3 and the
+//                                    core: Y3 = P1 x_2 F2^T (new F1, new F2)
+// so no thread walks a row of X. What bounds the sweep is the latency of its
+// small contractions, so everything that does not depend on each other shares an
+// interval between two barriers (15 of them; a barrier after every contraction
+// took 27) and the block is small enough for several per SM. Against the row pass
+// (ntd_l2_kernel: 32 rows a load, L1 63 % busy on 128 registers) and, for an X
+// in shared memory, ntd_small_kernel (four passes over X):
+//   1000 x 40^3, m (3, 4, 5), FP32, 100 sweeps       29.0 -> 9.3 ms
+//   200 x 24^3, m (12, 10, 8), FP32, 40 sweeps        8.9 -> 2.5 ms
+//   200 x 40^3, m (3, 4, 5), FP64, 20 sweeps         13.0 -> 7.1 ms
+//   1000 x 4^3, m (3, 3, 3), FP64, 400 sweeps         8.8 -> 7.9 ms
+//
+// Factor rows are padded with zeros to pitch fpitch(m) and read in 16-byte
+// pieces; the rows of T and P1 to a pitch that keeps the row reads of Y1 and Y2
+// free of bank conflicts. No sum depends on the block size, so a fit may be
+// split over launches of different ones.
+constexpr int kBlkMaxM = 16;
+__host__ __device__ inline int fpitch(int m) { return m <= 4 ? 4 : (m <= 8 ? 8 : 16); }
+// Row pitch of T and P1 for N3 columns: 16-byte reads of eight consecutive rows
+// fall on distinct banks (even 16-byte rows), single reads of 32 rows (odd).
+template <typename T>
+__host__ __device__ inline int rpitch(int n3) {
+  constexpr int VL = 16 / (int)sizeof(T);
+  if (n3 % VL) return n3 | 1;
+  const int v = n3 / VL;
+  return (v | 1) * VL;
+}
+
+struct NtdBlkSizes {
+  int f, g, s, y, p, nm, mm, u, total;
+};
+template <typename T>
+__host__ __device__ inline NtdBlkSizes ntd_blk_sizes(const int* N, const int* m) {
+  NtdBlkSizes z;
+  const int cp = rpitch<T>(N[2]);
+  z.f = z.s = z.nm = z.mm = 0;
+  for (int k = 0; k < 3; ++k) {
+    const int nf = N[k] * fpitch(m[k]);
+    z.f += nf;
+    z.nm = nf > z.nm ? nf : z.nm;
+    z.s += (m[k] * m[k] + 3) & ~3;
+    z.mm = m[k] * m[k] > z.mm ? m[k] * m[k] : z.mm;
+  }
+  z.mm = (z.mm + 3) & ~3;
+  z.g = (m[0] * m[1] * m[2] + 3) & ~3;
+  const int y1 = N[0] * m[1] * m[2], y2 = m[0] * N[1] * m[2], y3 = m[0] * m[1] * N[2];
+  z.y = y1 > y2 ? (y1 > y3 ? y1 : y3) : (y2 > y3 ? y2 : y3);
+  z.y = (z.y + 3) & ~3;
+  const int pa = N[0] * m[1] * cp, pb = m[0] * N[1] * cp;
+  z.p = ((pa > pb ? pa : pb) + 3) & ~3;
+  // U = G x_1 F1 x_2 F2 of the final residual overlays everything from P on.
+  z.u = N[0] * N[1] * m[2];
+  const int tail = z.p + z.nm + z.mm + 3 * z.g;
+  z.total = 2 * z.f + z.g + z.s + z.y + (tail > z.u ? tail : z.u);
+  return z;
+}
+
+template <typename T>
+__device__ __forceinline__ void ld4s(const T* p, T (&w)[4]) {
+  if constexpr (sizeof(T) == 4) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+  } else {
+    const double2 a = *reinterpret_cast<const double2*>(p);
+    const double2 b = *reinterpret_cast<const double2*>(p + 2);
+    w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y;
+  }
+}
+template <typename T, int VL>
+__device__ __forceinline__ void ldv(const T* p, T (&v)[VL]) {
+  if constexpr (VL == 4) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  } else if constexpr (VL == 2) {
+    const double2 t = *reinterpret_cast<const double2*>(p);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+    v[0] = *p;
+  }
+}
+template <typename T, int VL>
+__device__ __forceinline__ void ldg_v(const T* p, T (&v)[VL]) {
+  if constexpr (VL == 4) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  } else if constexpr (VL == 2) {
+    const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+    v[0] = t.x; v[1] = t.y;
+  } else {
+    v[0] = __ldg(p);
+  }
+}
+template <typename T, int VL>
+__device__ __forceinline__ void stv(T* p, const T (&v)[VL]) {
+  if constexpr (VL == 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  else if constexpr (VL == 2) *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+  else *p = v[0];
+}
+
+// out[l, p, c] = sum_j F[j, p] X[l, j, c], p < Q (F: J x QP in shared memory,
+// zero past Q), j in order, VL consecutive c per thread. Column c = (j', k) of
+// N3 entries per row k goes to out[((l Q + p) C / N3 + j') cp + k].
+template <typename T, int QP, int VL>
+__device__ __forceinline__ void col_pass_impl(const T* __restrict__ X, int L, int J, int C, int N3,
+                                              int cp, const T* F, int Q, T* out) {
+  const int cv = C / VL, rows = C / N3;
+  for (int t = threadIdx.x; t < L * cv; t += blockDim.x) {
+    const int l = t / cv, c = (t - l * cv) * VL;
+    const T* x = X + (int64_t)l * J * C + c;
+    T acc[QP][VL];
+#pragma unroll
+    for (int p = 0; p < QP; ++p)
+#pragma unroll
+      for (int u = 0; u < VL; ++u) acc[p][u] = T(0);
+    constexpr int U = VL == 4 ? 4 : 8;  // loads in flight
+    int j = 0;
+    for (; j + U <= J; j += U) {
+      T v[U][VL];
+#pragma unroll
+      for (int q = 0; q < U; ++q) ldg_v<T, VL>(x + (int64_t)(j + q) * C, v[q]);
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+#pragma unroll
+        for (int p = 0; p < QP; p += 4) {
+          T w[4];
+          ld4s(F + (j + q) * QP + p, w);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int u = 0; u < VL; ++u) acc[p + e][u] = fma(v[q][u], w[e], acc[p + e][u]);
+        }
+    }
+    for (; j < J; ++j) {
+      T v[VL];
+      ldg_v<T, VL>(x + (int64_t)j * C, v);
+#pragma unroll
+      for (int p = 0; p < QP; p += 4) {
+        T w[4];
+        ld4s(F + j * QP + p, w);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+          for (int u = 0; u < VL; ++u) acc[p + e][u] = fma(v[u], w[e], acc[p + e][u]);
+      }
+    }
+    const int jr = c / N3, k = c - jr * N3;
+    T* o = out + ((int64_t)l * Q * rows + jr) * cp + k;
+#pragma unroll
+    for (int p = 0; p < QP; ++p)
+      if (p < Q) stv<T, VL>(o + (int64_t)p * rows * cp, acc[p]);
+  }
+}
+
+template <typename T, int QM>
+__device__ void col_pass(const T* __restrict__ X, int L, int J, int C, int N3, int cp, const T* F,
+                         int Q, bool vec, T* out) {
+  constexpr int VL = 16 / (int)sizeof(T);
+  if (Q <= 4) {
+    if (vec) col_pass_impl<T, 4, VL>(X, L, J, C, N3, cp, F, Q, out);
+    else col_pass_impl<T, 4, 1>(X, L, J, C, N3, cp, F, Q, out);
+  } else if (Q <= 8) {
+    if (vec) col_pass_impl<T, 8, VL>(X, L, J, C, N3, cp, F, Q, out);
+    else col_pass_impl<T, 8, 1>(X, L, J, C, N3, cp, F, Q, out);
+  } else if constexpr (QM > 8) {
+    if (vec) col_pass_impl<T, 16, VL>(X, L, J, C, N3, cp, F, Q, out);
+    else col_pass_impl<T, 16, 1>(X, L, J, C, N3, cp, F, Q, out);
+  }
+}
+
+// Y[row, q] = sum_k P[row cp + k] F[k, q], rows < R, q < Q, k < K in order (F:
+// K x QP, zero past Q): one thread per row, all q.
+template <typename T, int QP>
+__device__ __forceinline__ void row_dots_impl(const T* P, int R, int cp, int K, const T* F, int Q,
+                                              T* Y) {
+  constexpr int VL = 16 / (int)sizeof(T);
+  for (int r = threadIdx.x; r < R; r += blockDim.x) {
+    T acc[QP];
+#pragma unroll
+    for (int q = 0; q < QP; ++q) acc[q] = T(0);
+    const T* x = P + r * cp;
+    auto add = [&](T v, const T* f) {
+#pragma unroll
+      for (int q = 0; q < QP; q += 4) {
+        T w[4];
+        ld4s(f + q, w);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[q + e] = fma(v, w[e], acc[q + e]);
+      }
+    };
+    int k = 0;
+    if (K % VL == 0) {  // cp is then a multiple of VL too
+      for (; k < K; k += VL) {
+        T v[VL];
+        ldv<T, VL>(x + k, v);
+#pragma unroll
+        for (int u = 0; u < VL; ++u) add(v[u], F + (k + u) * QP);
+      }
+    } else {
+#pragma unroll 4
+      for (; k < K; ++k) add(x[k], F + k * QP);
+    }
+#pragma unroll
+    for (int q = 0; q < QP; ++q)
+      if (q < Q) Y[r * Q + q] = acc[q];
+  }
+}
+template <typename T, int QM>
+__device__ void row_dots(const T* P, int R, int cp, int K, const T* F, int Q, T* Y) {
+  if (Q <= 4) row_dots_impl<T, 4>(P, R, cp, K, F, Q, Y);
+  else if (Q <= 8) row_dots_impl<T, 8>(P, R, cp, K, F, Q, Y);
+  else if constexpr (QM > 8) row_dots_impl<T, 16>(P, R, cp, K, F, Q, Y);
+}
+
+// S = F^T F (m x m; F: N rows of pitch fp): four lanes per entry, lane u adding
+// the rows u, u + 4, ... in order, the four sums by a fixed shuffle tree.
+template <typename T>
+__device__ void gram4(const T* F, int N, int fp, int m, T* S) {
+  const int u = threadIdx.x & 3;
+  for (int e0 = 0; e0 < m * m; e0 += blockDim.x / 4) {
+    const int e = e0 + (int)threadIdx.x / 4;
+    T s = T(0);
+    if (e < m * m) {
+      const int a = e / m, b = e - a * m;
+      for (int i = u; i < N; i += 4) s = fma(F[i * fp + a], F[i * fp + b], s);
+    }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if (e < m * m && u == 0) S[e] = s;
+  }
+}
+
+// out[l, p, c] = sum_j A[p, j] in[l, j, c] for a symmetric A (J x J), all in
+// shared memory (a core times a Gram along one mode).
+template <typename T>
+__device__ void core_gram(const T* in, int L, int J, int C, const T* A, T* out) {
+  for (int e = threadIdx.x; e < L * J * C; e += blockDim.x) {
+    const int c = e % C, lp = e / C, p = lp % J, l = lp / J;
+    const T* x = in + l * J * C + c;
+    T s = T(0);
+    for (int j = 0; j < J; ++j) s = fma(A[p * J + j], x[j * C], s);
+    out[e] = s;
+  }
+}
+
+// out[i, a] = sum over l, c of Y[l, i, c] G[l, a, c] (out: row pitch op).
+template <typename T>
+__device__ void unfold_dots(const T* Y, const T* G, int L, int NI, int MA, int C, int op, T* out) {
+  for (int e = threadIdx.x; e < NI * MA; e += blockDim.x) {
+    const int i = e / MA, a = e - i * MA;
+    T s = T(0);
+    for (int l = 0; l < L; ++l) {
+      const T* y = Y + (l * NI + i) * C;
+      const T* g = G + (l * MA + a) * C;
+      for (int c = 0; c < C; ++c) s = fma(y[c], g[c], s);
+    }
+    out[i * op + a] = s;
+  }
+}
+
+// The MU step of a factor: Fn[i, a] from the old F, the numerators (pitch fp) and
+// den = F H; Fn is another buffer, so every row of the old F stays readable.
+template <typename T>
+__device__ void mu_factor(const T* F, const T* num, const T* H, int N, int fp, int m, T eps,
+                          T* Fn) {
+  for (int e = threadIdx.x; e < N * m; e += blockDim.x) {
+    const int i = e / m, a = e - i * m;
+    const T* f = F + i * fp;
+    T den = T(0);
+    for (int w = 0; w < m; ++w) den = fma(f[w], H[w * m + a], den);
+    const T v = f[a] * num[i * fp + a] / (den > eps ? den : eps);
+    Fn[i * fp + a] = v > T(0) ? v : T(0);
+  }
+}
+
+template <typename T>
+int64_t ntd_blk_elems(const ntd_small_job& j) {
+  // The kernel's 32-bit sizes are formed only for jobs near a block's size.
+  for (int k = 0; k < 3; ++k)
+    if (j.dims[k] > 1 << 20) return 1LL << 40;
+  const int64_t N1 = j.dims[0], N2 = j.dims[1], N3 = j.dims[2] + 8LL;
+  const int64_t m1 = j.m[0], m2 = j.m[1], m3 = j.m[2];
+  const int64_t top = (N1 + N2 + N3) * kBlkMaxM + N1 * m2 * N3 + m1 * N2 * N3 + N1 * N2 * m3 +
+                      N1 * m2 * m3 + m1 * N2 * m3 + m1 * m2 * N3;
+  if (top > 1LL << 24) return top;
+  return ntd_blk_sizes<T>(j.dims, j.m).total;
+}
+
+template <typename T, int QM>
+__global__ void __launch_bounds__(kThreads, QM > 8 ? 2 : 3)
+ntd_blk_kernel(const ntd_small_job* __restrict__ jobs, int iters, T eps, double* rel_errs) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double red[2 * kFixedLanes];
+  __shared__ double nrm[2];
+  constexpr int VL = 16 / (int)sizeof(T);
+  const ntd_small_job& jb = jobs[blockIdx.x];
+  const int N1 = jb.dims[0], N2 = jb.dims[1], N3 = jb.dims[2];
+  const int m1 = jb.m[0], m2 = jb.m[1], m3 = jb.m[2];
+  const NtdBlkSizes z = ntd_blk_sizes<T>(jb.dims, jb.m);
+  const int p1 = fpitch(m1), p2 = fpitch(m2), p3 = fpitch(m3), cp = rpitch<T>(N3);
+  const int ng = m1 * m2 * m3;
+  // Every factor twice: a MU step writes the copy its old rows are not in.
+  T* F1 = reinterpret_cast<T*>(smem_raw);
+  T* F2 = F1 + N1 * p1;
+  T* F3 = F2 + N2 * p2;
+  T* F1n = F1 + z.f;
+  T* F2n = F2 + z.f;
+  T* F3n = F3 + z.f;
+  T* G = F1 + 2 * z.f;
+  T* S1 = G + z.g;
+  T* S2 = S1 + ((m1 * m1 + 3) & ~3);
+  T* S3 = S2 + ((m2 * m2 + 3) & ~3);
+  T* Y = S1 + z.s;
+  T* P = Y + z.y;
+  T* num = P + z.p;
+  T* H = num + z.nm;
+  T* W = H + z.mm;
+  T* W2 = W + z.g;
+  T* M = W2 + z.g;
+  const T* X = static_cast<const T*>(jb.X);
+  const bool vec = N3 % VL == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  auto load_factor = [&](T* F, T* other, const void* src, int N, int fp, int m) {
+    const T* f = static_cast<const T*>(src);
+    for (int e = threadIdx.x; e < N * fp; e += blockDim.x) {
+      const int i = e / fp, a = e - i * fp;
+      F[e] = a < m ? f[i * m + a] : T(0);
+      other[e] = T(0);
+    }
+  };
+  load_factor(F1, F1n, jb.F[0], N1, p1, m1);
+  load_factor(F2, F2n, jb.F[1], N2, p2, m2);
+  load_factor(F3, F3n, jb.F[2], N3, p3, m3);
+  load(G, static_cast<const T*>(jb.G), ng);
+  __syncthreads();
+  gram4(F1, N1, p1, m1, S1);
+  gram4(F2, N2, p2, m2, S2);
+  gram4(F3, N3, p3, m3, S3);
+  __syncthreads();
+  auto swap = [](T*& a, T*& b) {
+    T* t = a;
+    a = b;
+    b = t;
+  };
+
+  for (int it = 0; it < iters; ++it) {
+    // ---- mode 1
+    core_gram(G, m1, m2, m3, S2, W);
+    col_pass<T, QM>(X, N1, N2, N3, N3, cp, F2, m2, vec, P);  // T (N1, m2, N3)
+    __syncthreads();
+    core_gram(W, m1 * m2, m3, 1, S3, W2);
+    row_dots<T, QM>(P, N1 * m2, cp, N3, F3, m3, Y);  // Y1 (N1, m2, m3)
+    __syncthreads();
+    unfold_dots(W2, G, 1, m1, m1, m2 * m3, m1, H);
+    unfold_dots(Y, G, 1, N1, m1, m2 * m3, p1, num);
+    __syncthreads();
+    mu_factor(F1, num, H, N1, p1, m1, eps, F1n);
+    swap(F1, F1n);
+    __syncthreads();
+    // ---- mode 2
+    gram4(F1, N1, p1, m1, S1);
+    col_pass<T, QM>(X, 1, N1, N2 * N3, N3, cp, F1, m1, vec, P);  // P1 (m1, N2, N3)
+    __syncthreads();
+    core_gram(G, 1, m1, m2 * m3, S1, W);
+    row_dots<T, QM>(P, m1 * N2, cp, N3, F3, m3, Y);  // Y2 (m1, N2, m3)
+    __syncthreads();
+    core_gram(W, m1 * m2, m3, 1, S3, W2);
+    unfold_dots(Y, G, m1, N2, m2, m3, p2, num);
+    __syncthreads();
+    unfold_dots(W2, G, m1, m2, m2, m3, m2, H);
+    __syncthreads();
+    mu_factor(F2, num, H, N2, p2, m2, eps, F2n);
+    swap(F2, F2n);
+    __syncthreads();
+    // ---- mode 3: Y3 = P1 x_2 F2^T (m1, m2, N3)
+    gram4(F2, N2, p2, m2, S2);
+    for (int e = threadIdx.x; e < m1 * m2 * N3; e += blockDim.x) {
+      const int k = e % N3, ab = e / N3, b = ab % m2, a = ab / m2;
+      const T* x = P + (int64_t)a * N2 * cp + k;
+      T s = T(0);
+#pragma unroll 4
+      for (int j = 0; j < N2; ++j) s = fma(F2[j * p2 + b], x[j * cp], s);
+      Y[e] = s;
+    }
+    __syncthreads();
+    core_gram(W, m1, m2, m3, S2, W2);  // G x_1 S1 x_2 S2
+    for (int e = threadIdx.x; e < N3 * m3; e += blockDim.x) {
+      const int k = e / m3, c = e - k * m3;
+      T s = T(0);
+#pragma unroll 4
+      for (int ab = 0; ab < m1 * m2; ++ab) s = fma(Y[ab * N3 + k], G[ab * m3 + c], s);
+      num[k * p3 + c] = s;
+    }
+    __syncthreads();
+    unfold_dots(W2, G, m1 * m2, m3, m3, 1, m3, H);
+    __syncthreads();
+    mu_factor(F3, num, H, N3, p3, m3, eps, F3n);
+    swap(F3, F3n);
+    __syncthreads();
+    // ---- core: M = Y3 x_3 F3^T, D = W2 x_3 S3
+    gram4(F3, N3, p3, m3, S3);
+    for (int e = threadIdx.x; e < ng; e += blockDim.x) {
+      const int c = e % m3, ab = e / m3;
+      T s = T(0);
+#pragma unroll 4
+      for (int k = 0; k < N3; ++k) s = fma(Y[ab * N3 + k], F3[k * p3 + c], s);
+      M[e] = s;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < ng; e += blockDim.x) {
+      const int c = e % m3, ab = e / m3;
+      T den = T(0);
+      for (int w = 0; w < m3; ++w) den = fma(W2[ab * m3 + w], S3[w * m3 + c], den);
+      const T v = G[e] * M[e] / (den > eps ? den : eps);
+      G[e] = v > T(0) ? v : T(0);
+    }
+    __syncthreads();
+  }
+  if (rel_errs) {
+    // ||X - G x_k F_k|| / ||X||: U = G x_1 F1 x_2 F2 (N1, N2, m3), then X streamed.
+    for (int e = threadIdx.x; e < N1 * m2 * m3; e += blockDim.x) {
+      const int bc = e % (m2 * m3), i = e / (m2 * m3);
+      T s = T(0);
+      for (int a = 0; a < m1; ++a) s = fma(F1[i * p1 + a], G[a * m2 * m3 + bc], s);
+      Y[e] = s;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < N1 * N2 * m3; e += blockDim.x) {
+      const int c = e % m3, ij = e / m3, j = ij % N2, i = ij / N2;
+      T s = T(0);
+      for (int b = 0; b < m2; ++b) s = fma(F2[j * p2 + b], Y[(i * m2 + b) * m3 + c], s);
+      P[e] = s;
+    }
+    __syncthreads();
+    stream_residual(X, N1 * N2, N3, P, F3, m3, p3, red, nrm);
+    if (threadIdx.x == 0) rel_errs[blockIdx.x] = sqrt(nrm[0] / nrm[1]);
+  }
+  auto store_factor = [&](void* dst, const T* F, int N, int fp, int m) {
+    T* f = static_cast<T*>(dst);
+    for (int e = threadIdx.x; e < N * m; e += blockDim.x) f[e] = F[(e / m) * fp + e % m];
+  };
+  store_factor(jb.F[0], F1, N1, p1, m1);
+  store_factor(jb.F[1], F2, N2, p2, m2);
+  store_factor(jb.F[2], F3, N3, p3, m3);
+  store(static_cast<T*>(jb.G), G, ng);
 }
 
 // nnCPD of a 3-way tensor per block with the tensor in global memory (the
@@ -542,7 +999,7 @@ cpx_l2_kernel(const nncp_job* __restrict__ jobs, int iters, T eps, double* rel_e
     Tb[e] = A[0][i * r + q] * A[1][j * r + q];
   }
   __syncthreads();
-  stream_residual(X, N[0] * N[1], N[2], Tb, A[2], r, red, nrm);
+  stream_residual(X, N[0] * N[1], N[2], Tb, A[2], r, r, red, nrm);
   if (threadIdx.x == 0 && rel_errs) rel_errs[blockIdx.x] = sqrt(nrm[0] / nrm[1]);
   for (int k = 0; k < 3; ++k) store(static_cast<T*>(jb.B[k]), A[k], N[k] * r);
   if (statuses != nullptr) {
@@ -685,6 +1142,33 @@ int ntd_small_batched(int n_jobs, const ntd_small_job* jobs, int iters, double e
       mm = jobs[i].m[k] > mm ? jobs[i].m[k] : mm;
     }
     work = w * mm > work ? w * mm : work;
+  }
+  // Every multirank within kBlkMaxM and every job's state within a block: the
+  // two-pass form with 16-byte column reads.
+  size_t blk = 0;
+  int mtop = 0;
+  for (int i = 0; i < n_jobs; ++i) {
+    const size_t e = (size_t)ntd_blk_elems<T>(jobs[i]);
+    blk = e > blk ? e : blk;
+    for (int k = 0; k < 3; ++k) mtop = jobs[i].m[k] > mtop ? jobs[i].m[k] : mtop;
+  }
+  const size_t smem1 = blk * sizeof(T);
+  if (mtop <= kBlkMaxM && smem1 <= kSmemBudget) {
+    NNC_TRY(upload(jobs, n_jobs, sc, &dev, s));
+    const void* kern =
+        mtop <= 8 ? (const void*)ntd_blk_kernel<T, 8> : (const void*)ntd_blk_kernel<T, 16>;
+    NNC_CUDA_TRY(raise_smem_limit(kern, smem1));
+    const TuneKey key{kTuneNtdBlk, (int)sizeof(T), size_class(work), size_class(n_jobs)};
+    return run_tuned(key, iters, kThreads, s, [&](int threads, int sweeps, bool last) -> int {
+      double* out = last ? rel_errs : nullptr;
+      if (mtop <= 8)
+        ntd_blk_kernel<T, 8><<<n_jobs, threads, smem1, s>>>(dev, sweeps, (T)eps, out);
+      else
+        ntd_blk_kernel<T, 16><<<n_jobs, threads, smem1, s>>>(dev, sweeps, (T)eps, out);
+      note_launch(s);
+      NNC_CUDA_TRY(cudaGetLastError());
+      return NNC_OK;
+    });
   }
   if (smem <= kSmemBudget) {
     NNC_TRY(upload(jobs, n_jobs, sc, &dev, s));
