@@ -279,10 +279,8 @@ template <typename T>
 cudaError_t launch_nncp(const nncp_job* jobs_dev, int n_jobs, size_t smem, int iters, double eps,
                         double* rel_errs, int* statuses, cudaStream_t s, int threads) {
   if (threads < 32 || threads > kThreads || threads % 32 != 0) return cudaErrorInvalidValue;
-  if (smem > 48 * 1024) {
-    cudaError_t e = raise_smem_limit((const void*)nncp_kernel<T>, smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = raise_smem_limit((const void*)nncp_kernel<T>, smem);
+  if (e != cudaSuccess) return e;
   nncp_kernel<T><<<n_jobs, threads, smem, s>>>(jobs_dev, iters, (T)eps, rel_errs, statuses);
   note_launch(s);
   return cudaGetLastError();
