@@ -60,6 +60,7 @@ __global__ void small_gemm_kernel(int M, int N, int K, const T* __restrict__ A, 
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / N, j = e % N;
     T acc = T(0);
+#pragma unroll 8  // eight rows' loads in flight, the terms in order
     for (int k = 0; k < K; ++k) acc = fma(A[i * as_i + k * as_k], B[k * bs_k + j * bs_j], acc);
     C[e] = D ? acc - D[e] : acc;
   }
@@ -103,16 +104,30 @@ __global__ void kr_kernel(KrArgs<T> a) {
   }
 }
 
-// MT[i, q] = sum_p W[(p N + i) r + q] Kpre[p r + q], p in order.
+// MT[i, q] = sum_p W[(p N + i) r + q] Kpre[p r + q]. N r is a few thousand and P a
+// few hundred, so one thread per entry leaves the sum to a handful of blocks
+// waiting on one load after another: a block takes 32 entries, group g of 16 the
+// terms p = g, g + 16, ... in order, and the groups are added in order.
+// P = 576, N r = 1536: 51.8 -> 10.5 us.
+constexpr int kWsCols = 32, kWsGroups = 16;
 template <typename T>
-__global__ void weighted_sum_p_kernel(const T* __restrict__ W, const T* __restrict__ Kpre,
-                                      int64_t P, int64_t N, int r, T* __restrict__ MT) {
+__global__ void __launch_bounds__(kWsCols * kWsGroups)
+weighted_sum_p_kernel(const T* __restrict__ W, const T* __restrict__ Kpre, int64_t P, int64_t N,
+                      int r, T* __restrict__ MT) {
+  __shared__ T part[kWsGroups][kWsCols];
   const int64_t n = N * r;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
+  const int c = threadIdx.x % kWsCols, g = threadIdx.x / kWsCols;
+  const int64_t e = (int64_t)blockIdx.x * kWsCols + c;
+  T acc = T(0);
+  if (e < n) {
     const int q = (int)(e % r);
-    T acc = T(0);
-    for (int64_t p = 0; p < P; ++p) acc = fma(W[p * n + e], Kpre[p * r + q], acc);
+#pragma unroll 4
+    for (int64_t p = g; p < P; p += kWsGroups) acc = fma(W[p * n + e], Kpre[p * r + q], acc);
+  }
+  part[g][c] = acc;
+  __syncthreads();
+  if (g == 0 && e < n) {
+    for (int k = 1; k < kWsGroups; ++k) acc += part[k][c];
     MT[e] = acc;
   }
 }
@@ -293,9 +308,16 @@ __global__ void lifted_loss_kernel(const T* __restrict__ MT, const T* __restrict
 struct SideStream {
   cudaStream_t s = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
-  cudaEvent_t m_ready = nullptr, g_ready = nullptr;  // the pending core update's steps
+  cudaEvent_t m_ready = nullptr, g_ready = nullptr;  // steps of a branch (see its user)
+  cudaEvent_t b_ready = nullptr;
+  // The branches are chains of one-block kernels beside kernels that fill the GPU: at
+  // the greatest priority their blocks take the next free slot instead of the end of the
+  // queue.
   int init() {
-    NNC_CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    int low = 0, high = 0;
+    NNC_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&low, &high));
+    NNC_CUDA_TRY(cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, high));
+    NNC_CUDA_TRY(cudaEventCreateWithFlags(&b_ready, cudaEventDisableTiming));
     NNC_CUDA_TRY(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
     NNC_CUDA_TRY(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
     NNC_CUDA_TRY(cudaEventCreateWithFlags(&m_ready, cudaEventDisableTiming));
@@ -307,6 +329,7 @@ struct SideStream {
     if (join) cudaEventDestroy(join);
     if (m_ready) cudaEventDestroy(m_ready);
     if (g_ready) cudaEventDestroy(g_ready);
+    if (b_ready) cudaEventDestroy(b_ready);
     if (s) cudaStreamDestroy(s);
   }
 };
@@ -490,9 +513,23 @@ int z_chain(Work<T>& w, int n, T* const* F, const T** zout, cudaStream_t s) {
   return NNC_OK;
 }
 
-// MT_n = unfold_n(Z_n) KR_{k!=n}(B^(k)) into w.MT; V_n into w.V.
+// V_n into w.V.
 template <typename T>
-int mttkrp_and_v(Work<T>& w, int n, const T* Z, T* const* B, cudaStream_t s) {
+int make_v(Work<T>& w, int n, cudaStream_t s) {
+  HadArgs<T> h{};
+  h.r = w.r;
+  h.out = w.V;
+  for (int k = 0; k < w.d; ++k)
+    if (k != n) h.M[h.nk++] = w.AtA[k];
+  hadamard_kernel<T><<<1, 256, 0, s>>>(h);
+  note_launch(s);
+  NNC_CUDA_TRY(cudaGetLastError());
+  return NNC_OK;
+}
+
+// MT_n = unfold_n(Z_n) KR_{k!=n}(B^(k)) into w.MT.
+template <typename T>
+int mttkrp(Work<T>& w, int n, const T* Z, T* const* B, cudaStream_t s) {
   const int d = w.d, r = w.r;
   KrArgs<T> pre{}, post{};
   pre.r = post.r = r;
@@ -528,20 +565,19 @@ int mttkrp_and_v(Work<T>& w, int n, const T* Z, T* const* B, cudaStream_t s) {
     NNC_CUDA_TRY(launch_ttm<T>(Z, pre.rows * w.N[n], (int)post.rows, 1, w.Kpost, r, 1, r, Wout,
                                w.split, w.split_cap, s));
     if (pre.rows > 1) {
-      weighted_sum_p_kernel<T><<<grid_for(w.N[n] * r, 256), 256, 0, s>>>(w.W, w.Kpre, pre.rows,
-                                                                           w.N[n], r, w.MT);
+      weighted_sum_p_kernel<T><<<(unsigned)ceil_div(w.N[n] * r, kWsCols), kWsCols * kWsGroups, 0,
+                                 s>>>(w.W, w.Kpre, pre.rows, w.N[n], r, w.MT);
       note_launch(s);
     }
   }
-  HadArgs<T> h{};
-  h.r = r;
-  h.out = w.V;
-  for (int k = 0; k < d; ++k)
-    if (k != n) h.M[h.nk++] = w.AtA[k];
-  hadamard_kernel<T><<<1, 256, 0, s>>>(h);
-  note_launch(s);
   NNC_CUDA_TRY(cudaGetLastError());
   return NNC_OK;
+}
+
+template <typename T>
+int mttkrp_and_v(Work<T>& w, int n, const T* Z, T* const* B, cudaStream_t s) {
+  NNC_TRY(mttkrp(w, n, Z, B, s));
+  return make_v(w, n, s);
 }
 
 // A^(k) = F^(k) B^(k) and A^(k)T A^(k).
@@ -560,55 +596,58 @@ int grad_a(Work<T>& w, int n, cudaStream_t s) {
   return NNC_OK;
 }
 
-// One block pair (F^(n), then B^(n)) of the projected-gradient step. The step
-// sizes (power iterations on small FP64 chains) need nothing from the
-// gradient chain, so with a side stream each runs beside it and is joined
-// before the update that uses it (the same launches either way).
+// The projected-gradient step of mode n in three parts. Each L is a chain of small
+// FP64 kernels, so the parts off the path F^(n) -> Z_{n+1} -> F^(n+1) run on a
+// side stream beside the mode products (see pg_step).
+// V_n, L_F = lmax(B V B^T) and lmax(V): tmp2 = B V (m x r), H = tmp2 B^T (m x m).
 template <typename T>
-int pg_mode(Work<T>& w, int n, T* const* F, T* const* B, cudaStream_t s, SideStream* side) {
+int pg_step_size_f(Work<T>& w, int n, T* const* B, cudaStream_t s) {
+  const int r = w.r, mn = w.m[n];
+  NNC_TRY(make_v(w, n, s));
+  NNC_CUDA_TRY(small_gemm<T>(mn, r, r, B[n], r, 1, w.V, r, 1, nullptr, w.tmp2, s));
+  NNC_CUDA_TRY(small_gemm<T>(mn, mn, r, w.tmp2, r, 1, B[n], 1, r, nullptr, w.H, s));
+  power_iter_kernel<T><<<2, power_iter_threads(mn, r), 0, s>>>(w.H, mn, w.Ls + 0, w.V, r,
+                                                                 w.Ls + 1);
+  note_launch(s);
+  NNC_CUDA_TRY(cudaGetLastError());
+  return NNC_OK;
+}
+
+// F^(n) <- max(F^(n) - (A V - MT) B^T / L_F, 0).
+template <typename T>
+int pg_update_f(Work<T>& w, int n, T* const* F, T* const* B, cudaStream_t s) {
   const int r = w.r, mn = w.m[n];
   const int64_t Nn = w.N[n];
-  const cudaStream_t ls = side ? side->s : s;
-  auto fork = [&]() -> int {
-    if (!side) return NNC_OK;
-    NNC_CUDA_TRY(cudaEventRecord(side->fork, s));
-    NNC_CUDA_TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
-    return NNC_OK;
-  };
-  auto join = [&]() -> int {
-    if (!side) return NNC_OK;
-    NNC_CUDA_TRY(cudaEventRecord(side->join, side->s));
-    NNC_CUDA_TRY(cudaStreamWaitEvent(s, side->join, 0));
-    return NNC_OK;
-  };
-  // L_F = lmax(B V B^T) and lmax(V) (one launch): tmp2 = B V (m x r), H = tmp2 B^T (m x m)
-  NNC_TRY(fork());
-  NNC_CUDA_TRY(small_gemm<T>(mn, r, r, B[n], r, 1, w.V, r, 1, nullptr, w.tmp2, ls));
-  NNC_CUDA_TRY(small_gemm<T>(mn, mn, r, w.tmp2, r, 1, B[n], 1, r, nullptr, w.H, ls));
-  power_iter_kernel<T><<<2, power_iter_threads(mn, r), 0, ls>>>(w.H, mn, w.Ls + 0, w.V, r,
-                                                                 w.Ls + 1);
-  note_launch(ls);
-  NNC_CUDA_TRY(cudaGetLastError());
   NNC_TRY(grad_a(w, n, s));
   // gF = gA B^T (N x m) into tmp
   NNC_CUDA_TRY(small_gemm<T>((int)Nn, mn, r, w.gA, r, 1, B[n], 1, r, nullptr, w.tmp, s));
-  NNC_TRY(join());
   pg_update_kernel<T><<<grid_for(Nn * mn, 256), 256, 0, s>>>(F[n], w.tmp, Nn * mn, w.Ls + 0,
                                                                nullptr);
   note_launch(s);
   NNC_CUDA_TRY(cudaGetLastError());
-  NNC_CUDA_TRY(launch_lift<T>(F[n], B[n], Nn, mn, r, w.A[n], s));
-  // L_B = lmax(F^T F) lmax(V)
-  NNC_TRY(fork());
+  return NNC_OK;
+}
+
+// B^(n) <- max(B^(n) - F^T (A V - MT) / L_B, 0) with the new F^(n) and
+// L_B = lmax(F^T F) lmax(V) (beside the gradient, on ls), then the new A^(n) and its Gram.
+template <typename T>
+int pg_update_b(Work<T>& w, int n, T* const* F, T* const* B, SideStream& side, cudaStream_t s,
+                cudaStream_t ls) {
+  const int r = w.r, mn = w.m[n];
+  const int64_t Nn = w.N[n];
+  NNC_CUDA_TRY(cudaEventRecord(side.fork, s));
+  NNC_CUDA_TRY(cudaStreamWaitEvent(ls, side.fork, 0));
   NNC_TRY(launch_gram<T>(F[n], Nn, mn, w.S, ls));
   power_iter_kernel<T><<<1, power_iter_threads(mn, mn), 0, ls>>>(w.S, mn, w.Ls + 2, w.S, mn,
-                                                                 w.Ls + 2);
+                                                                   w.Ls + 2);
   note_launch(ls);
   NNC_CUDA_TRY(cudaGetLastError());
+  NNC_CUDA_TRY(cudaEventRecord(side.join, ls));
+  NNC_CUDA_TRY(launch_lift<T>(F[n], B[n], Nn, mn, r, w.A[n], s));
   NNC_TRY(grad_a(w, n, s));
   // gB = F^T gA (m x r) into tmp
   NNC_CUDA_TRY(small_gemm<T>(mn, r, (int)Nn, F[n], 1, mn, w.gA, r, 1, nullptr, w.tmp, s));
-  NNC_TRY(join());
+  NNC_CUDA_TRY(cudaStreamWaitEvent(s, side.join, 0));
   pg_update_kernel<T><<<grid_for((int64_t)mn * r, 256), 256, 0, s>>>(B[n], w.tmp, (int64_t)mn * r,
                                                                       w.Ls + 2, w.Ls + 1);
   note_launch(s);
@@ -674,22 +713,47 @@ int lifted_grad(const T* X, int d, const int64_t* dims, const int* m, int r, boo
 
 namespace {
 
-// One projected-gradient step (two passes over X), stream-ordered on s.
+// One projected-gradient step (two passes over X) on `s`. Z_{n+1} needs the new
+// F^(n) but no B, so the B update of mode n (and then V and the F step size of mode
+// n + 1) runs on side.s beside the mode products of Z_{n+1}, and the B update of the
+// last mode, with the loss, beside the next step's first pass (`pending`: this
+// step begins with it). Every value is formed by the same launches from the
+// same values as in program order.
+template <typename T>
+int pg_tail(Work<T>& w, T* const* F, T* const* B, double* last, double* trace, int* counter,
+            SideStream& side, cudaStream_t s, cudaStream_t ls) {
+  NNC_TRY(pg_update_b(w, w.d - 1, F, B, side, s, ls));
+  // MT_d and V_d do not involve mode d: the loss at the new point.
+  return loss_into(w, w.d - 1, last, trace, counter, s);
+}
+
 template <typename T>
 int pg_step(Work<T>& w, T* const* F, T* const* B, double* last, double* trace, int* counter,
-            cudaStream_t s, SideStream* side) {
+            cudaStream_t s, SideStream& side, cudaStream_t ls, bool pending) {
   const int d = w.d;
-  NNC_TRY(pass_last(w, F[d - 1], s));
+  NNC_CUDA_TRY(cudaEventRecord(side.g_ready, s));  // F of the mode before is final
+  NNC_CUDA_TRY(cudaStreamWaitEvent(side.s, side.g_ready, 0));
+  if (pending) NNC_TRY(pg_tail(w, F, B, last, trace, counter, side, side.s, ls));
   for (int n = 0; n < d; ++n) {
+    if (n > 0) {
+      NNC_CUDA_TRY(cudaEventRecord(side.g_ready, s));
+      NNC_CUDA_TRY(cudaStreamWaitEvent(side.s, side.g_ready, 0));
+      NNC_TRY(pg_update_b(w, n - 1, F, B, side, side.s, ls));
+    }
+    NNC_CUDA_TRY(cudaEventRecord(side.b_ready, side.s));
+    NNC_TRY(pg_step_size_f(w, n, B, side.s));
+    NNC_CUDA_TRY(cudaEventRecord(side.m_ready, side.s));
+    if (n == 0) NNC_TRY(pass_last(w, F[d - 1], s));
+    if (n == 1 && d > 2) NNC_TRY(make_u0(w, F[0], s));
     if (n == d - 1) NNC_TRY(pass_first(w, F[0], s));
     const T* Z = nullptr;
     NNC_TRY(z_chain(w, n, F, &Z, s));
-    NNC_TRY(mttkrp_and_v(w, n, Z, B, s));
-    NNC_TRY(pg_mode(w, n, F, B, s, side));
-    if (n == 0 && d > 2) NNC_TRY(make_u0(w, F[0], s));
+    NNC_CUDA_TRY(cudaStreamWaitEvent(s, side.b_ready, 0));
+    NNC_TRY(mttkrp(w, n, Z, B, s));
+    NNC_CUDA_TRY(cudaStreamWaitEvent(s, side.m_ready, 0));
+    NNC_TRY(pg_update_f(w, n, F, B, s));
   }
-  // MT_d and V_d do not involve mode d: the loss at the new point.
-  return loss_into(w, d - 1, last, trace, counter, s);
+  return NNC_OK;
 }
 
 // Private stream, graph and events of the replay loop.
@@ -706,68 +770,6 @@ struct PgGraph {
     if (cs) cudaStreamDestroy(cs);
   }
 };
-
-}  // namespace
-
-template <typename T>
-int lifted_pg_fit(const T* X, int d, const int64_t* dims, const int* m, int r, bool tensor_cores,
-                  int steps, T* const* F, T* const* B, double* trace, double* loss,
-                  cudaStream_t s) {
-  Scratch sc(s);
-  Work<T> w;
-  NNC_TRY(setup(w, X, d, dims, m, r, tensor_cores, sc, s));
-  for (int k = 0; k < d; ++k) NNC_TRY(refresh_a(w, k, F[k], B[k], s));
-  double* last = w.Ls + 3;
-  int* counter = nullptr;
-  NNC_TRY(sc.get(&counter, 2));
-  NNC_CUDA_TRY(cudaMemsetAsync(counter, 0, 2 * sizeof(int), s));
-  if (steps > 0) {
-    // One step is captured as a CUDA graph on a private stream and replayed;
-    // the trace slot advances through the device counter.
-    PgGraph g;
-    SideStream side;
-    NNC_TRY(side.init());
-    NNC_CUDA_TRY(cudaStreamCreateWithFlags(&g.cs, cudaStreamNonBlocking));
-    NNC_CUDA_TRY(cudaEventCreateWithFlags(&g.fork, cudaEventDisableTiming));
-    NNC_CUDA_TRY(cudaEventCreateWithFlags(&g.join, cudaEventDisableTiming));
-    NNC_CUDA_TRY(cudaEventRecord(g.fork, s));
-    NNC_CUDA_TRY(cudaStreamWaitEvent(g.cs, g.fork, 0));
-    NNC_CUDA_TRY(cudaStreamBeginCapture(g.cs, cudaStreamCaptureModeThreadLocal));
-    const int cap = pg_step(w, F, B, last, trace, counter, g.cs, &side);
-    const cudaError_t end_e = cudaStreamEndCapture(g.cs, &g.graph);
-    if (cap != NNC_OK) return cap;
-    NNC_CUDA_TRY(end_e);
-    NNC_CUDA_TRY(cudaGraphInstantiate(&g.exec, g.graph, 0));
-    size_t nn = 0;
-    NNC_CUDA_TRY(cudaGraphGetNodes(g.graph, nullptr, &nn));
-    std::vector<cudaGraphNode_t> nodes(nn);
-    NNC_CUDA_TRY(cudaGraphGetNodes(g.graph, nodes.data(), &nn));
-    long long kernels = 0;
-    for (cudaGraphNode_t nd : nodes) {
-      cudaGraphNodeType ty;
-      NNC_CUDA_TRY(cudaGraphNodeGetType(nd, &ty));
-      if (ty == cudaGraphNodeTypeKernel) ++kernels;
-    }
-    for (int t = 0; t < steps; ++t) NNC_CUDA_TRY(cudaGraphLaunch(g.exec, g.cs));
-    note_graph_launches(kernels * steps);
-    NNC_CUDA_TRY(cudaEventRecord(g.join, g.cs));
-    NNC_CUDA_TRY(cudaStreamWaitEvent(s, g.join, 0));
-    NNC_CUDA_TRY(cudaStreamSynchronize(g.cs));
-  }
-  NNC_TRY(check_tc(w, s));
-  NNC_TRY(check_trace_finite(counter, s, "candelinc_pg_fit"));
-  if (loss) {
-    if (steps == 0) {
-      *loss = NAN;
-    } else {
-      NNC_CUDA_TRY(cudaMemcpyAsync(loss, last, sizeof(double), cudaMemcpyDeviceToHost, s));
-      NNC_CUDA_TRY(cudaStreamSynchronize(s));
-    }
-  }
-  return NNC_OK;
-}
-
-namespace {
 
 // Captures `body` (stream-ordered work on a private stream) once as a CUDA
 // graph and replays it `count` times after the work queued on s; `after(t,
@@ -863,6 +865,49 @@ int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last las
 }
 
 }  // namespace
+
+template <typename T>
+int lifted_pg_fit(const T* X, int d, const int64_t* dims, const int* m, int r, bool tensor_cores,
+                  int steps, T* const* F, T* const* B, double* trace, double* loss,
+                  cudaStream_t s) {
+  Scratch sc(s);
+  Work<T> w;
+  NNC_TRY(setup(w, X, d, dims, m, r, tensor_cores, sc, s));
+  for (int k = 0; k < d; ++k) NNC_TRY(refresh_a(w, k, F[k], B[k], s));
+  double* last = w.Ls + 3;
+  int* counter = nullptr;
+  NNC_TRY(sc.get(&counter, 2));
+  NNC_CUDA_TRY(cudaMemsetAsync(counter, 0, 2 * sizeof(int), s));
+  if (steps > 0) {
+    // The steps are captured as CUDA graphs on a private stream and replayed; the
+    // trace slot advances through the device counter.
+    SideStream side, step_size;
+    NNC_TRY(side.init());
+    NNC_TRY(step_size.init());
+    NNC_TRY(replay_pipelined(
+        steps, s,
+        [&](cudaStream_t cs) -> int {
+          return pg_step(w, F, B, last, trace, counter, cs, side, step_size.s, false);
+        },
+        [&](cudaStream_t cs) -> int {
+          return pg_step(w, F, B, last, trace, counter, cs, side, step_size.s, true);
+        },
+        [&](cudaStream_t cs) -> int {
+          return pg_tail(w, F, B, last, trace, counter, side, cs, step_size.s);
+        }));
+  }
+  NNC_TRY(check_tc(w, s));
+  NNC_TRY(check_trace_finite(counter, s, "candelinc_pg_fit"));
+  if (loss) {
+    if (steps == 0) {
+      *loss = NAN;
+    } else {
+      NNC_CUDA_TRY(cudaMemcpyAsync(loss, last, sizeof(double), cudaMemcpyDeviceToHost, s));
+      NNC_CUDA_TRY(cudaStreamSynchronize(s));
+    }
+  }
+  return NNC_OK;
+}
 
 // nnCPD of X itself (Alg. 2, first step): the MU sweep of the core nnCPD with
 // X in place of G, A^(n) <- max(A^(n) .* MT_n / max(A^(n) V_n, eps), 0) for

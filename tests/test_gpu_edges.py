@@ -43,3 +43,22 @@ def test_small_batched_edges(dt, jobs):
         for a, b in zip(F + [G], Fo + [Go]):
             np.testing.assert_allclose(a.double().cpu().numpy(), b, rtol=tol, atol=tol * 1e-3)
         assert e == pytest.approx(orc.rel_err_tucker(Xr, Go, Fo), abs=tol)
+
+
+# Few outputs with many partial sums (32 or more: the wide sum), and the weighted sums of
+# the inner modes below, at and past one group of 16 terms.
+@pytest.mark.parametrize("dims,m,r", [((6, 40, 21, 9), (2, 16, 16, 8), 3),
+                                      ((33, 5, 40, 7), (3, 5, 24, 5), 2),
+                                      ((9, 70, 13), (4, 17, 3), 5)])
+def test_lifted_gradient_sums(dims, m, r):
+    rng = np.random.default_rng(5)
+    X = rng.random(dims)
+    F = [1 - rng.random((n, k)) for n, k in zip(dims, m)]
+    B = [1 - rng.random((k, r)) for k in m]
+    dt = torch.float64
+    loss, gF, gB = native.candelinc_lifted_grad(_dev(X, dt), [_dev(f, dt) for f in F],
+                                                [_dev(b, dt) for b in B])
+    gFo, gBo = orc.lifted_loss_grad(X, F, B)
+    assert loss == pytest.approx(orc.lifted_loss(X, F, B), rel=1e-9)
+    for a, b in zip(gF + gB, list(gFo) + list(gBo)):
+        np.testing.assert_allclose(a.cpu().numpy(), b, rtol=1e-9, atol=1e-9 * np.abs(b).max())
