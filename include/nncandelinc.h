@@ -20,8 +20,10 @@
  *  - `stream` is a cudaStream_t (NULL = legacy default stream). Work is
  *    stream-ordered. A call returns after its host outputs are written; it
  *    synchronises `stream` only when it has host outputs to write.
- *  - Scratch memory is taken from the stream-ordered allocator
- *    (cudaMallocAsync) on `stream` and released before the call returns.
+ *  - Scratch memory is taken, stream-ordered on `stream`, from a memory pool of
+ *    the library's own and returned to it before the call returns. The pool
+ *    keeps at most 4 GiB (or 1/64 of the device's memory, if less) between calls;
+ *    nnc_release_scratch() gives it back to the device.
  *  - Every call returns NNC_OK (0) or a negative NNC_ERR_* code; on error the
  *    caller's arrays may hold partial results. nnc_status_string() names it.
  *  - Update rule: multiplicative updates with a Gauss-Seidel order, guarded
@@ -519,6 +521,11 @@ int nnc_wait_selftest(long long cycles, void* stream);
  * every thread of the process. Returns the previous countdown.
  */
 int nnc_debug_fail_alloc(int nth);
+
+/* Gives the scratch memory that the library keeps for the current device between
+ * calls, and that no queued work still uses, back to the device (for another
+ * allocator of the process to use). Errors: CUDA. */
+int nnc_release_scratch(void);
 
 /* The sweep index (0-based) at which the last NNC_BF16_REFINE ntd_fit call of
  * this thread began its FP32 refinement sweeps (iters when it ran none), or -1

@@ -104,6 +104,56 @@ cudaError_t raise_smem_limit(const void* kernel, size_t bytes) {
   return e;
 }
 
+namespace {
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices];  // created by the first allocation on a device
+cudaError_t device_pool(cudaMemPool_t* pool) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (g_pool[dev] == nullptr) {
+    cudaDeviceProp prop;
+    e = cudaGetDeviceProperties(&prop, dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t made = nullptr;
+    e = cudaMemPoolCreate(&made, &props);
+    if (e != cudaSuccess) return e;
+    uint64_t keep = prop.totalGlobalMem / 64;
+    if (keep > kScratchKeepBytes) keep = kScratchKeepBytes;
+    e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) {
+      cudaMemPoolDestroy(made);
+      return e;
+    }
+    g_pool[dev] = made;
+  }
+  *pool = g_pool[dev];
+  return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  *p = nullptr;
+  cudaMemPool_t pool = nullptr;
+  cudaError_t e = device_pool(&pool);
+  if (e != cudaSuccess) return e;
+  e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  if (e == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();
+    (void)cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  }
+  return e;
+}
+
 int device_sm_count() {
   static std::atomic<int> cache[64];  // 0 until first read (zero-initialised static)
   int dev = 0;
@@ -223,6 +273,16 @@ const char* nnc_last_error_detail(void) { return g_detail.c_str(); }
 long long nnc_kernel_launches(void) { return g_kernel_launches.load(); }
 
 int nnc_last_refine_sweep(void) { return g_refine_sweep; }
+
+int nnc_release_scratch(void) {
+  int dev = 0;
+  nnc::clear_error_detail();
+  NNC_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= nnc::kMaxDevices) return NNC_OK;
+  std::lock_guard<std::mutex> lk(nnc::g_pool_mu);
+  if (nnc::g_pool[dev] != nullptr) NNC_CUDA_TRY(cudaMemPoolTrimTo(nnc::g_pool[dev], 0));
+  return NNC_OK;
+}
 
 int nnc_debug_fail_alloc(int nth) {
   return g_fail_alloc.exchange(nth > 0 ? nth : 0);

@@ -30,7 +30,7 @@ EXPORTED = ("ntd_fit", "ntd_fit_batched", "ntd_fit_small_batched", "nmf_fit_batc
             "nnc_status_string", "nnc_last_error_detail",
             "nnc_profile_enable", "nnc_profile_read", "nnc_kernel_launches",
             "nnc_autotune_enable", "nnc_wait_selftest", "nnc_debug_fail_alloc",
-            "nnc_last_refine_sweep")
+            "nnc_last_refine_sweep", "nnc_release_scratch")
 
 
 class NncError(RuntimeError):
@@ -141,6 +141,8 @@ def load(path: str | None = None):
     lib.nnc_wait_selftest.restype = ctypes.c_int
     lib.nnc_debug_fail_alloc.argtypes = [ctypes.c_int]
     lib.nnc_debug_fail_alloc.restype = ctypes.c_int
+    lib.nnc_release_scratch.argtypes = []
+    lib.nnc_release_scratch.restype = ctypes.c_int
     lib.nnc_last_refine_sweep.argtypes = []
     lib.nnc_last_refine_sweep.restype = ctypes.c_int
     _lib = lib
@@ -554,6 +556,11 @@ def nnc_autotune_enable(on=True):
 def nnc_last_refine_sweep():
     """Sweep at which this thread's last BF16 ntd_fit began its FP32 sweeps."""
     return int(load().nnc_last_refine_sweep())
+
+
+def nnc_release_scratch():
+    """Gives the scratch memory the library keeps between calls back to the device."""
+    _check("nnc_release_scratch", load().nnc_release_scratch())
 
 
 def nnc_debug_fail_alloc(nth):

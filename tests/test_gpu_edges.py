@@ -62,3 +62,17 @@ def test_lifted_gradient_sums(dims, m, r):
     assert loss == pytest.approx(orc.lifted_loss(X, F, B), rel=1e-9)
     for a, b in zip(gF + gB, list(gFo) + list(gBo)):
         np.testing.assert_allclose(a.cpu().numpy(), b, rtol=1e-9, atol=1e-9 * np.abs(b).max())
+
+
+def test_scratch_is_kept_bounded_and_given_back():
+    X = torch.rand(256, 256, 256, device="cuda")
+    F = [torch.rand(256, 8, device="cuda") + 0.1 for _ in range(3)]
+    G = torch.rand(8, 8, 8, device="cuda") + 0.1
+    native.ntd_fit(X, F, G, 2)
+    torch.cuda.synchronize()
+    held = torch.cuda.mem_get_info()[0]
+    native.nnc_release_scratch()
+    freed = torch.cuda.mem_get_info()[0] - held
+    # The scratch of the call holds a copy of X (64 MiB) and more; 4 GiB is the most
+    # the library keeps.
+    assert 64 << 20 <= freed <= 4 << 30
