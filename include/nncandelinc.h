@@ -51,10 +51,11 @@ typedef enum {
   NNC_FP64 = 0,        /* double storage and arithmetic (SIMT)               */
   NNC_FP32 = 1,        /* float storage, FP32-accurate arithmetic: the two
                           passes over X per sweep run on the tensor cores as
-                          three TF32 products per term (hi*hi + hi*lo + lo*hi
-                          of exact TF32 splits, FP32 accumulation); shapes the
-                          tensor-core path cannot take (N3 % 4 != 0) run the
-                          SIMT passes                                        */
+                          three products per term (hi*hi + hi*lo + lo*hi of
+                          splits into two FP16 parts, scaled by powers of two
+                          per slice, or into two TF32 parts; FP32
+                          accumulation); shapes the tensor-core path cannot
+                          take (N3 % 4 != 0) run the SIMT passes             */
   NNC_BF16_REFINE = 2, /* float storage; the passes over X use a BF16 copy of
                           X on the tensor cores (FP32 accumulation), then the
                           last `refine_iters` sweeps are NNC_FP32 sweeps     */

@@ -362,7 +362,7 @@ int64_t prod(const int64_t* v, int a, int b) {  // v[a] ... v[b-1]
 
 template <typename T>
 int setup(Work<T>& w, const T* X, int d, const int64_t* dims, const int* m, int r, bool want_tc,
-          Scratch& sc, cudaStream_t s) {
+          Scratch& sc, cudaStream_t s, bool one_pass = false) {
   w.d = d;
   w.r = r;
   w.X = X;
@@ -430,8 +430,12 @@ int setup(Work<T>& w, const T* X, int d, const int64_t* dims, const int* m, int 
   w.tc = false;
   if constexpr (std::is_same<T, float>::value) {
     if (want_tc) {
-      const int st2 = w.plan.init(tc::kKindTf32x3, X, dims[0], prod(dims, 1, d - 1),
-                                  dims[d - 1], m[0], m[d - 1], sc, s);
+      // One pass over X alone (the loss) is not worth a copy of X.
+      const int64_t n2 = prod(dims, 1, d - 1);
+      const int st2 = one_pass ? w.plan.init(tc::kKindTf32x3, X, dims[0], n2, dims[d - 1], m[0],
+                                             m[d - 1], sc, s, /*p1_kj=*/false, /*need_p1=*/false)
+                               : w.plan.init_fp32(X, dims[0], n2, dims[d - 1], m[0], m[d - 1],
+                                                  sc, s);
       if (st2 == NNC_OK) w.tc = true;
       else if (st2 != NNC_ERR_UNSUPPORTED) return st2;
     }
@@ -683,9 +687,9 @@ int lifted_grad(const T* X, int d, const int64_t* dims, const int* m, int r, boo
                 cudaStream_t s) {
   Scratch sc(s);
   Work<T> w;
-  NNC_TRY(setup(w, X, d, dims, m, r, tensor_cores, sc, s));
-  for (int k = 0; k < d; ++k) NNC_TRY(refresh_a(w, k, F[k], B[k], s));
   const bool grads = gF != nullptr;
+  NNC_TRY(setup(w, X, d, dims, m, r, tensor_cores, sc, s, /*one_pass=*/!grads));
+  for (int k = 0; k < d; ++k) NNC_TRY(refresh_a(w, k, F[k], B[k], s));
   double* dloss = w.Ls + 3;
   NNC_TRY(pass_last(w, F[d - 1], s));
   if (grads) {

@@ -91,18 +91,27 @@ __device__ __forceinline__ void step(float (&acc)[2][4][4], const float* a, cons
     for (int j = 0; j < 4; ++j)
 #pragma unroll
       for (int h = 0; h < 2; ++h) bl[j][h] = tf32_rn(xb[h][j] - __uint_as_float(bh[j][h]));
+    // A fresh fragment per step, added with round-to-nearest: the tensor core truncates
+    // as it accumulates, one-sided on nonnegative data, and a chain over the whole
+    // contraction biased the numerators of the modes formed here by more than the
+    // passes' own rounding.
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        mma_tf32(acc[i][j], al[i], bh[j][0], bh[j][1]);
-        mma_tf32(acc[i][j], ah[i], bl[j][0], bl[j][1]);
+        float part[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_tf32(part, al[i], bh[j][0], bh[j][1]);
+        mma_tf32(part, ah[i], bl[j][0], bl[j][1]);
+        mma_tf32(part, ah[i], bh[j][0], bh[j][1]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[i][j][q] += part[q];
       }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mma_tf32(acc[i][j], ah[i], bh[j][0], bh[j][1]);
   }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) mma_tf32(acc[i][j], ah[i], bh[j][0], bh[j][1]);
 }
 
 // Entry (s, c) of the tile in a 32 x 32 shared-memory buffer whose rows have

@@ -158,7 +158,7 @@ int sweep3(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double* tr
     u.err = tcp ? tcp->err : nullptr;
     u.ybuf = b.Yb;
     if constexpr (std::is_same<T, float>::value) {
-      if (tcp) {
+      if (tcp) {  // (all NULL for the FP16 pairs, whose passes form their operands)
         u.bt = tcp->Bt1;
         u.bhi = tcp->B1hi;
         u.blo = tcp->B1lo;
@@ -557,7 +557,13 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
       fast = &plan16;
     }
     if (passes >= 1 && (passes == 1 || o->refine_iters > 0 || trigger)) {
-      const int st = plan32.init(tc::kKindTf32x3, X, N1, N2, N3, m1, m3, sc, s, /*p1_kj=*/true);
+      const int st = plan32.init_fp32(X, N1, N2, N3, m1, m3, sc, s, /*p1_kj=*/true);
+      // The FP16 pair passes stream X fast enough that the side kernels would be the
+      // longer branch on the few SMs a full grid leaves: 512^3, m = 32, SMs left 0, 8,
+      // 16, 24, 32, 40: 265, 258, 250, 248, 253, 259 us per sweep; 256^3, m = 20
+      // (3.4 tiles per SM): 73.6 up to 24, 71.2 at 32 and 40.
+      if (plan32.kind == tc::kKindF16x3)
+        plan32.reserve_sms = N1 * N2 >= 128 * 8LL * device_sm_count() ? 24 : 32;
       if (st == NNC_OK) exact = &plan32;
       else if (st != NNC_ERR_UNSUPPORTED) return st;
     }

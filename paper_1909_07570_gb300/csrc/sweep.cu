@@ -793,25 +793,37 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) {
 template <int SPLIT>
 __device__ __forceinline__ void numu_mma(float (&acc)[4][4], float4 y, const float4 (&gv)[4]) {
   const float ya[4] = {y.x, y.y, y.z, y.w};
+  uint32_t ah[2][4], al[2][4];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    uint32_t ah[4] = {mma32::tf32_rn(ya[2 * h]), 0u, mma32::tf32_rn(ya[2 * h + 1]), 0u};
-    uint32_t al[4] = {0u, 0u, 0u, 0u};
-    if constexpr (SPLIT == 3) {
-      al[0] = mma32::tf32_rn(ya[2 * h] - __uint_as_float(ah[0]));
-      al[2] = mma32::tf32_rn(ya[2 * h + 1] - __uint_as_float(ah[2]));
-    }
+    ah[h][0] = mma32::tf32_rn(ya[2 * h]);
+    ah[h][2] = mma32::tf32_rn(ya[2 * h + 1]);
+    ah[h][1] = ah[h][3] = al[h][1] = al[h][3] = 0u;
+    al[h][0] = mma32::tf32_rn(ya[2 * h] - __uint_as_float(ah[h][0]));
+    al[h][2] = mma32::tf32_rn(ya[2 * h + 1] - __uint_as_float(ah[h][2]));
+  }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < 4; ++j) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
       const float g0 = h ? gv[j].z : gv[j].x, g1 = h ? gv[j].w : gv[j].y;
       const uint32_t bh0 = mma32::tf32_rn(g0), bh1 = mma32::tf32_rn(g1);
       if constexpr (SPLIT == 3) {
+        // A fresh fragment for every eight terms, added with round-to-nearest, as in
+        // mma32::step: the modes' numerators and the core's then carry the same
+        // truncation (a difference between them shifts scale from factor to factor
+        // with every sweep).
+        float part[4] = {0.f, 0.f, 0.f, 0.f};
         const uint32_t bl0 = mma32::tf32_rn(g0 - __uint_as_float(bh0));
         const uint32_t bl1 = mma32::tf32_rn(g1 - __uint_as_float(bh1));
-        mma32::mma_tf32(acc[j], al, bh0, bh1);
-        mma32::mma_tf32(acc[j], ah, bl0, bl1);
+        mma32::mma_tf32(part, al[h], bh0, bh1);
+        mma32::mma_tf32(part, ah[h], bl0, bl1);
+        mma32::mma_tf32(part, ah[h], bh0, bh1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] += part[q];
+      } else {
+        mma32::mma_tf32(acc[j], ah[h], bh0, bh1);
       }
-      mma32::mma_tf32(acc[j], ah, bh0, bh1);
     }
   }
 }

@@ -1,5 +1,7 @@
 // Tensor-core (tcgen05) mode products: the two passes over X of an nnTD sweep
-// (n-mode multiplication, Appendix A), in two number formats.
+// (n-mode multiplication, Appendix A), in three number formats. The first two are
+// described here, the FP16 pairs (F16x3, the FP32-accurate form of the fits) at
+// f16_pass_kernel.
 //
 //   BF16    X is kept as a BF16 copy Xb with per-slice power-of-two scales s_i
 //           (mode-1 slices), rows padded with zeros to Kp = roundup(N3, 64):
@@ -275,6 +277,62 @@ __device__ __forceinline__ bool epi_all(bool ok) {
 }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
+// FUSE: row j of the factor (zero past yf_m) into row lr of Fs: rows of 8
+// float4 chunks, chunk c stored at c ^ (row & 7), so that the row-per-thread
+// stores and the chunk reads of the contraction avoid bank conflicts.
+__device__ __forceinline__ void stage_factor_row(const TcEpilogue& ep, int64_t j, int lr,
+                                                 float* Fs) {
+  const float* f = ep.yf + j * ep.yf_m;
+  float fr[32];
+  if ((ep.yf_m & 3) == 0 && (reinterpret_cast<uintptr_t>(f) & 15) == 0) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float4 q = 4 * c < ep.yf_m ? *reinterpret_cast<const float4*>(f + 4 * c)
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+      fr[4 * c] = q.x; fr[4 * c + 1] = q.y; fr[4 * c + 2] = q.z; fr[4 * c + 3] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int b = 0; b < 32; ++b) fr[b] = b < ep.yf_m ? f[b] : 0.f;
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+    *reinterpret_cast<float4*>(Fs + lr * 32 + ((c ^ (lr & 7)) << 2)) =
+        make_float4(fr[4 * c], fr[4 * c + 1], fr[4 * c + 2], fr[4 * c + 3]);
+}
+
+// FUSE: contraction of the tile (one slab s, rows j0 .. j0 + 127) by the 128
+// epilogue threads:
+//   share[b, c] = sum_r F[j0 + r, b] P[(s, j0 + r), c]
+// on the tensor cores (mma32.cuh: SPLIT = 1, TF32 operands beside the BF16
+// rounding of X; 3, split TF32 in the FP32-accurate passes). The warp of quarter
+// q takes rows 32 q .. 32 q + 31 with the whole 32 x 32 share (zero past m2,
+// m3) in registers; the four partial shares are added in quarter order.
+template <int SPLIT>
+__device__ __forceinline__ void fused_share(const TcEpilogue& ep, int64_t tile, int lane,
+                                            int quarter, float* Ps, const float* Fs) {
+  const int et = threadIdx.x - 64;  // 0 .. 127
+  const int o0 = mma32::frag_off(lane, 0), o1 = mma32::frag_off(lane, 1);
+  float acc[2][4][4];
+  mma32::zero(acc);
+  epi_sync();  // Ps and Fs complete
+#pragma unroll
+  for (int ks = 4 * quarter; ks < 4 * quarter + 4; ++ks)
+    mma32::step<SPLIT>(acc, Fs + ks * 256, Ps + ks * 256, o0, o1);
+  epi_sync();  // Ps is reused for the partial shares
+  float* red = Ps;  // 4 x 32 x 32
+  mma32::store(red + quarter * 1024, acc, lane);
+  epi_sync();
+  const int m2 = ep.yf_m, m3 = ep.q, n = m2 * m3;
+  float* yo = ep.ysh + tile * n;
+  for (int e = et; e < n; e += 128) {
+    const int bb = e / m3, cc = e % m3, o = mma32::tile_index(bb, cc);
+    const float y = ((red[o] + red[o + 1024]) + red[o + 2048]) + red[o + 3072];
+    yo[ep.y_tr ? cc * m2 + bb : e] = y;
+  }
+  epi_sync();  // red and Fs are free for the next tile
+}
+
 template <int KIND, bool kMN, int NP, bool FUSE>
 __global__ void __launch_bounds__(kThreadsTc, 1)
 tc_pass_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -479,26 +537,7 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           // loaded when the range changes (never, when the grid is a multiple of
           // the tiles per slab); the previous tile ended with a barrier.
           fs_slice = tile % ep.y_nh;
-          const int64_t j = fs_slice * 128 + lr;
-          const float* f = ep.yf + j * ep.yf_m;
-          float fr[32];
-          if ((ep.yf_m & 3) == 0 && (reinterpret_cast<uintptr_t>(f) & 15) == 0) {
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const float4 q = 4 * c < ep.yf_m ? *reinterpret_cast<const float4*>(f + 4 * c)
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
-              fr[4 * c] = q.x; fr[4 * c + 1] = q.y; fr[4 * c + 2] = q.z; fr[4 * c + 3] = q.w;
-            }
-          } else {
-#pragma unroll
-            for (int b = 0; b < 32; ++b) fr[b] = b < ep.yf_m ? f[b] : 0.f;
-          }
-          // Rows of 8 float4 chunks, chunk c stored at c ^ (row & 7): the
-          // row-per-thread stores and the chunk reads below avoid bank conflicts.
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            *reinterpret_cast<float4*>(Fs + lr * 32 + ((c ^ (lr & 7)) << 2)) =
-                make_float4(fr[4 * c], fr[4 * c + 1], fr[4 * c + 2], fr[4 * c + 3]);
+          stage_factor_row(ep, fs_slice * 128 + lr, lr, Fs);
         }
       }
       const int64_t row = tile * 128 + lr;
@@ -590,35 +629,7 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&accempty[buf]);
-      if constexpr (FUSE) {
-        // Contraction of the tile (one slab s, rows j0 .. j0 + 127):
-        //   share[b, c] = sum_r F[j0 + r, b] P[(s, j0 + r), c]
-        // on the tensor cores (mma32.cuh: TF32 operands beside the BF16
-        // rounding of X, split TF32 in the FP32-accurate pass). The warp of
-        // quarter q takes rows 32 q .. 32 q + 31 with the whole 32 x 32 share
-        // (zero past m2, m3) in registers; the four partial shares are added
-        // in quarter order.
-        const int et = threadIdx.x - 64;  // 0 .. 127
-        const int o0 = mma32::frag_off(lane, 0), o1 = mma32::frag_off(lane, 1);
-        float acc[2][4][4];
-        mma32::zero(acc);
-        epi_sync();  // Ps and Fs complete
-#pragma unroll
-        for (int ks = 4 * quarter; ks < 4 * quarter + 4; ++ks)
-          mma32::step<L::kTf32 ? 3 : 1>(acc, Fs + ks * 256, Ps + ks * 256, o0, o1);
-        epi_sync();  // Ps is reused for the partial shares
-        float* red = Ps;  // 4 x 32 x 32
-        mma32::store(red + quarter * 1024, acc, lane);
-        epi_sync();
-        const int m2 = ep.yf_m, m3 = ep.q, n = m2 * m3;
-        float* yo = ep.ysh + tile * n;
-        for (int e = et; e < n; e += 128) {
-          const int bb = e / m3, cc = e % m3, o = mma32::tile_index(bb, cc);
-          const float y = ((red[o] + red[o + 1024]) + red[o + 2048]) + red[o + 3072];
-          yo[ep.y_tr ? cc * m2 + bb : e] = y;
-        }
-        epi_sync();  // red and Fs are free for the next tile
-      }
+      if constexpr (FUSE) fused_share<L::kTf32 ? 3 : 1>(ep, tile, lane, quarter, Ps, Fs);
     }
   } else if constexpr (L::kTf32) {
     // ---- TF32 split of A (warps 6-9): A <- x_hi in place, x_lo to its ring ----
@@ -668,6 +679,551 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(L::kTmemCols)
                  : "memory");
+  }
+}
+
+// ---- FP16 pair passes (kKindF16x3) ----------------------------------------------
+//
+// FP32-accurate passes on pairs of FP16 parts. X is kept as Xh + Xl, with
+//   x / (s_i t_j u_k) = x_hi + x_lo,   x_hi = fp16(.), x_lo = fp16(. - x_hi),
+// s, t, u powers of two that bring the largest entry of every slice of every mode
+// close below 2^15: where an entry is within 2^16 of the largest of its slices,
+// the pair holds 22 bits and a sign (as the TF32 pair does), below that the
+// error stays 2^-40 of the largest. B is split the same way with u or s folded in
+// and a power of two per column. x_hi [f_hi; f_lo] and x_lo f_hi are accumulated
+// as in the TF32x3 pass.
+// Why pairs made once per fit instead of TF32 parts made in every pass: the
+// TF32x3 stage moves each entry through shared memory five times (TMA in, read and
+// two writes of the split, two reads by the MMAs, 8 bytes an entry in the last
+// three) and no role of it bounds it alone, 137-151 us a pass at 512^3, m = 32. A pair
+// is as large as the FP32 entry, comes in by TMA and goes out by the MMAs, at half the
+// bytes. Both passes read the same copy: pass 1 K-major, pass 2 MN-major (no
+// transposed copy). 512^3, m = 32, in the sweep: 140 -> 105 us a pass (537 MB, 5.1
+// TB/s); 256^3, m = 20, where the pair (67 MB) stays in L2: 27 -> 20-23 us.
+//
+// Warps 0 and 1 as in tc_pass_kernel, warps 2-5 the epilogue. B stays in shared
+// memory for the whole pass: warps 2-9 read the factor, find each column's
+// largest entry, and write the split operand into the swizzled layout, while the first
+// stages of X are in flight (no operand is formed by the updates, and a stage
+// carries X alone).
+constexpr int kF16Stage = 2 * kTileBytes;  // x_hi, x_lo: 128 rows x 64 K entries
+constexpr int kF16MaxStages = 8;
+constexpr int kF16MinStages = 3;
+// Stages a set of accumulators sums before the epilogue adds them in FP32. The tensor
+// core truncates as it accumulates, one-sided on nonnegative data and more with every
+// product in an accumulator: at NP = 32 the four K steps of a stage go to four
+// accumulators, 32 products each in a group of two stages. With one group a
+// tile (64 products an accumulator at K = 256) the factors after 30 sweeps were
+// 1.5 times as far from 64 bits as with the TF32x3 passes.
+constexpr int kF16Group = 2;
+
+struct F16Operand {
+  const float* F;       // K x q row-major
+  const float* kscale;  // u or s by K index
+  int K, q;
+};
+
+template <int NP>
+__host__ __device__ constexpr int f16_b_bytes(int nk) { return nk * 2 * NP * 128; }
+// Stages that fit beside the operand and the epilogue's tiles.
+template <int NP, bool FUSE>
+__host__ __device__ inline int f16_stages(int nk) {
+  const int room = 227 * 1024 - 1536 - 1024 - f16_b_bytes<NP>(nk) - (FUSE ? 2 * 128 * 32 * 4 : 0);
+  const int n = room / kF16Stage;
+  return n > kF16MaxStages ? kF16MaxStages : n;
+}
+template <int NP, bool FUSE>
+__host__ __device__ inline int f16_smem(int nk) {
+  return 1024 + f16_stages<NP, FUSE>(nk) * kF16Stage + f16_b_bytes<NP>(nk) +
+         (FUSE ? 2 * 128 * 32 * 4 : 0);
+}
+
+__device__ __forceinline__ uint32_t f16_instr_desc(bool mn, int n) {
+  // FP16 operands (format 0), FP32 accumulator, M = 128, B K-major.
+  return (1u << 4) | ((mn ? 1u : 0u) << 15) | (static_cast<uint32_t>(n >> 3) << 17) |
+         (static_cast<uint32_t>(128 >> 4) << 24);
+}
+
+// Exponent e with 2^14 <= v 2^-e < 2^15 for the bits of a positive float, within
+// the range whose powers of two are normal floats; 0 for zero.
+__device__ __forceinline__ int f16_exponent(unsigned bits) {
+  const int e = (int)(bits >> 23) - 127 - 14;
+  return bits == 0u ? 0 : (e < -126 ? -126 : e);
+}
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+
+__device__ __forceinline__ void split_f16(float v, __half& hi, __half& lo) {
+  hi = __float2half_rn(v);
+  lo = __float2half_rn(v - __half2float(hi));
+}
+
+// The pass's B operand in shared memory (256 threads: warps 2-9): for each 64-entry
+// K chunk 2 NP rows of 128 bytes, rows [0, NP) f_hi and [NP, 2 NP) f_lo of
+// F[k, q] kscale[k] / cscale[q], in the 128-byte swizzle. cs[q] gets cscale.
+template <int NP>
+__device__ __forceinline__ void f16_operand(const F16Operand& fo, int nk, unsigned char* bs,
+                                            float* cs, unsigned* cmax) {
+  const int t = threadIdx.x - 64, lane = t & 31, w = t >> 5;
+  constexpr int NC = NP / 32;  // columns per lane
+  const int noct = nk * 8;     // octets of K entries
+  auto value = [&](int k, int n) {
+    return k < fo.K && n < fo.q ? fo.F[(int64_t)k * fo.q + n] * fo.kscale[k] : 0.f;
+  };
+  for (int n = t; n < NP; n += 256) cmax[n] = 0u;
+  asm volatile("bar.sync 2, 256;" ::: "memory");
+  float mx[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) mx[c] = 0.f;
+  for (int o = w; o < noct; o += 8) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = value(8 * o + u, lane + 32 * c);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) mx[c] = fmaxf(mx[c], fabsf(v[u]));
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) atomicMax(&cmax[lane + 32 * c], __float_as_uint(mx[c]));
+  asm volatile("bar.sync 2, 256;" ::: "memory");
+  float inv[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const int e = f16_exponent(cmax[lane + 32 * c]);
+    inv[c] = pow2f(-e);
+    if (w == 0) cs[lane + 32 * c] = pow2f(e);
+  }
+  for (int o = w; o < noct; o += 8) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int n = lane + 32 * c;
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = value(8 * o + u, n);
+      union { __half h[8]; uint4 q; } hi, lo;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) split_f16(v[u] * inv[c], hi.h[u], lo.h[u]);
+      unsigned char* row = bs + (o >> 3) * (2 * NP * 128) + n * 128 + (((o & 7) ^ (n & 7)) << 4);
+      *reinterpret_cast<uint4*>(row) = hi.q;
+      *reinterpret_cast<uint4*>(row + NP * 128) = lo.q;
+    }
+  }
+}
+
+template <bool kMN, int NP, bool FUSE>
+__global__ void __launch_bounds__(kThreadsTc, 1)
+f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__ CUtensorMap tmLo,
+                F16Operand fo, int nk, int64_t ntiles, TcEpilogue ep, int* err) {
+  static_assert(!FUSE || (NP == 32 && !kMN), "the fused contraction covers m3 <= 32 of pass 1");
+  constexpr int kAcc = 128 / NP;      // accumulators the K stages rotate over
+  constexpr int kAccCols = 2 * NP;    // [0, NP) x_hi f_hi, [NP, 2 NP) the small terms
+  constexpr int kTmemCols = 2 * kAcc * kAccCols;
+  static_assert(kTmemCols == 512, "all of the tensor memory");
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ uint64_t full[kF16MaxStages], empty[kF16MaxStages], accfull[2], accempty[2], bready;
+  __shared__ float cs[NP];
+  __shared__ unsigned cmax[NP];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int fail;
+
+  unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int nst = f16_stages<NP, FUSE>(nk);
+  unsigned char* bs = base + nst * kF16Stage;
+  unsigned char* epi = bs + f16_b_bytes<NP>(nk);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* vfail = &fail;
+  pdl_trigger();
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < nst; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&accfull[b], 1);
+      mbar_init(&accempty[b], 4);
+    }
+    mbar_init(&bready, 8);
+    fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_slot)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+
+  if (warp == 0) {
+    // ---- TMA producer ----------------------------------------------------------
+    // The pair of X is complete before any pass is launched, so its tiles are
+    // requested without waiting for the predecessor grid.
+    if (lane == 0) {
+      const int64_t my_tiles = (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
+      const uint64_t once = l2_evict_first();
+      auto load = [&](const CUtensorMap* tm, void* dst, int x, int y, uint64_t* bar) {
+        if (ep.x_resident) tma_load_2d(dst, tm, x, y, bar);
+        else tma_load_2d_hint(dst, tm, x, y, bar, once);
+      };
+      int64_t it = 0;
+      int s = 0;
+      uint32_t ph = 1;  // the first round's stages are free
+      bool ok = true;
+      for (int64_t q = 0; ok && q < my_tiles; ++q) {
+        const int m0 = static_cast<int>((blockIdx.x + q * gridDim.x) * 128);
+        for (int kc = 0; kc < nk; ++kc, ++it) {
+          if (it >= nst && !mbar_wait(&empty[s], ph, vfail)) {
+            ok = false;
+            break;
+          }
+          unsigned char* st = base + s * kF16Stage;
+          mbar_expect_tx(&full[s], kF16Stage);
+          if (!kMN) {
+            load(&tmHi, st, kc * 64, m0, &full[s]);
+            load(&tmLo, st + kTileBytes, kc * 64, m0, &full[s]);
+          } else {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              load(&tmHi, st + h * (kTileBytes / 2), m0 + h * 64, kc * 64, &full[s]);
+              load(&tmLo, st + kTileBytes + h * (kTileBytes / 2), m0 + h * 64, kc * 64, &full[s]);
+            }
+          }
+          if (++s == nst) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      if (!ok) {
+        // Let the copies this CTA started land before it can exit (bounded).
+        for (int back = 1; back <= nst && it - back >= 0; ++back) {
+          const int64_t j = it - back;
+          const long long t0 = clock64();
+          while (!mbar_try_wait(&full[j % nst], (j / nst) & 1) && clock64() - t0 < kWaitCycles) {
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ---- MMA issuer ----------------------------------------------------------------
+    if (lane == 0) {
+      const uint32_t idesc = f16_instr_desc(kMN, NP);
+      const uint32_t idesc2 = f16_instr_desc(kMN, 2 * NP);
+      const uint64_t bdesc_base = smem_desc(smem_u32(bs), 16, 1024);
+      bool ok = mbar_wait(&bready, 0, vfail);
+      int gcount = 0, rs = 0;  // groups of kF16Group stages; the ring's stage
+      uint32_t rph = 0;
+      for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+        for (int k0 = 0; ok && k0 < nk; k0 += kF16Group, ++gcount) {
+          const int buf = gcount & 1, kend = min(nk, k0 + kF16Group);
+          if (gcount >= 2 && !mbar_wait(&accempty[buf], ((gcount >> 1) - 1) & 1, vfail)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t acc0 = tmem + buf * kAcc * kAccCols;
+          for (int kc = k0; kc < kend; ++kc) {
+            if (!mbar_wait(&full[rs], rph, vfail)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t st = smem_u32(base + rs * kF16Stage);
+            const uint64_t hidesc = smem_desc(st, kMN ? kTileBytes / 2 : 16, 1024);
+            const uint64_t lodesc = smem_desc(st + kTileBytes, kMN ? kTileBytes / 2 : 16, 1024);
+            const uint64_t bdesc0 = bdesc_base + (uint64_t)((kc * 2 * NP * 128) >> 4);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+              constexpr uint32_t astep = kMN ? 2048 : 32;
+              const uint64_t astep16 = (uint64_t)((kk * astep) >> 4);
+              const uint64_t bdesc = bdesc0 + (uint64_t)((kk * 32) >> 4);
+              const uint32_t acc = acc0 + (kk & (kAcc - 1)) * kAccCols;
+              const uint32_t accum = (kc > k0 || kk >= kAcc) ? 1u : 0u;
+              mma<kKindBf16>(acc, hidesc + astep16, bdesc, idesc2, accum);
+              mma<kKindBf16>(acc + NP, lodesc + astep16, bdesc, idesc, 1u);
+            }
+            mma_commit(&empty[rs]);
+            if (++rs == nst) {
+              rs = 0;
+              rph ^= 1u;
+            }
+          }
+          if (ok) mma_commit(&accfull[buf]);
+        }
+      }
+    }
+  } else {
+    // ---- the B operand (warps 2-9) -------------------------------------------------
+    pdl_wait();
+    f16_operand<NP>(fo, nk, bs, cs, cmax);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bready);
+    asm volatile("bar.sync 2, 256;" ::: "memory");  // cs complete
+    if (warp < 6) {
+      // ---- epilogue (warps 2-5) ------------------------------------------------------
+      const int quarter = warp & 3;
+      const int lr = quarter * 32 + lane;
+      float* Ps = reinterpret_cast<float*>(epi);  // FUSE: 128 x 32 pass rows
+      float* Fs = Ps + 128 * 32;                  // FUSE: 128 x 32 factor rows
+      int gcount = 0;
+      int64_t fs_slice = -1;
+      for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        if constexpr (FUSE) {
+          if (tile % ep.y_nh != fs_slice) {
+            fs_slice = tile % ep.y_nh;
+            stage_factor_row(ep, fs_slice * 128 + lr, lr, Fs);
+          }
+        }
+        const int64_t row = tile * 128 + lr;
+        // Row (a, b) = (row / kp, row % kp): (i, j) of pass 1, (j, k) of pass 2.
+        const int64_t ra = row / ep.kp, rb = row % ep.kp;
+        const bool live = ra < ep.ra_n && rb < ep.rb_n;
+        int64_t orow = -1;
+        if (live) orow = ep.p1_layout == 2 ? rb * ep.n2 + ra : row;
+        const float rsc = live ? ep.ra_scale[ra] * ep.rb_scale[rb] : 1.f;
+        // The tile's sums: every group's accumulators added in FP32.
+        float sum[NP];
+#pragma unroll
+        for (int t = 0; t < NP; ++t) sum[t] = 0.f;
+        bool got = true;
+        for (int k0 = 0; k0 < nk; k0 += kF16Group, ++gcount) {
+          const int buf = gcount & 1;
+          got = mbar_wait(&accfull[buf], (gcount >> 1) & 1, vfail);
+          if constexpr (FUSE) got = epi_all(got);
+          else got = __all_sync(0xffffffffu, got);
+          if (!got) break;
+          tc_fence_after();
+          const uint32_t accb =
+              tmem + buf * kAcc * kAccCols + (static_cast<uint32_t>(quarter * 32) << 16);
+#pragma unroll
+          for (int c0 = 0; c0 < NP; c0 += 32) {
+#pragma unroll
+            for (int q = 0; q < kAcc; ++q) {
+              uint32_t h[32], w[32];
+              tmem_ld32(accb + q * kAccCols + c0, h);
+              tmem_ld32(accb + q * kAccCols + NP + c0, w);
+#pragma unroll
+              for (int t = 0; t < 32; ++t)
+                sum[c0 + t] += __uint_as_float(h[t]) + __uint_as_float(w[t]);
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&accempty[buf]);
+        }
+        if (!got) break;
+#pragma unroll
+        for (int c0 = 0; c0 < NP; c0 += 32) {
+          float* v = sum + c0;
+          // Powers of two: the column's first (its result is the entry without the
+          // row's scale), then the row's.
+#pragma unroll
+          for (int t = 0; t < 32; ++t)
+            v[t] = v[t] * cs[c0 + t] * rsc;
+          if (ep.p1_layout != 1) {
+            if (orow >= 0) {
+              float* o = ep.out + orow * ep.q;
+              if ((ep.q & 3) == 0) {
+#pragma unroll
+                for (int t = 0; t < 32; t += 4)
+                  if (c0 + t < ep.q)
+                    *reinterpret_cast<float4*>(o + c0 + t) =
+                        make_float4(v[t], v[t + 1],
+                                    v[t + 2], v[t + 3]);
+              } else {
+#pragma unroll
+                for (int t = 0; t < 32; ++t)
+                  if (c0 + t < ep.q) o[c0 + t] = v[t];
+              }
+            }
+            if constexpr (FUSE) {
+#pragma unroll
+              for (int t = 0; t < 32; t += 4)
+                *reinterpret_cast<float4*>(Ps + lr * 32 + (((t >> 2) ^ (lr & 7)) << 2)) =
+                    make_float4(t < ep.q ? v[t] : 0.f,
+                                t + 1 < ep.q ? v[t + 1] : 0.f,
+                                t + 2 < ep.q ? v[t + 2] : 0.f,
+                                t + 3 < ep.q ? v[t + 3] : 0.f);
+            }
+          } else if (live) {
+            float* o = ep.out + ra * ep.n3 + rb;
+#pragma unroll
+            for (int t = 0; t < 32; ++t)
+              if (c0 + t < ep.q) o[static_cast<int64_t>(c0 + t) * ep.slab] = v[t];
+          }
+        }
+        if constexpr (FUSE) fused_share<3>(ep, tile, lane, quarter, Ps, Fs);
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && fail) atomicExch(err, 1);
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"(kTmemCols)
+                 : "memory");
+  }
+}
+
+// ---- the FP16 pair of X ------------------------------------------------------------
+
+// rmax[r] = bits of max_k |X[r, k]| over the rows of X (R x N3): LW lanes a row (the
+// power of two at and above its 16-byte pieces, at most a warp), two rows in
+// flight per lane group.
+__global__ void __launch_bounds__(256)
+row_max_kernel(const float* __restrict__ X, int64_t R, int N3, int lw, unsigned* __restrict__ rmax) {
+  const int lane = threadIdx.x & (lw - 1);
+  const int64_t groups = (int64_t)gridDim.x * (blockDim.x / lw);
+  const int64_t g0 = (int64_t)blockIdx.x * (blockDim.x / lw) + threadIdx.x / lw;
+  const int nv = N3 >> 2;
+  // Every group runs the same number of rounds: the shuffles take whole warps.
+  const int64_t rounds = (R + 2 * groups - 1) / (2 * groups);
+  for (int64_t q0 = 0; q0 < rounds; ++q0) {
+    const int64_t r = g0 + q0 * 2 * groups;
+    const bool one = r < R, two = r + groups < R;
+    const float4* a = reinterpret_cast<const float4*>(X + (one ? r : 0) * N3);
+    const float4* b = reinterpret_cast<const float4*>(X + (two ? r + groups : 0) * N3);
+    float ma = 0.f, mb = 0.f;
+#pragma unroll 4
+    for (int v = lane; v < nv; v += lw) {
+      const float4 p = a[v], q = b[v];
+      ma = fmaxf(ma, fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fmaxf(fabsf(p.z), fabsf(p.w))));
+      mb = fmaxf(mb, fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fmaxf(fabsf(q.z), fabsf(q.w))));
+    }
+    for (int o = lw >> 1; o > 0; o >>= 1) {
+      ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+      mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+    }
+    if (lane == 0) {
+      if (one) rmax[r] = __float_as_uint(ma);
+      if (two) rmax[r + groups] = __float_as_uint(mb);
+    }
+  }
+}
+
+// s_i for mode-1 slice i: 2^e with 2^14 <= max 2^-e < 2^15, e >= kF16MinS so that
+// s_i t_j u_k stays a normal float.
+constexpr int kF16MinS = -96, kF16MinT = -15;
+__global__ void __launch_bounds__(256)
+slice_s_kernel(const unsigned* __restrict__ rmax, int64_t N2, float* __restrict__ s) {
+  __shared__ unsigned m;
+  if (threadIdx.x == 0) m = 0u;
+  __syncthreads();
+  unsigned v = 0u;
+  for (int64_t j = threadIdx.x; j < N2; j += blockDim.x) {
+    const unsigned x = rmax[(int64_t)blockIdx.x * N2 + j];
+    v = x > v ? x : v;
+  }
+  atomicMax(&m, __reduce_max_sync(0xffffffffu, v));
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int e = f16_exponent(m);
+    s[blockIdx.x] = pow2f(m == 0u ? 0 : (e < kF16MinS ? kF16MinS : e));
+  }
+}
+
+// The power of two t in [2^kF16MinT, 1] that brings a slice whose largest scaled entry
+// is max < 2^15 to 2^14 or more (1 for a slice of zeros).
+__device__ __forceinline__ float slice_t(float mx) {
+  if (!(mx > 0.f)) return 1.f;
+  const int e = f16_exponent(__float_as_uint(mx));
+  return pow2f(e > 0 ? 0 : (e < kF16MinT ? kF16MinT : e));
+}
+
+__global__ void __launch_bounds__(256)
+slice_t_kernel(const unsigned* __restrict__ rmax, const float* __restrict__ s, int64_t N1,
+               int64_t N2, float* __restrict__ t) {
+  const int64_t j = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  __shared__ float part[8][32];
+  float m = 0.f;
+  if (j < N2)
+    for (int64_t i = threadIdx.x >> 5; i < N1; i += 8)
+      m = fmaxf(m, __uint_as_float(rmax[i * N2 + j]) * (1.f / s[i]));
+  part[threadIdx.x >> 5][threadIdx.x & 31] = m;
+  __syncthreads();
+  if (threadIdx.x < 32 && j < N2) {
+    for (int w = 1; w < 8; ++w) m = fmaxf(m, part[w][threadIdx.x]);
+    t[j] = slice_t(m);
+  }
+}
+
+// umax[k] = bits of max over the rows (i, j) of |X| / (s_i t_j): a block takes
+// 4 tx columns k (tx a power of two, at most 64, so that short rows use every
+// thread too) and every gridDim.x-th group of 256 / tx rows.
+__global__ void __launch_bounds__(256)
+col_max_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int tx,
+               const float* __restrict__ s, const float* __restrict__ t,
+               unsigned* __restrict__ umax) {
+  const int k = 4 * (blockIdx.y * tx + (threadIdx.x & (tx - 1)));
+  const int ty = 256 / tx, sub = threadIdx.x / tx;
+  float m[4] = {0.f, 0.f, 0.f, 0.f};
+  if (k < N3) {
+#pragma unroll 4
+    for (int64_t r = (int64_t)blockIdx.x * ty + sub; r < R; r += (int64_t)ty * gridDim.x) {
+      const int i = (int)(r / N2);
+      const float inv = (1.f / s[i]) * (1.f / t[r - (int64_t)i * N2]);
+      const float4 x = *reinterpret_cast<const float4*>(X + r * N3 + k);
+      m[0] = fmaxf(m[0], fabsf(x.x) * inv);
+      m[1] = fmaxf(m[1], fabsf(x.y) * inv);
+      m[2] = fmaxf(m[2], fabsf(x.z) * inv);
+      m[3] = fmaxf(m[3], fabsf(x.w) * inv);
+    }
+  }
+  __shared__ float part[1024];  // [row group][4 tx]
+#pragma unroll
+  for (int c = 0; c < 4; ++c) part[threadIdx.x * 4 + c] = m[c];
+  __syncthreads();
+  const int col = blockIdx.y * 4 * tx + threadIdx.x;
+  if (threadIdx.x < 4 * tx && col < N3) {
+    float v = part[threadIdx.x];
+    for (int q = 1; q < ty; ++q) v = fmaxf(v, part[q * 4 * tx + threadIdx.x]);
+    if (v > 0.f) atomicMax(&umax[col], __float_as_uint(v));
+  }
+}
+
+__global__ void slice_u_kernel(const unsigned* __restrict__ umax, int N3, int n3p,
+                               float* __restrict__ u) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n3p) u[k] = k < N3 ? slice_t(__uint_as_float(umax[k])) : 1.f;
+}
+
+// Xh, Xl (rows of n3p entries, zero past N3) from X: eight entries a thread.
+__global__ void __launch_bounds__(256)
+x_to_pair_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int n3p,
+                 const float* __restrict__ s, const float* __restrict__ t,
+                 const float* __restrict__ u, __half* __restrict__ Xh, __half* __restrict__ Xl) {
+  const int oct = n3p >> 3;
+  const int64_t n = R * oct;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = e / oct;
+    const int k = (int)(e - r * oct) * 8;
+    const int64_t i = r / N2;
+    const float inv = (1.f / s[i]) * (1.f / t[r - i * N2]);
+    const float* x = X + r * N3 + k;
+    float v[8];
+    // N3 % 4 == 0: the first four entries exist, the last four all or none.
+    const float4 a = *reinterpret_cast<const float4*>(x);
+    const float4 b = k + 4 < N3 ? *reinterpret_cast<const float4*>(x + 4)
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    union { __half h[8]; uint4 q; } hi, lo;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) split_f16(v[q] * inv * (1.f / u[k + q]), hi.h[q], lo.h[q]);
+    *reinterpret_cast<uint4*>(Xh + r * n3p + k) = hi.q;
+    *reinterpret_cast<uint4*>(Xl + r * n3p + k) = lo.q;
   }
 }
 
@@ -805,28 +1361,45 @@ int make_map(CUtensorMap* tm, CUtensorMapDataType dt, const void* base, uint64_t
   return NNC_OK;
 }
 
+// Fewest CTAs that keep the largest tile count per CTA of a grid over the
+// SMs the pass may take: the time is the same, and the SMs left over run
+// the small kernels of the sweep that the graph places beside the pass.
+// With at least min_tiles tiles per SM the pass leaves `reserve` SMs to them. With y_nh
+// tiles per slab (a fused pass) a grid that is a multiple of them gives every
+// CTA tiles of one j range only, so it loads its factor rows once per pass.
+int64_t pass_grid(int64_t tiles, int reserve, int64_t y_nh, int min_tiles) {
+  const int sms = device_sm_count();
+  const int avail = (tiles >= (int64_t)min_tiles * sms && reserve > 0 && reserve < sms / 2) ? sms - reserve : sms;
+  const int64_t per = ceil_div(tiles, (int64_t)avail);
+  int64_t grid = ceil_div(tiles, per);
+  if (y_nh > 1) {
+    const int64_t up = ceil_div(grid, y_nh) * y_nh;
+    if (up <= avail) grid = up;
+    else if (avail >= y_nh) grid = avail / y_nh * y_nh;
+  }
+  return grid;
+}
+
 template <int KIND, bool kMN, int NP, bool FUSE>
 int launch_pass(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& blo, int nk,
                 int64_t tiles, const TcEpilogue& ep, int* err, int reserve, cudaStream_t s) {
   constexpr int smem = TcLayout<KIND, NP, FUSE>::kSmem;
   NNC_CUDA_TRY(raise_smem_limit((const void*)tc_pass_kernel<KIND, kMN, NP, FUSE>, smem));
-  // Fewest CTAs that keep the largest tile count per CTA of a grid over the
-  // SMs the pass may take: the time is the same, and the SMs left over run
-  // the small kernels of the sweep that the graph places beside the pass.
-  // With at least 8 tiles per SM the pass leaves `reserve` SMs to them.
-  const int sms = device_sm_count();
-  const int avail = (tiles >= 8LL * sms && reserve > 0 && reserve < sms / 2) ? sms - reserve : sms;
-  const int64_t per = ceil_div(tiles, (int64_t)avail);
-  int64_t grid = ceil_div(tiles, per);
-  if (FUSE && ep.y_nh > 1) {
-    // A grid that is a multiple of the tiles per slab gives every CTA tiles
-    // of one j range only, so it loads its factor rows once per pass.
-    const int64_t up = ceil_div(grid, ep.y_nh) * ep.y_nh;
-    if (up <= avail) grid = up;
-    else if (avail >= ep.y_nh) grid = avail / ep.y_nh * ep.y_nh;
-  }
+  const int64_t grid = pass_grid(tiles, reserve, FUSE ? ep.y_nh : 1, /*min_tiles=*/8);
   NNC_CUDA_TRY(launch_pdl(tc_pass_kernel<KIND, kMN, NP, FUSE>, dim3(static_cast<unsigned>(grid)),
                           dim3(kThreadsTc), smem, s, a, b, blo, nk, tiles, ep, err));
+  note_launch(s);
+  return NNC_OK;
+}
+
+template <bool kMN, int NP, bool FUSE>
+int launch_f16(const CUtensorMap& hi, const CUtensorMap& lo, const F16Operand& fo, int nk,
+               int64_t tiles, const TcEpilogue& ep, int* err, int reserve, cudaStream_t s) {
+  const int smem = f16_smem<NP, FUSE>(nk);
+  NNC_CUDA_TRY(raise_smem_limit((const void*)f16_pass_kernel<kMN, NP, FUSE>, smem));
+  const int64_t grid = pass_grid(tiles, reserve, FUSE ? ep.y_nh : 1, /*min_tiles=*/1);
+  NNC_CUDA_TRY(launch_pdl(f16_pass_kernel<kMN, NP, FUSE>, dim3(static_cast<unsigned>(grid)),
+                          dim3(kThreadsTc), smem, s, hi, lo, fo, nk, tiles, ep, err));
   note_launch(s);
   return NNC_OK;
 }
@@ -845,7 +1418,7 @@ int launch_np(int np, const CUtensorMap& a, const CUtensorMap& b, const CUtensor
 }  // namespace
 
 int TcPlan::init(int kind_, const float* X, int64_t N1_, int64_t N2_, int64_t N3_, int m1_,
-                 int m3_, Scratch& sc, cudaStream_t s, bool p1_kj_) {
+                 int m3_, Scratch& sc, cudaStream_t s, bool p1_kj_, bool need_p1) {
   kind = kind_;
   p1_kj = p1_kj_;
   N1 = N1_;
@@ -855,15 +1428,18 @@ int TcPlan::init(int kind_, const float* X, int64_t N1_, int64_t N2_, int64_t N3
   m3 = m3_;
   np1 = m1 <= 32 ? 32 : 64;
   np3 = m3 <= 32 ? 32 : 64;
-  const int kstage = kind == kKindBf16 ? 64 : 32;
+  const int kstage = kind == kKindTf32x3 ? 32 : 64;
   // K of pass 1 is N3 (BF16: padded rows of Xb), K of pass 2 is N1.
-  kp3 = kind == kKindBf16 ? static_cast<int>(ceil_div(N3, 64) * 64) : static_cast<int>(N3);
+  kp3 = kind == kKindBf16 ? static_cast<int>(ceil_div(N3, 64) * 64)
+        : kind == kKindF16x3 ? static_cast<int>(ceil_div(N3, 8) * 8)
+                             : static_cast<int>(N3);
   kb3 = static_cast<int>(ceil_div(N3, kstage) * kstage);
   kp1 = static_cast<int>(ceil_div(N1, kstage) * kstage);
   if (m1 > 64 || m3 > 64 || N1 * N2 > (1LL << 31) || N2 * kp3 > (1LL << 31)) {
     set_error_detail_text("tensor-core pass: shape outside the path (m <= 64)");
     return NNC_ERR_UNSUPPORTED;
   }
+  if (kind == kKindF16x3) return init_f16(X, sc, s);
   if (kind == kKindTf32x3 && (N3 % 4) != 0) {
     set_error_detail_text("tensor-core TF32 pass: N3 must be a multiple of 4");
     return NNC_ERR_UNSUPPORTED;
@@ -910,6 +1486,7 @@ int TcPlan::init(int kind_, const float* X, int64_t N1_, int64_t N2_, int64_t N3
     NNC_TRY(make_map(&mapA3, f32, X, N3, rows, static_cast<uint64_t>(N3) * 4, 32, 128));
     NNC_TRY(make_map(&mapB3, f32, B3hi, kb3, np3, static_cast<uint64_t>(kb3) * 4, 32, np3));
     NNC_TRY(make_map(&mapB3lo, f32, B3lo, kb3, np3, static_cast<uint64_t>(kb3) * 4, 32, np3));
+    if (!need_p1) return NNC_OK;
     // Pass 2 reads Xt = X viewed (N1 x N2 N3), transposed: K-major rows of N1p
     // in the order (j, k), or (k, j) for p1_kj.
     const int64_t C = N2 * N3, n1p = ceil_div(N1, 4) * 4;
@@ -931,7 +1508,81 @@ int TcPlan::init(int kind_, const float* X, int64_t N1_, int64_t N2_, int64_t N3
   return NNC_OK;
 }
 
+// The shapes the FP16 pair passes take: rows of X on 16 bytes, and both passes'
+// operands (K x m, split, in shared memory for the whole pass) beside three
+// stages at least: K up to 768 for m <= 32, 384 for m <= 64 (512 and 256 less the
+// fused contraction's tiles).
+int TcPlan::init_f16(const float* X, Scratch& sc, cudaStream_t s) {
+  const int64_t rows = N1 * N2;
+  const int nk3 = kb3 / 64, nk1 = kp1 / 64;
+  const int st3 = np3 == 32 ? f16_stages<32, true>(nk3) : f16_stages<64, false>(nk3);
+  const int st1 = np1 == 32 ? f16_stages<32, false>(nk1) : f16_stages<64, false>(nk1);
+  if (N3 % 4 != 0 || (reinterpret_cast<uintptr_t>(X) & 15) != 0 || st3 < kF16MinStages ||
+      st1 < kF16MinStages || N2 > (1LL << 30)) {
+    set_error_detail_text("FP16 pair pass: shape outside the path");
+    return NNC_ERR_UNSUPPORTED;
+  }
+  unsigned *rmax = nullptr, *umax = nullptr;
+  NNC_TRY(sc.get(&err, 1));
+  NNC_TRY(sc.get(&scale, static_cast<size_t>(N1)));
+  NNC_TRY(sc.get(&sc_t, static_cast<size_t>(N2)));
+  NNC_TRY(sc.get(&sc_u, static_cast<size_t>(kp3)));
+  NNC_TRY(sc.get(&rmax, static_cast<size_t>(rows)));
+  NNC_TRY(sc.get(&umax, static_cast<size_t>(N3)));
+  NNC_TRY(sc.get(&Xh, static_cast<size_t>(rows * kp3)));
+  NNC_TRY(sc.get(&Xl, static_cast<size_t>(rows * kp3)));
+  const int sms = device_sm_count();
+  int lw = 1;
+  while (lw < 32 && lw < N3 / 4) lw *= 2;
+  const int64_t per_block = 256 / lw;
+  const int64_t rb = ceil_div(rows, 2 * per_block);
+  row_max_kernel<<<(unsigned)(rb < 16LL * sms ? rb : 16LL * sms), 256, 0, s>>>(
+      X, rows, (int)N3, lw, rmax);
+  note_launch(s);
+  slice_s_kernel<<<(unsigned)N1, 256, 0, s>>>(rmax, N2, scale);
+  note_launch(s);
+  slice_t_kernel<<<(unsigned)ceil_div(N2, 32), 256, 0, s>>>(rmax, scale, N1, N2, sc_t);
+  note_launch(s);
+  NNC_CUDA_TRY(cudaMemsetAsync(umax, 0, sizeof(unsigned) * N3, s));
+  int tx = 1;
+  while (tx < 64 && 4 * tx < N3) tx *= 2;
+  const int64_t ky = ceil_div(N3, 4 * tx);
+  const int64_t cb = ceil_div(rows, 4 * (256 / tx));
+  const int64_t cx = ceil_div(8LL * sms, ky);
+  col_max_kernel<<<dim3((unsigned)(cb < cx ? cb : cx), (unsigned)ky), 256, 0, s>>>(
+      X, rows, (int)N2, (int)N3, tx, scale, sc_t, umax);
+  note_launch(s);
+  slice_u_kernel<<<(unsigned)ceil_div(kp3, 256), 256, 0, s>>>(umax, (int)N3, kp3, sc_u);
+  note_launch(s);
+  const int64_t n = rows * (kp3 / 8);
+  const int64_t xb = ceil_div(n, 256);
+  x_to_pair_kernel<<<(unsigned)(xb < 32LL * sms ? xb : 32LL * sms), 256, 0, s>>>(
+      X, rows, (int)N2, (int)N3, kp3, scale, sc_t, sc_u, Xh, Xl);
+  note_launch(s);
+  NNC_CUDA_TRY(cudaGetLastError());
+  // After the conversion: a pass launched as a programmatic dependent reads the pair
+  // before it waits for its predecessor, so that must not be the conversion.
+  NNC_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
+  // The pair stays in L2 (129 MB) from pass to pass with room for the pass results.
+  x_resident = 4 * rows * kp3 <= 80LL << 20;
+  const CUtensorMapDataType h = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+  const uint64_t ld = static_cast<uint64_t>(kp3) * 2, ldw = static_cast<uint64_t>(N2) * kp3 * 2;
+  NNC_TRY(make_map(&mapA3, h, Xh, kp3, rows, ld, 64, 128));
+  NNC_TRY(make_map(&mapL3, h, Xl, kp3, rows, ld, 64, 128));
+  NNC_TRY(make_map(&mapA1, h, Xh, static_cast<uint64_t>(N2) * kp3, N1, ldw, 64, 64));
+  NNC_TRY(make_map(&mapL1, h, Xl, static_cast<uint64_t>(N2) * kp3, N1, ldw, 64, 64));
+  return NNC_OK;
+}
+
+int TcPlan::init_fp32(const float* X, int64_t N1_, int64_t N2_, int64_t N3_, int m1_, int m3_,
+                      Scratch& sc, cudaStream_t s, bool p1_kj_) {
+  const int st = init(kKindF16x3, X, N1_, N2_, N3_, m1_, m3_, sc, s, p1_kj_);
+  if (st != NNC_ERR_UNSUPPORTED) return st;
+  return init(kKindTf32x3, X, N1_, N2_, N3_, m1_, m3_, sc, s, p1_kj_);
+}
+
 int TcPlan::convert_b3(const float* F3, cudaStream_t s) const {
+  if (kind == kKindF16x3) return NNC_OK;  // the pass forms its operand
   factor_b_kernel<<<64, 256, 0, s>>>(F3, static_cast<int>(N3), m3, kb3, np3, nullptr, Bt3, B3hi,
                                      B3lo);
   note_launch(s);
@@ -940,6 +1591,7 @@ int TcPlan::convert_b3(const float* F3, cudaStream_t s) const {
 }
 
 int TcPlan::convert_b1(const float* F1, cudaStream_t s) const {
+  if (kind == kKindF16x3) return NNC_OK;
   factor_b_kernel<<<64, 256, 0, s>>>(F1, static_cast<int>(N1), m1, kp1, np1,
                                      kind == kKindBf16 ? scale : nullptr, Bt1, B1hi, B1lo);
   note_launch(s);
@@ -977,6 +1629,19 @@ int TcPlan::pass3(const float* F3, float* P3, cudaStream_t s, bool convert, cons
     ep.y_nh = N2 / 128;
   }
   const int64_t tiles = ceil_div(N1 * N2, 128);
+  if (kind == kKindF16x3) {
+    ep.kp = N2;  // tile row (i, j)
+    ep.ra_scale = scale;
+    ep.ra_n = N1;
+    ep.rb_scale = sc_t;
+    ep.rb_n = N2;
+    ep.x_resident = x_resident;
+    const F16Operand fo{F3, sc_u, static_cast<int>(N3), m3};
+    const int nkf = kb3 / 64, rsv = reserve_sms;
+    if (ep.ysh) return launch_f16<false, 32, true>(mapA3, mapL3, fo, nkf, tiles, ep, err, rsv, s);
+    if (np3 == 32) return launch_f16<false, 32, false>(mapA3, mapL3, fo, nkf, tiles, ep, err, rsv, s);
+    return launch_f16<false, 64, false>(mapA3, mapL3, fo, nkf, tiles, ep, err, rsv, s);
+  }
   const int stagek = kind == kKindBf16 ? 64 : 32;
   const int nk = static_cast<int>(ceil_div(N3, stagek));
   if (kind == kKindBf16)
@@ -998,8 +1663,8 @@ int TcPlan::pass1(const float* F1, float* P1, cudaStream_t s, bool convert, cons
   ep.slab = N2 * N3;
   if (!p1_kj) {
     ep.p1_layout = 1;
-  } else if (kind == kKindBf16) {
-    ep.p1_layout = 2;  // MN-major tiles of Xb have rows (j, k)
+  } else if (kind != kKindTf32x3) {
+    ep.p1_layout = 2;  // MN-major tiles of Xb (Xh, Xl) have rows (j, k)
   } else {
     ep.p1_layout = 0;  // Xt already has rows (k, j)
     ep.rows = N2 * N3;
@@ -1013,6 +1678,17 @@ int TcPlan::pass1(const float* F1, float* P1, cudaStream_t s, bool convert, cons
     ep.y_nh = N2 / 128;
   }
   const int64_t tiles = ceil_div(N2 * kp3, 128);
+  if (kind == kKindF16x3) {
+    ep.ra_scale = sc_t;  // tile row (j, k)
+    ep.ra_n = N2;
+    ep.rb_scale = sc_u;
+    ep.rb_n = N3;
+    ep.x_resident = x_resident;
+    const F16Operand fo{F1, scale, static_cast<int>(N1), m1};
+    const int nkf = kp1 / 64, rsv = reserve_sms;
+    if (np1 == 32) return launch_f16<true, 32, false>(mapA1, mapL1, fo, nkf, tiles, ep, err, rsv, s);
+    return launch_f16<true, 64, false>(mapA1, mapL1, fo, nkf, tiles, ep, err, rsv, s);
+  }
   const int stagek = kind == kKindBf16 ? 64 : 32;
   const int nk = static_cast<int>(ceil_div(N1, stagek));
   if (kind == kKindBf16)

@@ -3,6 +3,7 @@
 
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "common.cuh"
 
@@ -11,6 +12,7 @@ namespace tc {
 
 constexpr int kKindBf16 = 0;
 constexpr int kKindTf32x3 = 1;
+constexpr int kKindF16x3 = 2;
 
 // Where and how the epilogue writes one pass's FP32 result.
 struct TcEpilogue {
@@ -41,6 +43,12 @@ struct TcEpilogue {
   int yf_m;
   int y_tr;
   int64_t y_nh;
+  // FP16 pairs: tile row = (a, b) = (row / kp, row % kp), written when a < ra_n
+  // and b < rb_n, times ra_scale[a] rb_scale[b]. x_resident: the pair stays in
+  // L2 from pass to pass (no evict-first hint).
+  const float *ra_scale, *rb_scale;
+  int64_t ra_n, rb_n;
+  int x_resident;
 };
 
 // Operands and TMA descriptors of the two passes over a 3-way FP32 X.
@@ -49,6 +57,9 @@ struct TcEpilogue {
 //   TF32x3: X itself for pass 1, a transposed copy Xt (N2 N3 x N1p, i
 //           contiguous; rows (j, k), or (k, j) with p1_kj) so that pass 2 is
 //           K-major too, and hi / lo TF32 operands B1hi/B1lo, B3hi/B3lo.
+//   F16x3:  X as a pair of FP16 copies Xh, Xl (rows padded to a multiple of 8,
+//           power-of-two scales s, t, u per slice of modes 1, 2, 3) that both
+//           passes read; they form their B operand themselves (tc_ttm.cu).
 // B operands are [np x k] row-major, zero outside the factor.
 struct TcPlan {
   int kind = kKindBf16;
@@ -60,17 +71,27 @@ struct TcPlan {
   __nv_bfloat16 *Xb = nullptr, *Bt1 = nullptr, *Bt3 = nullptr;
   float *B1hi = nullptr, *B1lo = nullptr, *B3hi = nullptr, *B3lo = nullptr, *Xt = nullptr;
   float *scale = nullptr, *inv_scale = nullptr;
+  __half *Xh = nullptr, *Xl = nullptr;
+  float *sc_t = nullptr, *sc_u = nullptr;  // F16x3: t and u (s is in `scale`)
+  int x_resident = 0;
+  CUtensorMap mapL3, mapL1;  // F16x3: Xl as operand A of pass 1 and pass 2
   int* err = nullptr;
-  // SMs a pass of at least 8 tiles per SM leaves to kernels that run beside
-  // it (the nnTD sweep's small kernels); 0: every SM.
+  // SMs a pass of at least 8 tiles per SM (F16x3: of any number) leaves to
+  // kernels that run beside it (the nnTD sweep's small kernels); 0: every SM.
   int reserve_sms = 0;
   CUtensorMap mapA3, mapB3, mapB3lo, mapA1, mapB1, mapB1lo;
 
   // Builds the operand buffers (BF16: Xb and the scales) from X, stream-ordered.
   // UNSUPPORTED when the shape is outside the path (m_n > 64; TF32x3 also
   // needs N3 % 4 == 0 for its TMA row strides).
+  // need_p1 = false: pass1 will not be called (TF32x3 then makes no copy of X).
   int init(int kind, const float* X, int64_t N1, int64_t N2, int64_t N3, int m1, int m3,
-           Scratch& sc, cudaStream_t s, bool p1_kj = false);
+           Scratch& sc, cudaStream_t s, bool p1_kj = false, bool need_p1 = true);
+  // FP32-accurate passes that a fit runs again and again: F16x3 where the shape
+  // allows it, else TF32x3.
+  int init_fp32(const float* X, int64_t N1, int64_t N2, int64_t N3, int m1, int m3, Scratch& sc,
+                cudaStream_t s, bool p1_kj = false);
+  int init_f16(const float* X, Scratch& sc, cudaStream_t s);  // part of init
   // B operands from the current factor (BF16: F^(1) scaled by s).
   int convert_b3(const float* F3, cudaStream_t s) const;
   int convert_b1(const float* F1, cudaStream_t s) const;

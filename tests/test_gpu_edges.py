@@ -76,3 +76,32 @@ def test_scratch_is_kept_bounded_and_given_back():
     # The scratch of the call holds a copy of X (64 MiB) and more; 4 GiB is the most
     # the library keeps.
     assert 64 << 20 <= freed <= 4 << 30
+
+
+# The FP16 pair passes through one nnTD sweep: K just past a 64-entry chunk and a group of
+# two, tiles with a remainder, NP = 64, the fused contraction (N2 % 128 == 0), slices of very
+# different magnitude and zero slices, and operands past what a block holds (TF32x3).
+# One sweep of FP32-accurate arithmetic on sums of up to a few thousand positive terms:
+# 1e-4 elementwise, as the other FP32 kernels.
+@pytest.mark.parametrize("dims,m,scaled", [
+    ((65, 33, 68), (5, 4, 3), False), ((130, 20, 132), (33, 5, 40), False),
+    ((24, 128, 72), (6, 8, 32), True), ((3, 256, 4), (2, 3, 4), True),
+    ((129, 7, 516), (8, 6, 20), True), ((800, 6, 20), (4, 4, 4), False),
+    ((17, 9, 900), (4, 4, 4), False)])
+def test_pair_passes_one_sweep(dims, m, scaled):
+    X, _, F0, G0, _ = inputs.small_problem(dims, 3, m, 2, seed=91)
+    if scaled:
+        rng = np.random.default_rng(3)
+        for n in range(3):
+            s = 10.0 ** rng.uniform(-3, 3, dims[n])
+            s[rng.integers(dims[n])] = 0.0
+            X = X * s.reshape([-1 if k == n else 1 for k in range(3)])
+    X = X.astype(np.float32).astype(np.float64)
+    F0 = [f.astype(np.float32).astype(np.float64) for f in F0]
+    G0 = G0.astype(np.float32).astype(np.float64)
+    F, G = [_dev(f, torch.float32) for f in F0], _dev(G0, torch.float32)
+    err, _ = native.ntd_fit(_dev(X, torch.float32), F, G, 1, precision="fp32")
+    Fo, Go, _ = orc.ntd_fit(X, F0, G0, 1)
+    for a, b in zip(F + [G], Fo + [Go]):
+        np.testing.assert_allclose(a.cpu().numpy(), b, rtol=1e-4, atol=1e-30)
+    assert abs(err - orc.rel_err_tucker(X, Go, Fo)) <= 1e-5
