@@ -557,6 +557,7 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
       fast = &plan16;
     }
     if (passes >= 1 && (passes == 1 || o->refine_iters > 0 || trigger)) {
+      plan32.rmax = plan16.rmax;
       const int st = plan32.init_fp32(X, N1, N2, N3, m1, m3, sc, s, /*p1_kj=*/true);
       // The FP16 pair passes stream X fast enough that the side kernels would be the
       // longer branch on the few SMs a full grid leaves: 512^3, m = 32, SMs left 0, 8,

@@ -10,6 +10,8 @@
 // a tile of rows (U rows in shared memory), forms X_hat in T and accumulates
 // (x - x_hat)^2 and x^2 (FP32 per thread for float data, FP64 across threads
 // and blocks); per-block partials are added in block order.
+#include <type_traits>
+
 #include "kernels.cuh"
 #include "residual.cuh"
 
@@ -29,22 +31,40 @@ __global__ void lift_kernel(const T* __restrict__ F, const T* __restrict__ B, in
   }
 }
 
-// out[l, q, c] = sum_j A[q, j] Y[l, j, c] for any Q (one thread per output).
+// out[l, q, c] = sum_j A[q, j] Y[l, j, c] for any Q, J <= 64: a block takes 256
+// flattened columns (l, c) and 16 outputs q, so an entry of Y serves 16 products and the
+// writes of out, the largest array here, are whole rows of c. (One thread per output
+// read Y once per product and divided for every output: the three products of a
+// 128^3 x 64 fit, 134 MB written by the last, 400 -> 98 us.)
+constexpr int kMpThreads = 256, kMpQ = 16;
 template <typename T>
-__global__ void mode_product_any_kernel(const T* __restrict__ Y, int64_t L, int J, int64_t C,
-                                        const T* __restrict__ A, int Q, T* __restrict__ out) {
-  const int64_t n = L * Q * C;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = e % C;
-    const int64_t q = (e / C) % Q;
-    const int64_t l = e / (C * Q);
-    const T* y = Y + l * J * C + c;
-    const T* a = A + q * J;
-    T s = T(0);
-    for (int j = 0; j < J; ++j) s = fma(a[j], y[(int64_t)j * C], s);
-    out[e] = s;
+__global__ void __launch_bounds__(kMpThreads)
+mode_product_any_kernel(const T* __restrict__ Y, int64_t L, int J, int64_t C,
+                        const T* __restrict__ A, int Q, T* __restrict__ out) {
+  __shared__ T as[64 * kMpQ];
+  const int q0 = blockIdx.y * kMpQ, qn = Q - q0 < kMpQ ? Q - q0 : kMpQ;
+  for (int e = threadIdx.x; e < J * kMpQ; e += kMpThreads) {
+    const int j = e / kMpQ, q = e % kMpQ;
+    as[e] = q < qn ? A[(int64_t)(q0 + q) * J + j] : T(0);
   }
+  __syncthreads();
+  const int64_t col = (int64_t)blockIdx.x * kMpThreads + threadIdx.x;
+  if (col >= L * C) return;
+  const int64_t l = col / C, c = col - l * C;
+  const T* y = Y + l * J * C + c;
+  T acc[kMpQ];
+#pragma unroll
+  for (int q = 0; q < kMpQ; ++q) acc[q] = T(0);
+#pragma unroll 4
+  for (int j = 0; j < J; ++j) {
+    const T v = y[(int64_t)j * C];
+#pragma unroll
+    for (int q = 0; q < kMpQ; ++q) acc[q] = fma(as[j * kMpQ + q], v, acc[q]);
+  }
+  T* o = out + (l * Q + q0) * C + c;
+#pragma unroll
+  for (int q = 0; q < kMpQ; ++q)
+    if (q < qn) o[q * C] = acc[q];
 }
 
 template <typename T>
@@ -60,75 +80,158 @@ __global__ void cp_rows_kernel(const T* __restrict__ A1, const T* __restrict__ A
   }
 }
 
-constexpr int kResThreads = 256;
-constexpr int kResRows = 64;
+constexpr int kResThreads = 128;
+// U rows staged at a time (16 KB of FP32: a thread of a short-rowed X walks few of them).
+__host__ __device__ constexpr int res_rows(int km) { return 4096 / km; }
 
-// Block (k tile of kResThreads, row tile of kResRows). Thread k keeps F3[k, :]
-// in registers (KM >= K entries, zero past K); the block's U rows sit in
-// shared memory and are read as broadcasts. Per element: x_hat = U[t, :] .
-// F3[k, :] in T, then (x - x_hat)^2 and x^2. For T = float the thread adds its
-// rows' terms in FP32 (rounded to nearest, so the errors are unbiased and
-// shrink in the FP64 sums that follow); GB300's FP64 rate is far below its
+// The k tile of a block: tx threads (a power of two, so that short rows of X use
+// every thread) times KT columns each; rows per block.
+template <typename T>
+__host__ __device__ constexpr int res_kt(int km) { return sizeof(T) == 8 ? 1 : 64 / km; }
+template <typename T>
+inline int res_km(int K) { return K <= 16 ? 16 : (K <= 32 ? 32 : 64); }
+struct ResGrid {
+  int tx, rows;
+  int64_t ktiles, blocks;
+};
+template <typename T>
+ResGrid res_grid(int64_t R, int64_t N3, int K) {
+  const int kt = res_kt<T>(res_km<T>(K));
+  ResGrid g;
+  g.tx = 1;
+  while (g.tx < kResThreads && (int64_t)g.tx * kt < N3) g.tx *= 2;
+  g.ktiles = ceil_div(N3, (int64_t)g.tx * kt);
+  // A block loads its columns' rows of F^(d) once: as many rows as still leave several
+  // blocks per SM.
+  const int chunk = res_rows(res_km<T>(K));
+  g.rows = 64;
+  while (g.rows < 2 * chunk && g.ktiles * ceil_div(R, 2 * g.rows) >= 6LL * device_sm_count())
+    g.rows *= 2;
+  g.blocks = g.ktiles * ceil_div(R, (int64_t)g.rows);
+  return g;
+}
+
+// Block (k tile, row tile). A thread keeps F3[k, :] of KT columns k = k0, k0 + tx, ...
+// in registers (KM >= K entries, zero past K); the block's U rows sit in shared
+// memory and are read in 16-byte broadcasts that serve KT products per entry
+// (one column a thread, one row at a time: 512^3, K = 32, 519 us and 128^3 x 64, K = 16,
+// 824 us, half of its threads past the row's end).
+// Per element: x_hat = U[t, :] . F3[k, :] in T, then (x - x_hat)^2 and x^2. For T =
+// float the thread adds its terms in FP32 (rounded to nearest, so the errors are unbiased
+// and shrink in the FP64 sums that follow); GB300's FP64 rate is far below its
 // FP32 rate, and FP64 arithmetic per element would bound the pass. The block
 // sums and the partials are FP64.
-template <typename T, int KM>
+template <typename T, int KM, int KT>
 __global__ void __launch_bounds__(kResThreads)
 residual_stream_kernel(const T* __restrict__ X, int64_t R, int64_t N3, const T* __restrict__ U,
-                       int K, const T* __restrict__ F3, double* __restrict__ part) {
-  __shared__ __align__(16) T us[kResRows * KM];
+                       int K, const T* __restrict__ F3, int tx, int64_t ktiles, int rows,
+                       double* __restrict__ part) {
+  constexpr int kRows = res_rows(KM);
+  __shared__ __align__(16) T us[kRows * KM];
   __shared__ double red[32];
-  const int64_t k = (int64_t)blockIdx.x * kResThreads + threadIdx.x;
-  const bool act = k < N3;
-  T f[KM];
+  const int ty = kResThreads / tx, sub = threadIdx.x / tx;
+  const int64_t k0 = (blockIdx.x % ktiles) * tx * KT + (threadIdx.x & (tx - 1));
+  T f[KT][KM];
+  bool act[KT];
 #pragma unroll
-  for (int c = 0; c < KM; ++c) f[c] = (act && c < K) ? F3[k * K + c] : T(0);
-  const int64_t r0 = (int64_t)blockIdx.y * kResRows;
-  const int nr = (int)(r0 + kResRows < R ? kResRows : R - r0);
-  for (int e = threadIdx.x; e < nr * KM; e += kResThreads) {
-    const int row = e / KM, c = e % KM;
-    us[e] = c < K ? U[(r0 + row) * K + c] : T(0);
+  for (int u = 0; u < KT; ++u) {
+    const int64_t k = k0 + (int64_t)u * tx;
+    act[u] = k < N3;
+#pragma unroll
+    for (int c = 0; c < KM; ++c) f[u][c] = (act[u] && c < K) ? F3[k * K + c] : T(0);
   }
-  __syncthreads();
-  T d2 = T(0), x2 = T(0);
-  if (act) {
-    const T* xp = X + r0 * N3 + k;
-#pragma unroll 4
-    for (int row = 0; row < nr; ++row) {
-      const T x = xp[(int64_t)row * N3];
-      const T* u = us + row * KM;
-      T h0 = T(0), h1 = T(0);
-#pragma unroll
-      for (int c = 0; c < KM; c += 2) {
-        h0 = fma(u[c], f[c], h0);
-        h1 = fma(u[c + 1], f[c + 1], h1);
-      }
-      const T dd = x - (h0 + h1);
-      d2 = fma(dd, dd, d2);
-      x2 = fma(x, x, x2);
+  const int64_t rb = (blockIdx.x / ktiles) * rows;
+  const int64_t rend = rb + rows < R ? rb + rows : R;
+  double td2 = 0.0, tx2 = 0.0;
+  for (int64_t r0 = rb; r0 < rend; r0 += kRows) {
+    const int nr = (int)(r0 + kRows < rend ? kRows : rend - r0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < nr * KM; e += kResThreads) {
+      const int row = e / KM, c = e % KM;
+      us[e] = c < K ? U[(r0 + row) * K + c] : T(0);
     }
-  }
-  double td2 = (double)d2, tx2 = (double)x2;
-  if (act && !(isfinite(d2) && isfinite(x2))) {
-    // The FP32 terms overflowed (entries beyond about 1e19): these rows again
-    // with FP64 terms. Non-finite data stays non-finite.
-    td2 = 0.0;
-    tx2 = 0.0;
-    const T* xp = X + r0 * N3 + k;
-    for (int row = 0; row < nr; ++row) {
-      const double x = (double)xp[(int64_t)row * N3];
-      double h = 0.0;
-      for (int c = 0; c < KM; ++c) h = fma((double)us[row * KM + c], (double)f[c], h);
-      const double dd = x - h;
-      td2 += dd * dd;
-      tx2 += x * x;
+    __syncthreads();
+    T d2 = T(0), x2 = T(0);
+    const T* xp = X + r0 * N3 + k0;
+    // Four rows at a time, their entries of X requested one round ahead.
+    constexpr int RU = 4;
+    T nx[RU][KT];
+    auto fetch = [&](int row) {
+#pragma unroll
+      for (int q = 0; q < RU; ++q)
+#pragma unroll
+        for (int u = 0; u < KT; ++u)
+          nx[q][u] = act[u] && row + q * ty < nr
+                         ? __ldg(xp + (int64_t)(row + q * ty) * N3 + (int64_t)u * tx)
+                         : T(0);
+    };
+    fetch(sub);
+    for (int row = sub; row < nr; row += RU * ty) {
+      T x[RU][KT];
+#pragma unroll
+      for (int q = 0; q < RU; ++q)
+#pragma unroll
+        for (int u = 0; u < KT; ++u) x[q][u] = nx[q][u];
+      fetch(row + RU * ty);
+#pragma unroll
+      for (int q = 0; q < RU; ++q) {
+        if (row + q * ty >= nr) break;
+        T h0[KT], h1[KT];
+#pragma unroll
+        for (int u = 0; u < KT; ++u) h0[u] = h1[u] = T(0);
+        const T* ur = us + (row + q * ty) * KM;
+#pragma unroll
+        for (int c = 0; c < KM; c += 4) {
+          T w[4];
+          if constexpr (sizeof(T) == 4) {
+            const float4 t = *reinterpret_cast<const float4*>(ur + c);
+            w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+          } else {
+            const double2 t0 = *reinterpret_cast<const double2*>(ur + c);
+            const double2 t1 = *reinterpret_cast<const double2*>(ur + c + 2);
+            w[0] = t0.x; w[1] = t0.y; w[2] = t1.x; w[3] = t1.y;
+          }
+#pragma unroll
+          for (int u = 0; u < KT; ++u) {
+            h0[u] = fma(w[0], f[u][c], h0[u]);
+            h1[u] = fma(w[1], f[u][c + 1], h1[u]);
+            h0[u] = fma(w[2], f[u][c + 2], h0[u]);
+            h1[u] = fma(w[3], f[u][c + 3], h1[u]);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < KT; ++u) {
+          // (a column past the end has x = 0 and f = 0)
+          const T dd = x[q][u] - (h0[u] + h1[u]);
+          d2 = fma(dd, dd, d2);
+          x2 = fma(x[q][u], x[q][u], x2);
+        }
+      }
+    }
+    if (isfinite(d2) && isfinite(x2)) {
+      td2 += (double)d2;
+      tx2 += (double)x2;
+    } else {
+      // The FP32 terms overflowed (entries beyond about 1e19): these rows again
+      // with FP64 terms. Non-finite data stays non-finite.
+      for (int row = sub; row < nr; row += ty)
+        for (int u = 0; u < KT; ++u) {
+          const int64_t k = k0 + (int64_t)u * tx;
+          if (k >= N3) continue;
+          const double x = (double)xp[(int64_t)row * N3 + (int64_t)u * tx];
+          double h = 0.0;
+          for (int c = 0; c < K; ++c) h = fma((double)us[row * KM + c], (double)F3[k * K + c], h);
+          const double dd = x - h;
+          td2 += dd * dd;
+          tx2 += x * x;
+        }
     }
   }
   const double bd2 = block_sum(td2, red);
   const double bx2 = block_sum(tx2, red);
   if (threadIdx.x == 0) {
-    const int64_t b = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-    part[2 * b] = bd2;
-    part[2 * b + 1] = bx2;
+    part[2 * (int64_t)blockIdx.x] = bd2;
+    part[2 * (int64_t)blockIdx.x + 1] = bx2;
   }
 }
 
@@ -194,8 +297,7 @@ int residual_prepare(int d, const int64_t* dims, int model, const int* m, int r,
       rows *= dims[k];
     }
   }
-  const int64_t Nd = dims[d - 1];
-  w->nblocks = ceil_div(Nd, kResThreads) * ceil_div(R, kResRows);
+  w->nblocks = res_grid<T>(R, dims[d - 1], K).blocks;
   NNC_TRY(sc.get(&w->part, (size_t)(2 * w->nblocks)));
   return NNC_OK;
 }
@@ -216,9 +318,11 @@ int residual_run(const T* X, int d, const int64_t* dims, int model, const int* m
     for (int k = 1; k < d; ++k) tail *= m[k];
     const T* src = G;
     for (int k = 0; k < d - 1; ++k) {
-      const int64_t n_out = lead * dims[k] * tail;
       T* dst = k < d - 2 ? w.tmp[k & 1] : U;
-      mode_product_any_kernel<T><<<grid_cap(n_out, 256), 256, 0, s>>>(
+      const int64_t cols = ceil_div(lead * tail, kMpThreads);
+      const int64_t qt = ceil_div(dims[k], kMpQ);
+      if (m[k] > 64 || cols > 0x7fffffffLL || qt > 65535) return NNC_ERR_UNSUPPORTED;
+      mode_product_any_kernel<T><<<dim3((unsigned)cols, (unsigned)qt), kMpThreads, 0, s>>>(
           src, lead, m[k], tail, factors[k], (int)dims[k], dst);
       note_launch(s);
       src = dst;
@@ -241,15 +345,17 @@ int residual_run(const T* X, int d, const int64_t* dims, int model, const int* m
   NNC_CUDA_TRY(cudaGetLastError());
   const T* Fd = factors[d - 1];  // F^(d) (Tucker) or A^(d) (CP): N_d x K
   const int64_t Nd = dims[d - 1];
-  dim3 grid((unsigned)ceil_div(Nd, kResThreads), (unsigned)ceil_div(R, kResRows));
-  if (K <= 16)
-    residual_stream_kernel<T, 16><<<grid, kResThreads, 0, s>>>(X, R, Nd, U, K, Fd, w.part);
-  else if (K <= 32)
-    residual_stream_kernel<T, 32><<<grid, kResThreads, 0, s>>>(X, R, Nd, U, K, Fd, w.part);
-  else if (K <= 64)
-    residual_stream_kernel<T, 64><<<grid, kResThreads, 0, s>>>(X, R, Nd, U, K, Fd, w.part);
-  else
-    return NNC_ERR_UNSUPPORTED;
+  if (K > 64) return NNC_ERR_UNSUPPORTED;
+  const ResGrid g = res_grid<T>(R, Nd, K);
+  if (g.blocks > 0x7fffffffLL) return NNC_ERR_UNSUPPORTED;
+  auto stream = [&](auto km) {
+    constexpr int KM = decltype(km)::value;
+    residual_stream_kernel<T, KM, res_kt<T>(KM)><<<(unsigned)g.blocks, kResThreads, 0, s>>>(
+        X, R, Nd, U, K, Fd, g.tx, g.ktiles, g.rows, w.part);
+  };
+  if (K <= 16) stream(std::integral_constant<int, 16>{});
+  else if (K <= 32) stream(std::integral_constant<int, 32>{});
+  else stream(std::integral_constant<int, 64>{});
   note_launch(s);
   residual_final_kernel<<<1, 1024, 0, s>>>(w.part, w.nblocks, out2, rel_out);
   note_launch(s);

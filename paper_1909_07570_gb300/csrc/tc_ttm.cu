@@ -1171,8 +1171,8 @@ col_max_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int tx,
   if (k < N3) {
 #pragma unroll 4
     for (int64_t r = (int64_t)blockIdx.x * ty + sub; r < R; r += (int64_t)ty * gridDim.x) {
-      const int i = (int)(r / N2);
-      const float inv = (1.f / s[i]) * (1.f / t[r - (int64_t)i * N2]);
+      const unsigned i = (unsigned)r / (unsigned)N2;  // R <= 2^31
+      const float inv = (1.f / s[i]) * (1.f / t[(unsigned)r - i * (unsigned)N2]);
       const float4 x = *reinterpret_cast<const float4*>(X + r * N3 + k);
       m[0] = fmaxf(m[0], fabsf(x.x) * inv);
       m[1] = fmaxf(m[1], fabsf(x.y) * inv);
@@ -1198,32 +1198,34 @@ __global__ void slice_u_kernel(const unsigned* __restrict__ umax, int N3, int n3
   if (k < n3p) u[k] = k < N3 ? slice_t(__uint_as_float(umax[k])) : 1.f;
 }
 
-// Xh, Xl (rows of n3p entries, zero past N3) from X: eight entries a thread.
+// Xh, Xl (rows of n3p entries, zero past N3) from X: eight entries a thread, tx threads
+// (a power of two) a row, one division per row.
 __global__ void __launch_bounds__(256)
-x_to_pair_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int n3p,
+x_to_pair_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int n3p, int tx,
                  const float* __restrict__ s, const float* __restrict__ t,
                  const float* __restrict__ u, __half* __restrict__ Xh, __half* __restrict__ Xl) {
-  const int oct = n3p >> 3;
-  const int64_t n = R * oct;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / oct;
-    const int k = (int)(e - r * oct) * 8;
-    const int64_t i = r / N2;
-    const float inv = (1.f / s[i]) * (1.f / t[r - i * N2]);
-    const float* x = X + r * N3 + k;
-    float v[8];
-    // N3 % 4 == 0: the first four entries exist, the last four all or none.
-    const float4 a = *reinterpret_cast<const float4*>(x);
-    const float4 b = k + 4 < N3 ? *reinterpret_cast<const float4*>(x + 4)
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    union { __half h[8]; uint4 q; } hi, lo;
+  const int oct = n3p >> 3, ty = 256 / tx;
+  for (int64_t r = (int64_t)blockIdx.x * ty + threadIdx.x / tx; r < R;
+       r += (int64_t)gridDim.x * ty) {
+    const unsigned i = (unsigned)r / (unsigned)N2;  // R <= 2^31
+    const float inv = (1.f / s[i]) * (1.f / t[(unsigned)r - i * (unsigned)N2]);
+#pragma unroll 2
+    for (int o = threadIdx.x & (tx - 1); o < oct; o += tx) {
+      const int k = 8 * o;
+      const float* x = X + r * N3 + k;
+      float v[8];
+      // N3 % 4 == 0: the first four entries exist, the last four all or none.
+      const float4 a = *reinterpret_cast<const float4*>(x);
+      const float4 b = k + 4 < N3 ? *reinterpret_cast<const float4*>(x + 4)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+      v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+      union { __half h[8]; uint4 q; } hi, lo;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) split_f16(v[q] * inv * (1.f / u[k + q]), hi.h[q], lo.h[q]);
-    *reinterpret_cast<uint4*>(Xh + r * n3p + k) = hi.q;
-    *reinterpret_cast<uint4*>(Xl + r * n3p + k) = lo.q;
+      for (int q = 0; q < 8; ++q) split_f16(v[q] * inv * (1.f / u[k + q]), hi.h[q], lo.h[q]);
+      *reinterpret_cast<uint4*>(Xh + r * n3p + k) = hi.q;
+      *reinterpret_cast<uint4*>(Xl + r * n3p + k) = lo.q;
+    }
   }
 }
 
@@ -1253,16 +1255,60 @@ __global__ void slice_scale_kernel(const float* __restrict__ X, int64_t slab, fl
   }
 }
 
-__global__ void x_to_bf16_kernel(const float* __restrict__ X, int64_t rows, int n3, int kp,
-                                 int rows_per_slice, const float* __restrict__ inv_scale,
-                                 __nv_bfloat16* __restrict__ Xb) {
-  const int64_t n = rows * kp;
-  for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t r = e / kp;
-    const int k = static_cast<int>(e % kp);
-    const float v = k < n3 ? X[r * n3 + k] * inv_scale[r / rows_per_slice] : 0.f;
-    Xb[e] = __float2bfloat16_rn(v);
+// The same scales from the rows' maxima.
+__global__ void __launch_bounds__(256)
+slice_scale_rows_kernel(const unsigned* __restrict__ rmax, int64_t N2, float* scale,
+                        float* inv_scale) {
+  __shared__ unsigned m;
+  if (threadIdx.x == 0) m = 0u;
+  __syncthreads();
+  unsigned v = 0u;
+  for (int64_t j = threadIdx.x; j < N2; j += blockDim.x) {
+    const unsigned x = rmax[(int64_t)blockIdx.x * N2 + j];
+    v = x > v ? x : v;
+  }
+  atomicMax(&m, __reduce_max_sync(0xffffffffu, v));
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const float mx = __uint_as_float(m);
+    int e = 0;
+    if (mx > 0.f && isfinite(mx)) frexpf(mx, &e);
+    scale[blockIdx.x] = ldexpf(1.f, e);
+    inv_scale[blockIdx.x] = ldexpf(1.f, -e);
+  }
+}
+
+// Xb (rows of kp entries, a multiple of 64, zero past n3) from X: eight entries a
+// thread, tx threads (a power of two) a row. 512^3: 358 -> 128 us (one entry a thread,
+// two divisions an entry).
+template <bool VEC>
+__global__ void __launch_bounds__(256)
+x_to_bf16_kernel(const float* __restrict__ X, int64_t rows, int n3, int kp, int rows_per_slice,
+                 int tx, const float* __restrict__ inv_scale, __nv_bfloat16* __restrict__ Xb) {
+  const int oct = kp >> 3, ty = 256 / tx;
+  for (int64_t r = (int64_t)blockIdx.x * ty + threadIdx.x / tx; r < rows;
+       r += (int64_t)gridDim.x * ty) {
+    const float inv = inv_scale[(unsigned)r / (unsigned)rows_per_slice];  // rows <= 2^31
+#pragma unroll 2
+    for (int o = threadIdx.x & (tx - 1); o < oct; o += tx) {
+      const int k = 8 * o;
+      const float* x = X + r * n3 + k;
+      float v[8];
+      if constexpr (VEC) {  // n3 % 4 == 0, rows on 16 bytes
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 a = k < n3 ? *reinterpret_cast<const float4*>(x) : z;
+        const float4 b = k + 4 < n3 ? *reinterpret_cast<const float4*>(x + 4) : z;
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+      } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = k + q < n3 ? x[q] : 0.f;
+      }
+      union { __nv_bfloat16 h[8]; uint4 q; } out;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) out.h[q] = __float2bfloat16_rn(v[q] * inv);
+      *reinterpret_cast<uint4*>(Xb + r * kp + k) = out.q;
+    }
   }
 }
 
@@ -1417,6 +1463,26 @@ int launch_np(int np, const CUtensorMap& a, const CUtensorMap& b, const CUtensor
 
 }  // namespace
 
+// Threads (a power of two, at most 256) that share a row of n pieces.
+static int row_threads(int n) {
+  int t = 1;
+  while (t < 256 && t < n) t *= 2;
+  return t;
+}
+
+// rmax: the largest magnitude of every row (i, j) of X (rows on 16 bytes).
+int TcPlan::row_maxima(const float* X, Scratch& sc, cudaStream_t s) {
+  const int64_t rows = N1 * N2;
+  NNC_TRY(sc.get(&rmax, static_cast<size_t>(rows)));
+  int lw = 1;
+  while (lw < 32 && lw < N3 / 4) lw *= 2;
+  const int64_t rb = ceil_div(rows, 2 * (256 / lw)), most = 16LL * device_sm_count();
+  row_max_kernel<<<(unsigned)(rb < most ? rb : most), 256, 0, s>>>(X, rows, (int)N3, lw, rmax);
+  note_launch(s);
+  NNC_CUDA_TRY(cudaGetLastError());
+  return NNC_OK;
+}
+
 int TcPlan::init(int kind_, const float* X, int64_t N1_, int64_t N2_, int64_t N3_, int m1_,
                  int m3_, Scratch& sc, cudaStream_t s, bool p1_kj_, bool need_p1) {
   kind = kind_;
@@ -1455,13 +1521,24 @@ int TcPlan::init(int kind_, const float* X, int64_t N1_, int64_t N2_, int64_t N3
     NNC_TRY(sc.get(&Bt3, static_cast<size_t>(np3) * kb3));
     NNC_CUDA_TRY(cudaMemsetAsync(Bt1, 0, sizeof(__nv_bfloat16) * np1 * kp1, s));
     NNC_CUDA_TRY(cudaMemsetAsync(Bt3, 0, sizeof(__nv_bfloat16) * np3 * kb3, s));
-    slice_scale_kernel<<<static_cast<unsigned>(N1), 256, 0, s>>>(X, N2 * N3, scale, inv_scale);
+    const bool vec = N3 % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    if (vec) {
+      NNC_TRY(row_maxima(X, sc, s));
+      slice_scale_rows_kernel<<<static_cast<unsigned>(N1), 256, 0, s>>>(rmax, N2, scale,
+                                                                        inv_scale);
+    } else {
+      slice_scale_kernel<<<static_cast<unsigned>(N1), 256, 0, s>>>(X, N2 * N3, scale, inv_scale);
+    }
     note_launch(s);
-    const int64_t n = rows * kp3;
-    const unsigned blocks =
-        static_cast<unsigned>(ceil_div(n, 256) < 16384 ? ceil_div(n, 256) : 16384);
-    x_to_bf16_kernel<<<blocks, 256, 0, s>>>(X, rows, static_cast<int>(N3), kp3,
-                                           static_cast<int>(N2), inv_scale, Xb);
+    const int ox = row_threads(kp3 / 8);
+    const int64_t xb = ceil_div(rows, 256 / ox), most = 32LL * device_sm_count();
+    const unsigned blocks = static_cast<unsigned>(xb < most ? xb : most);
+    if (vec)
+      x_to_bf16_kernel<true><<<blocks, 256, 0, s>>>(X, rows, static_cast<int>(N3), kp3,
+                                                    static_cast<int>(N2), ox, inv_scale, Xb);
+    else
+      x_to_bf16_kernel<false><<<blocks, 256, 0, s>>>(X, rows, static_cast<int>(N3), kp3,
+                                                     static_cast<int>(N2), ox, inv_scale, Xb);
     note_launch(s);
     NNC_CUDA_TRY(cudaGetLastError());
     const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
@@ -1522,23 +1599,16 @@ int TcPlan::init_f16(const float* X, Scratch& sc, cudaStream_t s) {
     set_error_detail_text("FP16 pair pass: shape outside the path");
     return NNC_ERR_UNSUPPORTED;
   }
-  unsigned *rmax = nullptr, *umax = nullptr;
+  unsigned* umax = nullptr;
   NNC_TRY(sc.get(&err, 1));
   NNC_TRY(sc.get(&scale, static_cast<size_t>(N1)));
   NNC_TRY(sc.get(&sc_t, static_cast<size_t>(N2)));
   NNC_TRY(sc.get(&sc_u, static_cast<size_t>(kp3)));
-  NNC_TRY(sc.get(&rmax, static_cast<size_t>(rows)));
   NNC_TRY(sc.get(&umax, static_cast<size_t>(N3)));
   NNC_TRY(sc.get(&Xh, static_cast<size_t>(rows * kp3)));
   NNC_TRY(sc.get(&Xl, static_cast<size_t>(rows * kp3)));
   const int sms = device_sm_count();
-  int lw = 1;
-  while (lw < 32 && lw < N3 / 4) lw *= 2;
-  const int64_t per_block = 256 / lw;
-  const int64_t rb = ceil_div(rows, 2 * per_block);
-  row_max_kernel<<<(unsigned)(rb < 16LL * sms ? rb : 16LL * sms), 256, 0, s>>>(
-      X, rows, (int)N3, lw, rmax);
-  note_launch(s);
+  if (rmax == nullptr) NNC_TRY(row_maxima(X, sc, s));
   slice_s_kernel<<<(unsigned)N1, 256, 0, s>>>(rmax, N2, scale);
   note_launch(s);
   slice_t_kernel<<<(unsigned)ceil_div(N2, 32), 256, 0, s>>>(rmax, scale, N1, N2, sc_t);
@@ -1554,10 +1624,10 @@ int TcPlan::init_f16(const float* X, Scratch& sc, cudaStream_t s) {
   note_launch(s);
   slice_u_kernel<<<(unsigned)ceil_div(kp3, 256), 256, 0, s>>>(umax, (int)N3, kp3, sc_u);
   note_launch(s);
-  const int64_t n = rows * (kp3 / 8);
-  const int64_t xb = ceil_div(n, 256);
+  const int ox = row_threads(kp3 / 8);
+  const int64_t xb = ceil_div(rows, 256 / ox);
   x_to_pair_kernel<<<(unsigned)(xb < 32LL * sms ? xb : 32LL * sms), 256, 0, s>>>(
-      X, rows, (int)N2, (int)N3, kp3, scale, sc_t, sc_u, Xh, Xl);
+      X, rows, (int)N2, (int)N3, kp3, ox, scale, sc_t, sc_u, Xh, Xl);
   note_launch(s);
   NNC_CUDA_TRY(cudaGetLastError());
   // After the conversion: a pass launched as a programmatic dependent reads the pair

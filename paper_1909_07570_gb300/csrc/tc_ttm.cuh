@@ -73,6 +73,9 @@ struct TcPlan {
   float *scale = nullptr, *inv_scale = nullptr;
   __half *Xh = nullptr, *Xl = nullptr;
   float *sc_t = nullptr, *sc_u = nullptr;  // F16x3: t and u (s is in `scale`)
+  // Bits of the largest magnitude of every row (i, j); another plan's for the same X
+  // may be handed in before init.
+  unsigned* rmax = nullptr;
   int x_resident = 0;
   CUtensorMap mapL3, mapL1;  // F16x3: Xl as operand A of pass 1 and pass 2
   int* err = nullptr;
@@ -91,7 +94,8 @@ struct TcPlan {
   // allows it, else TF32x3.
   int init_fp32(const float* X, int64_t N1, int64_t N2, int64_t N3, int m1, int m3, Scratch& sc,
                 cudaStream_t s, bool p1_kj = false);
-  int init_f16(const float* X, Scratch& sc, cudaStream_t s);  // part of init
+  int init_f16(const float* X, Scratch& sc, cudaStream_t s);  // parts of init
+  int row_maxima(const float* X, Scratch& sc, cudaStream_t s);
   // B operands from the current factor (BF16: F^(1) scaled by s).
   int convert_b3(const float* F3, cudaStream_t s) const;
   int convert_b1(const float* F1, cudaStream_t s) const;

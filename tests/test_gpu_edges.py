@@ -105,3 +105,26 @@ def test_pair_passes_one_sweep(dims, m, scaled):
     for a, b in zip(F + [G], Fo + [Go]):
         np.testing.assert_allclose(a.cpu().numpy(), b, rtol=1e-4, atol=1e-30)
     assert abs(err - orc.rel_err_tucker(X, Go, Fo)) <= 1e-5
+
+
+# The residual pass: rows of X shorter and longer than a block's columns, one row tile and
+# a remainder, every register tile (K = 16, 32, 64 entries), both models, d = 3 and 4. The sums
+# are FP64 (FP32 terms for FP32 data: 1e-5 of the norm is 100 times their rounding).
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+@pytest.mark.parametrize("dims,m", [((3, 5, 1), (2, 3, 1)), ((9, 15, 517), (4, 5, 17)),
+                                    ((40, 33, 30), (33, 3, 33)), ((6, 7, 5, 70), (3, 2, 5, 16)),
+                                    ((17, 70, 9, 3), (2, 17, 4, 3))])
+def test_residual_edges(dt, dims, m):
+    rng = np.random.default_rng(17)
+    X = rng.random(dims)
+    F = [rng.random((n, k)) / k for n, k in zip(dims, m)]
+    G = rng.random(m)
+    A = [rng.random((n, m[0])) for n in dims]
+    tol = 1e-11 if dt == torch.float64 else 1e-5
+    Xd = _dev(X, dt)
+    rn, xn = native.recon_residual(Xd, [_dev(f, dt) for f in F], _dev(G, dt))
+    Xr = Xd.double().cpu().numpy()
+    assert xn == pytest.approx(np.linalg.norm(Xr), rel=tol)
+    assert rn / xn == pytest.approx(orc.rel_err_tucker(Xr, G, F), rel=tol)
+    rn, xn = native.recon_residual(Xd, [_dev(a, dt) for a in A])
+    assert rn / xn == pytest.approx(orc.rel_err_cp(Xr, A), rel=tol)
