@@ -490,6 +490,35 @@ int run_sweeps(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double
   return NNC_OK;
 }
 
+// A fit on one cluster: the sweeps between two exact checkpoints are one launch.
+template <typename T>
+int ntd_fit3_small(const T* X, const int64_t* dims, const int* m, const nnc_opts* o, T* const* F,
+                   T* G, double* trace, double* rel_err, const NtdState<T>& b, Scratch& sc,
+                   cudaStream_t s) {
+  NNC_CUDA_TRY(cudaMemsetAsync(b.counter, 0, 2 * sizeof(int), s));
+  const bool exact = o->exact_every > 0 && trace;
+  ResidualWork<T> rw;
+  if (exact || rel_err) NNC_TRY(residual_prepare<T>(3, dims, 0, m, 0, sc, &rw));
+  const T* fac[3] = {F[0], F[1], F[2]};
+  for (int t = 0; t < o->iters;) {
+    const int n = exact ? std::min(o->iters - t, o->exact_every - t % o->exact_every)
+                        : o->iters - t;
+    NNC_TRY(ntd_cluster_sweeps<T>(X, dims, m, F, G, o->eps, n, b.stats, trace, b.counter, s));
+    t += n;
+    if (exact)
+      NNC_TRY(residual_run<T>(X, 3, dims, 0, m, 0, fac, G, rw, nullptr, trace + t - 1, s));
+  }
+  NNC_TRY(check_trace_finite(b.counter, s, "ntd_fit"));
+  if (rel_err) {
+    NNC_TRY(residual_run<T>(X, 3, dims, 0, m, 0, fac, G, rw, b.resid2, nullptr, s));
+    double h[2];
+    NNC_CUDA_TRY(cudaMemcpyAsync(h, b.resid2, sizeof(h), cudaMemcpyDeviceToHost, s));
+    NNC_CUDA_TRY(cudaStreamSynchronize(s));
+    *rel_err = sqrt(h[0] / h[1]);
+  }
+  return NNC_OK;
+}
+
 // passes: 0 = SIMT for every sweep; 1 = TF32x3 tensor cores for every sweep
 // (FP32-accurate); 2 = BF16 tensor cores, then TF32x3 for the refinement sweeps.
 // A tensor-core plan that the shape does not allow falls back to SIMT passes.
@@ -523,7 +552,8 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
   if (st[2] > 0.0) return NNC_ERR_NONFINITE;
   if (st[1] > 0.0) return NNC_ERR_NEGATIVE_INPUT;
   if (!(st[0] > 0.0)) return NNC_ERR_INVALID_ARG;  // X == 0: the relative error is undefined
-
+  if (passes != 2 && !profile_enabled() && ntd_cluster_fits<T>(dims, m))
+    return ntd_fit3_small<T>(X, dims, m, o, F, G, trace, rel_err, b, sc, s);
 
   NNC_TRY(sc.get(&b.P3, (size_t)(N1 * N2 * m3)));
   NNC_TRY(sc.get(&b.P1, (size_t)(m1 * N2 * N3)));

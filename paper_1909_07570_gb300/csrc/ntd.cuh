@@ -18,4 +18,14 @@ int ntd_fit3_bf16(const float* X, const int64_t* dims, const int* m, const nnc_o
                   float* const* F, float* G, double* trace, double* rel_err, int* refined_from,
                   cudaStream_t s);
 
+// Whole fits of small tensors on one thread-block cluster (ntd_cluster.cu).
+// ntd_cluster_fits: the shape is one it takes and is the faster form for.
+// ntd_cluster_sweeps: `sweeps` sweeps in place on F and G in one launch; counter is
+// trace_record's pair, x2 the device's ||X||^2, trace (device) may be NULL.
+template <typename T>
+bool ntd_cluster_fits(const int64_t* dims, const int* m);
+template <typename T>
+int ntd_cluster_sweeps(const T* X, const int64_t* dims, const int* m, T* const* F, T* G, double eps,
+                       int sweeps, const double* x2, double* trace, int* counter, cudaStream_t s);
+
 }  // namespace nnc

@@ -128,3 +128,35 @@ def test_residual_edges(dt, dims, m):
     assert rn / xn == pytest.approx(orc.rel_err_tucker(Xr, G, F), rel=tol)
     rn, xn = native.recon_residual(Xd, [_dev(a, dt) for a in A])
     assert rn / xn == pytest.approx(orc.rel_err_cp(Xr, A), rel=tol)
+
+
+# Whole fits on one cluster: modes shorter than the cluster (CTAs without slices), slices
+# with a remainder, 16-byte and single columns, every tile width, exact checkpoints; and the
+# same fit in pieces. The trace and factors against the oracle: FP64 rounding over a few
+# sweeps; FP32 1e-4 on factors after three sweeps, 1e-5 on the trace.
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+@pytest.mark.parametrize("dims,m", [((1, 1, 1), (1, 1, 1)), ((5, 61, 201), (3, 3, 3)),
+                                    ((40, 40, 40), (5, 5, 5)), ((17, 3, 33), (2, 3, 7)),
+                                    ((20, 18, 22), (8, 7, 4)), ((33, 16, 8), (1, 6, 4))])
+def test_cluster_fit_edges(dt, dims, m):
+    X, _, F0, G0, _ = inputs.small_problem(dims, 2, m, 2, seed=57)
+    X, F0, G0 = (_dev(X, dt).double().cpu().numpy(),
+                 [_dev(f, dt).double().cpu().numpy() for f in F0],
+                 _dev(G0, dt).double().cpu().numpy())
+    F, G = [_dev(f, dt) for f in F0], _dev(G0, dt)
+    err, tr = native.ntd_fit(_dev(X, dt), F, G, 3)
+    Fo, Go, tro = orc.ntd_fit(X, F0, G0, 3)
+    tol = _TOL[dt]
+    scale = max(1.0, float(np.max(tro)))
+    np.testing.assert_allclose(tr.cpu().numpy(), tro, rtol=1e-8 if dt == torch.float64 else 0,
+                               atol=(1e-8 if dt == torch.float64 else 1e-5) * scale)
+    for a, b in zip(F + [G], Fo + [Go]):
+        np.testing.assert_allclose(a.double().cpu().numpy(), b, rtol=tol, atol=tol * 1e-3)
+    assert err == pytest.approx(orc.rel_err_tucker(X, Go, Fo), abs=tol)
+    # In pieces, and with an exact checkpoint after every second sweep.
+    F2, G2 = [_dev(f, dt) for f in F0], _dev(G0, dt)
+    native.ntd_fit(_dev(X, dt), F2, G2, 1, trace=False, rel_err=False)
+    err2, tr2 = native.ntd_fit(_dev(X, dt), F2, G2, 2, exact_every=2)
+    for a, b in zip(F + [G], F2 + [G2]):
+        assert torch.equal(a, b)
+    assert tr2[1].item() == pytest.approx(err2, rel=1e-6)
