@@ -52,6 +52,10 @@ struct NtdState {
   // tensor-core passes (y_nh = N2 / 128 per slab; NULL: the update kernel forms them)
   T* Y1p;
   T* Y3p;
+  // Partial sums of the SIMT passes, which split the contraction of a tensor too small to
+  // fill the GPU otherwise (one pass at a time uses them).
+  T* split;
+  size_t split_cap;
   int y_nh;
   double *stats_part, *stats, *trace_dummy, *resid2, *dots;
   int* counter;
@@ -69,9 +73,8 @@ int pass_x3(const T* X, const NtdState<T>& b, const T* F3, const T* F2, const tc
       return tcp->pass3(F3, b.P3, s, /*convert=*/false);
     }
   }
-  // No split buffer: the passes fill the GPU without splitting the contraction.
   NNC_CUDA_TRY(launch_ttm<T>(X, b.N[0] * b.N[1], (int)b.N[2], 1, F3, b.m[2], 1, b.m[2], b.P3,
-                             nullptr, 0, s));
+                             b.split, b.split_cap, s));
   return NNC_OK;
 }
 
@@ -85,7 +88,7 @@ int pass_x1(const T* X, const NtdState<T>& b, const T* F1, const T* F2, const tc
     }
   }
   NNC_CUDA_TRY(launch_ttm<T>(X, 1, (int)b.N[0], b.N[1] * b.N[2], F1, b.m[0], 1, b.m[0], b.P1s,
-                             nullptr, 0, s));
+                             b.split, b.split_cap, s));
   return launch_p1_rows<T>(b.P1s, b.m[0], b.N[1], b.N[2], b.P1, s);
 }
 
@@ -600,8 +603,11 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
     }
   }
   const int n_fast_max = fast ? o->iters - o->refine_iters : 0;
-  if (!exact && (o->iters - n_fast_max > 0 || trigger))
+  if (!exact && (o->iters - n_fast_max > 0 || trigger)) {
     NNC_TRY(sc.get(&b.P1s, (size_t)(m1 * N2 * N3)));
+    b.split_cap = (size_t)1 << 20;
+    NNC_TRY(sc.get(&b.split, b.split_cap));
+  }
   ResidualWork<T> rw;
   Checkpoints<T> ck;
   if (o->exact_every > 0 && trace) {

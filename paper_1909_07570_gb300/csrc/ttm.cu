@@ -4,18 +4,15 @@
 //
 // A tensor is viewed as (L, J, C) with J the contracted mode:
 //   out[l, q, c] = sum_j Fm[j, q] * Y[l, j, c]
-// Two kernels cover the two memory patterns:
+// The kernels by memory pattern:
 //   * ttm_rows (C == 1): J is the contiguous axis (e.g. X x_3 F^(3)T). A block
-//     stages a BM x 32 tile of Y and a 32 x QP slice of Fm in shared memory;
+//     stages tiles of Y's rows and the slice of Fm in a 3-deep cp.async ring;
 //     each thread keeps TR rows x QP outputs in registers.
-//   * ttm_cols (C > 1): J is strided (e.g. X x_1 F^(1)T). Each thread owns TC
-//     flattened (l, c) columns, streams them along j with coalesced loads and
-//     keeps QP outputs per column in registers; Fm rows are broadcast from
-//     shared memory.
-//   * ttm_cols_pipe (C > 1, rows of C 16-byte aligned): the same register
-//     tiling, with the block's 256 TC flattened columns staged through a
-//     3-deep cp.async ring of 16 rows j, so that two chunks are in flight
-//     while the third is consumed.
+//   * ttm_cols_pipe (C > 1): J is strided (e.g. X x_1 F^(1)T). Each thread owns TC
+//     flattened (l, c) columns and keeps QP outputs per column in registers; the
+//     block's 256 TC columns are staged through a 3-deep cp.async ring of 16
+//     rows j, so that two chunks are in flight while the third is consumed, and
+//     Fm rows are broadcast from shared memory.
 //   * ttm_cols_tc (float, C % 4 == 0, Q <= 32): the column product as a GEMM on
 //     the tensor cores (TF32x3 on mma.sync, FP32-accurate), for the mode
 //     products of the compressed tensors in the tensor-core paths.
@@ -36,20 +33,53 @@ __host__ __device__ constexpr int rows_bk() { return sizeof(T) == 4 ? 32 : 16; }
 constexpr int kColsThreads = 256;
 constexpr int kColsBJ = 32;
 
+// Rows tile of BM = 128 TR rows x BK columns j in a 3-deep cp.async ring (single elements: a
+// row of Y starts anywhere), with the chunk's rows of Fm; each thread keeps TR rows x QP
+// outputs in registers, its terms in the order of k. What bounds it is the shared-memory
+// reads, 1 + QP / 4 per TR rows and k; staged by plain loads between two barriers it waited
+// on memory instead. 65317 x 255, Q = 12: 85.5 -> 32.7 us.
+constexpr int kRowsStages = 3;
+template <typename T, int QP, int TR>
+constexpr size_t rows_smem_bytes() {
+  constexpr size_t xs = (size_t)kRowsThreads * TR * (rows_bk<T>() + 1);
+  return sizeof(T) * kRowsStages * (((xs + 3) & ~(size_t)3) + (size_t)rows_bk<T>() * QP);
+}
+
 template <typename T, int QP, int TR>
 __global__ void __launch_bounds__(kRowsThreads)
 ttm_rows_kernel(const T* __restrict__ Y, int64_t R, int K, int k_per_split,
                 const T* __restrict__ Fm, int64_t fs_k, int64_t fs_q, int Q,
                 T* __restrict__ out) {
-  constexpr int BM = kRowsThreads * TR;
-  constexpr int BK = rows_bk<T>();
-  __shared__ T Xs[BM][BK + 1];
-  __shared__ __align__(16) T Fs[BK][QP];
+  constexpr int BM = kRowsThreads * TR, BK = rows_bk<T>(), LD = BK + 1;
+  constexpr int XS = (BM * LD + 3) & ~3;  // elements of one stage's Y tile
+  constexpr int V = 16 / (int)sizeof(T);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* Xs = reinterpret_cast<T*>(smem_raw);
+  T* Fs = Xs + kRowsStages * XS;
 
   const int tid = threadIdx.x;
   const int64_t r0 = (int64_t)blockIdx.x * BM;
   const int kbeg = blockIdx.y * k_per_split;
   const int kend = min(K, kbeg + k_per_split);
+  const int nch = (kend - kbeg + BK - 1) / BK;
+  const int rn = (int)min((int64_t)BM, R - r0);
+  const T* y0 = Y + r0 * K;
+  auto issue = [&](int c) {
+    const int k0 = kbeg + c * BK, slot = c % kRowsStages;
+    T* xs = Xs + slot * XS;
+    const int kk = tid % BK, k = k0 + kk;
+#pragma unroll 8
+    for (int rr = tid / BK; rr < BM; rr += kRowsThreads / BK) {
+      const bool ok = rr < rn && k < kend;
+      cp_elem(xs + rr * LD + kk, ok ? y0 + (int64_t)rr * K + k : Y, ok);
+    }
+    T* fs = Fs + slot * BK * QP;
+    for (int e = tid; e < BK * QP; e += kRowsThreads) {
+      const int fk = e / QP, q = e % QP;
+      const bool ok = q < Q && k0 + fk < kend;
+      cp_elem(fs + e, ok ? Fm + ((k0 + fk) * fs_k + q * fs_q) : Fm, ok);
+    }
+  };
 
   T acc[TR][QP];
 #pragma unroll
@@ -57,29 +87,37 @@ ttm_rows_kernel(const T* __restrict__ Y, int64_t R, int K, int k_per_split,
 #pragma unroll
     for (int q = 0; q < QP; ++q) acc[t][q] = T(0);
 
-  for (int k0 = kbeg; k0 < kend; k0 += BK) {
-    for (int e = tid; e < BM * BK; e += kRowsThreads) {
-      const int rr = e / BK, kk = e % BK;
-      const int64_t r = r0 + rr;
-      const int k = k0 + kk;
-      Xs[rr][kk] = (r < R && k < kend) ? Y[r * K + k] : T(0);
-    }
-    for (int e = tid; e < BK * QP; e += kRowsThreads) {
-      const int kk = e / QP, q = e % QP;
-      const int k = k0 + kk;
-      Fs[kk][q] = (q < Q && k < kend) ? Fm[k * fs_k + q * fs_q] : T(0);
-    }
+#pragma unroll
+  for (int c = 0; c < kRowsStages - 1; ++c) {
+    if (c < nch) issue(c);
+    cp_commit();
+  }
+  for (int c = 0; c < nch; ++c) {
+    if (c + kRowsStages - 1 < nch) issue(c + kRowsStages - 1);
+    cp_commit();
+    cp_wait<kRowsStages - 1>();
     __syncthreads();
+    const T* xs = Xs + (c % kRowsStages) * XS + tid * LD;
+    const T* fs = Fs + (c % kRowsStages) * BK * QP;
 #pragma unroll 4
     for (int kk = 0; kk < BK; ++kk) {
       T x[TR];
 #pragma unroll
-      for (int t = 0; t < TR; ++t) x[t] = Xs[tid + t * kRowsThreads][kk];
+      for (int t = 0; t < TR; ++t) x[t] = xs[t * kRowsThreads * LD + kk];
 #pragma unroll
-      for (int q = 0; q < QP; ++q) {
-        const T f = Fs[kk][q];
+      for (int q = 0; q < QP; q += V) {
+        T f[V];
+        if constexpr (sizeof(T) == 4) {
+          const float4 w = *reinterpret_cast<const float4*>(fs + kk * QP + q);
+          f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w;
+        } else {
+          const double2 w = *reinterpret_cast<const double2*>(fs + kk * QP + q);
+          f[0] = w.x; f[1] = w.y;
+        }
 #pragma unroll
-        for (int t = 0; t < TR; ++t) acc[t][q] = fma(x[t], f, acc[t][q]);
+        for (int u = 0; u < V; ++u)
+#pragma unroll
+          for (int t = 0; t < TR; ++t) acc[t][q + u] = fma(x[t], f[u], acc[t][q + u]);
       }
     }
     __syncthreads();
@@ -97,72 +135,6 @@ ttm_rows_kernel(const T* __restrict__ Y, int64_t R, int K, int k_per_split,
   }
 }
 
-template <typename T, int QP, int TC>
-__global__ void __launch_bounds__(kColsThreads)
-ttm_cols_kernel(const T* __restrict__ Y, int64_t L, int J, int64_t C, int j_per_split,
-                const T* __restrict__ Fm, int64_t fs_j, int64_t fs_q, int Q,
-                T* __restrict__ out) {
-  constexpr int BJ = kColsBJ;
-  __shared__ __align__(16) T Fs[BJ][QP];
-
-  const int64_t ncols = L * C;
-  const int64_t base = (int64_t)blockIdx.x * (kColsThreads * TC) + threadIdx.x;
-  const int jbeg = blockIdx.y * j_per_split;
-  const int jend = min(J, jbeg + j_per_split);
-
-  const T* y[TC];
-  int64_t col_l[TC], col_c[TC];
-  bool active[TC];
-#pragma unroll
-  for (int t = 0; t < TC; ++t) {
-    const int64_t g = base + (int64_t)t * kColsThreads;
-    active[t] = g < ncols;
-    const int64_t gg = active[t] ? g : 0;
-    col_l[t] = gg / C;
-    col_c[t] = gg % C;
-    y[t] = Y + col_l[t] * (int64_t)J * C + col_c[t];
-  }
-
-  T acc[TC][QP];
-#pragma unroll
-  for (int t = 0; t < TC; ++t)
-#pragma unroll
-    for (int q = 0; q < QP; ++q) acc[t][q] = T(0);
-
-  for (int j0 = jbeg; j0 < jend; j0 += BJ) {
-    for (int e = threadIdx.x; e < BJ * QP; e += kColsThreads) {
-      const int jj = e / QP, q = e % QP;
-      const int j = j0 + jj;
-      Fs[jj][q] = (q < Q && j < jend) ? Fm[j * fs_j + q * fs_q] : T(0);
-    }
-    __syncthreads();
-    const int jn = min(BJ, jend - j0);
-#pragma unroll 4
-    for (int jj = 0; jj < jn; ++jj) {
-      T v[TC];
-#pragma unroll
-      for (int t = 0; t < TC; ++t) v[t] = active[t] ? y[t][(int64_t)(j0 + jj) * C] : T(0);
-#pragma unroll
-      for (int q = 0; q < QP; ++q) {
-        const T f = Fs[jj][q];
-#pragma unroll
-        for (int t = 0; t < TC; ++t) acc[t][q] = fma(f, v[t], acc[t][q]);
-      }
-    }
-    __syncthreads();
-  }
-
-  T* o = out + (int64_t)blockIdx.y * L * Q * C;
-#pragma unroll
-  for (int t = 0; t < TC; ++t) {
-    if (!active[t]) continue;
-    T* ot = o + col_l[t] * Q * C + col_c[t];
-#pragma unroll
-    for (int q = 0; q < QP; ++q)
-      if (q < Q) ot[(int64_t)q * C] = acc[t][q];
-  }
-}
-
 constexpr int kPipeBJ = 16;
 constexpr int kPipeStages = 3;
 
@@ -172,16 +144,18 @@ constexpr size_t pipe_smem_bytes() {
 }
 
 // Flattened columns (l, c) col0 .. col0 + BC - 1 (BC = 256 TC, col0 =
-// blockIdx.x BC), rows j of split blockIdx.y. Each 16-byte copy stays in one
-// row (l, j) because C % V == 0. Rows and columns past the ends are staged as
+// blockIdx.x BC), rows j of split blockIdx.y. Copies of CV entries: 16 bytes where
+// C % CV == 0 keeps each in one row (l, j), else single entries (rows of Y that start
+// anywhere: 301 x 55335, Q = 24, 66.6 us with loads straight into registers, whose
+// latency nothing hid, 56.1 us through the ring, both beside the mode-2 branch). Rows and columns past the ends are staged as
 // zeros (Fm rows too), so every chunk runs all kPipeBJ rows.
-template <typename T, int QP, int TC>
+template <typename T, int QP, int TC, int CV>
 __global__ void __launch_bounds__(kColsThreads, QP * TC * sizeof(T) < 256 ? 2 : 1)
 ttm_cols_pipe_kernel(const T* __restrict__ Y, int64_t L, int J, int64_t C, int j_per_split, const T* __restrict__ Fm, int64_t fs_j, int64_t fs_q, int Q,
                      T* __restrict__ out) {
   constexpr int BC = kColsThreads * TC;
-  constexpr int V = 16 / (int)sizeof(T);  // elements per 16-byte copy
-  constexpr int CPR = BC / V;             // copies per staged row
+  constexpr int V = 16 / (int)sizeof(T);  // elements of a 16-byte read of Fm
+  constexpr int CPR = BC / CV;            // copies per staged row
   static_assert(QP % V == 0, "QP must be a whole number of 16-byte vectors");
   using Vec = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -198,19 +172,21 @@ ttm_cols_pipe_kernel(const T* __restrict__ Y, int64_t L, int J, int64_t C, int j
   constexpr int RP = kColsThreads / CPR;
   static_assert(kColsThreads % CPR == 0 && kPipeBJ % RP == 0, "copy layout");
   const int v = tid % CPR, jr = tid / CPR;
-  const int64_t vcol = col0 + (int64_t)v * V;
+  const int64_t vcol = col0 + (int64_t)v * CV;
   const bool cok = vcol < ncols;
   const int64_t vl = cok ? vcol / C : 0;
   const T* ysrc = Y + vl * (int64_t)J * C + (cok ? vcol - vl * C : 0);
   auto issue = [&](int chunk) {
     const int slot = chunk % kPipeStages;
     const int j0 = jbeg + chunk * kPipeBJ;
-    T* ys = Ys + slot * kPipeBJ * BC + v * V;
+    T* ys = Ys + slot * kPipeBJ * BC + v * CV;
 #pragma unroll
     for (int jj = jr; jj < kPipeBJ; jj += RP) {
       const int j = j0 + jj;
       const bool ok = cok && j < jend;
-      cp_vec(ys + jj * BC, ok ? ysrc + (int64_t)j * C : Y, ok ? V : 0);
+      const T* src = ok ? ysrc + (int64_t)j * C : Y;
+      if constexpr (CV == 1) cp_elem(ys + jj * BC, src, ok);
+      else cp_vec(ys + jj * BC, src, ok ? CV : 0);
     }
     // The Fm rows of the chunk go the same way (element copies), so that no
     // thread waits for them before the chunk it is about to consume.
@@ -519,59 +495,58 @@ cudaError_t ttm_dispatch(const T* Y, int64_t L, int J, int64_t C, const T* Fm, i
   const int64_t out_elems = L * Q * C;
   int per = J, splits = 1;
   if (C == 1) {
-    constexpr int TR = (sizeof(T) == 4 && QP <= 32) ? 2 : 1;
-    constexpr int BM = kRowsThreads * TR;
-    const int64_t blocks = ceil_div(L, BM);
+    // Two rows a thread (fewer reads of Fm) once the grid has four blocks per SM all the
+    // same.
+    constexpr bool two = sizeof(T) == 4 && QP <= 32;
+    const bool use2 = two && ceil_div(L, 2 * kRowsThreads) >= 4LL * device_sm_count();
+    const int64_t blocks = ceil_div(L, (use2 ? 2 : 1) * kRowsThreads);
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     splits = choose_splits(blocks, J, out_elems, split_cap, rows_bk<T>(), &per);
     T* dst = splits > 1 ? split_buf : out;
     dim3 grid((unsigned)blocks, (unsigned)splits);
-    ttm_rows_kernel<T, QP, TR><<<grid, kRowsThreads, 0, s>>>(Y, L, J, per, Fm, fs_j, fs_q, Q, dst);
+    auto run = [&](auto tr) -> cudaError_t {
+      constexpr int TR = decltype(tr)::value;
+      constexpr size_t smem = rows_smem_bytes<T, QP, TR>();
+      const cudaError_t e0 = raise_smem_limit((const void*)ttm_rows_kernel<T, QP, TR>, smem);
+      if (e0 != cudaSuccess) return e0;
+      ttm_rows_kernel<T, QP, TR><<<grid, kRowsThreads, smem, s>>>(Y, L, J, per, Fm, fs_j, fs_q, Q,
+                                                                  dst);
+      return cudaSuccess;
+    };
+    const cudaError_t e0 = use2 ? run(std::integral_constant<int, two ? 2 : 1>{})
+                                : run(std::integral_constant<int, 1>{});
+    if (e0 != cudaSuccess) return e0;
     note_launch(s);
   } else {
     const int64_t ncols = L * C;
-    const bool wide = (QP <= 32) && ceil_div(ncols, 2 * kColsThreads) >= 2LL * device_sm_count();
     constexpr int PV = 16 / (int)sizeof(T);
-    const bool pipe = C % PV == 0 && reinterpret_cast<uintptr_t>(Y) % 16 == 0;
-    if (pipe) {
-      // Two columns per thread when the grid still has two blocks per SM.
-      constexpr bool two = sizeof(T) == 4 && QP <= 32;
-      const bool use2 = two && ceil_div(ncols, 2 * kColsThreads) >= 2LL * device_sm_count();
-      const int64_t blocks = ceil_div(ncols, (int64_t)(use2 ? 2 : 1) * kColsThreads);
-      if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-      splits = choose_splits(blocks, J, out_elems, split_cap, kColsBJ, &per);
-      T* dst = splits > 1 ? split_buf : out;
-      dim3 grid((unsigned)blocks, (unsigned)splits);
-      if (use2) {
-        constexpr int PTC = two ? 2 : 1;
-        constexpr size_t smem = pipe_smem_bytes<T, QP, PTC>();
-        const cudaError_t e0 =
-            raise_smem_limit((const void*)ttm_cols_pipe_kernel<T, QP, PTC>, smem);
-        if (e0 != cudaSuccess) return e0;
-        ttm_cols_pipe_kernel<T, QP, PTC><<<grid, kColsThreads, smem, s>>>(
-            Y, L, J, C, per, Fm, fs_j, fs_q, Q, dst);
-      } else {
-        constexpr size_t smem = pipe_smem_bytes<T, QP, 1>();
-        const cudaError_t e0 = raise_smem_limit((const void*)ttm_cols_pipe_kernel<T, QP, 1>, smem);
-        if (e0 != cudaSuccess) return e0;
-        ttm_cols_pipe_kernel<T, QP, 1><<<grid, kColsThreads, smem, s>>>(Y, L, J, C, per, Fm, fs_j,
-                                                                         fs_q, Q, dst);
-      }
-      note_launch(s);
-    } else if (wide) {
-      const int64_t blocks = ceil_div(ncols, 2 * kColsThreads);
-      splits = choose_splits(blocks, J, out_elems, split_cap, kColsBJ, &per);
-      T* dst = splits > 1 ? split_buf : out;
-      dim3 grid((unsigned)blocks, (unsigned)splits);
-      ttm_cols_kernel<T, QP, 2><<<grid, kColsThreads, 0, s>>>(Y, L, J, C, per, Fm, fs_j, fs_q, Q, dst);
-      note_launch(s);
-    } else {
-      const int64_t blocks = ceil_div(ncols, kColsThreads);
-      splits = choose_splits(blocks, J, out_elems, split_cap, kColsBJ, &per);
-      T* dst = splits > 1 ? split_buf : out;
-      dim3 grid((unsigned)blocks, (unsigned)splits);
-      ttm_cols_kernel<T, QP, 1><<<grid, kColsThreads, 0, s>>>(Y, L, J, C, per, Fm, fs_j, fs_q, Q, dst);
-      note_launch(s);
-    }
+    const bool vec = C % PV == 0 && reinterpret_cast<uintptr_t>(Y) % 16 == 0;
+    // Two columns per thread (16-byte copies only) when the grid still has two blocks per
+    // SM.
+    constexpr bool two = sizeof(T) == 4 && QP <= 32;
+    const bool use2 = two && vec && ceil_div(ncols, 2 * kColsThreads) >= 2LL * device_sm_count();
+    const int64_t blocks = ceil_div(ncols, (int64_t)(use2 ? 2 : 1) * kColsThreads);
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    splits = choose_splits(blocks, J, out_elems, split_cap, kColsBJ, &per);
+    T* dst = splits > 1 ? split_buf : out;
+    dim3 grid((unsigned)blocks, (unsigned)splits);
+    auto run = [&](auto tc, auto cv) -> cudaError_t {
+      constexpr int TC = decltype(tc)::value, CV = decltype(cv)::value;
+      constexpr size_t smem = pipe_smem_bytes<T, QP, TC>();
+      const cudaError_t e0 = raise_smem_limit((const void*)ttm_cols_pipe_kernel<T, QP, TC, CV>, smem);
+      if (e0 != cudaSuccess) return e0;
+      ttm_cols_pipe_kernel<T, QP, TC, CV><<<grid, kColsThreads, smem, s>>>(Y, L, J, C, per, Fm, fs_j,
+                                                                           fs_q, Q, dst);
+      return cudaSuccess;
+    };
+    using One = std::integral_constant<int, 1>;
+    using Vec16 = std::integral_constant<int, PV>;
+    cudaError_t e0;
+    if (use2) e0 = run(std::integral_constant<int, two ? 2 : 1>{}, Vec16{});
+    else if (vec) e0 = run(One{}, Vec16{});
+    else e0 = run(One{}, One{});
+    if (e0 != cudaSuccess) return e0;
+    note_launch(s);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || splits == 1) return e;
@@ -614,6 +589,8 @@ cudaError_t launch_ttm(const T* Y, int64_t L, int J, int64_t C, const T* Fm, int
                        cudaStream_t s) {
   if (L <= 0 || J <= 0 || C <= 0 || Q <= 0) return cudaErrorInvalidValue;
   if (Q <= 8) return ttm_dispatch<T, 8>(Y, L, J, C, Fm, fs_j, fs_q, Q, out, split_buf, split_cap, s);
+  if (Q <= 12)
+    return ttm_dispatch<T, 12>(Y, L, J, C, Fm, fs_j, fs_q, Q, out, split_buf, split_cap, s);
   if (Q <= 16) return ttm_dispatch<T, 16>(Y, L, J, C, Fm, fs_j, fs_q, Q, out, split_buf, split_cap, s);
   if (Q <= 24) return ttm_dispatch<T, 24>(Y, L, J, C, Fm, fs_j, fs_q, Q, out, split_buf, split_cap, s);
   if (Q <= 32) return ttm_dispatch<T, 32>(Y, L, J, C, Fm, fs_j, fs_q, Q, out, split_buf, split_cap, s);

@@ -160,3 +160,24 @@ def test_cluster_fit_edges(dt, dims, m):
     for a, b in zip(F + [G], F2 + [G2]):
         assert torch.equal(a, b)
     assert tr2[1].item() == pytest.approx(err2, rel=1e-6)
+
+
+# SIMT mode products: rows of every start modulo 16 bytes, K and Q at and past the tiles, one
+# and two rows a thread, columns with a remainder and few enough rows j for one batch, and
+# contractions split over blocks. FP64: 1e-12 of the largest sum; FP32: 1e-5 (sums of a
+# few hundred positive terms in FP32).
+@pytest.mark.parametrize("dt,tol", [(torch.float64, 1e-12), (torch.float32, 1e-5)])
+@pytest.mark.parametrize("dims,Q", [((3, 5, 1), 1), ((2, 127, 33), 12), ((9, 43, 255), 13),
+                                    ((513, 310, 17), 8), ((31, 9, 7), 64), ((17, 257, 65), 24),
+                                    ((1, 129, 97), 9)])
+def test_simt_mode_products(dt, tol, dims, Q):
+    rng = np.random.default_rng(23)
+    X = rng.random(dims)
+    for mode in range(3):
+        F = rng.random((dims[mode], Q))
+        Y = native.mode_product(_dev(X, dt), _dev(F, dt), mode,
+                                precision="fp64" if dt == torch.float64 else "fp32_simt")
+        ref = np.moveaxis(np.tensordot(_dev(X, dt).double().cpu().numpy(),
+                                       _dev(F, dt).double().cpu().numpy(), axes=([mode], [0])),
+                          -1, mode)
+        np.testing.assert_allclose(Y.double().cpu().numpy(), ref, rtol=0, atol=tol * ref.max())
