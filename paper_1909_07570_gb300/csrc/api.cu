@@ -197,9 +197,9 @@ int nncp_run(int n_jobs, const nncp_job* jobs, const nnc_opts* o, double* rel_er
   std::vector<nncp_job> host(jobs, jobs + n_jobs);
   NNC_CUDA_TRY(cudaMemcpyAsync(dev, host.data(), sizeof(nncp_job) * n_jobs,
                                cudaMemcpyHostToDevice, s));
-  const TuneKey key = nncp_tune_key(jobs, n_jobs, sizeof(T));
+  const TuneKey key = nncp_tune_key(jobs, n_jobs, sizeof(T), rt.rp);
   NNC_TRY(run_tuned(key, o->iters, 256, s, [&](int threads, int sweeps, bool last) -> int {
-    NNC_CUDA_TRY(launch_nncp<T>(dev, n_jobs, rt.smem, sweeps, o->eps, last ? rel_errs : nullptr,
+    NNC_CUDA_TRY(launch_nncp<T>(dev, n_jobs, rt.smem, rt.rp, sweeps, o->eps, last ? rel_errs : nullptr,
                                 last ? statuses : nullptr, s, threads));
     return NNC_OK;
   }));

@@ -8,7 +8,7 @@
 namespace nnc {
 
 // The kernel family and the shape classes a choice is cached under.
-enum TuneKernel { kTuneNncp = 0, kTuneNtdSmall, kTuneNtdL2, kTuneCpxL2, kTuneNmfSmall, kTuneNtdBlk };
+enum TuneKernel { kTuneNncp = 0, kTuneNtdSmall, kTuneNtdL2, kTuneCpxL2, kTuneNmfSmall, kTuneNtdBlk, kTuneNncp3 };
 
 struct TuneKey {
   int kernel;    // TuneKernel

@@ -25,7 +25,8 @@ size_t nncp_smem_bytes(const nncp_job& j, size_t elem);
 // (nncp_core_fit_batched and its no-alloc variant) take their decision here,
 // so they cannot drift apart.
 struct NncpRoute {
-  size_t smem = 0;        // one-pass kernel: dynamic shared memory (largest valid job)
+  size_t smem = 0;        // one-pass kernels: dynamic shared memory (largest valid job)
+  int rp = 0;             // row tile of the jobs that run with their core in shared memory
   bool two_pass = false;  // the two-pass sweep (two passes over the tensor) takes the batch
   bool cluster = false;   // ... as one thread-block cluster per fit (nncp_cluster_batched)
   int invalid = 0;        // jobs that fail nncp_job_valid
@@ -36,7 +37,8 @@ struct NncpRoute {
 // mode and sweep), so a batch holding a tensor of 16384 entries or more goes
 // to the two-pass kernel when that kernel can take it (every valid job 3-way,
 // r <= 16, its arrays within one block), and so does a batch whose one-pass
-// state exceeds 200 KiB of shared memory. UNSUPPORTED (with a detail) when
+// state exceeds 200 KiB of shared memory. In the one-pass kernel a 3-way job
+// with r <= 16 that fits in a block's shared memory with its core runs from there. UNSUPPORTED (with a detail) when
 // neither kernel takes the batch. A two-pass batch runs one cluster of
 // cpx_cluster_ctas() CTAs per fit when the clusters of all its valid jobs fit
 // on the GPU at once and every job's slabs fit in a CTA's shared memory (a
@@ -46,7 +48,7 @@ struct NncpRoute {
 template <typename T>
 int nncp_route(int n_jobs, const nncp_job* jobs, bool skip_invalid, NncpRoute* rt);
 
-// One block of `threads` threads (32 .. 256) per job; jobs_dev is a device
+// One block of `threads` threads (32 .. 256) per job (smem and rp from the route); jobs_dev is a device
 // array of n_jobs descriptors whose cores and factors hold elements of type T.
 // rel_errs (device, n_jobs) may be NULL. statuses (device, n_jobs) may be
 // NULL; a block writes NNC_OK, NNC_ERR_NONFINITE (a non-finite entry in its
@@ -54,8 +56,9 @@ int nncp_route(int n_jobs, const nncp_job* jobs, bool skip_invalid, NncpRoute* r
 // NNC_ERR_INVALID_ARG (descriptor fails nncp_job_valid: nothing else done).
 // Results do not depend on `threads`.
 template <typename T>
-cudaError_t launch_nncp(const nncp_job* jobs_dev, int n_jobs, size_t smem, int iters, double eps,
-                        double* rel_errs, int* statuses, cudaStream_t s, int threads = 256);
+cudaError_t launch_nncp(const nncp_job* jobs_dev, int n_jobs, size_t smem, int rp, int iters,
+                        double eps, double* rel_errs, int* statuses, cudaStream_t s,
+                        int threads = 256);
 
 // The two-pass sweep with one thread-block cluster per fit (nncp_cluster.cu):
 // 3-way jobs, any r <= 32; jobs that fail nncp_job_valid are skipped
@@ -70,6 +73,6 @@ int cpx_cluster_ctas();
 
 // The tuning class of a batch (largest per-sweep work over the valid jobs,
 // number of jobs).
-TuneKey nncp_tune_key(const nncp_job* jobs, int n_jobs, size_t elem);
+TuneKey nncp_tune_key(const nncp_job* jobs, int n_jobs, size_t elem, int rp);
 
 }  // namespace nnc

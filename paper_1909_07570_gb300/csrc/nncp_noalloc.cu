@@ -75,8 +75,8 @@ int run_noalloc(int n_jobs, const nncp_job* jobs, const nnc_opts* o, double* rel
                                cudaMemcpyHostToDevice, s));
   // A block size tuned by an earlier allocating call of the same class is
   // reused; this call never times anything.
-  const int threads = tuned_threads(nncp_tune_key(jobs, n_jobs, sizeof(T)), 256);
-  NNC_CUDA_TRY(launch_nncp<T>(table, n_jobs, rt.smem, o->iters, o->eps, rel_errs, statuses, s,
+  const int threads = tuned_threads(nncp_tune_key(jobs, n_jobs, sizeof(T), rt.rp), 256);
+  NNC_CUDA_TRY(launch_nncp<T>(table, n_jobs, rt.smem, rt.rp, o->iters, o->eps, rel_errs, statuses, s,
                               threads));
   return NNC_OK;
 }

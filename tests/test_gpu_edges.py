@@ -181,3 +181,29 @@ def test_simt_mode_products(dt, tol, dims, Q):
                                        _dev(F, dt).double().cpu().numpy(), axes=([mode], [0])),
                           -1, mode)
         np.testing.assert_allclose(Y.double().cpu().numpy(), ref, rtol=0, atol=tol * ref.max())
+
+
+# Core fits with the core in shared memory: modes of one entry, modes longer and shorter than
+# a block, every row tile (r 1..4, 5..8, 9..16) in one batch, and a core that only the L1 form
+# takes. Five sweeps: FP64 1e-9, FP32 1e-4.
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+@pytest.mark.parametrize("jobs", [
+    [((1, 1, 1), 1), ((4, 4, 4), 3), ((5, 1, 3), 4)],
+    [((16, 16, 16), 8), ((2, 13, 7), 5), ((6, 5, 4), 2)],
+    [((9, 12, 17), 16), ((3, 33, 2), 9), ((8, 8, 8), 7), ((2, 2, 2), 1)],
+    [((40, 3, 64), 16), ((24, 24, 24), 12)],
+    [((6, 7, 5), 17), ((3, 3, 3), 2)]])
+def test_core_fits_in_shared_memory(dt, jobs):
+    rng = np.random.default_rng(29)
+    probs = [(rng.random(m), inputs.initial_cp(m, r, 7 + i)) for i, (m, r) in enumerate(jobs)]
+    dev = [(_dev(G, dt), [_dev(b, dt) for b in B]) for G, B in probs]
+    st = torch.full((len(jobs),), 9, dtype=torch.int32, device="cuda")
+    errs = native.nncp_core_fit_batched(dev, 5, statuses=st).cpu().numpy()
+    assert st.tolist() == [0] * len(jobs)
+    tol = _TOL[dt]
+    for (G, B0), (Gd, B), e in zip(probs, dev, errs):
+        Gr = Gd.double().cpu().numpy()
+        Bo, tro = orc.nncp_fit(Gr, [_dev(b, dt).double().cpu().numpy() for b in B0], 5)
+        for a, b in zip(B, Bo):
+            np.testing.assert_allclose(a.double().cpu().numpy(), b, rtol=tol, atol=tol * 1e-3)
+        assert e == pytest.approx(tro[-1], abs=tol)
