@@ -832,40 +832,39 @@ int graph_kernels(cudaGraph_t graph, long long* kernels) {
   return NNC_OK;
 }
 
-// Captures `first`, `rest` and `last` (stream-ordered work on one private
-// stream) as three CUDA graphs and runs first once, rest count - 1 times and
-// last once, after the work queued on s (count >= 1).
+// Runs `first`, count - 1 times `rest`, and `last` (stream-ordered work on one private
+// stream) after the work queued on s (count >= 1). `rest` is captured as a CUDA graph
+// and replayed; `first` and `last` run once and are launched as they are, `first` before
+// the capture, which the host makes while the device runs it.
 template <typename First, typename Rest, typename Last>
 int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last last) {
   if (count <= 0) return NNC_OK;
-  PgGraph g[3];
-  NNC_CUDA_TRY(cudaStreamCreateWithFlags(&g[0].cs, cudaStreamNonBlocking));
-  NNC_CUDA_TRY(cudaEventCreateWithFlags(&g[0].fork, cudaEventDisableTiming));
-  NNC_CUDA_TRY(cudaEventCreateWithFlags(&g[0].join, cudaEventDisableTiming));
-  cudaStream_t cs = g[0].cs;
-  NNC_CUDA_TRY(cudaEventRecord(g[0].fork, s));
-  NNC_CUDA_TRY(cudaStreamWaitEvent(cs, g[0].fork, 0));
-  long long kernels[3] = {0, 0, 0};
-  auto capture = [&](int i, auto& body) -> int {
-    NNC_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    const int st = body(cs);
-    const cudaError_t e = cudaStreamEndCapture(cs, &g[i].graph);
-    if (st != NNC_OK) return st;
-    NNC_CUDA_TRY(e);
-    NNC_CUDA_TRY(cudaGraphInstantiate(&g[i].exec, g[i].graph, 0));
-    return graph_kernels(g[i].graph, &kernels[i]);
-  };
-  NNC_TRY(capture(0, first));
-  NNC_TRY(capture(1, rest));
-  NNC_TRY(capture(2, last));
-  NNC_CUDA_TRY(cudaGraphLaunch(g[0].exec, cs));
-  for (int t = 1; t < count; ++t) NNC_CUDA_TRY(cudaGraphLaunch(g[1].exec, cs));
-  NNC_CUDA_TRY(cudaGraphLaunch(g[2].exec, cs));
-  note_graph_launches(kernels[0] + kernels[1] * (count - 1) + kernels[2]);
-  NNC_CUDA_TRY(cudaEventRecord(g[0].join, cs));
-  NNC_CUDA_TRY(cudaStreamWaitEvent(s, g[0].join, 0));
-  NNC_CUDA_TRY(cudaStreamSynchronize(cs));
-  return NNC_OK;
+  PgGraph g;
+  NNC_CUDA_TRY(cudaStreamCreateWithFlags(&g.cs, cudaStreamNonBlocking));
+  NNC_CUDA_TRY(cudaEventCreateWithFlags(&g.fork, cudaEventDisableTiming));
+  NNC_CUDA_TRY(cudaEventCreateWithFlags(&g.join, cudaEventDisableTiming));
+  NNC_CUDA_TRY(cudaEventRecord(g.fork, s));
+  NNC_CUDA_TRY(cudaStreamWaitEvent(g.cs, g.fork, 0));
+  const int st1 = first(g.cs);
+  int st2 = st1;
+  if (st1 == NNC_OK && count > 1) {
+    NNC_CUDA_TRY(cudaStreamBeginCapture(g.cs, cudaStreamCaptureModeThreadLocal));
+    st2 = rest(g.cs);
+    const cudaError_t e = cudaStreamEndCapture(g.cs, &g.graph);
+    if (st2 == NNC_OK) {
+      NNC_CUDA_TRY(e);
+      NNC_CUDA_TRY(cudaGraphInstantiate(&g.exec, g.graph, 0));
+      long long kernels = 0;
+      NNC_TRY(graph_kernels(g.graph, &kernels));
+      for (int t = 1; t < count; ++t) NNC_CUDA_TRY(cudaGraphLaunch(g.exec, g.cs));
+      note_graph_launches(kernels * (count - 1));
+    }
+  }
+  if (st2 == NNC_OK) st2 = last(g.cs);
+  NNC_CUDA_TRY(cudaEventRecord(g.join, g.cs));
+  NNC_CUDA_TRY(cudaStreamWaitEvent(s, g.join, 0));
+  NNC_CUDA_TRY(cudaStreamSynchronize(g.cs));
+  return st2;
 }
 
 }  // namespace

@@ -317,6 +317,10 @@ struct GraphRun {
   cudaGraphExec_t exec[3] = {};
   cudaEvent_t fork = nullptr, join = nullptr;
   ~GraphRun() {
+    // A call that fails half way leaves no work on its scratch behind (a call that ends
+    // well has waited already).
+    for (cudaStream_t q : {br.s2, br.s3, cs})
+      if (q) cudaStreamSynchronize(q);
     for (int k = 0; k < 3; ++k) {
       if (exec[k]) cudaGraphExecDestroy(exec[k]);
       if (graph[k]) cudaGraphDestroy(graph[k]);
@@ -388,8 +392,8 @@ struct Checkpoints {
   }
 };
 
-// Captures the sweep on a private stream and replays it `count` times after
-// the work already queued on `s`, runs the last sweep's core update, and makes
+// Runs the sweep `count` times on a private stream (the first few launched as they
+// are, the others replayed from captured graphs) after the work already queued on `s`, runs the last sweep's core update, and makes
 // `s` wait for all of it. The core update a replay runs first is the previous
 // sweep's; in the first replay there is none, and the core kernels see the
 // pending flag at 0 and return at once. `first` is the fit's index of the
@@ -415,13 +419,7 @@ int run_sweeps(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double
   NNC_CUDA_TRY(cudaEventRecord(g.fork, s));
   NNC_CUDA_TRY(cudaStreamWaitEvent(g.cs, g.fork, 0));
 
-  NNC_TRY(capture_sweep<T>(X, F, G, b, eps, trace, nullptr, tcp, true, g, 0));
   long long kn[3] = {0, 0, 0};
-  NNC_TRY(count_kernel_nodes(g.graph[0], &kn[0]));
-  if (count >= kSweepsPerGraph) {
-    NNC_TRY(capture_sweep<T>(X, F, G, b, eps, trace, nullptr, tcp, true, g, 2, kSweepsPerGraph));
-    NNC_TRY(count_kernel_nodes(g.graph[2], &kn[2]));
-  }
   const bool checkpoints = ck && ck->every > 0 && trace;
 
   // Sampled sweeps: the last of every kProfileEvery (an instrumented copy,
@@ -431,15 +429,28 @@ int run_sweeps(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double
   const int samples = profile_enabled() ? count / kProfileEvery : 0;
   long long kernels = 0;
   int t = 0;
+  // The first sweeps are launched as they are, so that the device is busy while the
+  // host captures the graph of the others (capturing and instantiating it takes the time
+  // of several sweeps of a mid-size tensor).
+  const int direct = samples > 0 ? 0 : std::min(count, kSweepsPerGraph);
   while (t < count) {
     const bool sampled = samples > 0 && t % kProfileEvery == kProfileEvery - 1;
     // A five-sweep replay must not pass a sampled sweep or a checkpoint (its
     // last sweep may be one).
-    bool five = !sampled && g.exec[2] && t + kSweepsPerGraph <= count &&
+    bool five = !sampled && t >= direct && t + kSweepsPerGraph <= count &&
                 (samples == 0 || t % kProfileEvery + kSweepsPerGraph <= kProfileEvery - 1);
     if (five && checkpoints)
       for (int u = t; u < t + kSweepsPerGraph - 1; ++u) five = five && !ck->at(first + u);
-    if (five) {
+    if (t < direct) {
+      NNC_TRY(sweep3<T>(X, F, G, b, eps, trace ? trace : b.trace_dummy, trace ? 1 : 0, nullptr, tcp,
+                        /*prev_core=*/true, g.br, g.cs));
+      ++t;
+    } else if (five) {
+      if (!g.exec[2]) {
+        NNC_TRY(capture_sweep<T>(X, F, G, b, eps, trace, nullptr, tcp, true, g, 2,
+                                 kSweepsPerGraph));
+        NNC_TRY(count_kernel_nodes(g.graph[2], &kn[2]));
+      }
       NNC_CUDA_TRY(cudaGraphLaunch(g.exec[2], g.cs));
       kernels += kn[2];
       t += kSweepsPerGraph;
@@ -456,6 +467,10 @@ int run_sweeps(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double
       kernels += kn[1];
       ++t;
     } else {
+      if (!g.exec[0]) {
+        NNC_TRY(capture_sweep<T>(X, F, G, b, eps, trace, nullptr, tcp, true, g, 0));
+        NNC_TRY(count_kernel_nodes(g.graph[0], &kn[0]));
+      }
       NNC_CUDA_TRY(cudaGraphLaunch(g.exec[0], g.cs));
       kernels += kn[0];
       ++t;
