@@ -471,12 +471,14 @@ int nncp_route(int n_jobs, const nncp_job* jobs, bool skip_invalid, NncpRoute* r
   // The cluster form: every valid job 3-way with slabs within a CTA, and a
   // cluster per valid job on the GPU at once.
   bool cl_ok = true;
-  int valid = 0;
+  int valid = 0, rmax = 1;
+  for (int i = 0; i < n_jobs; ++i)
+    if (nncp_job_valid(jobs[i])) rmax = std::max(rmax, (int)jobs[i].r);
   for (int i = 0; i < n_jobs; ++i) {
     const nncp_job& j = jobs[i];
     if (!nncp_job_valid(j)) continue;
     ++valid;
-    if (j.d != 3 || cpx_cluster_elems(j) * sizeof(T) > kSmemBudget) cl_ok = false;
+    if (j.d != 3 || cpx_cluster_elems(j, rmax) * sizeof(T) > kSmemBudget) cl_ok = false;
   }
   cl_ok = cl_ok && valid >= 1 && (int64_t)valid * cpx_cluster_ctas() <= device_sm_count();
   constexpr int64_t kTwoPassMinEntries = 16384;

@@ -61,14 +61,15 @@ cudaError_t launch_nncp(const nncp_job* jobs_dev, int n_jobs, size_t smem, int r
                         int threads = 256);
 
 // The two-pass sweep with one thread-block cluster per fit (nncp_cluster.cu):
-// 3-way jobs, any r <= 32; jobs that fail nncp_job_valid are skipped
+// 3-way jobs, r <= 16; jobs that fail nncp_job_valid are skipped
 // (statuses: INVALID_ARG); statuses and rel_errs as in nncp_l2_batched.
 template <typename T>
 int nncp_cluster_batched(int n_jobs, const nncp_job* jobs, int iters, double eps,
                          double* rel_errs, int* statuses, cudaStream_t s);
-// Shared-memory elements of one CTA of a cluster fit of job j, and the CTAs
+// Shared-memory elements of one CTA of a cluster fit of job j in a batch whose largest
+// rank is rmax, and the CTAs
 // of a cluster.
-size_t cpx_cluster_elems(const nncp_job& j);
+size_t cpx_cluster_elems(const nncp_job& j, int rmax);
 int cpx_cluster_ctas();
 
 // The tuning class of a batch (largest per-sweep work over the valid jobs,

@@ -1,28 +1,33 @@
 // nnCPD of a 3-way core by one thread-block cluster per fit (Alg. 1, step 2):
-// the Gauss-Seidel sweep of cpx_l2_kernel (small_batched.cu), a sweep
+// the Gauss-Seidel sweep
 //   T   = G x_3 A3^T              MT1[i, q] = sum_j T[i, j, q] A2[j, q]    A1 <- MU
-//                                 MT2[j, q] = sum_i T[i, j, q] A1[i, q]    A2 <- MU
-//   T'  = G x_1 A1^T              MT3[k, q] = sum_j T'[q, j, k] A2[j, q]   A3 <- MU
+//   T'  = G x_1 A1^T              MT2[j, q] = sum_k T'[j, k, q] A3[k, q]   A2 <- MU
+//                                 MT3[k, q] = sum_j T'[j, k, q] A2[j, q]   A3 <- MU
 // with A_n <- max(A_n * MT_n / max(A_n V_n, eps), 0), V_n the Hadamard product
-// of the other factors' Grams, spread over kCl CTAs instead of one.
+// of the other factors' Grams, spread over kCl CTAs.
 //
-// CTA c of the cluster keeps, in shared memory, the slab of the core with
-// i in [c ni, (c + 1) ni) (for T) and the slab with k in [c nk, (c + 1) nk)
-// (for T'), and a copy of every factor and Gram. It forms T and T' on its
-// slabs, MT1 and MT3 on its rows, and the new rows of A1 and A3 for its i and
-// k; the MU step of A2 (whose MT2 sums over every i) runs in every CTA on the
-// same data. Twice per sweep the CTAs exchange through distributed shared
-// memory what the others need:
-//   after A1:  its new A1 rows, its share of Gram1 and its share of MT2;
-//   after A3:  its new A3 rows and its share of Gram3;
-// each CTA writes them to an outbox of its own, the cluster synchronises, and
-// every CTA reads all outboxes, adding the shares in CTA order (so every CTA
-// holds bit-identical factors and Grams, and results do not depend on timing).
-// The second exchange's barrier also tells every CTA that the first outbox has
-// been read, and the next sweep's first barrier the same of the second, so two
-// barriers per sweep suffice.
+// CTA c of the cluster owns the rows of every factor in its ranges of i, j and k and keeps, in
+// shared memory, the slab of the core with its i (for T), the slab with its j (for
+// T'), and full copies of every factor and Gram. T and T' on its slabs give MT1 and MT2 on its
+// own rows and its share of MT3; new rows go to the other CTAs through distributed
+// shared memory, into the copy of the factor that no CTA reads any more (two
+// copies, swapped at the barrier), the shares of MT3 to the CTA that owns the row k, which
+// adds them in CTA order: every CTA holds the same bits and results do not depend
+// on timing. Three cluster barriers and three block barriers a sweep:
+//   T, Gram3 | MT1, MU on A1, rows sent   || T', Gram1 | MT2, MU on A2, rows sent |
+//   shares of MT3 sent || Gram2 | MT3, MU on A3, rows sent ||
+// Every contraction is short and latency bounds it: eight lanes share an output of a
+// MU step, one term in eight of the numerator and of the denominator each, and lane u
+// sends the new entry to CTA u. In FP64 the FP64 units bound the products (a warp-wide FMA
+// takes 16 cycles): no padded entry is formed and each Gram once, by symmetry.
+// A sweep, FP32, against the form that took mode 2 from T (its MTTKRP summed over every
+// CTA's slab and its MU step repeated in every CTA; two cluster barriers, twelve block barriers):
+//   32^3, r = 16    10.7 -> 7.7 us          40^3, r = 10     19.4 -> 9.1 us
+//   16 x 64 x 16    11.8 -> 6.8 us          64 x 4 x 64      10.5 -> 8.3 us (r = 13)
+// and in FP64 32^3 at r = 16 50.8 -> 50.8, at r = 5 22.3 -> 20.3 us.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "kernels.cuh"
@@ -37,127 +42,92 @@ constexpr int kClThreads = 512;
 
 __host__ __device__ constexpr size_t al4(size_t x) { return (x + 3) & ~static_cast<size_t>(3); }
 
-// Element offsets of one CTA's shared memory.
+// Element offsets of one CTA's shared memory; factors, Grams and products have rows of rp.
 struct ClLayout {
-  int ni, nk;  // slab widths
-  int xpitch;  // row pitch of the i-slab
-  size_t xi, xk, a[3], g[3], tb, mt, den, v, ob1, ob2, total;
-  __host__ __device__ explicit ClLayout(const int* N, int r) {
+  int ni, nj, nk;  // rows of each factor a CTA owns
+  int xpitch;      // row pitch of the i-slab
+  size_t xi, xj, a[2][3], g[3], tb, in, total;
+  __host__ __device__ explicit ClLayout(const int* N, int rp) {
     ni = (N[0] + kCl - 1) / kCl;
+    nj = (N[1] + kCl - 1) / kCl;
     nk = (N[2] + kCl - 1) / kCl;
-    int nmax = N[0] > N[1] ? N[0] : N[1];
-    nmax = nmax > N[2] ? nmax : N[2];
     size_t p = 0;
     xpitch = N[2] | 1;  // odd: the rows a warp reads fall on distinct banks
     xi = p;  p += al4((size_t)ni * N[1] * xpitch);  // [ii][j][k], rows xpitch apart
-    xk = p;  p += al4((size_t)N[0] * N[1] * nk);  // [i][j][kk]
-    for (int n = 0; n < 3; ++n) { a[n] = p;  p += al4((size_t)N[n] * r); }
-    for (int n = 0; n < 3; ++n) { g[n] = p;  p += al4((size_t)r * r); }
-    const size_t t3 = (size_t)ni * N[1] * r, t1 = (size_t)N[1] * nk * r;
-    tb = p;  p += al4(t3 > t1 ? t3 : t1);           // T [ii][j][q], then T' [j][kk][q]
-    mt = p;  p += al4((size_t)nmax * r);
-    den = p; p += al4((size_t)nmax * r);
-    v = p;   p += al4((size_t)r * r);
-    ob1 = p; p += al4((size_t)ni * r + (size_t)r * r + (size_t)N[1] * r);
-    ob2 = p; p += al4((size_t)nk * r + (size_t)r * r);
+    xj = p;  p += al4((size_t)N[0] * nj * N[2]);    // [i][jj][k]
+    for (int b = 0; b < 2; ++b)
+      for (int n = 0; n < 3; ++n) { a[b][n] = p;  p += (size_t)N[n] * rp; }
+    for (int n = 0; n < 3; ++n) { g[n] = p;  p += (size_t)rp * rp; }
+    const size_t t3 = (size_t)ni * N[1] * rp, t1 = (size_t)nj * N[2] * rp;
+    tb = p;  p += t3 > t1 ? t3 : t1;                // T [ii][j][q], then T' [jj][k][q]
+    in = p;  p += (size_t)kCl * nk * rp;            // shares of MT3 for this CTA's k
     total = p;
   }
 };
 
-// out[e] = sum_{t < len} term(e, t, .) for e < nout, with term(e, t, s) =
-// fma(x_t, y_t, s): for len >= 16 four consecutive lanes share an output,
-// lane u adds the terms t = u, u + 4, ... in order, and a fixed shuffle tree
-// adds the four partial sums (the reductions of the sweep are latency-bound;
-// this keeps four times more of them in flight); shorter ones take one lane
-// each, terms in order. Every thread of the block calls it.
-template <typename T, typename F>
-__device__ __forceinline__ void dots4(int nout, int len, F term, T* out) {
-  if (len < 16) {  // too short to share: one lane per output
-    for (int e = threadIdx.x; e < nout; e += blockDim.x) {
-      T s = T(0);
-      for (int t = 0; t < len; ++t) s = term(e, t, s);
-      out[e] = s;
-    }
-    return;
-  }
-  const int per = blockDim.x / 4, u = threadIdx.x & 3;
-  for (int e0 = 0; e0 < nout; e0 += per) {
-    const int e = e0 + (int)threadIdx.x / 4;
-    T s = T(0);
-    if (e < nout)
-      for (int t = u; t < len; t += 4) s = term(e, t, s);
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    if (e < nout && u == 0) out[e] = s;
-  }
-}
-
-// gram[a, b] = sum_{i < n} A[i, a] A[i, b] (A: n x r, row-major).
-template <typename T>
-__device__ void gram_rows(const T* A, int n, int r, T* gram) {
-  dots4<T>(r * r, n, [&](int e, int i, T s) {
-    const int a = e / r, b = e - a * r;
-    return fma(A[i * r + a], A[i * r + b], s);
-  }, gram);
-}
-
-// MU on rows [0, n) of A (row-major, r wide) with numerators MT (n x r):
-// A <- max(A * MT / max(A V, eps), 0). den is scratch, n x r.
-template <typename T>
-__device__ void mu_rows_local(T* A, const T* MT, const T* V, int n, int r, T eps, T* den) {
-  dots4<T>(n * r, r, [&](int e, int p, T s) {
-    const int i = e / r, q = e - i * r;
-    return fma(A[i * r + p], V[p * r + q], s);
-  }, den);
-  __syncthreads();
-  for (int e = threadIdx.x; e < n * r; e += blockDim.x) {
-    const T v = A[e] * MT[e] / (den[e] > eps ? den[e] : eps);
-    A[e] = v > T(0) ? v : T(0);
-  }
-  __syncthreads();
-}
-
-// P[row, q] = sum_{t < len} x[row, t] F[t, q] for row < nrow, q < r, where
-// x[row, t] = X[xo(row) + t xs] and F is len x r: four q per thread (four
-// independent accumulators, F read in 16-byte rows) when r % 4 == 0.
-template <typename T, typename XO>
-__device__ void pass_quads(int nrow, int len, int r, const T* X, XO xo, int64_t xs, const T* F,
-                           T* P) {
-  if ((r & 3) == 0) {
-    const int nq = r / 4;
-    for (int e = threadIdx.x; e < nrow * nq; e += blockDim.x) {
-      const int row = e / nq, q = 4 * (e - row * nq);
-      const T* x = X + xo(row);
-      T a0 = T(0), a1 = T(0), a2 = T(0), a3 = T(0);
-#pragma unroll 4
+// P[row, q] = sum_{t < len} x[t xs] F[t, q] for row < rows, q < r, x = X + xo(row), F and P
+// with rows of RP. FP32: a thread per 16-byte piece of a row; FP64: a thread per entry
+// (the FP64 units bound it, so no entry of the padding is formed).
+template <typename T, int RP, typename XO>
+__device__ __forceinline__ void row_products(int rows, int len, int r, const T* X, XO xo, int xs,
+                                             const T* F, T* P) {
+  constexpr int VW = sizeof(T) == 4 ? 4 : 1;
+  const int np = VW == 4 ? RP / 4 : r;
+  for (int e = threadIdx.x; e < rows * np; e += kClThreads) {
+    const int row = e / np, q = (e - row * np) * VW;
+    const T* x = X + xo(row);
+    if constexpr (VW == 4) {
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
       for (int t = 0; t < len; ++t) {
-        const T v = x[t * xs];
-        T f[4];
-        if constexpr (sizeof(T) == 4) {  // F rows start on 16 bytes (r % 4 == 0)
-          const float4 w = *reinterpret_cast<const float4*>(F + t * r + q);
-          f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w;
-        } else {
-          const double2 w0 = *reinterpret_cast<const double2*>(F + t * r + q);
-          const double2 w1 = *reinterpret_cast<const double2*>(F + t * r + q + 2);
-          f[0] = w0.x; f[1] = w0.y; f[2] = w1.x; f[3] = w1.y;
-        }
-        a0 = fma(v, f[0], a0);
-        a1 = fma(v, f[1], a1);
-        a2 = fma(v, f[2], a2);
-        a3 = fma(v, f[3], a3);
+        const float v = x[t * xs];
+        const float4 w = *reinterpret_cast<const float4*>(F + t * RP + q);
+        s.x = fmaf(v, w.x, s.x);
+        s.y = fmaf(v, w.y, s.y);
+        s.z = fmaf(v, w.z, s.z);
+        s.w = fmaf(v, w.w, s.w);
       }
-      T* o = P + (size_t)row * r + q;
-      o[0] = a0; o[1] = a1; o[2] = a2; o[3] = a3;
+      *reinterpret_cast<float4*>(P + row * RP + q) = s;
+    } else {
+      T s = T(0);
+#pragma unroll 8
+      for (int t = 0; t < len; ++t) s = fma(x[t * xs], F[t * RP + q], s);
+      P[row * RP + q] = s;
     }
-  } else {
-    dots4<T>(nrow * r, len, [&](int e, int t, T s) {
-      const int row = e / r, q = e - row * r;
-      return fma(X[xo(row) + t * xs], F[t * r + q], s);
-    }, P);
   }
 }
 
-template <typename T>
+// The entry (a, b), a <= b, of a Gram that a thread has a part in: four lanes an entry
+// where the block has the threads (r <= 12: 78 entries), two for up to 136 entries.
+template <int RP>
+struct GramLane {
+  int a = 0, b, u, nl;
+  bool on;
+  __device__ explicit GramLane(int r) {
+    const int ne = r * (r + 1) / 2;
+    nl = RP <= 12 || r <= 12 ? 4 : 2;  // by r alone: a batch's tile changes no bits
+    const int e = (int)threadIdx.x / nl;
+    u = (int)threadIdx.x % nl;
+    on = e < ne;
+    int k = e;
+    while (a < r && k >= r - a) k -= r - a++;
+    b = a + k;
+  }
+};
+
+// S[a, b] = S[b, a] = sum_{i < n} A[i, a] A[i, b], the lanes' sums added.
+template <typename T, int RP>
+__device__ __forceinline__ void gram_lanes(const GramLane<RP>& g, const T* A, int n, T* S) {
+  T s = T(0);
+  if (g.on) {
+#pragma unroll 4
+    for (int i = g.u; i < n; i += g.nl) s = fma(A[i * RP + g.a], A[i * RP + g.b], s);
+  }
+  for (int o = g.nl / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (g.on && g.u == 0) S[g.a * RP + g.b] = S[g.b * RP + g.a] = s;
+}
+
+template <typename T, int RP>
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     cpx_cluster_kernel(const nncp_job* __restrict__ jobs, int iters, T eps, double* rel_errs,
                        int* statuses) {
@@ -175,116 +145,125 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     return;
   }
   const int N1 = jb.m[0], N2 = jb.m[1], N3 = jb.m[2], r = jb.r;
-  const ClLayout L(jb.m, r);
+  const ClLayout L(jb.m, RP);
   T* sm = reinterpret_cast<T*>(smem_raw);
   T* Xi = sm + L.xi;
-  T* Xk = sm + L.xk;
-  T* A[3] = {sm + L.a[0], sm + L.a[1], sm + L.a[2]};
+  T* Xj = sm + L.xj;
+  T* A[3] = {sm + L.a[0][0], sm + L.a[0][1], sm + L.a[0][2]};
+  T* An[3] = {sm + L.a[1][0], sm + L.a[1][1], sm + L.a[1][2]};
   T* Gr[3] = {sm + L.g[0], sm + L.g[1], sm + L.g[2]};
   T* Tb = sm + L.tb;
-  T* MT = sm + L.mt;
-  T* den = sm + L.den;
-  T* V = sm + L.v;
-  T* ob1 = sm + L.ob1;  // [A1 rows: ni x r][Gram1 share: r x r][MT2 share: N2 x r]
-  T* ob2 = sm + L.ob2;  // [A3 rows: nk x r][Gram3 share: r x r]
-  const int i0 = c * L.ni, ni = max(0, min(L.ni, N1 - i0));
-  const int k0 = c * L.nk, nk = max(0, min(L.nk, N3 - k0));
+  T* In = sm + L.in;  // [CTA][kk][q]
+  const int i0 = min(c * L.ni, N1), ni = min(L.ni, N1 - i0);
+  const int j0 = min(c * L.nj, N2), nj = min(L.nj, N2 - j0);
+  const int k0 = min(c * L.nk, N3), nk = min(L.nk, N3 - k0);
   const T* X = static_cast<const T*>(jb.G);
-  const int tid = threadIdx.x, nt = blockDim.x;
+  const int tid = threadIdx.x, nt = kClThreads;
+  const GramLane<RP> gl(r);
 
   for (int e = tid; e < ni * N2 * N3; e += nt) {
     const int row = e / N3, k = e - row * N3;
     Xi[row * L.xpitch + k] = X[(int64_t)i0 * N2 * N3 + e];
   }
-  for (int e = tid; e < N1 * N2 * nk; e += nt) {
-    const int kk = e % nk, ij = e / nk;
-    Xk[e] = X[(int64_t)ij * N3 + k0 + kk];
+  for (int e = tid; e < N1 * nj * N3; e += nt) {
+    const int i = e / (nj * N3), jk = e - i * nj * N3;
+    Xj[e] = X[((int64_t)i * N2 + j0) * N3 + jk];
   }
   for (int n = 0; n < 3; ++n) {
     const T* src = static_cast<const T*>(jb.B[n]);
-    for (int e = tid; e < jb.m[n] * r; e += nt) A[n][e] = src[e];
+    for (int e = tid; e < jb.m[n] * RP; e += nt) {
+      const int i = e / RP, q = e % RP;
+      A[n][e] = q < r ? src[i * r + q] : T(0);
+      An[n][e] = T(0);
+    }
   }
   __syncthreads();
-  for (int n = 0; n < 3; ++n) gram_rows(A[n], jb.m[n], r, Gr[n]);
-  __syncthreads();
+  gram_lanes<T, RP>(gl, A[1], N2, Gr[1]);
+  // No CTA sends before every CTA's copies are zeroed.
+  cl.sync();
+
+  // The MU step on rows r0 .. r0 + rows - 1 of factor n: num(i, q, u) is lane u's part of
+  // the numerator of row r0 + i, Ga .* Gb = V_n. Eight lanes an entry; lane u sends
+  // it to CTA u.
+  const int u = tid & 7;
+  auto mu_rows = [&](int n, int r0, int rows, const T* Ga, const T* Gb, auto num) {
+    const T* f = A[n] + r0 * RP;
+    for (int e0 = 0; e0 < rows * r; e0 += nt / 8) {
+      const int e = e0 + tid / 8, i = e / r, q = e - i * r;
+      const bool on = e < rows * r;
+      T s = T(0), den = T(0);
+      if (on) {
+        s = num(i, q);
+        for (int p = u; p < r; p += 8) den = fma(f[i * RP + p], Ga[p * RP + q] * Gb[p * RP + q], den);
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+      }
+      if (on) {
+        T v = f[i * RP + q] * s / (den > eps ? den : eps);
+        v = v > T(0) ? v : T(0);
+        T* const dst = An[n] + (r0 + i) * RP + q;
+        if (u == c)
+          *dst = v;
+        else
+          *cl.map_shared_rank(dst, u) = v;
+      }
+    }
+  };
+  auto swap = [&](int n) {
+    T* t = A[n];
+    A[n] = An[n];
+    An[n] = t;
+  };
+  static_assert(kCl == 8, "lane u of an entry serves CTA u");
 
   for (int it = 0; it < iters; ++it) {
-    // ---- T[ii, j, q] = sum_k Xi[ii, j, k] A3[k, q]; MT1 on this CTA's rows --
-    pass_quads<T>(ni * N2, N3, r, Xi, [&](int row) { return (int64_t)row * L.xpitch; }, 1, A[2],
-                  Tb);
-    for (int e = tid; e < r * r; e += nt) V[e] = Gr[1][e] * Gr[2][e];
+    // ---- T[ii, j, :] on this CTA's i; Gram3
+    row_products<T, RP>(ni * N2, N3, r, Xi, [&](int row) { return row * L.xpitch; }, 1, A[2], Tb);
+    gram_lanes<T, RP>(gl, A[2], N3, Gr[2]);
     __syncthreads();
-    dots4<T>(ni * r, N2, [&](int e, int j, T s) {
-      const int ii = e / r, q = e - ii * r;
-      return fma(Tb[(ii * N2 + j) * r + q], A[1][j * r + q], s);
-    }, MT);
+    // ---- A1
+    mu_rows(0, i0, ni, Gr[1], Gr[2], [&](int i, int q) {
+      T s = T(0);
+#pragma unroll 4
+      for (int j = u; j < N2; j += 8) s = fma(Tb[(i * N2 + j) * RP + q], A[1][j * RP + q], s);
+      return s;
+    });
+    cl.sync();
+    swap(0);
+    // ---- T'[jj, k, :] on this CTA's j; Gram1
+    row_products<T, RP>(nj * N3, N1, r, Xj, [&](int jk) { return jk; }, nj * N3, A[0], Tb);
+    gram_lanes<T, RP>(gl, A[0], N1, Gr[0]);
     __syncthreads();
-    // ---- the new rows i0 .. i0 + ni - 1 of A1 ---------------------------------
-    mu_rows_local(A[0] + (size_t)i0 * r, MT, V, ni, r, eps, den);
-    // ---- outbox 1: those rows, their Gram share, their MT2 share --------------
+    // ---- A2
+    mu_rows(1, j0, nj, Gr[0], Gr[2], [&](int j, int q) {
+      T s = T(0);
+#pragma unroll 4
+      for (int k = u; k < N3; k += 8) s = fma(Tb[(j * N3 + k) * RP + q], A[2][k * RP + q], s);
+      return s;
+    });
+    __syncthreads();
+    // ---- this CTA's share of MT3 to the owners of the rows k
     {
-      const T* a1 = A[0] + (size_t)i0 * r;
-      for (int e = tid; e < ni * r; e += nt) ob1[e] = a1[e];
-      gram_rows(a1, ni, r, ob1 + L.ni * r);
-      dots4<T>(N2 * r, ni, [&](int e, int ii, T s) {
-        const int j = e / r, q = e - j * r;
-        return fma(Tb[(ii * N2 + j) * r + q], a1[ii * r + q], s);
-      }, ob1 + L.ni * r + r * r);
+      const T* a2 = An[1] + j0 * RP;  // its new rows of A2
+      for (int e = tid; e < N3 * r; e += nt) {
+        const int k = e / r, q = e - k * r, o = k / L.nk;
+        T s = T(0);
+#pragma unroll 4
+        for (int j = 0; j < nj; ++j) s = fma(Tb[(j * N3 + k) * RP + q], a2[j * RP + q], s);
+        *cl.map_shared_rank(In + (c * L.nk + k - o * L.nk) * RP + q, o) = s;
+      }
     }
     cl.sync();
-    // ---- gather A1, Gram1 and MT2 from every CTA, shares added in CTA order ---
-    for (int e = tid; e < r * r + N2 * r; e += nt) {
-      T v[kCl];
-#pragma unroll
-      for (int c2 = 0; c2 < kCl; ++c2) v[c2] = cl.map_shared_rank(ob1, c2)[L.ni * r + e];
-      T acc = v[0];
-#pragma unroll
-      for (int c2 = 1; c2 < kCl; ++c2) acc += v[c2];
-      if (e < r * r) Gr[0][e] = acc;
-      else MT[e - r * r] = acc;
-    }
-    for (int e = tid; e < N1 * r; e += nt) {
-      const int c2 = (e / r) / L.ni;
-      A[0][e] = cl.map_shared_rank(ob1, c2)[e - c2 * L.ni * r];
-    }
+    swap(1);
+    // ---- Gram2; A3
+    gram_lanes<T, RP>(gl, A[1], N2, Gr[1]);
     __syncthreads();
-    // ---- A2 in every CTA alike -------------------------------------------------
-    for (int e = tid; e < r * r; e += nt) V[e] = Gr[0][e] * Gr[2][e];
-    __syncthreads();
-    mu_rows_local(A[1], MT, V, N2, r, eps, den);
-    // ---- T'[j, kk, q] = sum_i A1[i, q] Xk[i, j, kk]; MT3 on this CTA's rows ---
-    gram_rows(A[1], N2, r, Gr[1]);
-    pass_quads<T>(N2 * nk, N1, r, Xk, [&](int jk) { return (int64_t)jk; }, (int64_t)N2 * nk,
-                  A[0], Tb);
-    __syncthreads();
-    for (int e = tid; e < r * r; e += nt) V[e] = Gr[0][e] * Gr[1][e];
-    dots4<T>(nk * r, N2, [&](int e, int j, T s) {
-      const int kk = e / r, q = e - kk * r;
-      return fma(Tb[(j * nk + kk) * r + q], A[1][j * r + q], s);
-    }, MT);
-    __syncthreads();
-    // ---- the new rows k0 .. k0 + nk - 1 of A3; outbox 2 -----------------------
-    mu_rows_local(A[2] + (size_t)k0 * r, MT, V, nk, r, eps, den);
-    {
-      const T* a3 = A[2] + (size_t)k0 * r;
-      for (int e = tid; e < nk * r; e += nt) ob2[e] = a3[e];
-      gram_rows(a3, nk, r, ob2 + L.nk * r);
-    }
+    mu_rows(2, k0, nk, Gr[0], Gr[1], [&](int k, int q) { return In[(u * L.nk + k) * RP + q]; });
     cl.sync();
-    for (int e = tid; e < r * r; e += nt) {
-      T v[kCl];
-#pragma unroll
-      for (int c2 = 0; c2 < kCl; ++c2) v[c2] = cl.map_shared_rank(ob2, c2)[L.nk * r + e];
-      T acc = v[0];
-#pragma unroll
-      for (int c2 = 1; c2 < kCl; ++c2) acc += v[c2];
-      Gr[2][e] = acc;
-    }
-    for (int e = tid; e < N3 * r; e += nt) {
-      const int c2 = (e / r) / L.nk;
-      A[2][e] = cl.map_shared_rank(ob2, c2)[e - c2 * L.nk * r];
-    }
-    __syncthreads();
+    swap(2);
   }
 
   // ||G - I x_k A_k||^2 and ||G||^2 on this CTA's slab (FP64, in an order fixed
@@ -293,7 +272,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     const int k = (int)(e % N3), ij = (int)(e / N3), j = ij % N2, ii = ij / N2;
     T hat = T(0);
     for (int q = 0; q < r; ++q)
-      hat = fma(A[0][(i0 + ii) * r + q] * A[1][j * r + q], A[2][k * r + q], hat);
+      hat = fma(A[0][(i0 + ii) * RP + q] * A[1][j * RP + q], A[2][k * RP + q], hat);
     const double g = (double)Xi[ij * L.xpitch + k], d = g - (double)hat;
     return make_double2(d * d, g * g);
   }, red);
@@ -307,8 +286,9 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     for (int n = 0; n < 3; ++n) {
       T* dst = static_cast<T*>(jb.B[n]);
       for (int e = tid; e < jb.m[n] * r; e += nt) {
-        dst[e] = A[n][e];
-        finite = finite && isfinite(A[n][e]);
+        const T v = A[n][(e / r) * RP + e % r];
+        dst[e] = v;
+        finite = finite && isfinite(v);
       }
     }
     const int ok = __syncthreads_and(finite ? 1 : 0);
@@ -330,24 +310,27 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
 
 }  // namespace
 
-size_t cpx_cluster_elems(const nncp_job& j) { return ClLayout(j.m, j.r).total; }
+size_t cpx_cluster_elems(const nncp_job& j, int rmax) {
+  return ClLayout(j.m, (rmax + 3) / 4 * 4).total;
+}
 
 int cpx_cluster_ctas() { return kCl; }
 
 template <typename T>
 int nncp_cluster_batched(int n_jobs, const nncp_job* jobs, int iters, double eps,
                          double* rel_errs, int* statuses, cudaStream_t s) {
-  size_t elems = 0;
+  int rmax = 1;
   for (int i = 0; i < n_jobs; ++i) {
-    const nncp_job& j = jobs[i];
-    if (!nncp_job_valid(j)) continue;  // the kernel reports it in its status
-    if (j.d != 3) {
-      set_error_detail_text("cluster nnCP: a 4-way job");
+    if (!nncp_job_valid(jobs[i])) continue;  // the kernel reports it in its status
+    rmax = jobs[i].r > rmax ? jobs[i].r : rmax;
+    if (jobs[i].d != 3 || jobs[i].r > 16) {
+      set_error_detail_text("cluster nnCP: a 4-way job or a rank above 16");
       return NNC_ERR_UNSUPPORTED;
     }
-    const size_t e = cpx_cluster_elems(j);
-    elems = e > elems ? e : elems;
   }
+  size_t elems = 0;
+  for (int i = 0; i < n_jobs; ++i)
+    if (nncp_job_valid(jobs[i])) elems = std::max(elems, cpx_cluster_elems(jobs[i], rmax));
   const size_t smem = elems * sizeof(T);
   if (smem > kSmemBudget) {
     set_error_detail_text("cluster nnCP: a job's slabs exceed one block of shared memory");
@@ -359,9 +342,14 @@ int nncp_cluster_batched(int n_jobs, const nncp_job* jobs, int iters, double eps
   std::vector<nncp_job> host(jobs, jobs + n_jobs);  // staged before cudaMemcpyAsync returns
   NNC_CUDA_TRY(cudaMemcpyAsync(dev, host.data(), sizeof(nncp_job) * n_jobs,
                                cudaMemcpyHostToDevice, s));
-  NNC_CUDA_TRY(raise_smem_limit((const void*)cpx_cluster_kernel<T>, smem));
-  cpx_cluster_kernel<T><<<(unsigned)(n_jobs * kCl), kClThreads, smem, s>>>(dev, iters, (T)eps,
-                                                                           rel_errs, statuses);
+  // rows of a multiple of four entries (16-byte reads), as few as the largest rank needs:
+  // the slabs' limit in shared memory stays where rows of r put it, but for a few per cent
+  const auto kern = rmax <= 4    ? cpx_cluster_kernel<T, 4>
+                    : rmax <= 8  ? cpx_cluster_kernel<T, 8>
+                    : rmax <= 12 ? cpx_cluster_kernel<T, 12>
+                                 : cpx_cluster_kernel<T, 16>;
+  NNC_CUDA_TRY(raise_smem_limit((const void*)kern, smem));
+  kern<<<(unsigned)(n_jobs * kCl), kClThreads, smem, s>>>(dev, iters, (T)eps, rel_errs, statuses);
   note_launch(s);
   NNC_CUDA_TRY(cudaGetLastError());
   return NNC_OK;

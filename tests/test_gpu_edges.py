@@ -207,3 +207,29 @@ def test_core_fits_in_shared_memory(dt, jobs):
         for a, b in zip(B, Bo):
             np.testing.assert_allclose(a.double().cpu().numpy(), b, rtol=tol, atol=tol * 1e-3)
         assert e == pytest.approx(tro[-1], abs=tol)
+
+
+# Core fits of 16384 entries or more, one cluster each: modes shorter than the cluster (CTAs
+# without rows of a factor), every row tile (4, 8, 12, 16), ranks that are not multiples of
+# four, and fits of several ranks and shapes in one batch (each keeps the bits of its own fit).
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+@pytest.mark.parametrize("jobs", [
+    [((64, 5, 64), 4)],
+    [((64, 5, 52), 12), ((64, 64, 4), 1), ((4, 64, 64), 4)],
+    [((64, 4, 64), 16)],
+    [((33, 9, 60), 11), ((26, 31, 27), 5), ((40, 17, 33), 13)]])
+def test_core_fits_on_clusters(dt, jobs):
+    rng = np.random.default_rng(37)
+    probs = [(rng.random(m), inputs.initial_cp(m, r, 11 + i)) for i, (m, r) in enumerate(jobs)]
+    dev = [(_dev(G, dt), [_dev(b, dt) for b in B]) for G, B in probs]
+    errs = native.nncp_core_fit_batched(dev, 5).cpu().numpy()
+    tol = _TOL[dt]
+    for (G, B0), (Gd, B), e in zip(probs, dev, errs):
+        Gr = Gd.double().cpu().numpy()
+        Bo, tro = orc.nncp_fit(Gr, [_dev(b, dt).double().cpu().numpy() for b in B0], 5)
+        for a, b in zip(B, Bo):
+            np.testing.assert_allclose(a.double().cpu().numpy(), b, rtol=tol, atol=tol * 1e-3)
+        assert e == pytest.approx(tro[-1], abs=tol)
+        one = [_dev(b, dt) for b in B0]
+        assert native.nncp_core_fit(Gd, one, 5) == e
+        assert all(torch.equal(a, b) for a, b in zip(one, B))
