@@ -118,10 +118,16 @@ struct GramLane {
 // S[a, b] = S[b, a] = sum_{i < n} A[i, a] A[i, b], the lanes' sums added.
 template <typename T, int RP>
 __device__ __forceinline__ void gram_lanes(const GramLane<RP>& g, const T* A, int n, T* S) {
-  T s = T(0);
+  T s = T(0), s1 = T(0);  // two sums a lane: half the chain, and half its rounding
   if (g.on) {
-#pragma unroll 4
-    for (int i = g.u; i < n; i += g.nl) s = fma(A[i * RP + g.a], A[i * RP + g.b], s);
+    int i = g.u;
+#pragma unroll 2
+    for (; i + g.nl < n; i += 2 * g.nl) {
+      s = fma(A[i * RP + g.a], A[i * RP + g.b], s);
+      s1 = fma(A[(i + g.nl) * RP + g.a], A[(i + g.nl) * RP + g.b], s1);
+    }
+    if (i < n) s = fma(A[i * RP + g.a], A[i * RP + g.b], s);
+    s += s1;
   }
   for (int o = g.nl / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (g.on && g.u == 0) S[g.a * RP + g.b] = S[g.b * RP + g.a] = s;
