@@ -714,8 +714,12 @@ constexpr int kF16MinStages = 3;
 // product in an accumulator: at NP = 32 the four K steps of a stage go to four
 // accumulators, 32 products each in a group of two stages. With one group a
 // tile (64 products an accumulator at K = 256) the factors after 30 sweeps were
-// 1.5 times as far from 64 bits as with the TF32x3 passes.
-constexpr int kF16Group = 2;
+// 1.5 times as far from 64 bits as with the TF32x3 passes. Up to 128 K entries the
+// TF32x3 pass puts 32 products in an accumulator too and the FP16 form is the less exact
+// per product: there a group is one stage (128^3 x 64, 30 sweeps: F4 1.24e-6 from 64 bits
+// with groups of two, 0.93e-6 with one, TF32x3 0.94e-6; 19.9 -> 20.4 ms). For longer K
+// groups of two are closer than TF32x3 (512^3: 9e-7 against 1.3e-5) and 5 % faster.
+__host__ __device__ constexpr int f16_group(int nk) { return nk <= 2 ? 1 : 2; }
 
 struct F16Operand {
   const float* F;       // K x q row-major
@@ -918,11 +922,12 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       const uint32_t idesc2 = f16_instr_desc(kMN, 2 * NP);
       const uint64_t bdesc_base = smem_desc(smem_u32(bs), 16, 1024);
       bool ok = mbar_wait(&bready, 0, vfail);
-      int gcount = 0, rs = 0;  // groups of kF16Group stages; the ring's stage
+      int gcount = 0, rs = 0;  // groups of stages; the ring's stage
+      const int group = f16_group(nk);
       uint32_t rph = 0;
       for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-        for (int k0 = 0; ok && k0 < nk; k0 += kF16Group, ++gcount) {
-          const int buf = gcount & 1, kend = min(nk, k0 + kF16Group);
+        for (int k0 = 0; ok && k0 < nk; k0 += group, ++gcount) {
+          const int buf = gcount & 1, kend = min(nk, k0 + group);
           if (gcount >= 2 && !mbar_wait(&accempty[buf], ((gcount >> 1) - 1) & 1, vfail)) {
             ok = false;
             break;
@@ -975,6 +980,7 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       float* Fs = Ps + 128 * 32;                  // FUSE: 128 x 32 factor rows
       int gcount = 0;
       int64_t fs_slice = -1;
+      const int group = f16_group(nk);
       for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         if constexpr (FUSE) {
           if (tile % ep.y_nh != fs_slice) {
@@ -994,7 +1000,7 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
 #pragma unroll
         for (int t = 0; t < NP; ++t) sum[t] = 0.f;
         bool got = true;
-        for (int k0 = 0; k0 < nk; k0 += kF16Group, ++gcount) {
+        for (int k0 = 0; k0 < nk; k0 += group, ++gcount) {
           const int buf = gcount & 1;
           got = mbar_wait(&accfull[buf], (gcount >> 1) & 1, vfail);
           if constexpr (FUSE) got = epi_all(got);
