@@ -8,7 +8,7 @@ per second over the timed steps (device time, inputs resident in HBM).
 
 The default workload is the 512^3 precision workload under the paper's
 protocol (5000 iterations per sub-solve, Sec. 4.1): the nnTD sweeps run on the
-BF16 copy of X except the last 200, which are FP32 (TF32x3) refinement sweeps.
+BF16 copy of X except the last 200, which are FP32 (FP16 pairs) refinement sweeps.
 The same step with FP32 passes throughout is timed beside it, and both final
 relative errors come from explicit FP64 passes: the comparison at equal
 relative error. Convergence records (exact checkpoints every 50 sweeps) give
@@ -278,9 +278,9 @@ def pass_rooflines(prof, w, dt_bytes, peaks, peak_src, workload):
     from paper_1909_07570_gb300 import native
     hbm = peak_value(peaks, "hbm_gbs", "hbm_GBps", "hbm") or FALLBACK_PEAKS["hbm_gbs"]
     nX = int(np.prod(w.dims))
-    names = {0: "ttm_rows_kernel", 1: "ttm_cols_kernel", 2: "tc_pass_kernel<bf16> (X x_3 F3^T)",
-             3: "tc_pass_kernel<bf16> (X x_1 F1^T)", 4: "tc_pass_kernel<tf32x3> (X x_3 F3^T)",
-             5: "tc_pass_kernel<tf32x3> (X x_1 F1^T)"}
+    names = {0: "ttm_rows_kernel", 1: "ttm_cols_pipe_kernel", 2: "tc_pass_kernel<bf16> (X x_3 F3^T)",
+             3: "tc_pass_kernel<bf16> (X x_1 F1^T)", 4: "f16_pass_kernel (X x_3 F3^T)",
+             5: "f16_pass_kernel (X x_1 F1^T)"}
     recs = []
     for kind in sorted(prof, key=lambda k: prof[k][1], reverse=True):
         n_l, ms_l = prof[kind]
@@ -375,9 +375,9 @@ def run_native(args, rank, world):
             "planted_rank": w.planted_rank, "ntd_sweeps_per_step": w.iters,
             "nncp_sweeps_per_step": w.cp_iters, "refine_sweeps": w.refine_iters,
             "step": "ntd_fit (with FP64 trace) + nncp_core_fit + candelinc_lift + recon_residual",
-            "passes": {"fp32": "tcgen05 TF32x3 (FP32-accurate, 3 products per term)",
+            "passes": {"fp32": "tcgen05 FP16 pairs (FP32-accurate, 3 products per term)",
                        "bf16": "tcgen05 BF16 with per-slice power-of-two scales; the last "
-                               f"{w.refine_iters} sweeps tcgen05 TF32x3 (FP32 refinement)",
+                               f"{w.refine_iters} sweeps tcgen05 FP16 pairs (FP32 refinement)",
                        "fp64": "SIMT FP64"}[precision],
             "l2": f"X ({X.numel() * X.element_size() >> 20} MiB) larger than L2, and flushed "
                   f"between timed steps ({L2_FLUSH_BYTES >> 20} MiB write)",
@@ -391,7 +391,7 @@ def run_native(args, rank, world):
     }
     peaks, peak_src = load_peaks()
 
-    # The same step with the plain FP32 (TF32x3) passes: the comparison at
+    # The same step with the plain FP32 (FP32-accurate) passes: the comparison at
     # equal relative error (same sweeps, same start; both final errors from an
     # explicit FP64 pass).
     if precision == "bf16" and rank == 0 and world == 1:
@@ -562,7 +562,7 @@ def line_40cube(dev, steps=5):
 
 def line_256cube(dev, steps=5):
     """The 256^3 FP32 workload (rank 10, m = 20, 500 + 500 sweeps): the whole
-    Alg. 1 step on the TF32x3 passes, device time, and its pass rooflines."""
+    Alg. 1 step on the FP32-accurate passes, device time, and its pass rooflines."""
     import torch
 
     from paper_1909_07570_gb300 import inputs, native
@@ -594,7 +594,7 @@ def line_256cube(dev, steps=5):
 
 
 def precision_form(dev):
-    """BF16 + FP32-refinement vs FP32 (TF32x3) nnTD on the 512^3 precision
+    """BF16 + FP32-refinement vs FP32 nnTD on the 512^3 precision
     workload: sweeps/s of device time and the final relative error of each."""
     import torch
 
@@ -632,7 +632,7 @@ def precision_form(dev):
 
 def differentiation_form(dev):
     """Block projected-gradient steps on the lifted loss (the hand-written
-    adjoint, two TF32x3 passes over X per step) on the 4-way 128^3 x 64
+    adjoint, two FP32-accurate passes over X per step) on the 4-way 128^3 x 64
     workload: steps/s of device time (marginal over the setup) and the fit."""
     import numpy as np
     import torch
@@ -668,7 +668,7 @@ def differentiation_form(dev):
 
 
 def ntd_4way(dev):
-    """nnTD of the 4-way 128^3 x 64 workload (two TF32x3 passes over X per
+    """nnTD of the 4-way 128^3 x 64 workload (two FP32-accurate passes over X per
     sweep, the d-way mode-product sweep): sweeps/s of device time (marginal
     over the setup) and the final relative error."""
     import numpy as np

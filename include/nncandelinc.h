@@ -100,7 +100,7 @@ typedef struct {
  *  X          device, dims[0] x ... x dims[d-1], entries >= 0 and finite
  *  d          3 or 4. d = 4 runs the same sweep on the d-way mode-product
  *             machinery of the differentiation form (two passes over X per
- *             sweep, the FP32 passes on the TF32x3 tensor-core kernel with X
+ *             sweep, the FP32 passes FP32-accurate on the tensor cores with X
  *             viewed as dims[0] x dims[1]*dims[2] x dims[3]); it has no
  *             NNC_BF16_REFINE form (UNSUPPORTED)
  *  dims, m    host arrays of d entries; 1 <= m[n] <= 64, dims[n] >= 1
@@ -238,7 +238,8 @@ typedef struct {
 /*
  * nncp_core_fit_batched - many independent nncp_core_fit problems (uneven
  * shapes and ranks: restarts, candidate ranks, several tensors) in one
- * launch, one thread block per job. Same update rule and options as
+ * launch, one thread block per job, the core and every array of a 3-way job
+ * with r <= 16 in shared memory where they fit. Same update rule and options as
  * nncp_core_fit. A batch holding a large tensor (16384 entries or more, such
  * as X itself in Alg. 2, e.g. 40 x 40 x 40) runs with the tensors read twice
  * per sweep from global memory when every job is 3-way with r <= 16 and its
@@ -279,7 +280,7 @@ int nncp_core_fit_batched(int n_jobs, const nncp_job* jobs, int precision, const
  * Who needs it: a host runtime that owns all device memory through its own
  * pool and forbids a library to allocate behind its back; a latency-critical
  * loop where an allocation may stall, or fail when the GPU's memory is nearly
- * all handed out. The allocating call takes its job table from cudaMallocAsync;
+ * all handed out. The allocating call takes its job table from the library's pool;
  * this one keeps the table in a fixed array inside the library's device memory
  * (4096 descriptors, 256 KiB, held on every GPU that loads the library until
  * the process exits) and calls no allocator at all.
@@ -362,8 +363,8 @@ int candelinc_lift(int d, const int64_t* dims, const int* m, int r, int precisio
  *  gF, gB     host arrays of d device pointers shaped like F and B (written),
  *             or both NULL for the loss alone
  *  loss       host, L with FP64 accumulation (may be NULL when gF is given)
- *  precision  NNC_FP64 (double); NNC_FP32 (float, TF32x3 tensor-core passes
- *             where the shape allows, else SIMT); NNC_FP32_SIMT (float)
+ *  precision  NNC_FP64 (double); NNC_FP32 (float, FP32-accurate tensor-core
+ *             passes where the shape allows, else SIMT); NNC_FP32_SIMT (float)
  * Errors: INVALID_ARG, NONFINITE (X), UNSUPPORTED (NNC_BF16_REFINE), CUDA,
  * ALLOC, TIMEOUT.
  */
@@ -408,7 +409,7 @@ int candelinc_pg_fit(const void* X, int d, const int64_t* dims, const int* m, in
  *             NULL
  *  rel_err    host, the final relative error from one explicit FP64 pass over
  *             X (NaN for 0 sweeps), or NULL
- *  precision  NNC_FP64, NNC_FP32 (TF32x3 tensor-core passes), NNC_FP32_SIMT
+ *  precision  NNC_FP64, NNC_FP32 (FP32-accurate tensor-core passes), NNC_FP32_SIMT
  * Errors: INVALID_ARG, NONFINITE (X, or a sweep whose FP64 residual terms
  * were not finite), UNSUPPORTED, CUDA, ALLOC, TIMEOUT.
  */
@@ -471,8 +472,9 @@ int recon_residual(const void* X, int d, const int64_t* dims, int precision, int
  *   1  X x_1 F^(1)T, SIMT passes
  *   2  X x_3 F^(3)T, BF16 tensor-core passes
  *   3  X x_1 F^(1)T, BF16 tensor-core passes
- *   4  X x_3 F^(3)T, TF32x3 tensor-core passes (NNC_FP32, refinement sweeps)
- *   5  X x_1 F^(1)T, TF32x3 tensor-core passes
+ *   4  X x_3 F^(3)T, FP32-accurate tensor-core passes (NNC_FP32, refinement
+ *      sweeps)
+ *   5  X x_1 F^(1)T, FP32-accurate tensor-core passes
  * nnc_profile_enable(on) switches it and clears the totals; nnc_profile_read
  * returns the number of timed launches and their total milliseconds of a
  * kind. Meant for one thread of control: concurrent ntd_fit calls while it is
@@ -516,7 +518,7 @@ int nnc_wait_selftest(long long cycles, void* stream);
 /*
  * Failure-injection hook for tests (not a step of the method; off by
  * default). Arms the nth scratch allocation from now (nth >= 1; 0 disarms) to
- * fail on the host as if cudaMallocAsync had returned an error, without
+ * fail on the host as if the pool had returned an error, without
  * calling the allocator: the call that makes it returns NNC_ERR_ALLOC, releases
  * the scratch it already holds, and leaves the CUDA context usable. Shared by
  * every thread of the process. Returns the previous countdown.

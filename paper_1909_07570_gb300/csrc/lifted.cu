@@ -12,8 +12,8 @@
 //
 // X is read twice per gradient: T_last = X x_d F^(d)T serves every Z_n with
 // n < d (further mode products on the compressed tensor), and
-// T_first = X x_1 F^(1)T serves Z_d. FP32 runs both passes on the TF32x3
-// tensor-core kernel with X viewed as 3-way (N_1, N_2 ... N_{d-1}, N_d); FP64
+// T_first = X x_1 F^(1)T serves Z_d. FP32 runs both passes on the
+// FP32-accurate tensor-core kernels with X viewed as 3-way (N_1, N_2 ... N_{d-1}, N_d); FP64
 // and FP32_SIMT run the SIMT mode products. The loss comes out of the same
 // terms in FP64: L = 1/2 ||X||^2 - <MT_n, A^(n)> + 1/2 sum(V_n .* A^(n)T A^(n)).
 //
@@ -882,8 +882,8 @@ int lifted_pg_fit(const T* X, int d, const int64_t* dims, const int* m, int r, b
   NNC_TRY(sc.get(&counter, 2));
   NNC_CUDA_TRY(cudaMemsetAsync(counter, 0, 2 * sizeof(int), s));
   if (steps > 0) {
-    // The steps are captured as CUDA graphs on a private stream and replayed; the
-    // trace slot advances through the device counter.
+    // The first and the last step are launched as they are, the others replayed from
+    // one CUDA graph on a private stream; the trace slot advances through the device counter.
     SideStream side, step_size;
     NNC_TRY(side.init());
     NNC_TRY(step_size.init());

@@ -2,7 +2,7 @@
 // not allocate device memory.
 //
 // nncp_core_fit_batched takes its job table (one descriptor per fit) from
-// cudaMallocAsync. Some callers cannot let a library allocate: a host runtime
+// the library's memory pool. Some callers cannot let a library allocate: a host runtime
 // that owns all device memory through its own pool or arena and forbids
 // allocations behind its back, a real-time or latency-critical loop where an
 // allocation may stall or fail under memory pressure, or a process that has

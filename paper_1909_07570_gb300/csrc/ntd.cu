@@ -19,11 +19,13 @@
 // BF16 copy of X (tc_ttm.cu). Two reads of X per sweep is the minimum under
 // the Gauss-Seidel order: pass 2 needs the F^(1) that pass 1 leads to.
 //
-// The sweep is captured as a CUDA graph on a private stream (several sweeps to
-// a graph) and replayed; the trace slot advances through a device counter. NNC_FP32 runs the passes
-// as FP32-accurate TF32x3 tensor-core products; NNC_BF16_REFINE replays the
-// BF16 tensor-core sweep for iters - refine_iters sweeps and then the TF32x3
-// sweep for the rest; NNC_FP32_SIMT and NNC_FP64 use the SIMT passes.
+// The sweep runs on private streams: the first few sweeps are launched as they are, while
+// the host captures a CUDA graph (several sweeps to a graph) that the others replay; the
+// trace slot advances through a device counter. Small tensors run all sweeps in one launch on
+// one cluster instead (ntd_cluster.cu). NNC_FP32 runs the passes as FP32-accurate
+// tensor-core products (FP16 pairs, or TF32x3 where a factor is too long for them);
+// NNC_BF16_REFINE runs the BF16 tensor-core sweep for iters - refine_iters sweeps and
+// then the FP32-accurate one for the rest; NNC_FP32_SIMT and NNC_FP64 use the SIMT passes.
 #include <algorithm>
 #include <type_traits>
 #include <vector>
@@ -94,7 +96,7 @@ int pass_x1(const T* X, const NtdState<T>& b, const T* F1, const T* F2, const tc
 
 // The tensor-core form of the factor updates' GEMMs (UpdArgs::tc): TF32
 // beside BF16 passes, whose rounding of X dominates; split TF32 (FP32-accurate)
-// beside TF32x3 passes; none on the SIMT path.
+// beside FP32-accurate passes; none on the SIMT path.
 inline int upd_tc(const tc::TcPlan* tcp) {
   return tcp ? (tcp->kind == tc::kKindBf16 ? 1 : 3) : 0;
 }
@@ -179,7 +181,7 @@ int sweep3(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double* tr
   // step.
   //   s2:  H2 ................ MU on F2 | H3 (S2 of the new F2)
   //   s3:  Num2 (P3, new F1) --^
-  // When pass 2 can also form the shares of Y3[k] = P1[k]^T F2 (TF32x3 with
+  // When pass 2 can also form the shares of Y3[k] = P1[k]^T F2 (FP32-accurate with
   // N2 % 128 == 0, m <= 32), it waits for the new F2 and the mode-3 update
   // only adds the shares; H3 runs beside the pass:
   //   s:   pass 2 (new F1, new F2) -- mode 3 (shares, H3)
@@ -393,8 +395,8 @@ struct Checkpoints {
 };
 
 // Runs the sweep `count` times on a private stream (the first few launched as they
-// are, the others replayed from captured graphs) after the work already queued on `s`, runs the last sweep's core update, and makes
-// `s` wait for all of it. The core update a replay runs first is the previous
+// are, the others replayed from captured graphs) after the work already queued on `s`,
+// runs the last sweep's core update, and makes `s` wait for all of it. The core update a replay runs first is the previous
 // sweep's; in the first replay there is none, and the core kernels see the
 // pending flag at 0 and return at once. `first` is the fit's index of the
 // first of these sweeps; *done gets the number of sweeps run, fewer than
@@ -537,8 +539,8 @@ int ntd_fit3_small(const T* X, const int64_t* dims, const int* m, const nnc_opts
   return NNC_OK;
 }
 
-// passes: 0 = SIMT for every sweep; 1 = TF32x3 tensor cores for every sweep
-// (FP32-accurate); 2 = BF16 tensor cores, then TF32x3 for the refinement sweeps.
+// passes: 0 = SIMT for every sweep; 1 = FP32-accurate tensor cores for every
+// sweep; 2 = BF16 tensor cores, then FP32-accurate ones for the refinement sweeps.
 // A tensor-core plan that the shape does not allow falls back to SIMT passes.
 template <typename T>
 int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts* o, T* const* F,
@@ -597,10 +599,10 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
   if constexpr (std::is_same<T, float>::value) {
     if (passes == 2 && o->iters > o->refine_iters) {
       NNC_TRY(plan16.init(tc::kKindBf16, X, N1, N2, N3, m1, m3, sc, s, /*p1_kj=*/true));
-      // The BF16 passes stream X about twice as fast as the TF32x3 ones and
+      // The BF16 passes stream X about twice as fast as FP32-accurate ones and
       // the small kernels beside them would otherwise hold SMs the pass
       // waits for: they leave 32 SMs to them (measured at 512^3, m = 32: 258
-      // -> 225 us per sweep; the TF32x3 sweep is fastest with every SM).
+      // -> 225 us per sweep).
       plan16.reserve_sms = 32;
       fast = &plan16;
     }
@@ -636,7 +638,7 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
   }
   if constexpr (std::is_same<T, float>::value) {
     // The tensor-core passes form the shares of Y1 when the shape allows it
-    // (y1_fusable), the TF32x3 passes also those of Y3 (y3_fusable).
+    // (y1_fusable), the FP32-accurate passes also those of Y3 (y3_fusable).
     const tc::TcPlan* any = exact ? exact : fast;
     if (any && any->y1_fusable(m2)) {
       b.y_nh = (int)(N2 / 128);

@@ -147,8 +147,9 @@ constexpr size_t pipe_smem_bytes() {
 // blockIdx.x BC), rows j of split blockIdx.y. Copies of CV entries: 16 bytes where
 // C % CV == 0 keeps each in one row (l, j), else single entries (rows of Y that start
 // anywhere: 301 x 55335, Q = 24, 66.6 us with loads straight into registers, whose
-// latency nothing hid, 56.1 us through the ring, both beside the mode-2 branch). Rows and columns past the ends are staged as
-// zeros (Fm rows too), so every chunk runs all kPipeBJ rows.
+// latency nothing hid, 56.1 us through the ring, both beside the mode-2 branch). Rows
+// and columns past the ends are staged as zeros (Fm rows too), so every chunk runs all
+// kPipeBJ rows.
 template <typename T, int QP, int TC, int CV>
 __global__ void __launch_bounds__(kColsThreads, QP * TC * sizeof(T) < 256 ? 2 : 1)
 ttm_cols_pipe_kernel(const T* __restrict__ Y, int64_t L, int J, int64_t C, int j_per_split, const T* __restrict__ Fm, int64_t fs_j, int64_t fs_q, int Q,
