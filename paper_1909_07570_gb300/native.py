@@ -410,7 +410,7 @@ def candelinc_lifted_grad(X, F, B, precision=None, grads=True, stream=None):
 
     Returns (loss, gF, gB) with gF[n], gB[n] shaped like F[n], B[n]; with
     grads=False only the loss is computed (gF = gB = None). precision: "fp64",
-    "fp32" (TF32x3 tensor-core passes) or "fp32_simt"."""
+    "fp32" (FP32-accurate tensor-core passes) or "fp32_simt"."""
     code, dtype = _precision(X, precision)
     _require(X, dtype, "X")
     d = X.dim()
