@@ -196,9 +196,12 @@ __device__ void fit_one(const nncp_job& job, int iters, T eps, unsigned char* sm
 //   1  T[i, j, :] = sum_k G[i, j, k] B3[k, :]        Gram3
 //   2  B1 <- MU (Num1[i, q] = sum_j T[i, j, q] B2[j, q])
 //   3  Num2[j, q] = sum_i T[i, j, q] B1[i, q]        Gram1
-//   4  B2 <- MU;  T'[j, k, :] = sum_i G[i, j, k] B1[i, :]
-//   5  Num3[k, q] = sum_j T'[j, k, q] B2[j, q]       Gram2
-//   6  B3 <- MU
+//   4  B2 <- MU
+//   5  T'[i, k, :] = sum_j G[i, j, k] B2[j, :]       Gram2
+//   6  B3 <- MU (Num3[k, q] = sum_i T'[i, k, q] B1[i, q])
+// Every sum has fit_one's terms in fit_one's order, and so its bits (T' = G x_1 B1, ready an
+// interval earlier, would sum mode 3 over i inside j; a few ill-conditioned fits among
+// thousands amplify that rounding to 1e-3 of an entry).
 // Rows of B and T are padded with zeros to RP entries and read in 16-byte pieces, a thread
 // forming a whole row of T; rows of G have an odd pitch. A MU step writes the copy of
 // the factor it does not read, and takes V as the product of two Grams in place. No sum
@@ -209,9 +212,9 @@ constexpr size_t kFit3Bytes = kSmemBudget;
 __host__ __device__ inline int fit3_rp(int r) { return r <= 4 ? 4 : (r <= 8 ? 8 : 16); }
 __host__ __device__ inline size_t fit3_elems(const nncp_job& j) {
   const int rp = fit3_rp(j.r), m1 = j.m[0], m2 = j.m[1], m3 = j.m[2];
-  const int msum = m1 + m2 + m3, mmax = m1 > m2 ? (m1 > m3 ? m1 : m3) : (m2 > m3 ? m2 : m3);
-  const size_t t = (size_t)m2 * (m1 > m3 ? m1 : m3) * rp;
-  return (size_t)2 * msum * rp + 3 * rp * rp + (size_t)mmax * rp + t + (size_t)m1 * m2 * (m3 | 1);
+  const int msum = m1 + m2 + m3;
+  const size_t t = (size_t)m1 * (m2 > m3 ? m2 : m3) * rp;
+  return (size_t)2 * msum * rp + 3 * rp * rp + (size_t)m2 * rp + t + (size_t)m1 * m2 * (m3 | 1);
 }
 __host__ __device__ inline bool fit3_takes(const nncp_job& j, size_t elem) {
   return j.d == 3 && j.r <= 16 && fit3_elems(j) * elem <= kFit3Bytes;
@@ -222,7 +225,7 @@ __device__ __forceinline__ void fit3(const nncp_job& job, int iters, T eps, unsi
                                      double* fpart, double* rel_err_out, int* status_out) {
   constexpr int VW = 16 / (int)sizeof(T);
   const int m1 = job.m[0], m2 = job.m[1], m3 = job.m[2], r = job.r, gp = m3 | 1;
-  const int mmax = max(m1, max(m2, m3)), tid = threadIdx.x, nt = blockDim.x;
+  const int tid = threadIdx.x, nt = blockDim.x;
   T* B[3];
   T* Bn[3];
   B[0] = reinterpret_cast<T*>(smem);
@@ -236,8 +239,8 @@ __device__ __forceinline__ void fit3(const nncp_job& job, int iters, T eps, unsi
   Gr[1] = Gr[0] + RP * RP;
   Gr[2] = Gr[1] + RP * RP;
   T* Num = Gr[2] + RP * RP;
-  T* Tb = Num + mmax * RP;
-  T* G = Tb + (size_t)m2 * max(m1, m3) * RP;
+  T* Tb = Num + m2 * RP;
+  T* G = Tb + (size_t)m1 * max(m2, m3) * RP;
   const T* Gg = static_cast<const T*>(job.G);
   for (int e = tid; e < m1 * m2 * m3; e += nt) G[(e / m3) * gp + e % m3] = Gg[e];
 #pragma unroll
@@ -337,17 +340,13 @@ __device__ __forceinline__ void fit3(const nncp_job& job, int iters, T eps, unsi
       mu(1, j, q, Num[j * RP + q], Gr[0], Gr[2]);
     }
     swap(1);
-    products(m2 * m3, m1, m2 * gp, [&](int row) { return (row / m3) * gp + row % m3; }, B[0]);
     __syncthreads();
     gram(B[1], m2, Gr[1]);
-    for (int e = tid; e < m3 * r; e += nt) {
-      const int k = e / r, q = e - k * r;
-      Num[k * RP + q] = numer(Tb + k * RP + q, m3 * RP, B[1] + q, m2);
-    }
+    products(m1 * m3, m2, gp, [&](int row) { return (row / m3) * m2 * gp + row % m3; }, B[1]);
     __syncthreads();
     for (int e = tid; e < m3 * r; e += nt) {
       const int k = e / r, q = e - k * r;
-      mu(2, k, q, Num[k * RP + q], Gr[0], Gr[1]);
+      mu(2, k, q, numer(Tb + k * RP + q, m3 * RP, B[0] + q, m1), Gr[0], Gr[1]);
     }
     swap(2);
     __syncthreads();

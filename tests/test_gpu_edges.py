@@ -233,3 +233,20 @@ def test_core_fits_on_clusters(dt, jobs):
         one = [_dev(b, dt) for b in B0]
         assert native.nncp_core_fit(Gd, one, 5) == e
         assert all(torch.equal(a, b) for a, b in zip(one, B))
+
+
+# A core fit in shared memory has the bits of the form that reads the core through L1, which a
+# zero column beyond rank 16 asks for: the column stays zero and adds exact zeros to every
+# sum.
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+@pytest.mark.parametrize("m,r", [((7, 8, 6), 3), ((4, 15, 9), 8), ((16, 3, 5), 5), ((2, 13, 7), 16),
+                                 ((1, 1, 1), 1), ((9, 4, 33), 11)])
+def test_core_fit_keeps_the_bits_of_the_general_form(dt, m, r):
+    rng = np.random.default_rng(41)
+    G = _dev(rng.random(m), dt)
+    B = [_dev(b, dt) for b in inputs.initial_cp(m, r, 13)]
+    wide = [torch.nn.functional.pad(b, (0, 17 - r)).contiguous() for b in B]
+    e, ew = native.nncp_core_fit(G, B, 60), native.nncp_core_fit(G, wide, 60)
+    assert e == ew
+    for a, b in zip(B, wide):
+        assert torch.equal(a, b[:, :r]) and not b[:, r:].any()
