@@ -77,13 +77,23 @@ class Scratch {
     return NNC_OK;
   }
 
+  // Gives one block back early (stream-ordered).
+  void drop(void* p) {
+    for (int i = 0; i < n_; ++i)
+      if (p != nullptr && blocks_[i] == p) {
+        cudaFreeAsync(p, stream_);
+        blocks_[i] = blocks_[--n_];
+        return;
+      }
+  }
+
   void release() {
     for (int i = n_ - 1; i >= 0; --i) cudaFreeAsync(blocks_[i], stream_);
     n_ = 0;
   }
 
  private:
-  static constexpr int kMax = 64;
+  static constexpr int kMax = 96;
   cudaStream_t stream_;
   void* blocks_[kMax] = {};
   int n_ = 0;

@@ -443,6 +443,31 @@ int setup(Work<T>& w, const T* X, int d, const int64_t* dims, const int* m, int 
   return NNC_OK;
 }
 
+// TF32x3 passes where the FP16 pairs do not hold X (*left). Otherwise, with a guard given, that
+// of the fit's sweeps in *use (NULL: no pairs).
+template <typename T>
+int settle_pairs(Work<T>& w, bool* left, Scratch& sc, cudaStream_t s, tc::PairGuard* guard = nullptr,
+                 tc::PairGuard** use = nullptr) {
+  *left = false;
+  if (use) *use = nullptr;
+  if constexpr (std::is_same<T, float>::value) {
+    if (!w.tc) return NNC_OK;
+    NNC_TRY(w.plan.wide(s, left));
+    if (*left) return w.plan.to_tf32(w.X, sc, s);
+    if (guard && w.plan.kind == tc::kKindF16x3) {
+      NNC_TRY(guard->start(&w.plan, sc));
+      *use = guard;
+    }
+  }
+  return NNC_OK;
+}
+
+template <typename T>
+int leave_pairs(Work<T>& w, Scratch& sc, cudaStream_t s) {
+  if constexpr (std::is_same<T, float>::value) return w.plan.to_tf32(w.X, sc, s);
+  return NNC_OK;
+}
+
 // T_last = X x_d F^(d)T laid out (N_1, ..., N_{d-1}, m_d).
 template <typename T>
 int pass_last(Work<T>& w, const T* Fd, cudaStream_t s) {
@@ -691,23 +716,31 @@ int lifted_grad(const T* X, int d, const int64_t* dims, const int* m, int r, boo
   NNC_TRY(setup(w, X, d, dims, m, r, tensor_cores, sc, s, /*one_pass=*/!grads));
   for (int k = 0; k < d; ++k) NNC_TRY(refresh_a(w, k, F[k], B[k], s));
   double* dloss = w.Ls + 3;
-  NNC_TRY(pass_last(w, F[d - 1], s));
-  if (grads) {
-    NNC_TRY(pass_first(w, F[0], s));
-    NNC_TRY(make_u0(w, F[0], s));
-  }
-  for (int n = 0; n < (grads ? d : 1); ++n) {
-    const T* Z = nullptr;
-    NNC_TRY(z_chain(w, n, F, &Z, s));
-    NNC_TRY(mttkrp_and_v(w, n, Z, B, s));
-    if (n == 0) NNC_TRY(loss_into(w, 0, dloss, nullptr, nullptr, s));
-    if (!grads) break;
-    NNC_TRY(grad_a(w, n, s));
-    const int mn = m[n];
-    NNC_CUDA_TRY(small_gemm<T>((int)dims[n], mn, r, w.gA, r, 1, B[n], 1, r, nullptr, gF[n], s));
-    NNC_CUDA_TRY(small_gemm<T>(mn, r, (int)dims[n], F[n], 1, mn, w.gA, r, 1, nullptr, gB[n], s));
-  }
-  NNC_TRY(check_tc(w, s));
+  auto evaluate = [&]() -> int {
+    NNC_TRY(pass_last(w, F[d - 1], s));
+    if (grads) {
+      NNC_TRY(pass_first(w, F[0], s));
+      NNC_TRY(make_u0(w, F[0], s));
+    }
+    for (int n = 0; n < (grads ? d : 1); ++n) {
+      const T* Z = nullptr;
+      NNC_TRY(z_chain(w, n, F, &Z, s));
+      NNC_TRY(mttkrp_and_v(w, n, Z, B, s));
+      if (n == 0) NNC_TRY(loss_into(w, 0, dloss, nullptr, nullptr, s));
+      if (!grads) break;
+      NNC_TRY(grad_a(w, n, s));
+      const int mn = m[n];
+      NNC_CUDA_TRY(small_gemm<T>((int)dims[n], mn, r, w.gA, r, 1, B[n], 1, r, nullptr, gF[n], s));
+      NNC_CUDA_TRY(small_gemm<T>(mn, r, (int)dims[n], F[n], 1, mn, w.gA, r, 1, nullptr, gB[n], s));
+    }
+    return check_tc(w, s);
+  };
+  NNC_TRY(evaluate());
+  // (asked afterwards, so that the device need not wait for the host between its setup and its
+  // many small launches)
+  bool left = false;
+  NNC_TRY(settle_pairs(w, &left, sc, s));
+  if (left) NNC_TRY(evaluate());
   if (loss) {
     NNC_CUDA_TRY(cudaMemcpyAsync(loss, dloss, sizeof(double), cudaMemcpyDeviceToHost, s));
     NNC_CUDA_TRY(cudaStreamSynchronize(s));
@@ -777,12 +810,14 @@ struct PgGraph {
 
 // Captures `body` (stream-ordered work on a private stream) once as a CUDA
 // graph and replays it `count` times after the work queued on s; `after(t,
-// cs)`, if given, queues work on the private stream after replay t.
+// cs)`, if given, queues work on the private stream after replay t. A look of `guard`, if
+// given, may end it early, after *done replays.
 struct NoAfter {
   int operator()(int, cudaStream_t) const { return NNC_OK; }
 };
 template <typename Body, typename After = NoAfter>
-int replay(int count, cudaStream_t s, Body body, After after = After()) {
+int replay(int count, cudaStream_t s, Body body, After after = After(),
+           tc::PairGuard* guard = nullptr, int* done = nullptr) {
   if (count <= 0) return NNC_OK;
   PgGraph g;
   NNC_CUDA_TRY(cudaStreamCreateWithFlags(&g.cs, cudaStreamNonBlocking));
@@ -806,11 +841,20 @@ int replay(int count, cudaStream_t s, Body body, After after = After()) {
     NNC_CUDA_TRY(cudaGraphNodeGetType(nd, &ty));
     if (ty == cudaGraphNodeTypeKernel) ++kernels;
   }
-  for (int t = 0; t < count; ++t) {
+  int t = 0;
+  while (t < count) {
     NNC_CUDA_TRY(cudaGraphLaunch(g.exec, g.cs));
     NNC_TRY(after(t, g.cs));
+    ++t;
+    if (guard && t < count) {
+      // looked at once the next sweep is queued
+      if (t % tc::kPairLook == 1) NNC_TRY(guard->mark(g.cs, t));
+      if (t % tc::kPairLook == 2) NNC_TRY(guard->look(s));
+      if (guard->slow) break;
+    }
   }
-  note_graph_launches(kernels * count);
+  if (done) *done = t;
+  note_graph_launches(kernels * t);
   NNC_CUDA_TRY(cudaEventRecord(g.join, g.cs));
   NNC_CUDA_TRY(cudaStreamWaitEvent(s, g.join, 0));
   NNC_CUDA_TRY(cudaStreamSynchronize(g.cs));
@@ -835,9 +879,12 @@ int graph_kernels(cudaGraph_t graph, long long* kernels) {
 // Runs `first`, count - 1 times `rest`, and `last` (stream-ordered work on one private
 // stream) after the work queued on s (count >= 1). `rest` is captured as a CUDA graph
 // and replayed; `first` and `last` run once and are launched as they are, `first` before
-// the capture, which the host makes while the device runs it.
+// the capture, which the host makes while the device runs it. A look of `guard`, if given, may
+// end it early (`last` runs in any case), after *done of the `count`.
 template <typename First, typename Rest, typename Last>
-int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last last) {
+int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last last,
+                     tc::PairGuard* guard, int* done) {
+  *done = 0;
   if (count <= 0) return NNC_OK;
   PgGraph g;
   NNC_CUDA_TRY(cudaStreamCreateWithFlags(&g.cs, cudaStreamNonBlocking));
@@ -847,7 +894,9 @@ int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last las
   NNC_CUDA_TRY(cudaStreamWaitEvent(g.cs, g.fork, 0));
   const int st1 = first(g.cs);
   int st2 = st1;
+  int t = 1;
   if (st1 == NNC_OK && count > 1) {
+    if (guard) NNC_TRY(guard->mark(g.cs, t));
     NNC_CUDA_TRY(cudaStreamBeginCapture(g.cs, cudaStreamCaptureModeThreadLocal));
     st2 = rest(g.cs);
     const cudaError_t e = cudaStreamEndCapture(g.cs, &g.graph);
@@ -856,10 +905,17 @@ int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last las
       NNC_CUDA_TRY(cudaGraphInstantiate(&g.exec, g.graph, 0));
       long long kernels = 0;
       NNC_TRY(graph_kernels(g.graph, &kernels));
-      for (int t = 1; t < count; ++t) NNC_CUDA_TRY(cudaGraphLaunch(g.exec, g.cs));
-      note_graph_launches(kernels * (count - 1));
+      while (t < count && !(guard && guard->slow)) {
+        NNC_CUDA_TRY(cudaGraphLaunch(g.exec, g.cs));
+        ++t;
+        // looked at once the next sweep is queued
+        if (guard && t % tc::kPairLook == 1) NNC_TRY(guard->mark(g.cs, t));
+        if (guard && t % tc::kPairLook == 2) NNC_TRY(guard->look(s));
+      }
+      note_graph_launches(kernels * (t - 1));
     }
   }
+  *done = t;
   if (st2 == NNC_OK) st2 = last(g.cs);
   NNC_CUDA_TRY(cudaEventRecord(g.join, g.cs));
   NNC_CUDA_TRY(cudaStreamWaitEvent(s, g.join, 0));
@@ -887,19 +943,31 @@ int lifted_pg_fit(const T* X, int d, const int64_t* dims, const int* m, int r, b
     SideStream side, step_size;
     NNC_TRY(side.init());
     NNC_TRY(step_size.init());
-    NNC_TRY(replay_pipelined(
-        steps, s,
-        [&](cudaStream_t cs) -> int {
-          return pg_step(w, F, B, last, trace, counter, cs, side, step_size.s, false);
-        },
-        [&](cudaStream_t cs) -> int {
-          return pg_step(w, F, B, last, trace, counter, cs, side, step_size.s, true);
-        },
-        [&](cudaStream_t cs) -> int {
-          return pg_tail(w, F, B, last, trace, counter, side, cs, step_size.s);
-        }));
+    int done = 0;
+    auto run = [&](int count, tc::PairGuard* guard) -> int {
+      NNC_TRY(replay_pipelined(
+          count, s,
+          [&](cudaStream_t cs) -> int {
+            return pg_step(w, F, B, last, trace, counter, cs, side, step_size.s, false);
+          },
+          [&](cudaStream_t cs) -> int {
+            return pg_step(w, F, B, last, trace, counter, cs, side, step_size.s, true);
+          },
+          [&](cudaStream_t cs) -> int {
+            return pg_tail(w, F, B, last, trace, counter, side, cs, step_size.s);
+          },
+          guard, &done));
+      return check_tc(w, s);
+    };
+    tc::PairGuard guard, *use = nullptr;
+    bool left = false;
+    NNC_TRY(settle_pairs(w, &left, sc, s, &guard, &use));
+    NNC_TRY(run(steps, use));
+    if (done < steps) {
+      NNC_TRY(leave_pairs(w, sc, s));
+      NNC_TRY(run(steps - done, nullptr));
+    }
   }
-  NNC_TRY(check_tc(w, s));
   NNC_TRY(check_trace_finite(counter, s, "candelinc_pg_fit"));
   if (loss) {
     if (steps == 0) {
@@ -952,21 +1020,39 @@ int nncp_tensor_fit(const T* X, int d, const int64_t* dims, int r, bool tensor_c
       NNC_TRY(residual_run<T>(X, d, dims, 1, m, r, fac, nullptr, rw, nullptr, trace + t, cs));
     return NNC_OK;
   };
-  NNC_TRY(replay(iters, s, [&](cudaStream_t cs) -> int {
-    NNC_TRY(pass_last(w, A[d - 1], cs));
-    for (int n = 0; n < d; ++n) {
-      if (n == d - 1) NNC_TRY(pass_first(w, A[0], cs));
-      const T* Z = nullptr;
-      NNC_TRY(z_chain(w, n, A, &Z, cs));
-      NNC_TRY(mttkrp_and_v(w, n, Z, B, cs));
-      // Den = A^(n) V_n into gA; MU in place.
-      NNC_CUDA_TRY(small_gemm<T>((int)w.N[n], r, r, A[n], r, 1, w.V, r, 1, nullptr, w.gA, cs));
-      NNC_CUDA_TRY(launch_elementwise_mu<T>(A[n], w.MT, w.gA, w.N[n] * r, eps, cs));
-      NNC_TRY(refresh_a(w, n, A[n], B[n], cs));
-      if (n == 0 && d > 2) NNC_TRY(make_u0(w, A[0], cs));
+  int base = 0, done = 0;  // sweeps done before the present replay, and in it
+  auto run = [&](int count, tc::PairGuard* guard) -> int {
+    NNC_TRY(replay(
+        count, s,
+        [&](cudaStream_t cs) -> int {
+          NNC_TRY(pass_last(w, A[d - 1], cs));
+          for (int n = 0; n < d; ++n) {
+            if (n == d - 1) NNC_TRY(pass_first(w, A[0], cs));
+            const T* Z = nullptr;
+            NNC_TRY(z_chain(w, n, A, &Z, cs));
+            NNC_TRY(mttkrp_and_v(w, n, Z, B, cs));
+            // Den = A^(n) V_n into gA; MU in place.
+            NNC_CUDA_TRY(small_gemm<T>((int)w.N[n], r, r, A[n], r, 1, w.V, r, 1, nullptr, w.gA, cs));
+            NNC_CUDA_TRY(launch_elementwise_mu<T>(A[n], w.MT, w.gA, w.N[n] * r, eps, cs));
+            NNC_TRY(refresh_a(w, n, A[n], B[n], cs));
+            if (n == 0 && d > 2) NNC_TRY(make_u0(w, A[0], cs));
+          }
+          return loss_into(w, d - 1, last, trace, counter, cs, /*rel=*/1);
+        },
+        [&](int t, cudaStream_t cs) -> int { return after(base + t, cs); }, guard, &done));
+    return check_tc(w, s);
+  };
+  if (iters > 0) {
+    tc::PairGuard guard, *use = nullptr;
+    bool left = false;
+    NNC_TRY(settle_pairs(w, &left, sc, s, &guard, &use));
+    NNC_TRY(run(iters, use));
+    if (done < iters) {
+      NNC_TRY(leave_pairs(w, sc, s));
+      base = done;
+      NNC_TRY(run(iters - base, nullptr));
     }
-    return loss_into(w, d - 1, last, trace, counter, cs, /*rel=*/1);
-  }, after));
+  }
   NNC_TRY(check_tc(w, s));
   NNC_TRY(check_trace_finite(counter, s, "nncp_tensor_fit"));
   if (rel_err) {
@@ -1186,10 +1272,24 @@ int ntd_fit_nway(const T* X, int d, const int64_t* dims, const int* m, bool tens
     zlast = Z;
     return NNC_OK;
   };
-  NNC_TRY(replay_pipelined(
-      iters, s, [&](cudaStream_t cs) -> int { return sweep(cs, false); },
-      [&](cudaStream_t cs) -> int { return sweep(cs, true); },
-      [&](cudaStream_t cs) -> int { return core_update(cs, w.split, false); }));
+  int done = 0;
+  auto run = [&](int count, tc::PairGuard* guard) -> int {
+    NNC_TRY(replay_pipelined(
+        count, s, [&](cudaStream_t cs) -> int { return sweep(cs, false); },
+        [&](cudaStream_t cs) -> int { return sweep(cs, true); },
+        [&](cudaStream_t cs) -> int { return core_update(cs, w.split, false); }, guard, &done));
+    return check_tc(w, s);
+  };
+  if (iters > 0) {
+    tc::PairGuard guard, *use = nullptr;
+    bool left = false;
+    NNC_TRY(settle_pairs(w, &left, sc, s, &guard, &use));
+    NNC_TRY(run(iters, use));
+    if (done < iters) {
+      NNC_TRY(leave_pairs(w, sc, s));
+      NNC_TRY(run(iters - done, nullptr));
+    }
+  }
   NNC_TRY(check_tc(w, s));
   NNC_TRY(check_trace_finite(counter, s, "ntd_fit"));
   if (rel_err) {

@@ -400,11 +400,11 @@ struct Checkpoints {
 // sweep's; in the first replay there is none, and the core kernels see the
 // pending flag at 0 and return at once. `first` is the fit's index of the
 // first of these sweeps; *done gets the number of sweeps run, fewer than
-// `count` when the refinement trigger of `ck` stopped them.
+// `count` when the refinement trigger of `ck` or a look of `guard` (NULL: none) stopped them.
 template <typename T>
 int run_sweeps(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double* trace,
                int count, int first, Checkpoints<T>* ck, const tc::TcPlan* tcp, cudaStream_t s,
-               int* done) {
+               int* done, tc::PairGuard* guard = nullptr) {
   *done = 0;
   if (count <= 0) return NNC_OK;
   GraphRun g;
@@ -435,7 +435,20 @@ int run_sweeps(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double
   // host captures the graph of the others (capturing and instantiating it takes the time
   // of several sweeps of a mid-size tensor).
   const int direct = samples > 0 ? 0 : std::min(count, kSweepsPerGraph);
+  int look = direct > 0 ? direct : kSweepsPerGraph;
+  bool marked = false;
   while (t < count) {
+    if (guard && t >= look) {
+      if (!marked) {
+        NNC_TRY(guard->mark(g.cs, t));
+        look = t + 1;  // looked at once the next sweeps are queued
+      } else {
+        NNC_TRY(guard->look(s));
+        if (guard->slow) break;
+        look = t + tc::kPairLook;
+      }
+      marked = !marked;
+    }
     const bool sampled = samples > 0 && t % kProfileEvery == kProfileEvery - 1;
     // A five-sweep replay must not pass a sampled sweep or a checkpoint (its
     // last sweep may be one).
@@ -636,19 +649,21 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
     ck.m = m;
     ck.rw = &rw;
   }
-  if constexpr (std::is_same<T, float>::value) {
-    // The tensor-core passes form the shares of Y1 when the shape allows it
-    // (y1_fusable), the FP32-accurate passes also those of Y3 (y3_fusable).
-    const tc::TcPlan* any = exact ? exact : fast;
-    if (any && any->y1_fusable(m2)) {
+  // The tensor-core passes form the shares of Y1 when the shape allows it
+  // (y1_fusable), the TF32x3 passes also those of Y3 (y3_fusable).
+  auto shares = [&](const tc::TcPlan* p) -> int {
+    if (p && !b.Y1p && p->y1_fusable(m2)) {
       b.y_nh = (int)(N2 / 128);
       NNC_TRY(sc.get(&b.Y1p, (size_t)(N1 * b.y_nh) * m2 * m3));
     }
-    if ((exact && exact->y3_fusable(m2)) || (fast && fast->y3_fusable(m2))) {
+    if (p && !b.Y3p && p->y3_fusable(m2)) {
       b.y_nh = (int)(N2 / 128);
       NNC_TRY(sc.get(&b.Y3p, (size_t)(N3 * b.y_nh) * m1 * m2));
     }
-  }
+    return NNC_OK;
+  };
+  NNC_TRY(shares(exact));
+  NNC_TRY(shares(fast));
 
   // Prologue: S_k = F_k^T F_k, H1 = unfold_1(G x_2 S2 x_3 S3) unfold_1(G)^T,
   // the BF16 operand of F^(3), the trace counter.
@@ -678,10 +693,34 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
     // The FP32-accurate sweeps start from the factors the fast sweeps left.
     if (exact && fast && o->iters - n_fast > 0) NNC_TRY(exact->convert_b3(F[2], s));
   }
-  int n_rest = 0;
-  NNC_TRY(run_sweeps<T>(X, F, G, b, o->eps, trace, o->iters - n_fast, n_fast, &ck, exact, s,
-                        &n_rest));
-  if (exact) NNC_TRY(exact->check(s));
+  // Sweeps from `at` on; with TF32x3 passes where the FP16 pairs do not hold X, and once
+  // wide factors make the pairs' passes slow.
+  int at = n_fast;
+  if (at < o->iters) {
+    if constexpr (std::is_same<T, float>::value) {
+      auto leave_pairs = [&]() -> int {
+        NNC_TRY(plan32.to_tf32(X, sc, s));
+        NNC_TRY(shares(exact));
+        return exact->convert_b3(F[2], s);
+      };
+      bool wide = false;
+      if (exact) NNC_TRY(exact->wide(s, &wide));
+      if (wide) NNC_TRY(leave_pairs());
+      if (exact && exact->kind == tc::kKindF16x3) {
+        tc::PairGuard guard;
+        NNC_TRY(guard.start(exact, sc));
+        int n = 0;
+        NNC_TRY(run_sweeps<T>(X, F, G, b, o->eps, trace, o->iters - at, at, &ck, exact, s, &n,
+                              &guard));
+        NNC_TRY(exact->check(s));
+        at += n;
+        if (at < o->iters) NNC_TRY(leave_pairs());
+      }
+    }
+    int n = 0;
+    NNC_TRY(run_sweeps<T>(X, F, G, b, o->eps, trace, o->iters - at, at, &ck, exact, s, &n));
+    if (exact) NNC_TRY(exact->check(s));
+  }
   NNC_TRY(check_trace_finite(b.counter, s, "ntd_fit"));
 
   if (rel_err) {

@@ -49,6 +49,7 @@
 
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 
 #include "kernels.cuh"
 #include "mma32.cuh"
@@ -307,10 +308,12 @@ __device__ __forceinline__ void stage_factor_row(const TcEpilogue& ep, int64_t j
 // on the tensor cores (mma32.cuh: SPLIT = 1, TF32 operands beside the BF16
 // rounding of X; 3, split TF32 in the FP32-accurate passes). The warp of quarter
 // q takes rows 32 q .. 32 q + 31 with the whole 32 x 32 share (zero past m2,
-// m3) in registers; the four partial shares are added in quarter order.
+// m3) in registers; the four partial shares are added in quarter order (`add`: onto what a
+// round before wrote).
 template <int SPLIT>
 __device__ __forceinline__ void fused_share(const TcEpilogue& ep, int64_t tile, int lane,
-                                            int quarter, float* Ps, const float* Fs) {
+                                            int quarter, float* Ps, const float* Fs,
+                                            bool add = false) {
   const int et = threadIdx.x - 64;  // 0 .. 127
   const int o0 = mma32::frag_off(lane, 0), o1 = mma32::frag_off(lane, 1);
   float acc[2][4][4];
@@ -328,7 +331,8 @@ __device__ __forceinline__ void fused_share(const TcEpilogue& ep, int64_t tile, 
   for (int e = et; e < n; e += 128) {
     const int bb = e / m3, cc = e % m3, o = mma32::tile_index(bb, cc);
     const float y = ((red[o] + red[o + 1024]) + red[o + 2048]) + red[o + 3072];
-    yo[ep.y_tr ? cc * m2 + bb : e] = y;
+    float* z = yo + (ep.y_tr ? cc * m2 + bb : e);
+    *z = add ? *z + y : y;
   }
   epi_sync();  // red and Fs are free for the next tile
 }
@@ -685,13 +689,19 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // ---- FP16 pair passes (kKindF16x3) ----------------------------------------------
 //
 // FP32-accurate passes on pairs of FP16 parts. X is kept as Xh + Xl, with
-//   x / (s_i t_j u_k) = x_hi + x_lo,   x_hi = fp16(.), x_lo = fp16(. - x_hi),
+//   v = x / (s_i t_j u_k) = x_hi + 2^-11 x_lo,   x_hi = fp16(v), x_lo = fp16(2^11 (v - x_hi)),
 // s, t, u powers of two that bring the largest entry of every slice of every mode
-// close below 2^15: where an entry is within 2^16 of the largest of its slices,
-// the pair holds 22 bits and a sign (as the TF32 pair does), below that the
-// error stays 2^-40 of the largest. B is split the same way with u or s folded in
-// and a power of two per column. x_hi [f_hi; f_lo] and x_lo f_hi are accumulated
-// as in the TF32x3 pass.
+// close below 2^15. B is split the same way with u or s folded in and a power of two per
+// column. x_hi [f_hi; f_lo] and x_lo f_hi are accumulated as in the TF32x3 pass, the last
+// two in accumulators of their own that count 2^-11.
+// Range: a pair holds 22 bits and a sign, as the TF32 pair does, from 2^-13 up (x_lo's
+// factor takes it out of the subnormals: without it only from 2^-1), 28 powers of two
+// below the largest entry; zeros are exact. The TF32 pair holds them at every magnitude. An X
+// with a nonzero entry below that range is flagged by x_to_pair_kernel, and the fit starts again
+// with TF32x3 passes. Factor entries below it (updates drive entries to zero; a block of X
+// may have no other terms) are the operand of another round over the tiles, scaled up
+// by 2^28, whose results are added: every entry keeps its 22 bits at the price of a pass per 28
+// powers of two, and a fit whose passes take many rounds goes on with TF32x3 (PairGuard).
 // Why pairs made once per fit instead of TF32 parts made in every pass: the
 // TF32x3 stage moves each entry through shared memory five times (TMA in, read and
 // two writes of the split, two reads by the MMAs, 8 bytes an entry in the last
@@ -757,23 +767,31 @@ __device__ __forceinline__ int f16_exponent(unsigned bits) {
 }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
+// v = hi + lo / kF16LoScale; 22 bits for |v| in [kF16Least, 2^15).
+constexpr float kF16LoScale = 2048.f;
+constexpr float kF16Least = 1.f / 8192.f;
 __device__ __forceinline__ void split_f16(float v, __half& hi, __half& lo) {
   hi = __float2half_rn(v);
-  lo = __float2half_rn(v - __half2float(hi));
+  lo = __float2half_rn((v - __half2float(hi)) * kF16LoScale);
 }
 
 // The pass's B operand in shared memory (256 threads: warps 2-9): for each 64-entry
 // K chunk 2 NP rows of 128 bytes, rows [0, NP) f_hi and [NP, 2 NP) f_lo of
-// F[k, q] kscale[k] / cscale[q], in the 128-byte swizzle. cs[q] gets cscale.
+// F[k, q] kscale[k] / cscale[q], in the 128-byte swizzle. cs[q] gets cscale. *more gets 1 when
+// a nonzero entry below the range is left for another round (zero here). A column whose largest
+// entry is so small that products with kscale may be subnormal is left whole.
+constexpr int kF16RoundBits = 28, kF16MaxRounds = 14;  // every product of two floats
+constexpr int kF16LeaveExp = -112;
+__device__ __forceinline__ unsigned char* f16_b_row(unsigned char* bs, int np, int o, int n) {
+  return bs + (o >> 3) * (2 * np * 128) + n * 128 + (((o & 7) ^ (n & 7)) << 4);
+}
 template <int NP>
 __device__ __forceinline__ void f16_operand(const F16Operand& fo, int nk, unsigned char* bs,
-                                            float* cs, unsigned* cmax) {
+                                            float* cs, unsigned* cmax, int* more) {
   const int t = threadIdx.x - 64, lane = t & 31, w = t >> 5;
   constexpr int NC = NP / 32;  // columns per lane
   const int noct = nk * 8;     // octets of K entries
-  auto value = [&](int k, int n) {
-    return k < fo.K && n < fo.q ? fo.F[(int64_t)k * fo.q + n] * fo.kscale[k] : 0.f;
-  };
+  auto in = [&](int k, int n) { return k < fo.K && n < fo.q; };
   for (int n = t; n < NP; n += 256) cmax[n] = 0u;
   asm volatile("bar.sync 2, 256;" ::: "memory");
   float mx[NC];
@@ -784,7 +802,10 @@ __device__ __forceinline__ void f16_operand(const F16Operand& fo, int nk, unsign
     for (int c = 0; c < NC; ++c) {
       float v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = value(8 * o + u, lane + 32 * c);
+      for (int u = 0; u < 8; ++u) {
+        const int k = 8 * o + u, n = lane + 32 * c;
+        v[u] = in(k, n) ? fo.F[(int64_t)k * fo.q + n] * fo.kscale[k] : 0.f;
+      }
 #pragma unroll
       for (int u = 0; u < 8; ++u) mx[c] = fmaxf(mx[c], fabsf(v[u]));
     }
@@ -796,24 +817,93 @@ __device__ __forceinline__ void f16_operand(const F16Operand& fo, int nk, unsign
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
     const int e = f16_exponent(cmax[lane + 32 * c]);
-    inv[c] = pow2f(-e);
-    if (w == 0) cs[lane + 32 * c] = pow2f(e);
+    const bool leave = e < kF16LeaveExp;
+    inv[c] = leave ? 0.f : pow2f(-e);
+    if (w == 0) cs[lane + 32 * c] = pow2f(leave ? e + kF16RoundBits : e);
   }
+  bool low = false;
   for (int o = w; o < noct; o += 8) {
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       const int n = lane + 32 * c;
-      float v[8];
+      float f[8], ks[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = value(8 * o + u, n);
+      for (int u = 0; u < 8; ++u) {  // sixteen loads in flight
+        const int k = 8 * o + u;
+        f[u] = in(k, n) ? fo.F[(int64_t)k * fo.q + n] : 0.f;
+        ks[u] = in(k, n) ? fo.kscale[k] : 0.f;
+      }
       union { __half h[8]; uint4 q; } hi, lo;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) split_f16(v[u] * inv[c], hi.h[u], lo.h[u]);
-      unsigned char* row = bs + (o >> 3) * (2 * NP * 128) + n * 128 + (((o & 7) ^ (n & 7)) << 4);
+      for (int u = 0; u < 8; ++u) {
+        const float y = f[u] * ks[u] * inv[c];
+        const bool under = fabsf(y) < kF16Least;
+        low |= under && f[u] != 0.f;
+        split_f16(under ? 0.f : y, hi.h[u], lo.h[u]);
+      }
+      unsigned char* row = f16_b_row(bs, NP, o, n);
       *reinterpret_cast<uint4*>(row) = hi.q;
       *reinterpret_cast<uint4*>(row + NP * 128) = lo.q;
     }
   }
+  if (low) *more = 1;
+}
+
+// The operand of round w > 0: the entries of the w-th range of 28 powers of two below the
+// column's largest (of the one before for a column that was left), scaled into the first, zero
+// for the others; *more as above.
+__device__ __noinline__ void f16_operand_round(const F16Operand& fo, int np, int nk,
+                                               unsigned char* bs, const unsigned* cmax, int round,
+                                               int* more) {
+  const int t = threadIdx.x - 64, lane = t & 31;
+  bool low = false;
+  for (int o = t >> 5; o < nk * 8; o += 8)
+    for (int n = lane; n < np; n += 32) {
+      const int e = f16_exponent(cmax[n]);
+      const int up = kF16RoundBits * (e < kF16LeaveExp ? round - 1 : round) - e;
+      float f[8], ks[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = 8 * o + u;
+        f[u] = k < fo.K && n < fo.q ? fo.F[(int64_t)k * fo.q + n] : 0.f;
+        ks[u] = k < fo.K ? fo.kscale[k] : 1.f;
+      }
+      union { __half h[8]; uint4 q; } hi, lo;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        // f 2^x in steps that stay within the result's magnitude and f's: exact where the
+        // result is in the range, infinite or below it otherwise.
+        int x = (__float_as_int(ks[u]) >> 23) - 127 + up;
+        float y = f[u];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          const int step = max(-126, min(127, x));
+          y *= pow2f(step);
+          x -= step;
+        }
+        const float m = fabsf(y);
+        low |= f[u] != 0.f && m < kF16Least;
+        split_f16(m >= kF16Least && m < 32768.f ? y : 0.f, hi.h[u], lo.h[u]);
+      }
+      unsigned char* row = f16_b_row(bs, np, o, n);
+      *reinterpret_cast<uint4*>(row) = hi.q;
+      *reinterpret_cast<uint4*>(row + np * 128) = lo.q;
+    }
+  if (low && round + 1 < kF16MaxRounds) *more = 1;
+}
+
+// AND of `ok` over warps 2-9 (named barrier 2).
+__device__ __forceinline__ bool all_of_256(bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred q, p;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "bar.red.and.pred p, 2, 256, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r)
+      : "r"(ok ? 1u : 0u)
+      : "memory");
+  return r != 0;
 }
 
 template <bool kMN, int NP, bool FUSE>
@@ -829,6 +919,7 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
   __shared__ uint64_t full[kF16MaxStages], empty[kF16MaxStages], accfull[2], accempty[2], bready;
   __shared__ float cs[NP];
   __shared__ unsigned cmax[NP];
+  __shared__ int more[kF16MaxRounds];  // of each round of f16_operand; the last stays 0
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
 
@@ -850,6 +941,7 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       mbar_init(&accempty[b], 4);
     }
     mbar_init(&bready, 8);
+    for (int w = 0; w < kF16MaxRounds; ++w) more[w] = 0;
     fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -880,29 +972,41 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       int64_t it = 0;
       int s = 0;
       uint32_t ph = 1;  // the first round's stages are free
-      bool ok = true;
-      for (int64_t q = 0; ok && q < my_tiles; ++q) {
-        const int m0 = static_cast<int>((blockIdx.x + q * gridDim.x) * 128);
-        for (int kc = 0; kc < nk; ++kc, ++it) {
-          if (it >= nst && !mbar_wait(&empty[s], ph, vfail)) {
-            ok = false;
-            break;
-          }
-          unsigned char* st = base + s * kF16Stage;
-          mbar_expect_tx(&full[s], kF16Stage);
-          if (!kMN) {
-            load(&tmHi, st, kc * 64, m0, &full[s]);
-            load(&tmLo, st + kTileBytes, kc * 64, m0, &full[s]);
-          } else {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              load(&tmHi, st + h * (kTileBytes / 2), m0 + h * 64, kc * 64, &full[s]);
-              load(&tmLo, st + kTileBytes + h * (kTileBytes / 2), m0 + h * 64, kc * 64, &full[s]);
+      bool ok = true, again = true;
+      for (int round = 0; ok && again; ++round) {
+        // Whether another round follows is known when this round's operand is; asked before
+        // the round's last load, so that the next operand's phase cannot end meanwhile.
+        int64_t ask = my_tiles * nk - 1;
+        ask = ask < nst ? ask : nst;
+        int64_t c = 0;
+        for (int64_t q = 0; ok && q < my_tiles; ++q) {
+          const int m0 = static_cast<int>((blockIdx.x + q * gridDim.x) * 128);
+          for (int kc = 0; kc < nk; ++kc, ++it, ++c) {
+            if (c == ask) {
+              ok = mbar_wait(&bready, round & 1, vfail);
+              again = ok && more[round] != 0;
             }
-          }
-          if (++s == nst) {
-            s = 0;
-            ph ^= 1u;
+            if (!ok || (it >= nst && !mbar_wait(&empty[s], ph, vfail))) {
+              ok = false;
+              break;
+            }
+            unsigned char* st = base + s * kF16Stage;
+            mbar_expect_tx(&full[s], kF16Stage);
+            if (!kMN) {
+              load(&tmHi, st, kc * 64, m0, &full[s]);
+              load(&tmLo, st + kTileBytes, kc * 64, m0, &full[s]);
+            } else {
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                load(&tmHi, st + h * (kTileBytes / 2), m0 + h * 64, kc * 64, &full[s]);
+                load(&tmLo, st + kTileBytes + h * (kTileBytes / 2), m0 + h * 64, kc * 64,
+                     &full[s]);
+              }
+            }
+            if (++s == nst) {
+              s = 0;
+              ph ^= 1u;
+            }
           }
         }
       }
@@ -922,64 +1026,65 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       const uint32_t idesc = f16_instr_desc(kMN, NP);
       const uint32_t idesc2 = f16_instr_desc(kMN, 2 * NP);
       const uint64_t bdesc_base = smem_desc(smem_u32(bs), 16, 1024);
-      bool ok = mbar_wait(&bready, 0, vfail);
       int gcount = 0, rs = 0;  // groups of stages; the ring's stage
       const int group = f16_group(nk);
       uint32_t rph = 0;
-      for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-        for (int k0 = 0; ok && k0 < nk; k0 += group, ++gcount) {
-          const int buf = gcount & 1, kend = min(nk, k0 + group);
-          if (gcount >= 2 && !mbar_wait(&accempty[buf], ((gcount >> 1) - 1) & 1, vfail)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t acc0 = tmem + buf * kAcc * kAccCols;
-          for (int kc = k0; kc < kend; ++kc) {
-            if (!mbar_wait(&full[rs], rph, vfail)) {
+      bool ok = true, again = true;
+      for (int round = 0; ok && again; ++round) {
+        ok = mbar_wait(&bready, round & 1, vfail);
+        again = ok && more[round] != 0;
+        for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+          for (int k0 = 0; ok && k0 < nk; k0 += group, ++gcount) {
+            const int buf = gcount & 1, kend = min(nk, k0 + group);
+            if (gcount >= 2 && !mbar_wait(&accempty[buf], ((gcount >> 1) - 1) & 1, vfail)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            const uint32_t st = smem_u32(base + rs * kF16Stage);
-            const uint64_t hidesc = smem_desc(st, kMN ? kTileBytes / 2 : 16, 1024);
-            const uint64_t lodesc = smem_desc(st + kTileBytes, kMN ? kTileBytes / 2 : 16, 1024);
-            const uint64_t bdesc0 = bdesc_base + (uint64_t)((kc * 2 * NP * 128) >> 4);
+            const uint32_t acc0 = tmem + buf * kAcc * kAccCols;
+            for (int kc = k0; kc < kend; ++kc) {
+              if (!mbar_wait(&full[rs], rph, vfail)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              const uint32_t st = smem_u32(base + rs * kF16Stage);
+              const uint64_t hidesc = smem_desc(st, kMN ? kTileBytes / 2 : 16, 1024);
+              const uint64_t lodesc = smem_desc(st + kTileBytes, kMN ? kTileBytes / 2 : 16, 1024);
+              const uint64_t bdesc0 = bdesc_base + (uint64_t)((kc * 2 * NP * 128) >> 4);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              constexpr uint32_t astep = kMN ? 2048 : 32;
-              const uint64_t astep16 = (uint64_t)((kk * astep) >> 4);
-              const uint64_t bdesc = bdesc0 + (uint64_t)((kk * 32) >> 4);
-              const uint32_t acc = acc0 + (kk & (kAcc - 1)) * kAccCols;
-              const uint32_t accum = (kc > k0 || kk >= kAcc) ? 1u : 0u;
-              mma<kKindBf16>(acc, hidesc + astep16, bdesc, idesc2, accum);
-              mma<kKindBf16>(acc + NP, lodesc + astep16, bdesc, idesc, 1u);
+              for (int kk = 0; kk < 4; ++kk) {
+                constexpr uint32_t astep = kMN ? 2048 : 32;
+                const uint64_t astep16 = (uint64_t)((kk * astep) >> 4);
+                const uint64_t bdesc = bdesc0 + (uint64_t)((kk * 32) >> 4);
+                const uint32_t acc = acc0 + (kk & (kAcc - 1)) * kAccCols;
+                const uint32_t accum = (kc > k0 || kk >= kAcc) ? 1u : 0u;
+                mma<kKindBf16>(acc, hidesc + astep16, bdesc, idesc2, accum);
+                mma<kKindBf16>(acc + NP, lodesc + astep16, bdesc, idesc, 1u);
+              }
+              mma_commit(&empty[rs]);
+              if (++rs == nst) {
+                rs = 0;
+                rph ^= 1u;
+              }
             }
-            mma_commit(&empty[rs]);
-            if (++rs == nst) {
-              rs = 0;
-              rph ^= 1u;
-            }
+            if (ok) mma_commit(&accfull[buf]);
           }
-          if (ok) mma_commit(&accfull[buf]);
         }
       }
     }
   } else {
     // ---- the B operand (warps 2-9) -------------------------------------------------
     pdl_wait();
-    f16_operand<NP>(fo, nk, bs, cs, cmax);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&bready);
-    asm volatile("bar.sync 2, 256;" ::: "memory");  // cs complete
-    if (warp < 6) {
-      // ---- epilogue (warps 2-5) ------------------------------------------------------
+    int gcount = 0;
+    // ---- epilogue of a round (warps 2-5); false: a wait gave up ------------------------
+    auto epilogue = [&](auto first, int round) -> bool {
+      constexpr bool kFirst = decltype(first)::value;
+      bool got = true;
       const int quarter = warp & 3;
       const int lr = quarter * 32 + lane;
       float* Ps = reinterpret_cast<float*>(epi);  // FUSE: 128 x 32 pass rows
       float* Fs = Ps + 128 * 32;                  // FUSE: 128 x 32 factor rows
-      int gcount = 0;
       int64_t fs_slice = -1;
       const int group = f16_group(nk);
       for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -1000,7 +1105,6 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
         float sum[NP];
 #pragma unroll
         for (int t = 0; t < NP; ++t) sum[t] = 0.f;
-        bool got = true;
         for (int k0 = 0; k0 < nk; k0 += group, ++gcount) {
           const int buf = gcount & 1;
           got = mbar_wait(&accfull[buf], (gcount >> 1) & 1, vfail);
@@ -1019,7 +1123,8 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
               tmem_ld32(accb + q * kAccCols + NP + c0, w);
 #pragma unroll
               for (int t = 0; t < 32; ++t)
-                sum[c0 + t] += __uint_as_float(h[t]) + __uint_as_float(w[t]);
+                sum[c0 + t] += fmaf(__uint_as_float(w[t]), 1.f / kF16LoScale,
+                                    __uint_as_float(h[t]));
             }
           }
           tc_fence_before();
@@ -1032,13 +1137,22 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
           float* v = sum + c0;
           // Powers of two: the column's first (its result is the entry without the
           // row's scale), then the row's.
+          if constexpr (kFirst) {
 #pragma unroll
-          for (int t = 0; t < 32; ++t)
-            v[t] = v[t] * cs[c0 + t] * rsc;
+            for (int t = 0; t < 32; ++t) v[t] = v[t] * cs[c0 + t] * rsc;
+          } else {
+            const double down = ldexp((double)rsc, -kF16RoundBits * round);
+#pragma unroll
+            for (int t = 0; t < 32; ++t) v[t] = (float)((double)v[t] * cs[c0 + t] * down);
+          }
           if (ep.p1_layout != 1) {
             if (orow >= 0) {
               float* o = ep.out + orow * ep.q;
-              if ((ep.q & 3) == 0) {
+              if constexpr (!kFirst) {
+#pragma unroll
+                for (int t = 0; t < 32; ++t)
+                  if (c0 + t < ep.q) o[c0 + t] += v[t];
+              } else if ((ep.q & 3) == 0) {
 #pragma unroll
                 for (int t = 0; t < 32; t += 4)
                   if (c0 + t < ep.q)
@@ -1064,12 +1178,39 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
             float* o = ep.out + ra * ep.n3 + rb;
 #pragma unroll
             for (int t = 0; t < 32; ++t)
-              if (c0 + t < ep.q) o[static_cast<int64_t>(c0 + t) * ep.slab] = v[t];
+              if (c0 + t < ep.q) {
+                float* z = o + static_cast<int64_t>(c0 + t) * ep.slab;
+                *z = kFirst ? v[t] : *z + v[t];
+              }
           }
         }
-        if constexpr (FUSE) fused_share<3>(ep, tile, lane, quarter, Ps, Fs);
+        if constexpr (FUSE) fused_share<3>(ep, tile, lane, quarter, Ps, Fs, !kFirst);
       }
+      return got;
+    };
+    // Whether another round follows (in all of warps 2-9 alike). Every MMA of the round is
+    // done: warps 2-5 have read its last accumulators.
+    auto round_done = [&](bool got, int round) -> bool {
+      return all_of_256(got && *vfail == 0) && more[round] != 0;
+    };
+    auto operand_done = [&]() {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bready);
+      asm volatile("bar.sync 2, 256;" ::: "memory");  // cs and more[round] complete
+    };
+    f16_operand<NP>(fo, nk, bs, cs, cmax, more);
+    operand_done();
+    bool got = true;
+    if (warp < 6) got = epilogue(std::true_type{}, 0);
+    int round = 0;
+    while (round_done(got, round)) {
+      ++round;
+      f16_operand_round(fo, NP, nk, bs, cmax, round, more + round);
+      operand_done();
+      if (warp < 6) got = epilogue(std::false_type{}, round);
     }
+    if (threadIdx.x == 64 && blockIdx.x == 0 && round > 0) atomicAdd(err + kFlagRounds, round);
   }
 
   tc_fence_before();
@@ -1206,12 +1347,15 @@ __global__ void slice_u_kernel(const unsigned* __restrict__ umax, int N3, int n3
 }
 
 // Xh, Xl (rows of n3p entries, zero past N3) from X: eight entries a thread, tx threads
-// (a power of two) a row, one division per row.
+// (a power of two) a row, one division per row. *wide gets 1 when the pair of a nonzero entry
+// holds less than 22 bits.
 __global__ void __launch_bounds__(256)
 x_to_pair_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int n3p, int tx,
                  const float* __restrict__ s, const float* __restrict__ t,
-                 const float* __restrict__ u, __half* __restrict__ Xh, __half* __restrict__ Xl) {
+                 const float* __restrict__ u, __half* __restrict__ Xh, __half* __restrict__ Xl,
+                 int* __restrict__ wide) {
   const int oct = n3p >> 3, ty = 256 / tx;
+  bool low = false;
   for (int64_t r = (int64_t)blockIdx.x * ty + threadIdx.x / tx; r < R;
        r += (int64_t)gridDim.x * ty) {
     const unsigned i = (unsigned)r / (unsigned)N2;  // R <= 2^31
@@ -1229,11 +1373,16 @@ x_to_pair_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int n3p
       v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
       union { __half h[8]; uint4 q; } hi, lo;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) split_f16(v[q] * inv * (1.f / u[k + q]), hi.h[q], lo.h[q]);
+      for (int q = 0; q < 8; ++q) {
+        const float y = v[q] * inv * (1.f / u[k + q]);
+        low |= v[q] != 0.f && fabsf(y) < kF16Least;
+        split_f16(y, hi.h[q], lo.h[q]);
+      }
       *reinterpret_cast<uint4*>(Xh + r * n3p + k) = hi.q;
       *reinterpret_cast<uint4*>(Xl + r * n3p + k) = lo.q;
     }
   }
+  if (low) *wide = 1;
 }
 
 // ---- conversions -------------------------------------------------------------
@@ -1607,14 +1756,17 @@ int TcPlan::init_f16(const float* X, Scratch& sc, cudaStream_t s) {
     return NNC_ERR_UNSUPPORTED;
   }
   unsigned* umax = nullptr;
-  NNC_TRY(sc.get(&err, 1));
+  NNC_TRY(sc.get(&err, kFlags));
   NNC_TRY(sc.get(&scale, static_cast<size_t>(N1)));
   NNC_TRY(sc.get(&sc_t, static_cast<size_t>(N2)));
   NNC_TRY(sc.get(&sc_u, static_cast<size_t>(kp3)));
   NNC_TRY(sc.get(&umax, static_cast<size_t>(N3)));
-  NNC_TRY(sc.get(&Xh, static_cast<size_t>(rows * kp3)));
-  NNC_TRY(sc.get(&Xl, static_cast<size_t>(rows * kp3)));
+  // One block, so that Xt fits where the pair was when the plan becomes TF32x3.
+  const int64_t half = ceil_div(rows * kp3, 64) * 64;
+  NNC_TRY(sc.get(&Xh, static_cast<size_t>(2 * half)));
+  Xl = Xh + half;
   const int sms = device_sm_count();
+  NNC_CUDA_TRY(cudaMemsetAsync(err, 0, kFlags * sizeof(int), s));
   if (rmax == nullptr) NNC_TRY(row_maxima(X, sc, s));
   slice_s_kernel<<<(unsigned)N1, 256, 0, s>>>(rmax, N2, scale);
   note_launch(s);
@@ -1634,11 +1786,11 @@ int TcPlan::init_f16(const float* X, Scratch& sc, cudaStream_t s) {
   const int ox = row_threads(kp3 / 8);
   const int64_t xb = ceil_div(rows, 256 / ox);
   x_to_pair_kernel<<<(unsigned)(xb < 32LL * sms ? xb : 32LL * sms), 256, 0, s>>>(
-      X, rows, (int)N2, (int)N3, kp3, ox, scale, sc_t, sc_u, Xh, Xl);
+      X, rows, (int)N2, (int)N3, kp3, ox, scale, sc_t, sc_u, Xh, Xl, err + kFlagWideX);
   note_launch(s);
   NNC_CUDA_TRY(cudaGetLastError());
-  // After the conversion: a pass launched as a programmatic dependent reads the pair
-  // before it waits for its predecessor, so that must not be the conversion.
+  // A pass launched as a programmatic dependent reads the pair before it waits for its
+  // predecessor, so that must not be the conversion: the error flag once more.
   NNC_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
   // The pair stays in L2 (129 MB) from pass to pass with room for the pass results.
   x_resident = 4 * rows * kp3 <= 80LL << 20;
@@ -1656,6 +1808,13 @@ int TcPlan::init_fp32(const float* X, int64_t N1_, int64_t N2_, int64_t N3_, int
   const int st = init(kKindF16x3, X, N1_, N2_, N3_, m1_, m3_, sc, s, p1_kj_);
   if (st != NNC_ERR_UNSUPPORTED) return st;
   return init(kKindTf32x3, X, N1_, N2_, N3_, m1_, m3_, sc, s, p1_kj_);
+}
+
+int TcPlan::to_tf32(const float* X, Scratch& sc, cudaStream_t s) {
+  sc.drop(Xh);
+  Xh = Xl = nullptr;
+  reserve_sms = 0;
+  return init(kKindTf32x3, X, N1, N2, N3, m1, m3, sc, s, p1_kj);
 }
 
 int TcPlan::convert_b3(const float* F3, cudaStream_t s) const {
@@ -1812,15 +1971,54 @@ int wait_selftest(long long cycles, cudaStream_t s) {
   return NNC_OK;
 }
 
+namespace {
+int timed_out(int flag) {
+  if (flag == 0) return NNC_OK;
+  set_error_detail_text("tensor-core mode product: a pipeline wait timed out");
+  return NNC_ERR_TIMEOUT;
+}
+}  // namespace
+
+int TcPlan::wide(cudaStream_t s, bool* w) const {
+  int h = 0;
+  *w = false;
+  if (kind != kKindF16x3) return NNC_OK;
+  NNC_CUDA_TRY(cudaMemcpyAsync(&h, err + kFlagWideX, sizeof(int), cudaMemcpyDeviceToHost, s));
+  NNC_CUDA_TRY(cudaStreamSynchronize(s));
+  *w = h != 0;
+  return NNC_OK;
+}
+
+int PairGuard::start(const TcPlan* p, Scratch& sc) {
+  NNC_TRY(sc.get(&seen, kFlags));
+  NNC_CUDA_TRY(cudaEventCreateWithFlags(&at, cudaEventDisableTiming));
+  plan = p;
+  return NNC_OK;
+}
+
+int PairGuard::mark(cudaStream_t cs, int sweeps) {
+  NNC_CUDA_TRY(cudaMemcpyAsync(seen, plan->err, kFlags * sizeof(int), cudaMemcpyDeviceToDevice, cs));
+  NNC_CUDA_TRY(cudaEventRecord(at, cs));
+  marked = sweeps;
+  return NNC_OK;
+}
+
+int PairGuard::look(cudaStream_t s) {
+  int h[kFlags] = {};
+  NNC_CUDA_TRY(cudaStreamWaitEvent(s, at, 0));
+  NNC_CUDA_TRY(cudaMemcpyAsync(h, seen, sizeof(h), cudaMemcpyDeviceToHost, s));
+  NNC_CUDA_TRY(cudaStreamSynchronize(s));
+  slow = 4 * (h[kFlagRounds] - rounds) > 2 * (marked - looked);
+  rounds = h[kFlagRounds];
+  looked = marked;
+  return timed_out(h[0]);
+}
+
 int TcPlan::check(cudaStream_t s) const {
   int h = 0;
   NNC_CUDA_TRY(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
   NNC_CUDA_TRY(cudaStreamSynchronize(s));
-  if (h != 0) {
-    set_error_detail_text("tensor-core mode product: a pipeline wait timed out");
-    return NNC_ERR_TIMEOUT;
-  }
-  return NNC_OK;
+  return timed_out(h);
 }
 
 }  // namespace tc

@@ -14,6 +14,10 @@ constexpr int kKindBf16 = 0;
 constexpr int kKindTf32x3 = 1;
 constexpr int kKindF16x3 = 2;
 
+// The device words of a plan (TcPlan::err): a pipeline wait timed out; F16x3 only: an entry of X
+// lies outside the range of a pair; rounds that passes took beyond the first (tc_ttm.cu).
+constexpr int kFlagWideX = 1, kFlagRounds = 2, kFlags = 3;
+
 // Where and how the epilogue writes one pass's FP32 result.
 struct TcEpilogue {
   float* out;
@@ -78,7 +82,7 @@ struct TcPlan {
   unsigned* rmax = nullptr;
   int x_resident = 0;
   CUtensorMap mapL3, mapL1;  // F16x3: Xl as operand A of pass 1 and pass 2
-  int* err = nullptr;
+  int* err = nullptr;  // F16x3: kFlags entries, else one
   // SMs a pass of at least 8 tiles per SM (F16x3: of any number) leaves to
   // kernels that run beside it (the nnTD sweep's small kernels); 0: every SM.
   int reserve_sms = 0;
@@ -91,9 +95,15 @@ struct TcPlan {
   int init(int kind, const float* X, int64_t N1, int64_t N2, int64_t N3, int m1, int m3,
            Scratch& sc, cudaStream_t s, bool p1_kj = false, bool need_p1 = true);
   // FP32-accurate passes that a fit runs again and again: F16x3 where the shape
-  // allows it, else TF32x3.
+  // allows it, else TF32x3. Whether the values of X allow it the device knows after init
+  // (`wide`: an entry outside the range of a pair, whose results are then not FP32-accurate;
+  // synchronises s): the caller then turns the plan into the TF32x3 one.
   int init_fp32(const float* X, int64_t N1, int64_t N2, int64_t N3, int m1, int m3, Scratch& sc,
                 cudaStream_t s, bool p1_kj = false);
+  int wide(cudaStream_t s, bool* w) const;
+  // An F16x3 plan becomes the TF32x3 plan of the same tensor; no work that reads the pair
+  // is in flight but on `s`.
+  int to_tf32(const float* X, Scratch& sc, cudaStream_t s);
   int init_f16(const float* X, Scratch& sc, cudaStream_t s);  // parts of init
   int row_maxima(const float* X, Scratch& sc, cudaStream_t s);
   // B operands from the current factor (BF16: F^(1) scaled by s).
@@ -113,6 +123,33 @@ struct TcPlan {
   bool y3_fusable(int m2) const;
   // Synchronises s and turns a device-side pipeline time-out into NNC_ERR_TIMEOUT.
   int check(cudaStream_t s) const;
+};
+
+// Watches a fit whose passes read FP16 pairs: once more than every fourth pass since the last
+// look took another round for wide factors (at 512^3 a round takes 100-120 us, a TF32x3 pass 140), the
+// fit does better with TF32x3 passes. The host looks every kPairLook sweeps, and once the next
+// ones are queued, so that the device does not wait for it; what it sees is as of the mark, so
+// it depends on the data alone.
+constexpr int kPairLook = 20;
+struct PairGuard {
+  bool slow = false;  // at the last look
+  PairGuard() = default;
+  PairGuard(const PairGuard&) = delete;
+  PairGuard& operator=(const PairGuard&) = delete;
+  ~PairGuard() {
+    if (at) cudaEventDestroy(at);
+  }
+  int start(const TcPlan* p, Scratch& sc);
+  // The device's words after the work queued so far on `cs`, `sweeps` sweeps (mark), and what
+  // they say (look, in the order of `s`, which it synchronises; NNC_ERR_TIMEOUT as TcPlan::check).
+  int mark(cudaStream_t cs, int sweeps);
+  int look(cudaStream_t s);
+
+ private:
+  const TcPlan* plan = nullptr;
+  int marked = 0, looked = 0, rounds = 0;
+  int* seen = nullptr;
+  cudaEvent_t at = nullptr;
 };
 
 // Runs the pass kernel's bounded mbarrier wait once, with a limit of `cycles`,

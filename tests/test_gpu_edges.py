@@ -250,3 +250,123 @@ def test_core_fit_keeps_the_bits_of_the_general_form(dt, m, r):
     assert e == ew
     for a, b in zip(B, wide):
         assert torch.equal(a, b[:, :r]) and not b[:, r:].any()
+
+
+# Data and factors beyond the range of the FP16 pairs (28 powers of two below the largest entry
+# of a slice or column): every sum is of nonnegative terms, so FP32-accurate arithmetic keeps the
+# relative error of every entry: 1e-4 a sweep, as in the other one-sweep tests.
+def _f32(a):
+    return np.asarray(a).astype(np.float32).astype(np.float64)
+
+
+def _entrywise(dev, ref, tol):
+    for a, b in zip(dev, ref):
+        np.testing.assert_allclose(a.cpu().numpy(), b, rtol=tol, atol=1e-30)
+
+
+@pytest.mark.parametrize("spike", [1e8, 1e12])
+def test_pair_range_one_large_entry(spike):
+    rng = np.random.default_rng(43)
+    X = rng.random((64, 64, 64))
+    X[11, 23, 42] = spike
+    X, F0 = _f32(X), [_f32(1 - rng.random((64, 10))) for _ in range(3)]
+    G0 = _f32(1 - rng.random((10, 10, 10)))
+    F, G = [_dev(f, torch.float32) for f in F0], _dev(G0, torch.float32)
+    native.ntd_fit(_dev(X, torch.float32), F, G, 3)
+    Fo, Go, _ = orc.ntd_fit(X, F0, G0, 3)
+    _entrywise(F + [G], list(Fo) + [Go], 3e-4)
+
+
+# X in three blocks along its first and last mode, and a factor that is smaller by 1e12 on each
+# block's slices than on the one's before: every term of a later block's numerators is tiny, and
+# none may be lost beside the first block's.
+def _three_blocks(dims, seed):
+    rng = np.random.default_rng(seed)
+    X = rng.random(dims)
+    b = [np.arange(n) * 3 // n for n in dims]
+    X *= (b[0][:, None] == b[-1][None, :]).reshape(dims[0], *[1] * (len(dims) - 2), dims[-1])
+    return _f32(X), b, rng
+
+
+@pytest.mark.parametrize("tiny", [0, -1])
+@pytest.mark.parametrize("call,dims,m", [
+    ("ntd", (48, 40, 68), (9, 10, 11)), ("ntd7", (48, 40, 68), (9, 10, 11)),
+    ("ntd", (24, 128, 72), (9, 20, 32)),       # the fused contraction
+    ("ntd", (130, 20, 132), (33, 5, 40)),      # columns of 64
+    ("ntd4", (20, 12, 14, 36), (9, 10, 11, 12)), ("ntd4x3", (20, 12, 14, 36), (9, 10, 11, 12)),
+    ("cp", (48, 40, 68), (9, 9, 9)), ("cp3", (48, 40, 68), (9, 9, 9))])
+def test_pair_range_wide_factors(call, dims, m, tiny):
+    X, b, rng = _three_blocks(dims, 47)
+    iters = {"ntd7": 7, "ntd4x3": 3, "cp3": 3}.get(call, 1)
+    F0 = [1 - rng.random((n, k)) for n, k in zip(dims, m)]
+    F0[tiny] *= 10.0 ** (-12 * b[tiny])[:, None]
+    F0, Xd = [_f32(f) for f in F0], _dev(X, torch.float32)
+    F = [_dev(f, torch.float32) for f in F0]
+    if call.startswith("cp"):
+        err, tr = native.nncp_tensor_fit(Xd, F, iters)
+        Fo, tro = orc.nncp_fit(X, F0, iters)
+        out, ref = F, list(Fo)
+    else:
+        G0 = _f32(1 - rng.random(m))
+        G = _dev(G0, torch.float32)
+        err, tr = native.ntd_fit(Xd, F, G, iters)
+        Fo, Go, tro = orc.ntd_fit(X, F0, G0, iters)
+        out, ref = F + [G], list(Fo) + [Go]
+    _entrywise(out, ref, 1e-4 * iters)
+    np.testing.assert_allclose(tr.cpu().numpy(), tro, rtol=0, atol=1e-5)
+
+
+def test_pair_range_lifted_gradient():
+    dims, m, r = (48, 40, 68), (9, 10, 11), 5
+    X, b, rng = _three_blocks(dims, 53)
+    F = [1 - rng.random((n, k)) for n, k in zip(dims, m)]
+    B = [_f32(1 - rng.random((k, r))) for k in m]
+    F[0][b[0] > 0] = 0.0  # A^(1) is zero there and the gradient -MT B^T: nonnegative sums
+    F[2] *= 10.0 ** (-12 * b[2])[:, None]
+    F = [_f32(f) for f in F]
+    _, gF, _ = native.candelinc_lifted_grad(_dev(X, torch.float32),
+                                            [_dev(f, torch.float32) for f in F],
+                                            [_dev(v, torch.float32) for v in B])
+    gFo, _ = orc.lifted_loss_grad(X, F, B)
+    np.testing.assert_allclose(gF[0].cpu().numpy()[b[0] > 0], gFo[0][b[0] > 0], rtol=1e-4)
+
+
+# The pairs are left after the first step (an X of wide range), and every step counts once: four
+# steps have the bits of twice two.
+@pytest.mark.parametrize("dims", [(48, 40, 68), (12, 10, 9, 16)])
+def test_pair_range_projected_gradient(dims):
+    rng = np.random.default_rng(59)
+    m, r = (9, 10, 11, 7)[:len(dims)], 5
+    X = rng.random(dims)
+    X[(3,) * len(dims)] = 1e10
+    X = _dev(X, torch.float32)
+    F0 = [_dev(1 - rng.random((n, k)), torch.float32) for n, k in zip(dims, m)]
+    B0 = [_dev(1 - rng.random((k, r)), torch.float32) for k in m]
+    F, B = [f.clone() for f in F0], [b.clone() for b in B0]
+    loss, tr = native.candelinc_pg_fit(X, F, B, 4)
+    F2, B2 = [f.clone() for f in F0], [b.clone() for b in B0]
+    _, tr2 = native.candelinc_pg_fit(X, F2, B2, 2)
+    loss2, tr3 = native.candelinc_pg_fit(X, F2, B2, 2)
+    assert loss == loss2 and torch.equal(tr, torch.cat([tr2, tr3]))
+    for a, b in zip(F + B, F2 + B2):
+        assert torch.equal(a, b)
+
+
+# Factors that leave the range of one round late in a long fit (between sweeps 250 and 300 on
+# these data), which then goes on with the other passes. The trace to 1e-5, as everywhere on the
+# FP32 path.
+def test_pair_range_left_late():
+    dims, m, iters = (48, 40, 68), (9, 10, 11), 620
+    rng = np.random.default_rng(7)
+    X = np.zeros(dims)
+    X[:24, :, :34] = rng.random((24, 40, 34))
+    X[24:, :, 34:] = rng.random((24, 40, 34))
+    X = _f32(X + 0.08 * rng.random(dims))
+    F0, G0 = [_f32(1 - rng.random((n, k))) for n, k in zip(dims, m)], _f32(1 - rng.random(m))
+    F, G = [_dev(f, torch.float32) for f in F0], _dev(G0, torch.float32)
+    err, tr = native.ntd_fit(_dev(X, torch.float32), F, G, iters, exact_every=60)
+    Fo, Go, tro = orc.ntd_fit(X, F0, G0, iters)
+    least = min((np.where(f > 0, f, np.inf) / f.max(0)).min() for f in Fo)
+    assert least < 2.0 ** -28
+    np.testing.assert_allclose(tr.cpu().numpy(), tro, rtol=0, atol=1e-5)
+    assert abs(err - orc.rel_err_tucker(X, Go, Fo)) <= 1e-5
