@@ -522,10 +522,11 @@ int nnc_wait_selftest(long long cycles, void* stream);
 
 /*
  * Failure-injection hook for tests (not a step of the method; off by
- * default). Arms the nth scratch allocation from now (nth >= 1; 0 disarms) to
- * fail on the host as if the pool had returned an error, without
- * calling the allocator: the call that makes it returns NNC_ERR_ALLOC, releases
- * the scratch it already holds, and leaves the CUDA context usable. Shared by
+ * default). Arms the nth scratch allocation or graph instantiation from now
+ * (nth >= 1; 0 disarms) to fail on the host as if the pool (the driver) had
+ * returned an error, without calling it: the call that makes it returns
+ * NNC_ERR_ALLOC, waits for the work it has queued on streams of its own,
+ * releases the scratch it already holds, and leaves the CUDA context usable. Shared by
  * every thread of the process. Returns the previous countdown.
  */
 int nnc_debug_fail_alloc(int nth);

@@ -71,6 +71,15 @@ bool alloc_injection_fires() {
   return false;
 }
 
+int graph_instantiate(cudaGraphExec_t* exec, cudaGraph_t graph) {
+  if (alloc_injection_fires()) {
+    set_error_detail_text("graph instantiation failed (injected by nnc_debug_fail_alloc)");
+    return NNC_ERR_ALLOC;
+  }
+  NNC_CUDA_TRY(cudaGraphInstantiate(exec, graph, 0));
+  return NNC_OK;
+}
+
 void note_launch(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone) return;

@@ -33,6 +33,9 @@ void set_error_detail_text(const std::string& s);
 // allocation (host-side failure injection; off unless a caller arms it).
 bool alloc_injection_fires();
 
+// Instantiates a captured graph (an allocation for the test hook).
+int graph_instantiate(cudaGraphExec_t* exec, cudaGraph_t graph);
+
 // Stream-ordered allocation from the library's own memory pool of the current
 // device (never the process's default pool). The pool keeps up to
 // kScratchKeepBytes, or 1/64 of the device's memory if that is less, across

@@ -325,6 +325,9 @@ struct SideStream {
     return NNC_OK;
   }
   ~SideStream() {
+    // A call that fails half way leaves no work on its scratch behind (a call that ends
+    // well has waited already).
+    if (s) cudaStreamSynchronize(s);
     if (fork) cudaEventDestroy(fork);
     if (join) cudaEventDestroy(join);
     if (m_ready) cudaEventDestroy(m_ready);
@@ -800,6 +803,7 @@ struct PgGraph {
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
   ~PgGraph() {
+    if (cs) cudaStreamSynchronize(cs);  // as ~SideStream
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
     if (fork) cudaEventDestroy(fork);
@@ -830,7 +834,7 @@ int replay(int count, cudaStream_t s, Body body, After after = After(),
   const cudaError_t end_e = cudaStreamEndCapture(g.cs, &g.graph);
   if (cap != NNC_OK) return cap;
   NNC_CUDA_TRY(end_e);
-  NNC_CUDA_TRY(cudaGraphInstantiate(&g.exec, g.graph, 0));
+  NNC_TRY(graph_instantiate(&g.exec, g.graph));
   size_t nn = 0;
   NNC_CUDA_TRY(cudaGraphGetNodes(g.graph, nullptr, &nn));
   std::vector<cudaGraphNode_t> nodes(nn);
@@ -902,7 +906,7 @@ int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last las
     const cudaError_t e = cudaStreamEndCapture(g.cs, &g.graph);
     if (st2 == NNC_OK) {
       NNC_CUDA_TRY(e);
-      NNC_CUDA_TRY(cudaGraphInstantiate(&g.exec, g.graph, 0));
+      NNC_TRY(graph_instantiate(&g.exec, g.graph));
       long long kernels = 0;
       NNC_TRY(graph_kernels(g.graph, &kernels));
       while (t < count && !(guard && guard->slow)) {

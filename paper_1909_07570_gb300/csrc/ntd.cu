@@ -365,8 +365,7 @@ int capture_sweep(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, dou
   const cudaError_t end_e = cudaStreamEndCapture(g.cs, &g.graph[slot]);
   if (cap_st != NNC_OK) return cap_st;
   NNC_CUDA_TRY(end_e);
-  NNC_CUDA_TRY(cudaGraphInstantiate(&g.exec[slot], g.graph[slot], 0));
-  return NNC_OK;
+  return graph_instantiate(&g.exec[slot], g.graph[slot]);
 }
 
 // Exact checkpoints of the trace and the refinement trigger (nnc_opts

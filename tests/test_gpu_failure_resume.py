@@ -99,3 +99,46 @@ def test_refinement_trigger_switches_early_and_stays_within_bf16_bound():
     assert np.abs(tr[ck] - tro[ck]).max() <= 1e-3
     assert np.abs(tr[sweep:] - tro[sweep:]).max() <= 1e-3
     assert abs(err - tro[-1]) <= 1e-3
+
+
+# A fit that fails on the host after its first step is queued (the graph of the others cannot be
+# instantiated: the last allocation that such a call makes) waits for that step before it
+# returns: nothing writes the caller's arrays, or scratch that has been given back, afterwards.
+@pytest.mark.parametrize("call", ["pg", "ntd"])
+def test_a_failing_fit_leaves_no_work_behind(call):
+    g = torch.Generator(device="cuda").manual_seed(5)
+    dims, m, r = (128, 128, 128, 128), (24, 24, 24, 24), 12  # a step of a millisecond
+    X = torch.rand(dims, generator=g, device="cuda")
+    F0 = [1 - torch.rand(n, k, generator=g, device="cuda") for n, k in zip(dims, m)]
+    B0 = [1 - torch.rand(k, r, generator=g, device="cuda") for k in m]
+    G0 = 1 - torch.rand(m, generator=g, device="cuda")
+
+    def run():
+        F, B, G = [f.clone() for f in F0], [b.clone() for b in B0], G0.clone()
+        torch.cuda.synchronize()
+        try:
+            if call == "pg":
+                native.candelinc_pg_fit(X, F, B, 3, trace=False)
+            else:
+                native.ntd_fit(X, F, G, 3, trace=False, rel_err=False)
+        except native.NncError as e:
+            return e, F + B + [G]
+        return None, F + B + [G]
+
+    assert native.nnc_debug_fail_alloc(100000) == 0
+    ok, want = run()
+    assert ok is None
+    count = 100000 - native.nnc_debug_fail_alloc(0)
+    native.nnc_debug_fail_alloc(count)
+    e, got = run()
+    with torch.cuda.stream(torch.cuda.Stream()):  # ordered after nothing of the library's
+        now = [a.clone() for a in got]
+    torch.cuda.synchronize()
+    assert e is not None and "graph instantiation failed" in str(e)
+    for a, b in zip(now, got):
+        assert torch.equal(a, b)
+    assert any(not torch.equal(a, f) for a, f in zip(got, F0))  # the step was under way
+    ok, again = run()
+    assert ok is None
+    for a, b in zip(again, want):
+        assert torch.equal(a, b)
