@@ -39,16 +39,17 @@ __global__ void lift_kernel(const T* __restrict__ F, const T* __restrict__ B, in
 constexpr int kMpThreads = 256, kMpQ = 16;
 template <typename T>
 __global__ void __launch_bounds__(kMpThreads)
-mode_product_any_kernel(const T* __restrict__ Y, int64_t L, int J, int64_t C,
+mode_product_any_kernel(const T* __restrict__ Y, int64_t L, int J, int64_t C, unsigned col_blocks,
                         const T* __restrict__ A, int Q, T* __restrict__ out) {
   __shared__ T as[64 * kMpQ];
-  const int q0 = blockIdx.y * kMpQ, qn = Q - q0 < kMpQ ? Q - q0 : kMpQ;
+  // Tiles of q and of columns in one grid dimension: a mode may have any length.
+  const int q0 = (int)(blockIdx.x / col_blocks) * kMpQ, qn = Q - q0 < kMpQ ? Q - q0 : kMpQ;
   for (int e = threadIdx.x; e < J * kMpQ; e += kMpThreads) {
     const int j = e / kMpQ, q = e % kMpQ;
     as[e] = q < qn ? A[(int64_t)(q0 + q) * J + j] : T(0);
   }
   __syncthreads();
-  const int64_t col = (int64_t)blockIdx.x * kMpThreads + threadIdx.x;
+  const int64_t col = (int64_t)(blockIdx.x % col_blocks) * kMpThreads + threadIdx.x;
   if (col >= L * C) return;
   const int64_t l = col / C, c = col - l * C;
   const T* y = Y + l * J * C + c;
@@ -321,9 +322,9 @@ int residual_run(const T* X, int d, const int64_t* dims, int model, const int* m
       T* dst = k < d - 2 ? w.tmp[k & 1] : U;
       const int64_t cols = ceil_div(lead * tail, kMpThreads);
       const int64_t qt = ceil_div(dims[k], kMpQ);
-      if (m[k] > 64 || cols > 0x7fffffffLL || qt > 65535) return NNC_ERR_UNSUPPORTED;
-      mode_product_any_kernel<T><<<dim3((unsigned)cols, (unsigned)qt), kMpThreads, 0, s>>>(
-          src, lead, m[k], tail, factors[k], (int)dims[k], dst);
+      if (m[k] > 64 || cols * qt > 0x7fffffffLL) return NNC_ERR_UNSUPPORTED;
+      mode_product_any_kernel<T><<<(unsigned)(cols * qt), kMpThreads, 0, s>>>(
+          src, lead, m[k], tail, (unsigned)cols, factors[k], (int)dims[k], dst);
       note_launch(s);
       src = dst;
       lead *= dims[k];

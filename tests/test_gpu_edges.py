@@ -130,6 +130,20 @@ def test_residual_edges(dt, dims, m):
     assert rn / xn == pytest.approx(orc.rel_err_cp(Xr, A), rel=tol)
 
 
+# A mode past 65535 tiles of 16 entries, as the first and as a middle mode. Tolerances as above.
+@pytest.mark.parametrize("dims", [(1048593, 2, 3), (2, 1048577, 1)])
+def test_residual_of_a_long_mode(dims):
+    rng = np.random.default_rng(19)
+    m = (2, 2, 1)
+    X = rng.random(dims)
+    F = [rng.random((n, k)) for n, k in zip(dims, m)]
+    G = rng.random(m)
+    rn, xn = native.recon_residual(_dev(X, torch.float64), [_dev(f, torch.float64) for f in F],
+                                   _dev(G, torch.float64))
+    assert xn == pytest.approx(np.linalg.norm(X), rel=1e-11)
+    assert rn / xn == pytest.approx(orc.rel_err_tucker(X, G, F), rel=1e-11)
+
+
 # Whole fits on one cluster: modes shorter than the cluster (CTAs without slices), slices
 # with a remainder, 16-byte and single columns, every tile width, exact checkpoints; and the
 # same fit in pieces. The trace and factors against the oracle: FP64 rounding over a few
