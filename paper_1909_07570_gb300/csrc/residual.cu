@@ -118,9 +118,11 @@ ResGrid res_grid(int64_t R, int64_t N3, int K) {
 // (one column a thread, one row at a time: 512^3, K = 32, 519 us and 128^3 x 64, K = 16,
 // 824 us, half of its threads past the row's end).
 // Per element: x_hat = U[t, :] . F3[k, :] in T, then (x - x_hat)^2 and x^2. For T =
-// float the thread adds its terms in FP32 (rounded to nearest, so the errors are unbiased
-// and shrink in the FP64 sums that follow); GB300's FP64 rate is far below its
-// FP32 rate, and FP64 arithmetic per element would bound the pass. The block
+// float the thread adds at most 64 terms in one FP32 chain (rounded to nearest, so the errors
+// are mostly unbiased; equal terms round alike, and 64 of them stay within 33 roundings), the chains
+// of a chunk in a pair of floats with the error of every addition kept, the chunks in FP64:
+// GB300's FP64 rate is far below its FP32 rate, and FP64 arithmetic per element would bound the
+// pass (one FP64 addition and conversion a chain: 424 -> 446 us at 512^3, this 426 us). The block
 // sums and the partials are FP64.
 template <typename T, int KM, int KT>
 __global__ void __launch_bounds__(kResThreads)
@@ -153,9 +155,21 @@ residual_stream_kernel(const T* __restrict__ X, int64_t R, int64_t N3, const T* 
     }
     __syncthreads();
     T d2 = T(0), x2 = T(0);
+    T cd[2] = {T(0), T(0)}, cx[2] = {T(0), T(0)};  // sum and what its additions rounded off
     const T* xp = X + r0 * N3 + k0;
     // Four rows at a time, their entries of X requested one round ahead.
-    constexpr int RU = 4;
+    constexpr int RU = 4, kRounds = 64 / (RU * KT);
+    int rounds = 0;
+    auto add = [](T (&c)[2], T v) {
+      const T t = c[0] + v, b = t - c[0];
+      c[1] += (c[0] - (t - b)) + (v - b);
+      c[0] = t;
+    };
+    auto flush = [&]() {
+      add(cd, d2);
+      add(cx, x2);
+      d2 = x2 = T(0);
+    };
     T nx[RU][KT];
     auto fetch = [&](int row) {
 #pragma unroll
@@ -208,10 +222,16 @@ residual_stream_kernel(const T* __restrict__ X, int64_t R, int64_t N3, const T* 
           x2 = fma(x[q][u], x[q][u], x2);
         }
       }
+      if (++rounds == kRounds) {
+        flush();
+        rounds = 0;
+      }
     }
-    if (isfinite(d2) && isfinite(x2)) {
-      td2 += (double)d2;
-      tx2 += (double)x2;
+    flush();
+    const double cd2 = (double)cd[0] + (double)cd[1], cx2 = (double)cx[0] + (double)cx[1];
+    if (isfinite(cd2) && isfinite(cx2)) {
+      td2 += cd2;
+      tx2 += cx2;
     } else {
       // The FP32 terms overflowed (entries beyond about 1e19): these rows again
       // with FP64 terms. Non-finite data stays non-finite.

@@ -144,6 +144,22 @@ def test_residual_of_a_long_mode(dims):
     assert rn / xn == pytest.approx(orc.rel_err_tucker(X, G, F), rel=1e-11)
 
 
+# FP32 terms are added in chains of at most 64 before FP64: equal terms, whose roundings add up.
+# The i-th rounding of a chain is at most 2^-24 of the i terms so far, 32.5 2^-24 of the chain in
+# all, and half of that in a norm. (Values whose chains of 1024 and 256 would be off by 7.6e-6
+# and 1.9e-6.)
+@pytest.mark.parametrize("value,last,dims", [(1.9976487, 16, (1000, 480, 512)),
+                                             (1.9550849, 32, (1000, 480, 256))])
+def test_residual_chains_are_short(value, last, dims):
+    v = float(np.float32(value))
+    X = torch.full(dims, v, device="cuda")
+    F = [torch.zeros(n, k, device="cuda") for n, k in zip(dims, (2, 2, last))]
+    rn, xn = native.recon_residual(X, F, torch.zeros(2, 2, last, device="cuda"))
+    want = v * np.sqrt(np.prod(dims, dtype=np.float64))
+    assert xn == pytest.approx(want, rel=32.5 * 2.0 ** -25)
+    assert rn == pytest.approx(want, rel=32.5 * 2.0 ** -25)
+
+
 # Whole fits on one cluster: modes shorter than the cluster (CTAs without slices), slices
 # with a remainder, 16-byte and single columns, every tile width, exact checkpoints; and the
 # same fit in pieces. The trace and factors against the oracle: FP64 rounding over a few
