@@ -400,3 +400,57 @@ def test_pair_range_left_late():
     assert least < 2.0 ** -28
     np.testing.assert_allclose(tr.cpu().numpy(), tro, rtol=0, atol=1e-5)
     assert abs(err - orc.rel_err_tucker(X, Go, Fo)) <= 1e-5
+
+
+# The tensor-core passes on shapes that no one-cluster fit takes (a multirank above 8): pairs with
+# the fused contraction over two tiles a slab, on data whose magnitudes are no product of
+# scales; and operands past what a block holds, which run as TF32x3: with the mode-3 shares formed
+# by the pass (N2 % 128 == 0, N3 > 768 or N1 > 1024), without them, and with columns of 64
+# (N1 > 512). One sweep to 1e-4 elementwise, as the pair passes above.
+@pytest.mark.parametrize("dims,m,scaled", [
+    ((3, 256, 4), (9, 3, 4), True), ((20, 128, 68), (10, 12, 9), True),
+    ((17, 128, 900), (12, 10, 12), False), ((1100, 128, 8), (9, 6, 4), False),
+    ((1030, 9, 20), (9, 4, 4), False), ((600, 9, 20), (40, 4, 4), True)])
+def test_passes_past_the_cluster_and_the_pairs(dims, m, scaled):
+    X, _, F0, G0, _ = inputs.small_problem(dims, 3, m, 2, seed=97)
+    if scaled:
+        X = X * 10.0 ** np.random.default_rng(61).uniform(-2, 2, dims)
+    X, F0, G0 = _f32(X), [_f32(f) for f in F0], _f32(G0)
+    F, G = [_dev(f, torch.float32) for f in F0], _dev(G0, torch.float32)
+    err, _ = native.ntd_fit(_dev(X, torch.float32), F, G, 1, precision="fp32")
+    Fo, Go, _ = orc.ntd_fit(X, F0, G0, 1)
+    _entrywise(F + [G], list(Fo) + [Go], 1e-4)
+    assert abs(err - orc.rel_err_tucker(X, Go, Fo)) <= 1e-5
+
+
+# The sweep of separate kernels on small and degenerate shapes: a multirank above 8 keeps them off
+# the cluster. Three sweeps, no sweep, and a fit whose residual overflows.
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+@pytest.mark.parametrize("dims,m", [((1, 7, 12), (1, 2, 9)),
+                                    ((12, 40, 1), (10, 3, 1)), ((37, 29, 23), (9, 6, 7)),
+                                    ((5, 61, 201), (3, 9, 3))])
+def test_separate_kernels_on_small_shapes(dt, dims, m):
+    X, _, F0, G0, _ = inputs.small_problem(dims, 2, m, 2, seed=67)
+    X, F0, G0 = (_dev(X, dt).double().cpu().numpy(),
+                 [_dev(f, dt).double().cpu().numpy() for f in F0],
+                 _dev(G0, dt).double().cpu().numpy())
+    F, G = [_dev(f, dt) for f in F0], _dev(G0, dt)
+    err, tr = native.ntd_fit(_dev(X, dt), F, G, 3)
+    Fo, Go, tro = orc.ntd_fit(X, F0, G0, 3)
+    tol = _TOL[dt]
+    for a, b in zip(F + [G], Fo + [Go]):
+        np.testing.assert_allclose(a.double().cpu().numpy(), b, rtol=tol, atol=tol * 1e-3)
+    np.testing.assert_allclose(tr.cpu().numpy(), tro, rtol=0,
+                               atol=(1e-8 if dt == torch.float64 else 1e-5) * max(1.0, tro.max()))
+    F, G = [_dev(f, dt) for f in F0], _dev(G0, dt)
+    err, _ = native.ntd_fit(_dev(X, dt), F, G, 0)
+    assert err == pytest.approx(orc.rel_err_tucker(X, G0, F0), abs=tol)
+    assert all(torch.equal(f, _dev(b, dt)) for f, b in zip(F + [G], F0 + [G0]))
+
+
+def test_separate_kernels_report_an_overflow():
+    X, _, F0, G0, _ = inputs.small_problem((24, 20, 16), 3, (9, 4, 4), 2, seed=21)
+    with pytest.raises(native.NncError) as ei:
+        native.ntd_fit(_dev(X * 1e30, torch.float32), [_dev(f, torch.float32) for f in F0],
+                       _dev(G0, torch.float32), 10)
+    assert ei.value.status == -3 and "sweep" in str(ei.value)
