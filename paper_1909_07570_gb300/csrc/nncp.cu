@@ -477,7 +477,7 @@ int nncp_route(int n_jobs, const nncp_job* jobs, bool skip_invalid, NncpRoute* r
     const nncp_job& j = jobs[i];
     if (!nncp_job_valid(j)) continue;
     ++valid;
-    if (j.d != 3 || cpx_cluster_elems(j, rmax) * sizeof(T) > kSmemBudget) cl_ok = false;
+    if (j.d != 3 || cpx_cluster_elems(j, rmax, false) * sizeof(T) > kClusterSmem) cl_ok = false;
   }
   cl_ok = cl_ok && valid >= 1 && (int64_t)valid * cpx_cluster_ctas() <= device_sm_count();
   constexpr int64_t kTwoPassMinEntries = 16384;

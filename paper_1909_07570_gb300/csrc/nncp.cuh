@@ -67,10 +67,15 @@ template <typename T>
 int nncp_cluster_batched(int n_jobs, const nncp_job* jobs, int iters, double eps,
                          double* rel_errs, int* statuses, cudaStream_t s);
 // Shared-memory elements of one CTA of a cluster fit of job j in a batch whose largest
-// rank is rmax, and the CTAs
+// rank is rmax, with the slab for mode 2 in shared memory or read from L2 in place, and the CTAs
 // of a cluster.
-size_t cpx_cluster_elems(const nncp_job& j, int rmax);
+size_t cpx_cluster_elems(const nncp_job& j, int rmax, bool slab_j);
 int cpx_cluster_ctas();
+// Shared memory a CTA of a cluster fit may ask for: with the kernel's static 4 KB nearly all that a
+// block can have, since the other form (one block a fit, the tensor read from L2 by one SM) is far
+// slower: us a sweep, FP64 38 x 44 x 53 at r = 1 423 against 16, 51 x 25 x 63 at r = 7 366 against 57, FP32
+// 61 x 53 x 52 at r = 5 94 against 9.3.
+constexpr size_t kClusterSmem = 222 * 1024;
 
 // The tuning class of a batch (largest per-sweep work over the valid jobs,
 // number of jobs).

@@ -8,7 +8,8 @@
 //
 // CTA c of the cluster owns the rows of every factor in its ranges of i, j and k and keeps, in
 // shared memory, the slab of the core with its i (for T), the slab with its j (for
-// T'), and full copies of every factor and Gram. T and T' on its slabs give MT1 and MT2 on its
+// T'; read from L2 in place where it does not fit beside the rest), and full copies of every
+// factor and Gram. T and T' on its slabs give MT1 and MT2 on its
 // own rows and its share of MT3; new rows go to the other CTAs through distributed
 // shared memory, into the copy of the factor that no CTA reads any more (two
 // copies, swapped at the barrier), the shares of MT3 to the CTA that owns the row k, which
@@ -47,14 +48,14 @@ struct ClLayout {
   int ni, nj, nk;  // rows of each factor a CTA owns
   int xpitch;      // row pitch of the i-slab
   size_t xi, xj, a[2][3], g[3], tb, in, total;
-  __host__ __device__ explicit ClLayout(const int* N, int rp) {
+  __host__ __device__ ClLayout(const int* N, int rp, bool slab_j) {
     ni = (N[0] + kCl - 1) / kCl;
     nj = (N[1] + kCl - 1) / kCl;
     nk = (N[2] + kCl - 1) / kCl;
     size_t p = 0;
     xpitch = N[2] | 1;  // odd: the rows a warp reads fall on distinct banks
     xi = p;  p += al4((size_t)ni * N[1] * xpitch);  // [ii][j][k], rows xpitch apart
-    xj = p;  p += al4((size_t)N[0] * nj * N[2]);    // [i][jj][k]
+    xj = p;  p += slab_j ? al4((size_t)N[0] * nj * N[2]) : 0;  // [i][jj][k]
     for (int b = 0; b < 2; ++b)
       for (int n = 0; n < 3; ++n) { a[b][n] = p;  p += (size_t)N[n] * rp; }
     for (int n = 0; n < 3; ++n) { g[n] = p;  p += (size_t)rp * rp; }
@@ -135,8 +136,8 @@ __device__ __forceinline__ void gram_lanes(const GramLane<RP>& g, const T* A, in
 
 template <typename T, int RP>
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
-    cpx_cluster_kernel(const nncp_job* __restrict__ jobs, int iters, T eps, double* rel_errs,
-                       int* statuses) {
+    cpx_cluster_kernel(const nncp_job* __restrict__ jobs, int iters, T eps, bool slab_j,
+                       double* rel_errs, int* statuses) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[2 * kFixedLanes];
   __shared__ double sums[2];
@@ -151,7 +152,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     return;
   }
   const int N1 = jb.m[0], N2 = jb.m[1], N3 = jb.m[2], r = jb.r;
-  const ClLayout L(jb.m, RP);
+  const ClLayout L(jb.m, RP, slab_j);
   T* sm = reinterpret_cast<T*>(smem_raw);
   T* Xi = sm + L.xi;
   T* Xj = sm + L.xj;
@@ -171,10 +172,11 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     const int row = e / N3, k = e - row * N3;
     Xi[row * L.xpitch + k] = X[(int64_t)i0 * N2 * N3 + e];
   }
-  for (int e = tid; e < N1 * nj * N3; e += nt) {
-    const int i = e / (nj * N3), jk = e - i * nj * N3;
-    Xj[e] = X[((int64_t)i * N2 + j0) * N3 + jk];
-  }
+  if (slab_j)
+    for (int e = tid; e < N1 * nj * N3; e += nt) {
+      const int i = e / (nj * N3), jk = e - i * nj * N3;
+      Xj[e] = X[((int64_t)i * N2 + j0) * N3 + jk];
+    }
   for (int n = 0; n < 3; ++n) {
     const T* src = static_cast<const T*>(jb.B[n]);
     for (int e = tid; e < jb.m[n] * RP; e += nt) {
@@ -240,7 +242,11 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
     cl.sync();
     swap(0);
     // ---- T'[jj, k, :] on this CTA's j; Gram1
-    row_products<T, RP>(nj * N3, N1, r, Xj, [&](int jk) { return jk; }, nj * N3, A[0], Tb);
+    if (slab_j)
+      row_products<T, RP>(nj * N3, N1, r, Xj, [&](int jk) { return jk; }, nj * N3, A[0], Tb);
+    else
+      row_products<T, RP>(nj * N3, N1, r, X + j0 * N3, [&](int jk) { return jk; }, N2 * N3, A[0],
+                          Tb);
     gram_lanes<T, RP>(gl, A[0], N1, Gr[0]);
     __syncthreads();
     // ---- A2
@@ -316,8 +322,8 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kClThreads)
 
 }  // namespace
 
-size_t cpx_cluster_elems(const nncp_job& j, int rmax) {
-  return ClLayout(j.m, (rmax + 3) / 4 * 4).total;
+size_t cpx_cluster_elems(const nncp_job& j, int rmax, bool slab_j) {
+  return ClLayout(j.m, (rmax + 3) / 4 * 4, slab_j).total;
 }
 
 int cpx_cluster_ctas() { return kCl; }
@@ -334,11 +340,15 @@ int nncp_cluster_batched(int n_jobs, const nncp_job* jobs, int iters, double eps
       return NNC_ERR_UNSUPPORTED;
     }
   }
-  size_t elems = 0;
-  for (int i = 0; i < n_jobs; ++i)
-    if (nncp_job_valid(jobs[i])) elems = std::max(elems, cpx_cluster_elems(jobs[i], rmax));
-  const size_t smem = elems * sizeof(T);
-  if (smem > kSmemBudget) {
+  auto smem_of = [&](bool slab_j) {
+    size_t elems = 0;
+    for (int i = 0; i < n_jobs; ++i)
+      if (nncp_job_valid(jobs[i])) elems = std::max(elems, cpx_cluster_elems(jobs[i], rmax, slab_j));
+    return elems * sizeof(T);
+  };
+  const bool slab_j = smem_of(true) <= kClusterSmem;
+  const size_t smem = smem_of(slab_j);
+  if (smem > kClusterSmem) {
     set_error_detail_text("cluster nnCP: a job's slabs exceed one block of shared memory");
     return NNC_ERR_UNSUPPORTED;
   }
@@ -355,7 +365,8 @@ int nncp_cluster_batched(int n_jobs, const nncp_job* jobs, int iters, double eps
                     : rmax <= 12 ? cpx_cluster_kernel<T, 12>
                                  : cpx_cluster_kernel<T, 16>;
   NNC_CUDA_TRY(raise_smem_limit((const void*)kern, smem));
-  kern<<<(unsigned)(n_jobs * kCl), kClThreads, smem, s>>>(dev, iters, (T)eps, rel_errs, statuses);
+  kern<<<(unsigned)(n_jobs * kCl), kClThreads, smem, s>>>(dev, iters, (T)eps, slab_j, rel_errs,
+                                                          statuses);
   note_launch(s);
   NNC_CUDA_TRY(cudaGetLastError());
   return NNC_OK;

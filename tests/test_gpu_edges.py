@@ -454,3 +454,21 @@ def test_separate_kernels_report_an_overflow():
         native.ntd_fit(_dev(X * 1e30, torch.float32), [_dev(f, torch.float32) for f in F0],
                        _dev(G0, torch.float32), 10)
     assert ei.value.status == -3 and "sweep" in str(ei.value)
+
+
+# Cluster core fits near and past the shared memory of a CTA: the slab of the second product
+# there and, where it does not fit, read in place. Bounds as for the other cluster fits.
+@pytest.mark.parametrize("dt,m,r", [(torch.float64, (38, 44, 53), 1), (torch.float64, (45, 33, 62), 1),
+                                    (torch.float64, (59, 26, 56), 5), (torch.float64, (64, 17, 60), 13),
+                                    (torch.float32, (61, 53, 52), 5), (torch.float32, (64, 63, 64), 4)])
+def test_cluster_core_fits_at_the_shared_memory_limit(dt, m, r):
+    rng = np.random.default_rng(71)
+    G, B0 = rng.random(m), inputs.initial_cp(m, r, 17)
+    B = [_dev(b, dt) for b in B0]
+    err = native.nncp_core_fit(_dev(G, dt), B, 5)
+    Bo, tro = orc.nncp_fit(_dev(G, dt).double().cpu().numpy(),
+                           [_dev(b, dt).double().cpu().numpy() for b in B0], 5)
+    tol = _TOL[dt]
+    for a, b in zip(B, Bo):
+        np.testing.assert_allclose(a.double().cpu().numpy(), b, rtol=tol, atol=tol * 1e-3)
+    assert err == pytest.approx(tro[-1], abs=tol)
