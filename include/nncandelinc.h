@@ -482,7 +482,9 @@ int recon_residual(const void* X, int d, const int64_t* dims, int precision, int
  *   5  X x_1 F^(1)T, FP32-accurate tensor-core passes
  * nnc_profile_enable(on) switches it and clears the totals; nnc_profile_read
  * returns the number of timed launches and their total milliseconds of a
- * kind. Meant for one thread of control: concurrent ntd_fit calls while it is
+ * kind. A small 3-way fit that otherwise runs as one launch has no passes to
+ * time: while profiling is on it runs as separate kernels, with the same
+ * results up to rounding. Meant for one thread of control: concurrent ntd_fit calls while it is
  * enabled share one event pool and give meaningless totals.
  */
 int nnc_profile_enable(int on);

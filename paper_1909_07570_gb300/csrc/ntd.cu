@@ -181,7 +181,7 @@ int sweep3(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double* tr
   // step.
   //   s2:  H2 ................ MU on F2 | H3 (S2 of the new F2)
   //   s3:  Num2 (P3, new F1) --^
-  // When pass 2 can also form the shares of Y3[k] = P1[k]^T F2 (FP32-accurate with
+  // When pass 2 can also form the shares of Y3[k] = P1[k]^T F2 (TF32x3 with
   // N2 % 128 == 0, m <= 32), it waits for the new F2 and the mode-3 update
   // only adds the shares; H3 runs beside the pass:
   //   s:   pass 2 (new F1, new F2) -- mode 3 (shares, H3)

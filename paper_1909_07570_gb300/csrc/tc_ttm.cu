@@ -1743,8 +1743,8 @@ int TcPlan::init(int kind_, const float* X, int64_t N1_, int64_t N2_, int64_t N3
 
 // The shapes the FP16 pair passes take: rows of X on 16 bytes, and both passes'
 // operands (K x m, split, in shared memory for the whole pass) beside three
-// stages at least: K up to 768 for m <= 32, 384 for m <= 64 (512 and 256 less the
-// fused contraction's tiles).
+// stages at least: N3 up to 768 for m3 <= 32 (room for the fused contraction's tiles is
+// kept), N1 up to 1024 for m1 <= 32, 512 each for m <= 64.
 int TcPlan::init_f16(const float* X, Scratch& sc, cudaStream_t s) {
   const int64_t rows = N1 * N2;
   const int nk3 = kb3 / 64, nk1 = kp1 / 64;

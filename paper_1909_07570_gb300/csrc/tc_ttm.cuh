@@ -116,7 +116,7 @@ struct TcPlan {
             const float* F2 = nullptr, int m2 = 0, float* Y1 = nullptr) const;
   bool y1_fusable(int m2) const;
   // P1 = X x_1 F1^T (FP32; m1 x N2 x N3, or rows (k, j) with p1_kj).
-  // With Y3 (y3_fusable(m2) only: FP32-accurate with p1_kj) the pass also writes the
+  // With Y3 (y3_fusable(m2) only: TF32x3 with p1_kj) the pass also writes the
   // per-tile shares of Y3[k] = P1[k, :, :]^T F2 (m1 x m2 each).
   int pass1(const float* F1, float* P1, cudaStream_t s, bool convert = true,
             const float* F2 = nullptr, int m2 = 0, float* Y3 = nullptr) const;
