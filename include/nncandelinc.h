@@ -54,13 +54,14 @@ typedef enum {
                           three products per term (hi*hi + hi*lo + lo*hi of
                           splits into two FP16 parts, scaled by powers of two
                           per slice, or into two TF32 parts; FP32
-                          accumulation). Either split holds 22 bits of every
-                          entry: an X with nonzero entries more than 28 powers
-                          of two below the largest of their slices runs with
-                          TF32 parts, smaller factor entries take further
+                          accumulation). Either way a sum is as exact as with
+                          22 bits of every entry: an X with nonzero entries
+                          more than 28 powers of two below the largest of
+                          their slices runs with TF32 parts; for sums without
+                          larger terms, smaller factor entries take further
                           rounds of a pass, and a fit with many such rounds
                           goes on with TF32 parts. Shapes the tensor-core path
-                          cannot take (N3 % 4 != 0) run the SIMT passes        */
+                          cannot take (N3 % 4 != 0) run the SIMT passes      */
   NNC_BF16_REFINE = 2, /* float storage; the passes over X use a BF16 copy of
                           X on the tensor cores (FP32 accumulation), then the
                           last `refine_iters` sweeps are NNC_FP32 sweeps     */

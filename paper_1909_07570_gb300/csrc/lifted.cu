@@ -458,7 +458,7 @@ int settle_pairs(Work<T>& w, bool* left, Scratch& sc, cudaStream_t s, tc::PairGu
     NNC_TRY(w.plan.wide(s, left));
     if (*left) return w.plan.to_tf32(w.X, sc, s);
     if (guard && w.plan.kind == tc::kKindF16x3) {
-      NNC_TRY(guard->start(&w.plan, sc));
+      NNC_TRY(guard->start(&w.plan, 1));
       *use = guard;
     }
   }
@@ -851,9 +851,7 @@ int replay(int count, cudaStream_t s, Body body, After after = After(),
     NNC_TRY(after(t, g.cs));
     ++t;
     if (guard && t < count) {
-      // looked at once the next sweep is queued
-      if (t % tc::kPairLook == 1) NNC_TRY(guard->mark(g.cs, t));
-      if (t % tc::kPairLook == 2) NNC_TRY(guard->look(s));
+      NNC_TRY(guard->step(g.cs, t));
       if (guard->slow) break;
     }
   }
@@ -900,7 +898,7 @@ int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last las
   int st2 = st1;
   int t = 1;
   if (st1 == NNC_OK && count > 1) {
-    if (guard) NNC_TRY(guard->mark(g.cs, t));
+    if (guard) NNC_TRY(guard->step(g.cs, t));
     NNC_CUDA_TRY(cudaStreamBeginCapture(g.cs, cudaStreamCaptureModeThreadLocal));
     st2 = rest(g.cs);
     const cudaError_t e = cudaStreamEndCapture(g.cs, &g.graph);
@@ -912,9 +910,7 @@ int replay_pipelined(int count, cudaStream_t s, First first, Rest rest, Last las
       while (t < count && !(guard && guard->slow)) {
         NNC_CUDA_TRY(cudaGraphLaunch(g.exec, g.cs));
         ++t;
-        // looked at once the next sweep is queued
-        if (guard && t % tc::kPairLook == 1) NNC_TRY(guard->mark(g.cs, t));
-        if (guard && t % tc::kPairLook == 2) NNC_TRY(guard->look(s));
+        if (guard) NNC_TRY(guard->step(g.cs, t));
       }
       note_graph_launches(kernels * (t - 1));
     }

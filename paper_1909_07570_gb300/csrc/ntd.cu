@@ -434,19 +434,10 @@ int run_sweeps(const T* X, T* const* F, T* G, NtdState<T>& b, double eps, double
   // host captures the graph of the others (capturing and instantiating it takes the time
   // of several sweeps of a mid-size tensor).
   const int direct = samples > 0 ? 0 : std::min(count, kSweepsPerGraph);
-  int look = direct > 0 ? direct : kSweepsPerGraph;
-  bool marked = false;
   while (t < count) {
-    if (guard && t >= look) {
-      if (!marked) {
-        NNC_TRY(guard->mark(g.cs, t));
-        look = t + 1;  // looked at once the next sweeps are queued
-      } else {
-        NNC_TRY(guard->look(s));
-        if (guard->slow) break;
-        look = t + tc::kPairLook;
-      }
-      marked = !marked;
+    if (guard && t > 0) {
+      NNC_TRY(guard->step(g.cs, t));
+      if (guard->slow) break;
     }
     const bool sampled = samples > 0 && t % kProfileEvery == kProfileEvery - 1;
     // A five-sweep replay must not pass a sampled sweep or a checkpoint (its
@@ -707,7 +698,7 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
       if (wide) NNC_TRY(leave_pairs());
       if (exact && exact->kind == tc::kKindF16x3) {
         tc::PairGuard guard;
-        NNC_TRY(guard.start(exact, sc));
+        NNC_TRY(guard.start(exact, kSweepsPerGraph));
         int n = 0;
         NNC_TRY(run_sweeps<T>(X, F, G, b, o->eps, trace, o->iters - at, at, &ck, exact, s, &n,
                               &guard));

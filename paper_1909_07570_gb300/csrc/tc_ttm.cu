@@ -698,10 +698,15 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // factor takes it out of the subnormals: without it only from 2^-1), 28 powers of two
 // below the largest entry; zeros are exact. The TF32 pair holds them at every magnitude. An X
 // with a nonzero entry below that range is flagged by x_to_pair_kernel, and the fit starts again
-// with TF32x3 passes. Factor entries below it (updates drive entries to zero; a block of X
-// may have no other terms) are the operand of another round over the tiles, scaled up
-// by 2^28, whose results are added: every entry keeps its 22 bits at the price of a pass per 28
-// powers of two, and a fit whose passes take many rounds goes on with TF32x3 (PairGuard).
+// with TF32x3 passes. Factor entries below it (updates drive entries to zero) matter to an output
+// that has no larger terms, as in a block of X of its own. What the products make of them is
+// off by less than 2^-20 in the scales' units a term (the pair's 2^-36 of an entry of F times 2^15
+// of X, the product of two low parts, which is not formed, and the tensor core's alignment of
+// subnormal operands, whose products lose bits below 2^-23), so an output of 2^3 K or more over K
+// terms is as exact as with 22 bits of every entry. A CTA that finds a smaller one goes
+// over its tiles again, in rounds that take the entries of 28 powers of two each, scaled up into
+// the range: the first overwrites the results, the others add to them, until no entry or no output
+// is left below. A fit whose passes take such rounds often goes on with TF32x3 passes (PairGuard).
 // Why pairs made once per fit instead of TF32 parts made in every pass: the
 // TF32x3 stage moves each entry through shared memory five times (TMA in, read and
 // two writes of the split, two reads by the MMAs, 8 bytes an entry in the last
@@ -777,17 +782,17 @@ __device__ __forceinline__ void split_f16(float v, __half& hi, __half& lo) {
 
 // The pass's B operand in shared memory (256 threads: warps 2-9): for each 64-entry
 // K chunk 2 NP rows of 128 bytes, rows [0, NP) f_hi and [NP, 2 NP) f_lo of
-// F[k, q] kscale[k] / cscale[q], in the 128-byte swizzle. cs[q] gets cscale. *more gets 1 when
-// a nonzero entry below the range is left for another round (zero here). A column whose largest
-// entry is so small that products with kscale may be subnormal is left whole.
-constexpr int kF16RoundBits = 28, kF16MaxRounds = 14;  // every product of two floats
+// F[k, q] kscale[k] / cscale[q], in the 128-byte swizzle. cs[q] gets cscale. *low gets 1 when
+// a nonzero entry lies below the range. A column whose largest entry is so small that products
+// with kscale may be subnormal is left to the rounds.
+constexpr int kF16RoundBits = 28, kF16MaxRounds = 16;  // every product of two floats
 constexpr int kF16LeaveExp = -112;
 __device__ __forceinline__ unsigned char* f16_b_row(unsigned char* bs, int np, int o, int n) {
   return bs + (o >> 3) * (2 * np * 128) + n * 128 + (((o & 7) ^ (n & 7)) << 4);
 }
 template <int NP>
 __device__ __forceinline__ void f16_operand(const F16Operand& fo, int nk, unsigned char* bs,
-                                            float* cs, unsigned* cmax, int* more) {
+                                            float* cs, unsigned* cmax, int* low_out) {
   const int t = threadIdx.x - 64, lane = t & 31, w = t >> 5;
   constexpr int NC = NP / 32;  // columns per lane
   const int noct = nk * 8;     // octets of K entries
@@ -819,7 +824,7 @@ __device__ __forceinline__ void f16_operand(const F16Operand& fo, int nk, unsign
     const int e = f16_exponent(cmax[lane + 32 * c]);
     const bool leave = e < kF16LeaveExp;
     inv[c] = leave ? 0.f : pow2f(-e);
-    if (w == 0) cs[lane + 32 * c] = pow2f(leave ? e + kF16RoundBits : e);
+    if (w == 0) cs[lane + 32 * c] = pow2f(e);
   }
   bool low = false;
   for (int o = w; o < noct; o += 8) {
@@ -837,59 +842,56 @@ __device__ __forceinline__ void f16_operand(const F16Operand& fo, int nk, unsign
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const float y = f[u] * ks[u] * inv[c];
-        const bool under = fabsf(y) < kF16Least;
-        low |= under && f[u] != 0.f;
-        split_f16(under ? 0.f : y, hi.h[u], lo.h[u]);
+        low |= fabsf(y) < kF16Least && f[u] != 0.f;
+        split_f16(y, hi.h[u], lo.h[u]);
       }
       unsigned char* row = f16_b_row(bs, NP, o, n);
       *reinterpret_cast<uint4*>(row) = hi.q;
       *reinterpret_cast<uint4*>(row + NP * 128) = lo.q;
     }
   }
-  if (low) *more = 1;
+  if (low) *low_out = 1;
 }
 
-// The operand of round w > 0: the entries of the w-th range of 28 powers of two below the
-// column's largest (of the one before for a column that was left), scaled into the first, zero
-// for the others; *more as above.
+// m 2^x: exact where the result is a normal float, else infinite or about as small as it is.
+__device__ __forceinline__ float scaled(float m, int x) {
+  for (; x > 127; x -= 127) m *= 0x1p127f;
+  for (; x < -126; x += 126) m *= 0x1p-126f;
+  return m * pow2f(x);
+}
+
+// The operand of round w > 0: the entries of the w-th 28 powers of two below the column's
+// largest (and whatever is not below them, in round 1), scaled up into the first, zero for the
+// others; *low_out as above.
 __device__ __noinline__ void f16_operand_round(const F16Operand& fo, int np, int nk,
                                                unsigned char* bs, const unsigned* cmax, int round,
-                                               int* more) {
+                                               int* low_out) {
   const int t = threadIdx.x - 64, lane = t & 31;
   bool low = false;
   for (int o = t >> 5; o < nk * 8; o += 8)
     for (int n = lane; n < np; n += 32) {
-      const int e = f16_exponent(cmax[n]);
-      const int up = kF16RoundBits * (e < kF16LeaveExp ? round - 1 : round) - e;
+      const int up = kF16RoundBits * (round - 1) - f16_exponent(cmax[n]);
       float f[8], ks[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int k = 8 * o + u;
-        f[u] = k < fo.K && n < fo.q ? fo.F[(int64_t)k * fo.q + n] : 0.f;
-        ks[u] = k < fo.K ? fo.kscale[k] : 1.f;
+        const bool in = k < fo.K && n < fo.q;
+        f[u] = in ? fo.F[(int64_t)k * fo.q + n] : 0.f;
+        ks[u] = in ? fo.kscale[k] : 1.f;
       }
       union { __half h[8]; uint4 q; } hi, lo;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        // f 2^x in steps that stay within the result's magnitude and f's: exact where the
-        // result is in the range, infinite or below it otherwise.
-        int x = (__float_as_int(ks[u]) >> 23) - 127 + up;
-        float y = f[u];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const int step = max(-126, min(127, x));
-          y *= pow2f(step);
-          x -= step;
-        }
-        const float m = fabsf(y);
-        low |= f[u] != 0.f && m < kF16Least;
-        split_f16(m >= kF16Least && m < 32768.f ? y : 0.f, hi.h[u], lo.h[u]);
+        const float y = scaled(f[u], (__float_as_int(ks[u]) >> 23) - 127 + up);
+        const bool under = fabsf(y) < kF16Least;
+        low |= under && f[u] != 0.f;
+        split_f16(under || (round > 1 && !(fabsf(y) < 32768.f)) ? 0.f : y, hi.h[u], lo.h[u]);
       }
       unsigned char* row = f16_b_row(bs, np, o, n);
       *reinterpret_cast<uint4*>(row) = hi.q;
       *reinterpret_cast<uint4*>(row + np * 128) = lo.q;
     }
-  if (low && round + 1 < kF16MaxRounds) *more = 1;
+  if (low && round + 1 < kF16MaxRounds) *low_out = 1;
 }
 
 // AND of `ok` over warps 2-9 (named barrier 2).
@@ -919,7 +921,9 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
   __shared__ uint64_t full[kF16MaxStages], empty[kF16MaxStages], accfull[2], accempty[2], bready;
   __shared__ float cs[NP];
   __shared__ unsigned cmax[NP];
-  __shared__ int more[kF16MaxRounds];  // of each round of f16_operand; the last stays 0
+  // Of each round: an entry below the range (f16_operand), and another round to follow.
+  __shared__ int low[kF16MaxRounds], again[kF16MaxRounds];
+  __shared__ uint64_t decided;
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
 
@@ -941,7 +945,8 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       mbar_init(&accempty[b], 4);
     }
     mbar_init(&bready, 8);
-    for (int w = 0; w < kF16MaxRounds; ++w) more[w] = 0;
+    mbar_init(&decided, 1);
+    for (int w = 0; w < kF16MaxRounds; ++w) low[w] = again[w] = 0;
     fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -972,9 +977,9 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       int64_t it = 0;
       int s = 0;
       uint32_t ph = 1;  // the first round's stages are free
-      bool ok = true, again = true;
-      for (int round = 0; ok && again; ++round) {
-        // Whether another round follows is known when this round's operand is; asked before
+      bool ok = true, more = true;
+      for (int round = 0; ok && more; ++round) {
+        // Whether another round may follow is known when this round's operand is; asked before
         // the round's last load, so that the next operand's phase cannot end meanwhile.
         int64_t ask = my_tiles * nk - 1;
         ask = ask < nst ? ask : nst;
@@ -984,7 +989,7 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
           for (int kc = 0; kc < nk; ++kc, ++it, ++c) {
             if (c == ask) {
               ok = mbar_wait(&bready, round & 1, vfail);
-              again = ok && more[round] != 0;
+              more = ok && low[round] != 0;
             }
             if (!ok || (it >= nst && !mbar_wait(&empty[s], ph, vfail))) {
               ok = false;
@@ -1009,6 +1014,10 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
             }
           }
         }
+        if (ok && more) {
+          ok = mbar_wait(&decided, round & 1, vfail);
+          more = ok && again[round] != 0;
+        }
       }
       if (!ok) {
         // Let the copies this CTA started land before it can exit (bounded).
@@ -1029,10 +1038,10 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       int gcount = 0, rs = 0;  // groups of stages; the ring's stage
       const int group = f16_group(nk);
       uint32_t rph = 0;
-      bool ok = true, again = true;
-      for (int round = 0; ok && again; ++round) {
+      bool ok = true, more = true;
+      for (int round = 0; ok && more; ++round) {
         ok = mbar_wait(&bready, round & 1, vfail);
-        again = ok && more[round] != 0;
+        more = ok && low[round] != 0;
         for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
           for (int k0 = 0; ok && k0 < nk; k0 += group, ++gcount) {
             const int buf = gcount & 1, kend = min(nk, k0 + group);
@@ -1071,6 +1080,10 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
             if (ok) mma_commit(&accfull[buf]);
           }
         }
+        if (ok && more) {
+          ok = mbar_wait(&decided, round & 1, vfail);
+          more = ok && again[round] != 0;
+        }
       }
     }
   } else {
@@ -1078,8 +1091,12 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
     pdl_wait();
     int gcount = 0;
     // ---- epilogue of a round (warps 2-5); false: a wait gave up ------------------------
-    auto epilogue = [&](auto first, int round) -> bool {
-      constexpr bool kFirst = decltype(first)::value;
+    bool starved = false;  // an output of the round's tiles is too small for what it lacks
+    auto epilogue = [&](auto first, auto asked, int round) -> bool {
+      constexpr bool kFirst = decltype(first)::value, kAsk = decltype(asked)::value;
+      // The least output that needs none of what its round leaves out (see above): of the low
+      // entries in round 0, of those of the ranges to come after it.
+      const float enough = round == 0 ? 8.f * fo.K : 0x1p24f * fo.K;
       bool got = true;
       const int quarter = warp & 3;
       const int lr = quarter * 32 + lane;
@@ -1137,21 +1154,30 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
           float* v = sum + c0;
           // Powers of two: the column's first (its result is the entry without the
           // row's scale), then the row's.
+          const double down = kFirst ? 0.0 : ldexp((double)rsc, -kF16RoundBits * (round - 1));
           if constexpr (kFirst) {
+            if (kAsk && live) {
+#pragma unroll
+              for (int t = 0; t < 32; ++t) starved |= c0 + t < ep.q && fabsf(v[t]) < enough;
+            }
 #pragma unroll
             for (int t = 0; t < 32; ++t) v[t] = v[t] * cs[c0 + t] * rsc;
           } else {
-            const double down = ldexp((double)rsc, -kF16RoundBits * round);
 #pragma unroll
             for (int t = 0; t < 32; ++t) v[t] = (float)((double)v[t] * cs[c0 + t] * down);
           }
+          // A later round adds to what is there.
+          auto add = [&](float* z, int t) {
+            *z += v[t];
+            starved |= kAsk && fabsf(*z) < (double)enough * cs[c0 + t] * down;
+          };
           if (ep.p1_layout != 1) {
             if (orow >= 0) {
               float* o = ep.out + orow * ep.q;
               if constexpr (!kFirst) {
 #pragma unroll
                 for (int t = 0; t < 32; ++t)
-                  if (c0 + t < ep.q) o[c0 + t] += v[t];
+                  if (c0 + t < ep.q) add(o + c0 + t, t);
               } else if ((ep.q & 3) == 0) {
 #pragma unroll
                 for (int t = 0; t < 32; t += 4)
@@ -1180,7 +1206,8 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
             for (int t = 0; t < 32; ++t)
               if (c0 + t < ep.q) {
                 float* z = o + static_cast<int64_t>(c0 + t) * ep.slab;
-                *z = kFirst ? v[t] : *z + v[t];
+                if constexpr (kFirst) *z = v[t];
+                else add(z, t);
               }
           }
         }
@@ -1188,29 +1215,39 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
       }
       return got;
     };
-    // Whether another round follows (in all of warps 2-9 alike). Every MMA of the round is
-    // done: warps 2-5 have read its last accumulators.
-    auto round_done = [&](bool got, int round) -> bool {
-      return all_of_256(got && *vfail == 0) && more[round] != 0;
+    // Whether another round follows (in all of warps 2-9 alike; the other roles are told). Every
+    // MMA of the round is done: warps 2-5 have read its last accumulators.
+    auto next_round = [&](bool got, int round) -> bool {
+      if (low[round] == 0) return false;
+      if (!all_of_256(got && *vfail == 0)) return false;  // the other roles stop at their waits
+      const bool more = !all_of_256(!starved);
+      if (threadIdx.x == 64) {
+        again[round] = more ? 1 : 0;
+        mbar_arrive(&decided);
+      }
+      starved = false;
+      return more;
     };
     auto operand_done = [&]() {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&bready);
-      asm volatile("bar.sync 2, 256;" ::: "memory");  // cs and more[round] complete
+      asm volatile("bar.sync 2, 256;" ::: "memory");  // cs and low[round] complete
     };
-    f16_operand<NP>(fo, nk, bs, cs, cmax, more);
+    f16_operand<NP>(fo, nk, bs, cs, cmax, low);
     operand_done();
     bool got = true;
-    if (warp < 6) got = epilogue(std::true_type{}, 0);
+    const auto yes = std::true_type{};
+    const auto no = std::false_type{};
+    if (warp < 6) got = low[0] == 0 ? epilogue(yes, no, 0) : epilogue(yes, yes, 0);
     int round = 0;
-    while (round_done(got, round)) {
+    while (next_round(got, round)) {
       ++round;
-      f16_operand_round(fo, NP, nk, bs, cmax, round, more + round);
+      f16_operand_round(fo, NP, nk, bs, cmax, round, low + round);
       operand_done();
-      if (warp < 6) got = epilogue(std::false_type{}, round);
+      if (warp < 6) got = round == 1 ? epilogue(yes, yes, 1) : epilogue(no, yes, round);
     }
-    if (threadIdx.x == 64 && blockIdx.x == 0 && round > 0) atomicAdd(err + kFlagRounds, round);
+    if (threadIdx.x == 64 && round > 0) atomicAdd(err + kFlagRounds, round);
   }
 
   tc_fence_before();
@@ -1989,29 +2026,70 @@ int TcPlan::wide(cudaStream_t s, bool* w) const {
   return NNC_OK;
 }
 
-int PairGuard::start(const TcPlan* p, Scratch& sc) {
-  NNC_TRY(sc.get(&seen, kFlags));
+// Page-locked words for the looks, one slot a fit: a copy to them and a wait for an event take no
+// lock that other threads' launches wait for, as a copy to pageable memory does.
+namespace {
+constexpr int kSlots = 64;
+std::mutex g_slot_mu;
+int* g_slots = nullptr;  // kSlots x kFlags, allocated by the first fit that looks
+bool g_slot_used[kSlots];
+int* take_slot() {
+  std::lock_guard<std::mutex> lk(g_slot_mu);
+  if (g_slots == nullptr &&
+      cudaHostAlloc(reinterpret_cast<void**>(&g_slots), kSlots * kFlags * sizeof(int),
+                    cudaHostAllocPortable) != cudaSuccess) {
+    (void)cudaGetLastError();
+    g_slots = nullptr;
+    return nullptr;
+  }
+  for (int k = 0; k < kSlots; ++k)
+    if (!g_slot_used[k]) {
+      g_slot_used[k] = true;
+      return g_slots + k * kFlags;
+    }
+  return nullptr;
+}
+void give_slot(int* p) {
+  std::lock_guard<std::mutex> lk(g_slot_mu);
+  g_slot_used[(p - g_slots) / kFlags] = false;
+}
+}  // namespace
+
+int PairGuard::start(const TcPlan* p, int first) {
+  slot = take_slot();
+  if (slot == nullptr) return NNC_OK;  // more fits at once than slots: this one does not look
   NNC_CUDA_TRY(cudaEventCreateWithFlags(&at, cudaEventDisableTiming));
   plan = p;
+  next = first;
   return NNC_OK;
 }
 
-int PairGuard::mark(cudaStream_t cs, int sweeps) {
-  NNC_CUDA_TRY(cudaMemcpyAsync(seen, plan->err, kFlags * sizeof(int), cudaMemcpyDeviceToDevice, cs));
-  NNC_CUDA_TRY(cudaEventRecord(at, cs));
-  marked = sweeps;
-  return NNC_OK;
+PairGuard::~PairGuard() {
+  if (at) {
+    // (a copy to the slot may be under way when a call ends early)
+    if (pending) cudaEventSynchronize(at);
+    cudaEventDestroy(at);
+  }
+  if (slot) give_slot(slot);
 }
 
-int PairGuard::look(cudaStream_t s) {
-  int h[kFlags] = {};
-  NNC_CUDA_TRY(cudaStreamWaitEvent(s, at, 0));
-  NNC_CUDA_TRY(cudaMemcpyAsync(h, seen, sizeof(h), cudaMemcpyDeviceToHost, s));
-  NNC_CUDA_TRY(cudaStreamSynchronize(s));
-  slow = 4 * (h[kFlagRounds] - rounds) > 2 * (marked - looked);
-  rounds = h[kFlagRounds];
-  looked = marked;
-  return timed_out(h[0]);
+int PairGuard::step(cudaStream_t cs, int t) {
+  if (slot == nullptr) return NNC_OK;
+  if (!pending && t >= next) {
+    NNC_CUDA_TRY(cudaMemcpyAsync(slot, plan->err, kFlags * sizeof(int), cudaMemcpyDeviceToHost, cs));
+    NNC_CUDA_TRY(cudaEventRecord(at, cs));
+    marked = t;
+    pending = true;
+  } else if (pending && t > marked) {
+    NNC_CUDA_TRY(cudaEventSynchronize(at));
+    pending = false;
+    slow = 4LL * (slot[kFlagRounds] - rounds) > 2LL * (marked - looked);
+    rounds = slot[kFlagRounds];
+    looked = marked;
+    next = t + (t > 80 ? t / 4 : 20);
+    return timed_out(slot[0]);
+  }
+  return NNC_OK;
 }
 
 int TcPlan::check(cudaStream_t s) const {

@@ -15,7 +15,7 @@ constexpr int kKindTf32x3 = 1;
 constexpr int kKindF16x3 = 2;
 
 // The device words of a plan (TcPlan::err): a pipeline wait timed out; F16x3 only: an entry of X
-// lies outside the range of a pair; rounds that passes took beyond the first (tc_ttm.cu).
+// lies outside the range of a pair; rounds that CTAs of passes took beyond the first (tc_ttm.cu).
 constexpr int kFlagWideX = 1, kFlagRounds = 2, kFlags = 3;
 
 // Where and how the epilogue writes one pass's FP32 result.
@@ -125,30 +125,29 @@ struct TcPlan {
   int check(cudaStream_t s) const;
 };
 
-// Watches a fit whose passes read FP16 pairs: once more than every fourth pass since the last
-// look took another round for wide factors (at 512^3 a round takes 100-120 us, a TF32x3 pass 140), the
-// fit does better with TF32x3 passes. The host looks every kPairLook sweeps, and once the next
-// ones are queued, so that the device does not wait for it; what it sees is as of the mark, so
-// it depends on the data alone.
-constexpr int kPairLook = 20;
+// Watches a fit whose passes read FP16 pairs: once some CTA took another round for wide factors
+// in every fourth pass (as far as the sum of rounds says) since the last look, the fit does
+// better with TF32x3 passes (at 512^3 a round takes 100-120 us, a TF32x3 pass 140). A look is of
+// the first sweeps, then of 20 more, then of a quarter of those done; it comes once the next sweeps
+// are queued, so that the device does not wait; what it sees is as of its mark, so it depends
+// on the data alone.
 struct PairGuard {
   bool slow = false;  // at the last look
   PairGuard() = default;
   PairGuard(const PairGuard&) = delete;
   PairGuard& operator=(const PairGuard&) = delete;
-  ~PairGuard() {
-    if (at) cudaEventDestroy(at);
-  }
-  int start(const TcPlan* p, Scratch& sc);
-  // The device's words after the work queued so far on `cs`, `sweeps` sweeps (mark), and what
-  // they say (look, in the order of `s`, which it synchronises; NNC_ERR_TIMEOUT as TcPlan::check).
-  int mark(cudaStream_t cs, int sweeps);
-  int look(cudaStream_t s);
+  ~PairGuard();
+  // The first look is of `first` sweeps.
+  int start(const TcPlan* p, int first);
+  // After every launch on `cs`, with `t` sweeps queued: marks, or looks, when that is due
+  // (NNC_ERR_TIMEOUT as TcPlan::check).
+  int step(cudaStream_t cs, int t);
 
  private:
   const TcPlan* plan = nullptr;
-  int marked = 0, looked = 0, rounds = 0;
-  int* seen = nullptr;
+  int next = 0, marked = 0, looked = 0, rounds = 0;
+  bool pending = false;
+  int* slot = nullptr;
   cudaEvent_t at = nullptr;
 };
 

@@ -361,6 +361,24 @@ def test_pair_range_lifted_gradient():
     np.testing.assert_allclose(gF[0].cpu().numpy()[b[0] > 0], gFo[0][b[0] > 0], rtol=1e-4)
 
 
+# The same through the other pass, with slices and columns so small that the products of the two
+# scales leave the normal floats: such a column is left whole for the second round.
+def test_pair_range_small_columns():
+    dims, m, r = (48, 40, 68), (9, 10, 11), 5
+    X, b, rng = _three_blocks(dims, 79)
+    X = _f32(X * 1e-15)
+    F = [1 - rng.random((n, k)) for n, k in zip(dims, m)]
+    B = [_f32(1 - rng.random((k, r))) for k in m]
+    F[2][b[2] > 0] = 0.0
+    F[0] *= 10.0 ** (-6 - 6 * b[0])[:, None]
+    F = [_f32(f) for f in F]
+    _, gF, _ = native.candelinc_lifted_grad(_dev(X, torch.float32),
+                                            [_dev(f, torch.float32) for f in F],
+                                            [_dev(v, torch.float32) for v in B])
+    gFo, _ = orc.lifted_loss_grad(X, F, B)
+    np.testing.assert_allclose(gF[2].cpu().numpy()[b[2] > 0], gFo[2][b[2] > 0], rtol=1e-4)
+
+
 # The pairs are left after the first step (an X of wide range), and every step counts once: four
 # steps have the bits of twice two.
 @pytest.mark.parametrize("dims", [(48, 40, 68), (12, 10, 9, 16)])
@@ -472,3 +490,20 @@ def test_cluster_core_fits_at_the_shared_memory_limit(dt, m, r):
     for a, b in zip(B, Bo):
         np.testing.assert_allclose(a.double().cpu().numpy(), b, rtol=tol, atol=tol * 1e-3)
     assert err == pytest.approx(tro[-1], abs=tol)
+
+
+# Wide factors beside data without small entries: every sum has terms of the column's largest
+# entry, and no more rounds are taken. Bounds as above.
+@pytest.mark.parametrize("dims,m", [((48, 40, 68), (9, 10, 11)), ((24, 128, 72), (9, 20, 32)),
+                                    ((12, 10, 14, 36), (9, 10, 11, 12))])
+def test_pair_range_wide_factors_beside_dense_data(dims, m):
+    rng = np.random.default_rng(73)
+    X = _f32(0.25 + rng.random(dims))
+    F0 = [_f32((1 - rng.random((n, k))) * 10.0 ** rng.uniform(-30, 0, (n, 1)))
+          for n, k in zip(dims, m)]
+    G0 = _f32(1 - rng.random(m))
+    F, G = [_dev(f, torch.float32) for f in F0], _dev(G0, torch.float32)
+    native.ntd_fit(_dev(X, torch.float32), F, G, 1)
+    Fo, Go, _ = orc.ntd_fit(X, F0, G0, 1)
+    for a, b in zip(F + [G], list(Fo) + [Go]):  # (FP32 ends at 1e-38)
+        np.testing.assert_allclose(a.cpu().numpy(), b, rtol=1e-4, atol=1e-30)
