@@ -56,7 +56,7 @@ typedef enum {
                           per slice, or into two TF32 parts; FP32
                           accumulation). Either way a sum is as exact as with
                           22 bits of every entry: an X with nonzero entries
-                          more than 28 powers of two below the largest of
+                          more than 32 powers of two below the largest of
                           their slices runs with TF32 parts; for sums without
                           larger terms, smaller factor entries take further
                           rounds of a pass, and a fit with many such rounds

@@ -697,8 +697,12 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // Range: a pair holds 22 bits and a sign, as the TF32 pair does, from 2^-13 up (x_lo's
 // factor takes it out of the subnormals: without it only from 2^-1), 28 powers of two
 // below the largest entry; zeros are exact. The TF32 pair holds them at every magnitude. An X
-// with a nonzero entry below that range is flagged by x_to_pair_kernel, and the fit starts again
-// with TF32x3 passes. Factor entries below it (updates drive entries to zero) matter to an output
+// with a nonzero entry below 2^-18 is flagged by x_to_pair_kernel and runs with TF32x3 passes: down
+// to there a pair loses a bit per power of two and is off by at most 2^-18 of the entry, no more
+// than the truncating sums (over random tensors in blocks, with entries of X down to 2^-32 and rows
+// of F down to 2^-66, the largest error of an entry of F from 64 bits after one to three
+// sweeps is on average 0.85 times that of TF32x3 passes), and uniform 32-bit random numbers stay above
+// it. Factor entries below the range (updates drive entries to zero) matter to an output
 // that has no larger terms, as in a block of X of its own. What the products make of them is
 // off by less than 2^-20 in the scales' units a term (the pair's 2^-36 of an entry of F times 2^15
 // of X, the product of two low parts, which is not formed, and the tensor core's alignment of
@@ -774,7 +778,7 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 
 // v = hi + lo / kF16LoScale; 22 bits for |v| in [kF16Least, 2^15).
 constexpr float kF16LoScale = 2048.f;
-constexpr float kF16Least = 1.f / 8192.f;
+constexpr float kF16Least = 0x1p-13f, kF16LeastX = 0x1p-18f;
 __device__ __forceinline__ void split_f16(float v, __half& hi, __half& lo) {
   hi = __float2half_rn(v);
   lo = __float2half_rn((v - __half2float(hi)) * kF16LoScale);
@@ -1384,8 +1388,8 @@ __global__ void slice_u_kernel(const unsigned* __restrict__ umax, int N3, int n3
 }
 
 // Xh, Xl (rows of n3p entries, zero past N3) from X: eight entries a thread, tx threads
-// (a power of two) a row, one division per row. *wide gets 1 when the pair of a nonzero entry
-// holds less than 22 bits.
+// (a power of two) a row, one division per row. *wide gets 1 when a nonzero entry lies below
+// kF16LeastX.
 __global__ void __launch_bounds__(256)
 x_to_pair_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int n3p, int tx,
                  const float* __restrict__ s, const float* __restrict__ t,
@@ -1412,7 +1416,7 @@ x_to_pair_kernel(const float* __restrict__ X, int64_t R, int N2, int N3, int n3p
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const float y = v[q] * inv * (1.f / u[k + q]);
-        low |= v[q] != 0.f && fabsf(y) < kF16Least;
+        low |= v[q] != 0.f && fabsf(y) < kF16LeastX;
         split_f16(y, hi.h[q], lo.h[q]);
       }
       *reinterpret_cast<uint4*>(Xh + r * n3p + k) = hi.q;
