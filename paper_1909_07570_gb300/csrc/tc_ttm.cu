@@ -717,8 +717,8 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // three) and no role of it bounds it alone, 137-151 us a pass at 512^3, m = 32. A pair
 // is as large as the FP32 entry, comes in by TMA and goes out by the MMAs, at half the
 // bytes. Both passes read the same copy: pass 1 K-major, pass 2 MN-major (no
-// transposed copy). 512^3, m = 32: 137 -> 122 us (pass 1, with its shares) and
-// 141 -> 98 us (pass 2) for 537 MB, 4.4 and 5.5 TB/s; 256^3, m = 20, where the pair (67 MB)
+// transposed copy). 512^3, m = 32: 137 -> 124 us (pass 1, with its shares) and
+// 141 -> 97 us (pass 2) for 537 MB, 4.3 and 5.5 TB/s; 256^3, m = 20, where the pair (67 MB)
 // stays in L2 from pass to pass: 27 -> 20-23 us in the sweep.
 //
 // Warps 0 and 1 as in tc_pass_kernel, warps 2-5 the epilogue. B stays in shared
