@@ -446,21 +446,18 @@ int setup(Work<T>& w, const T* X, int d, const int64_t* dims, const int* m, int 
   return NNC_OK;
 }
 
-// TF32x3 passes where the FP16 pairs do not hold X (*left). Otherwise, with a guard given, that
-// of the fit's sweeps in *use (NULL: no pairs).
+// TF32x3 passes where the FP16 pairs do not hold X; otherwise the guard of the fit's sweeps in
+// *use (NULL: no pairs).
 template <typename T>
-int settle_pairs(Work<T>& w, bool* left, Scratch& sc, cudaStream_t s, tc::PairGuard* guard = nullptr,
-                 tc::PairGuard** use = nullptr) {
-  *left = false;
-  if (use) *use = nullptr;
+int settle_pairs(Work<T>& w, tc::PairGuard* guard, tc::PairGuard** use, Scratch& sc, cudaStream_t s) {
+  *use = nullptr;
   if constexpr (std::is_same<T, float>::value) {
-    if (!w.tc) return NNC_OK;
-    NNC_TRY(w.plan.wide(s, left));
-    if (*left) return w.plan.to_tf32(w.X, sc, s);
-    if (guard && w.plan.kind == tc::kKindF16x3) {
-      NNC_TRY(guard->start(&w.plan, 1));
-      *use = guard;
-    }
+    if (!w.tc || w.plan.kind != tc::kKindF16x3) return NNC_OK;
+    bool wide = false;
+    NNC_TRY(guard->start(&w.plan, 1, s));
+    NNC_TRY(guard->wide(s, &wide));
+    if (wide) return w.plan.to_tf32(w.X, sc, s);
+    *use = guard;
   }
   return NNC_OK;
 }
@@ -699,9 +696,10 @@ int loss_into(Work<T>& w, int n, double* out, double* trace, int* counter, cudaS
 }
 
 template <typename T>
-int check_tc(Work<T>& w, cudaStream_t s) {
+int check_tc(Work<T>& w, cudaStream_t s, bool* wide = nullptr) {
+  if (wide) *wide = false;
   if constexpr (std::is_same<T, float>::value) {
-    if (w.tc) return w.plan.check(s);
+    if (w.tc) return w.plan.check(s, wide);
   }
   NNC_CUDA_TRY(cudaStreamSynchronize(s));
   return NNC_OK;
@@ -736,14 +734,18 @@ int lifted_grad(const T* X, int d, const int64_t* dims, const int* m, int r, boo
       NNC_CUDA_TRY(small_gemm<T>((int)dims[n], mn, r, w.gA, r, 1, B[n], 1, r, nullptr, gF[n], s));
       NNC_CUDA_TRY(small_gemm<T>(mn, r, (int)dims[n], F[n], 1, mn, w.gA, r, 1, nullptr, gB[n], s));
     }
-    return check_tc(w, s);
+    return NNC_OK;
   };
+  // (The range of X is asked afterwards, so that the device need not wait for the host between its
+  // setup and its many small launches.)
+  bool wide = false;
   NNC_TRY(evaluate());
-  // (asked afterwards, so that the device need not wait for the host between its setup and its
-  // many small launches)
-  bool left = false;
-  NNC_TRY(settle_pairs(w, &left, sc, s));
-  if (left) NNC_TRY(evaluate());
+  NNC_TRY(check_tc(w, s, &wide));
+  if (wide) {
+    NNC_TRY(leave_pairs(w, sc, s));
+    NNC_TRY(evaluate());
+    NNC_TRY(check_tc(w, s));
+  }
   if (loss) {
     NNC_CUDA_TRY(cudaMemcpyAsync(loss, dloss, sizeof(double), cudaMemcpyDeviceToHost, s));
     NNC_CUDA_TRY(cudaStreamSynchronize(s));
@@ -960,8 +962,7 @@ int lifted_pg_fit(const T* X, int d, const int64_t* dims, const int* m, int r, b
       return check_tc(w, s);
     };
     tc::PairGuard guard, *use = nullptr;
-    bool left = false;
-    NNC_TRY(settle_pairs(w, &left, sc, s, &guard, &use));
+    NNC_TRY(settle_pairs(w, &guard, &use, sc, s));
     NNC_TRY(run(steps, use));
     if (done < steps) {
       NNC_TRY(leave_pairs(w, sc, s));
@@ -1044,8 +1045,7 @@ int nncp_tensor_fit(const T* X, int d, const int64_t* dims, int r, bool tensor_c
   };
   if (iters > 0) {
     tc::PairGuard guard, *use = nullptr;
-    bool left = false;
-    NNC_TRY(settle_pairs(w, &left, sc, s, &guard, &use));
+    NNC_TRY(settle_pairs(w, &guard, &use, sc, s));
     NNC_TRY(run(iters, use));
     if (done < iters) {
       NNC_TRY(leave_pairs(w, sc, s));
@@ -1282,8 +1282,7 @@ int ntd_fit_nway(const T* X, int d, const int64_t* dims, const int* m, bool tens
   };
   if (iters > 0) {
     tc::PairGuard guard, *use = nullptr;
-    bool left = false;
-    NNC_TRY(settle_pairs(w, &left, sc, s, &guard, &use));
+    NNC_TRY(settle_pairs(w, &guard, &use, sc, s));
     NNC_TRY(run(iters, use));
     if (done < iters) {
       NNC_TRY(leave_pairs(w, sc, s));

@@ -597,6 +597,7 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
   tc::TcPlan plan16, plan32;
   const tc::TcPlan* fast = nullptr;   // the first iters - refine sweeps
   const tc::TcPlan* exact = nullptr;  // FP32-accurate sweeps
+  tc::PairGuard guard;                // of those with FP16 pairs
   // The refinement trigger may end the fast sweeps early (exact checkpoints needed).
   const bool trigger = passes == 2 && o->refine_tol > 0.0 && o->exact_every > 0 && trace;
   if constexpr (std::is_same<T, float>::value) {
@@ -615,11 +616,13 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
       // The FP16 pair passes stream X fast enough that the side kernels would be the
       // longer branch on the few SMs a full grid leaves: 512^3, m = 32, SMs left 0, 8,
       // 16, 24, 32, 40: 265, 258, 250, 248, 253, 259 us per sweep; 256^3, m = 20
-      // (3.4 tiles per SM): 73.6 up to 24, 71.2 at 32 and 40.
+      // (3.4 tiles per SM): 73.6 up to 24, 71.2 at 32 and 40 (the check of the factors' range
+      // has added 1 to 3 us to all of them).
       if (plan32.kind == tc::kKindF16x3)
         plan32.reserve_sms = N1 * N2 >= 128 * 8LL * device_sm_count() ? 24 : 32;
       if (st == NNC_OK) exact = &plan32;
       else if (st != NNC_ERR_UNSUPPORTED) return st;
+      if (exact && exact->kind == tc::kKindF16x3) NNC_TRY(guard.start(exact, kSweepsPerGraph, s));
     }
   }
   const int n_fast_max = fast ? o->iters - o->refine_iters : 0;
@@ -694,11 +697,10 @@ int ntd_fit3_impl(const T* X, const int64_t* dims, const int* m, const nnc_opts*
         return exact->convert_b3(F[2], s);
       };
       bool wide = false;
-      if (exact) NNC_TRY(exact->wide(s, &wide));
+      const bool pair = exact && exact->kind == tc::kKindF16x3;
+      if (pair) NNC_TRY(guard.wide(s, &wide));
       if (wide) NNC_TRY(leave_pairs());
-      if (exact && exact->kind == tc::kKindF16x3) {
-        tc::PairGuard guard;
-        NNC_TRY(guard.start(exact, kSweepsPerGraph));
+      if (pair && !wide) {
         int n = 0;
         NNC_TRY(run_sweeps<T>(X, F, G, b, o->eps, trace, o->iters - at, at, &ck, exact, s, &n,
                               &guard));

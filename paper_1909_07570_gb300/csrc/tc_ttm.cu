@@ -2020,16 +2020,6 @@ int timed_out(int flag) {
 }
 }  // namespace
 
-int TcPlan::wide(cudaStream_t s, bool* w) const {
-  int h = 0;
-  *w = false;
-  if (kind != kKindF16x3) return NNC_OK;
-  NNC_CUDA_TRY(cudaMemcpyAsync(&h, err + kFlagWideX, sizeof(int), cudaMemcpyDeviceToHost, s));
-  NNC_CUDA_TRY(cudaStreamSynchronize(s));
-  *w = h != 0;
-  return NNC_OK;
-}
-
 // Page-locked words for the looks, one slot a fit: a copy to them and a wait for an event take no
 // lock that other threads' launches wait for, as a copy to pageable memory does.
 namespace {
@@ -2059,12 +2049,23 @@ void give_slot(int* p) {
 }
 }  // namespace
 
-int PairGuard::start(const TcPlan* p, int first) {
+int PairGuard::start(const TcPlan* p, int first, cudaStream_t s) {
+  plan = p;
+  next = first;
   slot = take_slot();
   if (slot == nullptr) return NNC_OK;  // more fits at once than slots: this one does not look
   NNC_CUDA_TRY(cudaEventCreateWithFlags(&at, cudaEventDisableTiming));
-  plan = p;
-  next = first;
+  NNC_CUDA_TRY(cudaMemcpyAsync(slot, plan->err, kFlags * sizeof(int), cudaMemcpyDeviceToHost, s));
+  NNC_CUDA_TRY(cudaEventRecord(at, s));
+  pending = true;
+  return NNC_OK;
+}
+
+int PairGuard::wide(cudaStream_t s, bool* w) {
+  if (slot == nullptr) return plan->check(s, w);
+  NNC_CUDA_TRY(cudaEventSynchronize(at));
+  pending = false;
+  *w = slot[kFlagWideX] != 0;
   return NNC_OK;
 }
 
@@ -2096,11 +2097,13 @@ int PairGuard::step(cudaStream_t cs, int t) {
   return NNC_OK;
 }
 
-int TcPlan::check(cudaStream_t s) const {
-  int h = 0;
-  NNC_CUDA_TRY(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+int TcPlan::check(cudaStream_t s, bool* wide) const {
+  const bool pair = wide != nullptr && kind == kKindF16x3;
+  int h[kFlags] = {};
+  NNC_CUDA_TRY(cudaMemcpyAsync(h, err, (pair ? kFlags : 1) * sizeof(int), cudaMemcpyDeviceToHost, s));
   NNC_CUDA_TRY(cudaStreamSynchronize(s));
-  return timed_out(h);
+  if (wide) *wide = pair && h[kFlagWideX] != 0;
+  return timed_out(h[0]);
 }
 
 }  // namespace tc

@@ -96,11 +96,10 @@ struct TcPlan {
            Scratch& sc, cudaStream_t s, bool p1_kj = false, bool need_p1 = true);
   // FP32-accurate passes that a fit runs again and again: F16x3 where the shape
   // allows it, else TF32x3. Whether the values of X allow it the device knows after init
-  // (`wide`: an entry outside the range of a pair, whose results are then not FP32-accurate;
-  // synchronises s): the caller then turns the plan into the TF32x3 one.
+  // (PairGuard::wide, check: an entry outside the range of a pair, whose results are then
+  // not FP32-accurate): the caller then turns the plan into the TF32x3 one.
   int init_fp32(const float* X, int64_t N1, int64_t N2, int64_t N3, int m1, int m3, Scratch& sc,
                 cudaStream_t s, bool p1_kj = false);
-  int wide(cudaStream_t s, bool* w) const;
   // An F16x3 plan becomes the TF32x3 plan of the same tensor; no work that reads the pair
   // is in flight but on `s`.
   int to_tf32(const float* X, Scratch& sc, cudaStream_t s);
@@ -122,7 +121,8 @@ struct TcPlan {
             const float* F2 = nullptr, int m2 = 0, float* Y3 = nullptr) const;
   bool y3_fusable(int m2) const;
   // Synchronises s and turns a device-side pipeline time-out into NNC_ERR_TIMEOUT.
-  int check(cudaStream_t s) const;
+  // *wide (F16x3): X has an entry outside the pairs' range.
+  int check(cudaStream_t s, bool* wide = nullptr) const;
 };
 
 // Watches a fit whose passes read FP16 pairs: once some CTA took another round for wide factors
@@ -137,8 +137,10 @@ struct PairGuard {
   PairGuard(const PairGuard&) = delete;
   PairGuard& operator=(const PairGuard&) = delete;
   ~PairGuard();
-  // The first look is of `first` sweeps.
-  int start(const TcPlan* p, int first);
+  // Right after the plan's init on `s`; the first look is of `first` sweeps.
+  int start(const TcPlan* p, int first, cudaStream_t s);
+  // Whether X has an entry outside the pairs' range (waits for the init alone).
+  int wide(cudaStream_t s, bool* w);
   // After every launch on `cs`, with `t` sweeps queued: marks, or looks, when that is due
   // (NNC_ERR_TIMEOUT as TcPlan::check).
   int step(cudaStream_t cs, int t);
