@@ -1161,8 +1161,16 @@ f16_pass_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant_
           const double down = kFirst ? 0.0 : ldexp((double)rsc, -kF16RoundBits * (round - 1));
           if constexpr (kFirst) {
             if (kAsk && live) {
+              float least = INFINITY;
+              if (c0 + 32 <= ep.q) {
 #pragma unroll
-              for (int t = 0; t < 32; ++t) starved |= c0 + t < ep.q && fabsf(v[t]) < enough;
+                for (int t = 0; t < 32; ++t) least = fminf(least, fabsf(v[t]));
+              } else {
+#pragma unroll
+                for (int t = 0; t < 32; ++t)
+                  if (c0 + t < ep.q) least = fminf(least, fabsf(v[t]));
+              }
+              starved |= least < enough;
             }
 #pragma unroll
             for (int t = 0; t < 32; ++t) v[t] = v[t] * cs[c0 + t] * rsc;
@@ -2029,12 +2037,18 @@ int* g_slots = nullptr;  // kSlots x kFlags, allocated by the first fit that loo
 bool g_slot_used[kSlots];
 int* take_slot() {
   std::lock_guard<std::mutex> lk(g_slot_mu);
-  if (g_slots == nullptr &&
-      cudaHostAlloc(reinterpret_cast<void**>(&g_slots), kSlots * kFlags * sizeof(int),
-                    cudaHostAllocPortable) != cudaSuccess) {
-    (void)cudaGetLastError();
-    g_slots = nullptr;
-    return nullptr;
+  if (g_slots == nullptr) {
+    // (relaxed: the allocation must not break a capture of another thread)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&g_slots),
+                                        kSlots * kFlags * sizeof(int), cudaHostAllocPortable);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+      (void)cudaGetLastError();
+      g_slots = nullptr;
+      return nullptr;
+    }
   }
   for (int k = 0; k < kSlots; ++k)
     if (!g_slot_used[k]) {
